@@ -5,26 +5,32 @@
 // 128-key tiles through a ring of 128B-swizzled shared-memory slots (K and V tiles alternate in the
 // ring; eight 16-token pages per tile, fetched page by page with TMA through the block table).
 //
-// Warp roles (384 threads, three warpgroups):
-//   warp 0        TMA producer for the K tiles (warp 3 for the V tiles): runs ahead across unit boundaries, limited only
-//                 by the ring
-//   warp 1        MMA issuer (one lane): S = Q K^T into TMEM, then O += P V with P read from TMEM;
-//                 owns the TMEM allocation (S0, S1, O0, O1: 4 x 128 columns)
-//   warp 2        TMA loader for the query tiles of each unit; in launches where every unit has one row tile it also issues
-//                 S = Q K^T, and warp 1 only O += P V (two issuing threads, see two_issuers below)
-//   warp 3        writes the zero rows of padding nodes (node >= n_nodes), then TMA producer for the V tiles
-//   warps 4..7    softmax warpgroup 0, warps 8..11 softmax warpgroup 1: one thread per query row; S from
-//                 TMEM to registers, fp32 online softmax in the log2 domain with lazy rescaling of O,
-//                 P written back to TMEM as packed bf16 over S; epilogue of the unit
-// A unit with two valid row tiles gives one to each softmax warpgroup (both consume every key tile, so
-// the tensor pipe works on one tile's MMAs while the other tile is in softmax).  A unit with one valid
-// row tile is handled by warpgroup 0 alone with S double-buffered over S0/S1.
+// What bounds it is the chain of a score tile, S = Q K^T -> softmax -> O += P V -> next S (P overlays S in TMEM, so the next S
+// follows the product that reads P), against 1,024 cycles of tensor work (16 products of 64 cycles) and 1,024 of the exponential
+// unit per 128 x 128 tile.  Two chains run side by side so that one is in the tensor pipe while the other is in softmax; each
+// has an S/P buffer, an accumulator and a pair of softmax warpgroups of its own:
+//   * a unit with two row tiles gives each chain a row tile, and both walk all key tiles;
+//   * a unit with one row tile deals its key tiles to the two chains in turn; every chain keeps its own reference maximum and
+//     accumulator and the two are put together at the end of the unit.
+// A row's 128 scores are split over two threads (64 each): one warp per scheduler and chain left half of the issue slots empty
+// (2.1 k cycles a tile with a row per thread, spills included).
+//
+// Warp roles (640 threads, five warpgroups):
+//   warp 0        TMA producer for the K tiles: runs ahead across unit boundaries, limited only by the ring
+//   warp 1        MMA issuer (one elected lane): O += P V of a chain, with P read from TMEM, then the chain's next S = Q K^T;
+//                 the chains take turns, so that their products do not interleave in the tensor pipe (with a thread per chain they
+//                 did: both chains ended together and then went through softmax together); owns the TMEM allocation (S0, S1, O0, O1)
+//   warp 2        publishes the units to the softmax warps and loads their query tiles
+//   warp 3        TMA producer for the V tiles
+//   warps 4..19   softmax warpgroups: 4..7 and 8..11 chain 0 (keys 0-63 and 64-127 of a tile), 12..15 and 16..19 chain 1;
+//                 fp32 online softmax in the log2 domain with lazy rescaling of O, P written back to TMEM as packed bf16 over S;
+//                 epilogue of the unit.  Before that they write the zero rows of padding nodes (node >= n_nodes).
 // All waits are bounded; a wait that runs out records CB_ERR_TIMEOUT and the CTA drains and exits.
 //
 // Cluster mode.  When a launch has so few units that the split above would make every unit a shared one (batch 1), the
 // kernel is launched as thread-block clusters instead: cluster k works on unit k, its CTAs take equal parts of the unit's
-// key tiles, and at the end they combine their shares through distributed shared memory: row block r of the 128 rows is
-// gathered in CTA r, which merges the contributions and writes the output.  No partials go to HBM and no merge pass runs.
+// key tiles, and at the end they combine their shares through distributed shared memory: row i of the 128 rows is
+// gathered in CTA i mod cs, which merges the contributions and writes the output.  No partials go to HBM and no merge pass runs.
 #include <cuda.h>
 
 #include <mutex>
@@ -32,6 +38,10 @@
 #include "cb_tc_dev.cuh"
 
 namespace {
+
+struct UnitDesc { int b, kh, rg, t0, t1, tiles, n, ctx, nrt, pad; };   // nrt = 0: no more units
+constexpr int kFmaExpPhase = 3;                              // of every four pairs of exponentials this one is taken by the FMA pipe
+constexpr int kUnitRing = 4;                                 // units published ahead of the slowest softmax thread: at most two
 
 template <int D>
 struct Cfg {
@@ -42,11 +52,14 @@ struct Cfg {
     static constexpr uint32_t OFF_Q = 0;                     // two row tiles
     static constexpr uint32_t OFF_RING = 2 * Q_BYTES;
     static constexpr uint32_t OFF_BAR = OFF_RING + NSLOT * TILE_BYTES;
-    // slot_full[NSLOT], slot_free[NSLOT], q_full, q_free, s_full0, p_ready[2], o_free[2], cluster_ready, cluster_data
-    static constexpr int NBAR = 2 * NSLOT + 2 + 7 + 2;       // ... and pv_done[2]
-    static constexpr uint32_t OFF_MISC = OFF_BAR + NBAR * 8;  // schedule, tmem base, abort flag
-    static constexpr uint32_t SMEM = OFF_MISC + 96;
-    static constexpr uint32_t SMEM_ALLOC = SMEM + 1024;      // slack to align the base to 1024 bytes
+    // slot_full[NSLOT], slot_free[NSLOT], q_full, q_free, s_full[2], p_ready[2], o_done[2], o_done_both, o_free[2], sums,
+    // unit_full[kUnitRing], cluster_ready, cluster_data
+    static constexpr int NBAR = 2 * NSLOT + 12 + kUnitRing + 2;
+    static constexpr uint32_t OFF_UNITS = OFF_BAR + NBAR * 8;
+    static constexpr uint32_t OFF_X = OFF_UNITS + kUnitRing * sizeof(UnitDesc);      // [2 chains][2][128 rows]: row sums, then reference and sum
+    static constexpr uint32_t OFF_MISC = OFF_X + 2 * 2 * CB_MT * 4;                  // schedule, tmem base, abort flag, pair counters
+    static constexpr uint32_t SMEM = OFF_MISC + 96 + 64;
+    static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
     static constexpr uint32_t O_COL = 256;                   // TMEM columns: S0 at 0, S1 at 128, O0 at 256, O1 at 256 + D
 };
 
@@ -63,28 +76,33 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
     using C = Cfg<D>;
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
+    extern __shared__ __align__(1024) uint8_t attn_smem[];
+    uint8_t* const sgen = attn_smem;
+    const uint32_t sbase = smem_u32(attn_smem);
+    if (sbase & 1023u) {                                      // the swizzled tiles need it; every thread sees the same address
+        if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)CB_ERR_UNSUPPORTED);
+        return;
+    }
     const uint32_t bar0 = sbase + C::OFF_BAR;
-    auto bar_full = [&](int s) { return bar0 + 8u * s; };
-    auto bar_free = [&](int s) { return bar0 + 8u * (C::NSLOT + s); };
+    auto bar_full = [&](uint32_t s) { return bar0 + 8u * s; };
+    auto bar_free = [&](uint32_t s) { return bar0 + 8u * (C::NSLOT + s); };
     auto slot_base = [&](uint32_t s) { return sbase + C::OFF_RING + s * C::TILE_BYTES; };
-    const uint32_t bar_qfull = bar0 + 8u * (2 * C::NSLOT), bar_qfree = bar_qfull + 8u;
-    // Completion of the tensor core's work is signalled with as few commits as possible (a second commit behind the
-    // same MMA block stalls the issuer): a ring slot's "free" barrier doubles as "the S product that read this K tile is
-    // done" and "the PV product that read this V tile is done".  Its phases are a ring revolution apart, so a softmax
-    // thread can wait on it by the slot's sequence number alone.  Only row tile 0 of a two-row-tile unit needs a
-    // barrier of its own for S, because its S is finished before the K tile is released.
-    const uint32_t bar_sfull0 = bar0 + 8u * (2 * C::NSLOT + 2);
-    auto bar_pready = [&](int s) { return bar0 + 8u * (2 * C::NSLOT + 3 + s); };
-    auto bar_ofree = [&](int s) { return bar0 + 8u * (2 * C::NSLOT + 5 + s); };
-    const uint32_t bar_cready = bar0 + 8u * (2 * C::NSLOT + 7), bar_cdata = bar_cready + 8u;   // cluster mode only
-    auto bar_pvdone = [&](int s) { return bar0 + 8u * (2 * C::NSLOT + 9 + s); };               // two issuing threads only (see below)
+    constexpr uint32_t B1 = 2 * C::NSLOT;
+    const uint32_t bar_qfull = bar0 + 8u * B1, bar_qfree = bar_qfull + 8u;
+    auto bar_sfull = [&](int l) { return bar0 + 8u * (B1 + 2 + l); };
+    auto bar_pready = [&](int l) { return bar0 + 8u * (B1 + 4 + l); };
+    auto bar_odone = [&](int l) { return bar0 + 8u * (B1 + 6 + l); };
+    const uint32_t bar_odone_both = bar0 + 8u * (B1 + 8);
+    auto bar_ofree = [&](int l) { return bar0 + 8u * (B1 + 9 + l); };
+    const uint32_t bar_sums = bar0 + 8u * (B1 + 11);
+    auto bar_ufull = [&](uint32_t k) { return bar0 + 8u * (B1 + 12 + k); };
+    const uint32_t bar_cready = bar0 + 8u * (B1 + 12 + kUnitRing), bar_cdata = bar_cready + 8u;   // cluster mode only
+    UnitDesc* s_units = reinterpret_cast<UnitDesc*>(sgen + C::OFF_UNITS);
+    volatile float* s_x = reinterpret_cast<volatile float*>(sgen + C::OFF_X);
     SchedSmem* s_sched = reinterpret_cast<SchedSmem*>(sgen + C::OFF_MISC);
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sgen + C::OFF_MISC + 64);
     volatile int* s_abort = reinterpret_cast<volatile int*>(sgen + C::OFF_MISC + 68);
-    volatile int* s_one_row = reinterpret_cast<volatile int*>(sgen + C::OFF_MISC + 72);   // every unit of the launch has one row tile
+    volatile int* s_pair = reinterpret_cast<volatile int*>(sgen + C::OFF_MISC + 96);   // [16 softmax warps]: pair barriers entered, -1 = left
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cta = blockIdx.x;
@@ -99,17 +117,20 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
     } else if (warp == 2) {
         if (lane == 0) {
             for (int s = 0; s < C::NSLOT; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_free(s), 1); }
-            mbar_init(bar_qfull, 1); mbar_init(bar_qfree, 1); mbar_init(bar_sfull0, 1);
-            for (int s = 0; s < 2; ++s) {
-                mbar_init(bar_pready(s), 256); mbar_init(bar_ofree(s), 128);
+            mbar_init(bar_qfull, 1); mbar_init(bar_qfree, 1);
+            for (int l = 0; l < 2; ++l) {
+                mbar_init(bar_sfull(l), 1); mbar_init(bar_pready(l), 256);
+                mbar_init(bar_odone(l), 1); mbar_init(bar_ofree(l), 512);
             }
-            mbar_init(bar_cready, p.cs > 0 ? (uint32_t)p.cs : 1u); mbar_init(bar_cdata, 128);
-            mbar_init(bar_pvdone(0), 1); mbar_init(bar_pvdone(1), 1);
+            mbar_init(bar_odone_both, 1); mbar_init(bar_sums, 512);
+            for (int k = 0; k < kUnitRing; ++k) mbar_init(bar_ufull(k), 1);
+            mbar_init(bar_cready, p.cs > 0 ? (uint32_t)p.cs : 1u); mbar_init(bar_cdata, 512);
             *s_abort = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             tma_prefetch_desc(&maps.k_pool); tma_prefetch_desc(&maps.v_pool); tma_prefetch_desc(&maps.q);
             tma_prefetch_desc(&maps.k_tree); tma_prefetch_desc(&maps.v_tree);
         }
+        if (lane < 16) s_pair[lane] = 0;
     }
     CB_PDL_ENTRY();
 
@@ -124,67 +145,44 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             s_sched->c_t0 = sh.RG > 0 ? (int)((long long)sh.tiles * rank / p.cs) : 0;
             s_sched->c_t1 = sh.RG > 0 ? (int)((long long)sh.tiles * (rank + 1) / p.cs) : 0;
             s_sched->g0 = 0; s_sched->g1 = 0; s_sched->pre0 = 0; s_sched->b0 = 0; s_sched->rg0 = 0;
-            *s_one_row = 1;
         }
     } else if (warp == 0) {
         // this CTA's range of the global tile sequence
-        int max_rt = 0;
-        const long long tot = cb_sched_total(p, lane, &max_rt);
+        const long long tot = cb_sched_total(p, lane);
         const long long g0 = cb_range_start(tot, p.nc, cta), g1 = cb_range_start(tot, p.nc, cta + 1);
         int b0 = 0, rg0 = 0;
         long long pre0 = 0;
         if (g0 < g1) cb_sched_locate(p, g0, lane, &rg0, &b0, &pre0);
-        if (lane == 0) {
-            s_sched->g0 = g0; s_sched->g1 = g1; s_sched->b0 = b0; s_sched->rg0 = rg0; s_sched->pre0 = pre0;
-            *s_one_row = (p.MT == 1 || max_rt <= 1) ? 1 : 0;
-        }
+        if (lane == 0) { s_sched->g0 = g0; s_sched->g1 = g1; s_sched->b0 = b0; s_sched->rg0 = rg0; s_sched->pre0 = pre0; }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
-    const long long g0 = s_sched->g0, g1 = s_sched->g1, pre0 = s_sched->pre0;
-    const int b0 = s_sched->b0, rg0 = s_sched->rg0;
-    // When no unit of the launch has two row tiles (the same for every CTA: it follows from n_nodes alone), the products of a
-    // key tile get an issuing thread each: warp 2's thread, which loads the query tile, issues S = Q K^T, warp 1's thread
-    // issues O += P V.  One thread issuing both spends about 2.0 k cycles per key tile in the two blocks and its loop, and the
-    // next S follows the P.V it has to wait for; with two threads the next S only waits for the completion of the P.V that
-    // read its buffer two tiles before, and the softmax warpgroup (1.9 k cycles per tile) is what a tile costs.
-    const bool two_issuers = *s_one_row != 0;
     constexpr uint32_t ns = (uint32_t)C::NSLOT;
-    CbWalker wk;
     if (p.cs > 0) {
         // the peers' barriers must exist before anything arrives on them
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        CbUnit u0;
-        u0.b = s_sched->c_b; u0.kh = s_sched->c_kh; u0.rg = 0; u0.t0 = s_sched->c_t0; u0.t1 = s_sched->c_t1;
-        u0.tiles = s_sched->c_tiles; u0.n = s_sched->c_n; u0.ctx = s_sched->c_ctx; u0.nrt = 1;
-        wk.init_fixed(u0);
-    } else {
-        wk.init(p, g0, g1, rg0, b0, pre0);
     }
-    CbUnit u;
 
     if (warp < 4) {
-        reg_dealloc<120>();
+        reg_dealloc<64>();
+        CbWalker wk;
+        if (p.cs > 0) {
+            CbUnit u0;
+            u0.b = s_sched->c_b; u0.kh = s_sched->c_kh; u0.rg = 0; u0.t0 = s_sched->c_t0; u0.t1 = s_sched->c_t1;
+            u0.tiles = s_sched->c_tiles; u0.n = s_sched->c_n; u0.ctx = s_sched->c_ctx; u0.nrt = 1;
+            wk.init_fixed(u0);
+        } else {
+            wk.init(p, s_sched->g0, s_sched->g1, s_sched->rg0, s_sched->b0, s_sched->pre0);
+        }
+        CbUnit u;
         if (warp == 0 || warp == 3) {
             // ------------------------------------------------------------------ K/V producers: warp 0 the K tiles, warp 3 the V tiles
             // A tile is 8 * DB boxes of 16 keys x 64 dims, one copy instruction each, and the copies of one warp instruction
             // are issued one after the other: two warps issue the two tiles of a key tile side by side.
             const bool isV = warp == 3;
-            if (isV) {
-                // rows of padding nodes (node >= n_nodes) are written as zeros: once, before the first V tile is wanted
-                const int per_row = p.Hq * D / 8;            // 16-byte chunks per node row
-                for (int idx = cta; idx < p.B * p.T; idx += gridDim.x) {
-                    const int b = idx / p.T, node = idx % p.T;
-                    const int n = min(max(p.n_nodes[b], 0), p.T);
-                    if (node < n) continue;
-                    uint4* op = reinterpret_cast<uint4*>(p.out + (size_t)idx * p.Hq * D);
-                    for (int k = lane; k < per_row; k += 32) op[k] = make_uint4(0, 0, 0, 0);
-                    if (p.lse) for (int h = lane; h < p.Hq; h += 32) p.lse[((size_t)b * p.Hq + h) * p.T + node] = 0.f;
-                }
-            }
             constexpr int NB = 8 * C::DB;                    // boxes per tile
             const bool active = lane < NB;
             const int j = lane % 8, dblk = (lane % NB) / 8;
@@ -223,149 +221,61 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             }
         } else if (warp == 1) {
             // ------------------------------------------------------------------ MMA issuer
-            if (lane == 0) {
+            if (elect_one()) {
                 constexpr uint32_t idesc_s = make_idesc(128, CB_KT, false);
                 constexpr uint32_t idesc_o = make_idesc(128, D, true);
-                uint32_t seq = 0, uq = 0, c_p[2] = {0u, 0u}, c_of[2] = {0u, 0u};
+                uint32_t seq0 = 0, uq = 0, c_p[2] = {0u, 0u};
                 bool ok = true;
-                const uint32_t q_lo0 = desc_lo(sbase + C::OFF_Q, 16), k_lo0 = desc_lo(sbase + C::OFF_RING, 16);
-                const uint32_t v_lo0 = desc_lo(sbase + C::OFF_RING, CB_KT * 128);
-                auto issue_s = [&](int rt, int buf, uint32_t kslot) {
-                    mma_s_block<D>(tmem + buf * 128, q_lo0 + rt * (C::Q_BYTES >> 4), k_lo0 + kslot * (C::TILE_BYTES >> 4), idesc_s);
-                };
-                auto issue_pv = [&](int ol, int buf, uint32_t vslot, bool accum) {
-                    mma_pv_block(tmem + C::O_COL + ol * D, tmem + buf * 128, v_lo0 + vslot * (C::TILE_BYTES >> 4), idesc_o, accum ? 1u : 0u);
-                };
-                if (two_issuers) {
-                    // O += P V only (S is issued by warp 2's thread).  After every product one more commit reports it on the
-                    // barrier of the S buffer whose P it read: the next S into that buffer waits for it.
-                    uint32_t c_of0 = 0;
-                    while (ok && wk.next(p, &u)) {
-                        const uint32_t seq0 = seq;
-                        for (int i = u.t0; ok && i < u.t1; ++i) {
-                            const int buf = (i - u.t0) & 1;
-                            const uint32_t vseq = seq0 + 2u * (uint32_t)(i - u.t0) + 1u, vs = vseq % ns;
-                            if (!(ok = mbar_wait(bar_full(vs), (vseq / ns) & 1, s_abort, p.status))) break;
-                            if (!(ok = mbar_wait(bar_pready(buf), c_p[buf] & 1, s_abort, p.status))) break;
-                            ++c_p[buf];
-                            if (i == u.t0) {
-                                if (c_of0 > 0 && !(ok = mbar_wait(bar_ofree(0), (c_of0 - 1) & 1, s_abort, p.status))) break;
-                                ++c_of0;
-                            }
-                            tc_fence_after();
-                            mma_pv_block(tmem + C::O_COL, tmem + buf * 128, desc_lo(slot_base(vs), CB_KT * 128), idesc_o, i > u.t0 ? 1u : 0u);
-                            tc_commit(bar_free(vs));
-                            tc_commit(bar_pvdone(buf));
-                        }
-                        seq = seq0 + 2u * (uint32_t)(u.t1 - u.t0);
-                    }
-                }
-                CbUnit un;
-                    bool have = !two_issuers && wk.next(p, &un);
-                while (ok && have) {
-                    u = un;
+                while (ok && wk.next(p, &u)) {
                     const bool two = u.nrt == 2;
+                    const int nt = u.t1 - u.t0, nev = two ? 2 * nt : nt;   // products of either kind in this unit
                     if (!(ok = mbar_wait(bar_qfull, uq & 1, s_abort, p.status))) break;
-                    tc_fence_after();
-                    const uint32_t seq0 = seq;
-                    for (int i = u.t0; ok && i <= u.t1; ++i) {
-                        if (i == u.t1) have = wk.next(p, &un);   // its loads overlap the wait for the last P
-                        const uint32_t kseq = seq0 + 2 * (i - u.t0), vseq_prev = kseq - 1;
-                        const uint32_t ks = kseq % C::NSLOT, vs = vseq_prev % C::NSLOT;
-                        if (two) {
-                            // per row tile l: PV of the previous key tile, then S of this one, so that the other
-                            // tile's softmax always has MMAs to overlap with
-                            for (int l = 0; l < 2; ++l) {
-                                if (i > u.t0) {
-                                    if (l == 0 && !(ok = mbar_wait(bar_full(vs), (vseq_prev / C::NSLOT) & 1, s_abort, p.status))) break;
-                                    if (!(ok = mbar_wait(bar_pready(l), c_p[l] & 1, s_abort, p.status))) break;
-                                    ++c_p[l];
-                                    if (i == u.t0 + 1) {
-                                        if (c_of[l] > 0 && !(ok = mbar_wait(bar_ofree(l), (c_of[l] - 1) & 1, s_abort, p.status))) break;
-                                        ++c_of[l];
-                                    }
-                                    tc_fence_after();
-                                    issue_pv(l, l, vs, i > u.t0 + 1);
-                                    if (l == 1) tc_commit(bar_free(vs));
-                                }
-                                if (i < u.t1) {
-                                    if (l == 0) {
-                                        if (!(ok = mbar_wait(bar_full(ks), (kseq / C::NSLOT) & 1, s_abort, p.status))) break;
-                                        tc_fence_after();
-                                    }
-                                    issue_s(l, l, ks);
-                                    if (l == 0) {
-                                        tc_commit(bar_sfull0);
-                                    } else {
-                                        tc_commit(bar_free(ks));
-                                        if (i == u.t1 - 1) tc_commit(bar_qfree);
-                                    }
-                                }
-                            }
-                        } else {
-                            if (i < u.t1) {
-                                const int buf = (i - u.t0) & 1;
-                                if (!(ok = mbar_wait(bar_full(ks), (kseq / C::NSLOT) & 1, s_abort, p.status))) break;
+                    // Turn e belongs to chain e & 1: the P V of its turn before (key tile iv), then S of this turn's key tile ik.
+                    for (int e = 0; e < nev + 2; ++e) {
+                        const int l = e & 1, ik = two ? e >> 1 : e, iv = two ? ik - 1 : ik - 2;
+                        if (e >= 2) {
+                            const uint32_t vseq = seq0 + 2u * (uint32_t)iv + 1u, vs = vseq % ns;
+                            if (iv < nt) {
+                                if ((!two || l == 0) && !(ok = mbar_wait(bar_full(vs), (vseq / ns) & 1, s_abort, p.status))) break;
+                                if (!(ok = mbar_wait(bar_pready(l), c_p[l] & 1, s_abort, p.status))) break;
+                                ++c_p[l];
+                                if (e < 4 && uq > 0 && !(ok = mbar_wait(bar_ofree(l), (uq - 1) & 1, s_abort, p.status))) break;
                                 tc_fence_after();
-                                issue_s(0, buf, ks);
+                                mma_pv_halves_block(tmem + C::O_COL + l * D, tmem + l * 128, desc_lo(slot_base(vs), CB_KT * 128), idesc_o, e < 4 ? 0u : 1u);
+                                if (!two || l == 1) tc_commit(bar_free(vs));
+                                if (two ? iv == nt - 1 : iv == nt - 1) tc_commit(two ? bar_odone(l) : bar_odone_both);
+                            }
+                        }
+                        if (ik < nt) {
+                            const uint32_t kseq = seq0 + 2u * (uint32_t)ik, ks = kseq % ns;
+                            if (!two || l == 0) {
+                                if (!(ok = mbar_wait(bar_full(ks), (kseq / ns) & 1, s_abort, p.status))) break;
+                                tc_fence_after();
+                            }
+                            mma_s_block<D>(tmem + l * 128, desc_lo(sbase + C::OFF_Q + (two ? l : 0) * C::Q_BYTES, 16), desc_lo(slot_base(ks), 16), idesc_s);
+                            tc_commit(bar_sfull(l));
+                            if (!two || l == 1) {
                                 tc_commit(bar_free(ks));
-                                if (i == u.t1 - 1) tc_commit(bar_qfree);
-                            }
-                            if (i > u.t0) {
-                                const int buf = (i - 1 - u.t0) & 1;
-                                if (!(ok = mbar_wait(bar_full(vs), (vseq_prev / C::NSLOT) & 1, s_abort, p.status))) break;
-                                if (!(ok = mbar_wait(bar_pready(buf), c_p[buf] & 1, s_abort, p.status))) break;
-                                ++c_p[buf];
-                                if (i == u.t0 + 1) {
-                                    if (c_of[0] > 0 && !(ok = mbar_wait(bar_ofree(0), (c_of[0] - 1) & 1, s_abort, p.status))) break;
-                                    ++c_of[0];
-                                }
-                                tc_fence_after();
-                                issue_pv(0, buf, vs, i > u.t0 + 1);
-                                tc_commit(bar_free(vs));
+                                if (ik == nt - 1) tc_commit(bar_qfree);
                             }
                         }
                     }
-                    seq = seq0 + 2 * (u.t1 - u.t0);
+                    // a chain without a tile in this unit still takes its turn on the accumulator's barrier
+                    if (ok && nev < 2 && uq > 0 && !(ok = mbar_wait(bar_ofree(1), (uq - 1) & 1, s_abort, p.status))) break;
+                    seq0 += 2u * (uint32_t)nt;
                     ++uq;
                 }
             }
-            __syncwarp();
-        } else if (warp == 2) {
-            // ------------------------------------------------------------------ query loader
+        } else {
+            // ------------------------------------------------------------------ units for the softmax warps, query tiles
             if (lane == 0) {
                 uint32_t uq = 0;
-                if (two_issuers) {
-                    // query tile, then S = Q K^T of every key tile of the unit.  The k-th S into a buffer waits for the
-                    // completion of the P.V that read the (k-1)-th P from it.
-                    constexpr uint32_t idesc_s = make_idesc(128, CB_KT, false);
-                    const uint32_t q_lo0 = desc_lo(sbase + C::OFF_Q, 16);
-                    uint32_t seq = 0, c_s[2] = {0u, 0u};
-                    bool ok = true;
-                    while (ok && wk.next(p, &u)) {
-                        if (uq > 0 && !(ok = mbar_wait(bar_qfree, (uq - 1) & 1, s_abort, p.status))) break;
-                        mbar_expect_tx(bar_qfull, (uint32_t)(C::DB * RT * 128));
-                        for (int db = 0; db < C::DB; ++db)
-                            tma_load_4d(sbase + C::OFF_Q + db * (CB_MT * 128), &maps.q, bar_qfull, db * 64, u.kh * p.G, u.rg * 2 * p.NPT, u.b);
-                        if (!(ok = mbar_wait(bar_qfull, uq & 1, s_abort, p.status))) break;
-                        ++uq;
-                        const uint32_t seq0 = seq;
-                        for (int i = u.t0; ok && i < u.t1; ++i) {
-                            const int buf = (i - u.t0) & 1;
-                            const uint32_t kseq = seq0 + 2u * (uint32_t)(i - u.t0), ks = kseq % ns;
-                            if (!(ok = mbar_wait(bar_full(ks), (kseq / ns) & 1, s_abort, p.status))) break;
-                            if (c_s[buf] > 0 && !(ok = mbar_wait(bar_pvdone(buf), (c_s[buf] - 1) & 1, s_abort, p.status))) break;
-                            ++c_s[buf];
-                            tc_fence_after();
-                            mma_s_block<D>(tmem + buf * 128, q_lo0, desc_lo(slot_base(ks), 16), idesc_s);
-                            tc_commit(bar_free(ks));
-                            if (i == u.t1 - 1) tc_commit(bar_qfree);
-                        }
-                        seq = seq0 + 2u * (uint32_t)(u.t1 - u.t0);
-                    }
-                }
-                while (!two_issuers && wk.next(p, &u)) {
-                    if (uq > 0 && !mbar_wait(bar_qfree, (uq - 1) & 1, s_abort, p.status)) break;
+                bool ok = true;
+                while (ok && wk.next(p, &u)) {
+                    volatile UnitDesc* d = &s_units[uq % kUnitRing];
+                    d->b = u.b; d->kh = u.kh; d->rg = u.rg; d->t0 = u.t0; d->t1 = u.t1; d->tiles = u.tiles; d->n = u.n; d->ctx = u.ctx; d->nrt = u.nrt;
+                    mbar_arrive(bar_ufull(uq % kUnitRing));
+                    if (uq > 0 && !(ok = mbar_wait(bar_qfree, (uq - 1) & 1, s_abort, p.status))) break;
                     mbar_expect_tx(bar_qfull, (uint32_t)(u.nrt * C::DB * RT * 128));
                     for (int rt = 0; rt < u.nrt; ++rt)
                         for (int db = 0; db < C::DB; ++db)
@@ -373,9 +283,13 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                                         (u.rg * 2 + rt) * p.NPT, u.b);
                     ++uq;
                 }
+                if (ok) {
+                    s_units[uq % kUnitRing].nrt = 0;
+                    mbar_arrive(bar_ufull(uq % kUnitRing));
+                }
                 if (p.cs > 0 && s_sched->c_has) {
                     // Cluster mode: the peers write their rows into this CTA's query tiles, so it reports itself ready to
-                    // receive as soon as its last S product has released them (long before its last P.V is done).
+                    // receive as soon as its last S product has released them (before its last P.V is done).
                     const int Rv = (min(RT, p.T * p.G) + p.cs - 1) / p.cs;
                     if ((uint32_t)(p.cs * Rv) * (uint32_t)((D + 4) * 4) <= 2u * C::Q_BYTES) {
                         if (uq == 0 || mbar_wait(bar_qfree, 0, s_abort, p.status))
@@ -383,308 +297,299 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     }
                 }
             }
-            __syncwarp();
         }
+        __syncwarp();
     } else {
         // ---------------------------------------------------------------------- softmax / correction / epilogue
-        reg_alloc<192>();
-        const int wg = (warp - 4) >> 2;                       // softmax warpgroup = row tile of a two-tile unit
+        reg_alloc<104>();
+        const int sw = warp - 4, l = sw >> 3, hf = (sw >> 2) & 1;   // chain, half of the tile's keys
         const int wq = warp & 3;                              // TMEM lane quarter this warp may access
         const int row = wq * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
-        const uint32_t tm_O = tmem + C::O_COL + wg * D + lane_addr;
-        uint32_t c_s0 = 0;                                    // completions of s_full0 consumed so far (warpgroup 0 only)
-        uint32_t seq = 0;                                     // ring sequence number of the next unit's first K tile
-        bool ok = true;
-        // The next unit's shape and this row's ancestor bits are fetched while the current unit is still being finished,
-        // so that their memory round trips do not sit between two units.
-        CbUnit un;
-        uint32_t mrow_n[4] = {0u, 0u, 0u, 0u};
-        auto fetch_next = [&]() {
-            const bool have = wk.next(p, &un);
-            mrow_n[0] = mrow_n[1] = mrow_n[2] = mrow_n[3] = 0u;
-            if (have && (wg == 0 || un.nrt == 2)) {
-                const int nnode = (un.rg * 2 + wg) * p.NPT + row / p.G;
-                if (row < RT && nnode < un.n) {
-                    const uint32_t* mp = p.tree_mask + ((size_t)un.b * p.T + nnode) * p.W;
-                    mrow_n[0] = mp[0];
-                    if (p.W > 1) mrow_n[1] = mp[1];
-                    if (p.W > 2) mrow_n[2] = mp[2];
-                    if (p.W > 3) mrow_n[3] = mp[3];
-                }
+        const int pair_id = 1 + l * 4 + wq;                   // named barrier of the two warps that share these rows
+        constexpr int CW = D / 4;                             // accumulator columns handled at a time
+        {
+            // rows of padding nodes (node >= n_nodes) are written as zeros while the first tiles are on their way
+            const int per_row = p.Hq * D / 8;                 // 16-byte chunks per node row
+            for (int idx = cta * 16 + sw; idx < p.B * p.T; idx += gridDim.x * 16) {
+                const int b = idx / p.T, nd = idx % p.T;
+                const int n = min(max(p.n_nodes[b], 0), p.T);
+                if (nd < n) continue;
+                uint4* op = reinterpret_cast<uint4*>(p.out + (size_t)idx * p.Hq * D);
+                for (int k = lane; k < per_row; k += 32) op[k] = make_uint4(0, 0, 0, 0);
+                if (p.lse) for (int h = lane; h < p.Hq; h += 32) p.lse[((size_t)b * p.Hq + h) * p.T + nd] = 0.f;
             }
-            return have;
+        }
+        int entered = 0;                                      // pair barriers entered
+        auto pair_sync = [&](bool v) {
+            ++entered;
+            if (lane == 0) s_pair[sw] = entered;
+            return pair_or(pair_id, v);
         };
-        float c_m = -INFINITY, c_l = 0.f;                     // cluster mode: this CTA's share of the unit, kept for the exchange
-        bool c_share = false;
-        bool have = fetch_next();
-        while (ok && have) {
-            u = un;
-            const uint32_t mrow[4] = {mrow_n[0], mrow_n[1], mrow_n[2], mrow_n[3]};
-            const bool two = u.nrt == 2;
-            const int nt = u.t1 - u.t0;
-            const uint32_t seq0 = seq;
-            seq += 2u * (uint32_t)nt;
-            if (wg == 1 && !two) {
-                // Handled by warpgroup 0 alone.  This warpgroup still watches every S completion, in order: waiting on a
-                // barrier by parity is only sound for a thread that is at most one phase away from it, and a thread that
-                // ran ahead over this unit would later meet ring barriers that are whole revolutions behind it.  It must
-                // not fall behind either (it may start late, after a long epilogue): half of every "P ready" arrival is
-                // its own, given when it has seen the tile's S, so the products cannot run more than a tile ahead of it.
-                for (int i = u.t0; ok && i < u.t1; ++i) {
-                    const uint32_t kseq = seq0 + 2u * (uint32_t)(i - u.t0);
-                    ok = mbar_wait(bar_free(kseq % ns), (kseq / ns) & 1, s_abort, p.status);
-                    mbar_arrive(bar_pready((i - u.t0) & 1));
-                }
-                have = fetch_next();
-                continue;
+        uint32_t c_s = 0, c_od = 0, c_ob = 0;                 // completions consumed: S of this chain, o_done of this chain, o_done_both
+        bool ok = true;
+        float x_m = -INFINITY, x_l = 0.f, x_w0 = 0.f, x_w1 = 0.f;   // one-row-tile unit: combined reference and sum, weights of O0 and O1
+        bool c_share = false;                                 // cluster mode: this CTA has a share of the unit
+        for (uint32_t uq = 0; ok; ++uq) {
+            if (!(ok = mbar_wait(bar_ufull(uq % kUnitRing), (uq / kUnitRing) & 1, s_abort, p.status))) break;
+            const volatile UnitDesc* u = &s_units[uq % kUnitRing];   // read again where it is needed: registers are short
+            if (u->nrt == 0) break;
+            const bool two = u->nrt == 2;
+            const int step = two ? 1 : 2, tfirst = u->t0 + (two ? 0 : l), t1 = u->t1, nfull = min(u->ctx / CB_KT, u->tiles - 1);
+            const int node = (u->rg * 2 + (two ? l : 0)) * p.NPT + row / p.G;
+            const bool row_valid = row < RT && node < u->n;
+            const bool warp_active = (wq * 32) < RT && node - row / p.G + (wq * 32) / p.G < u->n;   // row 0 of the warp is valid
+            // this row's ancestor bits: word 0 (the reference is taken from the tile's first 32 keys) and this half's two words
+            uint32_t mref = 0u, mlo = 0u, mhi = 0u;
+            if (row_valid && t1 == u->tiles) {
+                const uint32_t* mp = p.tree_mask + ((size_t)u->b * p.T + node) * p.W;
+                mref = mp[0];
+                if (2 * hf < p.W) mlo = mp[2 * hf];
+                if (2 * hf + 1 < p.W) mhi = mp[2 * hf + 1];
             }
-            // S(i) is done when tile i's K slot is released (or, for row tile 0 of two, when s_full0 completes);
-            // every PV up to tile i is done when tile i's V slot is released.
-            auto wait_pv = [&](int i) {
-                const uint32_t vseq = seq0 + 2u * (uint32_t)(i - u.t0) + 1u;
-                return mbar_wait(bar_free(vseq % ns), (vseq / ns) & 1, s_abort, p.status);
-            };
-            const int rt = u.rg * 2 + wg;
-            const int node = rt * p.NPT + row / p.G, g = row % p.G, h = u.kh * p.G + g;
-            const bool row_valid = row < RT && node < u.n;
-            const bool warp_active = (wq * 32) < RT && (rt * p.NPT + (wq * 32) / p.G) < u.n;   // row 0 of the warp is valid
-            const int nct = u.tiles - 1;
-            float m_used = -INFINITY, l = 0.f;
-            for (int i = u.t0; i < u.t1; ++i) {
-                const int buf = two ? wg : ((i - u.t0) & 1);
-                if (two && wg == 0) {
-                    if (!(ok = mbar_wait(bar_sfull0, c_s0 & 1, s_abort, p.status))) break;
-                    ++c_s0;
-                } else {
-                    const uint32_t kseq = seq0 + 2u * (uint32_t)(i - u.t0);
-                    if (!(ok = mbar_wait(bar_free(kseq % ns), (kseq / ns) & 1, s_abort, p.status))) break;
-                }
+            const uint32_t ts = tmem + l * 128 + lane_addr, tsh = ts + 64 * hf;
+            const uint32_t tm_O = tmem + C::O_COL + l * D + lane_addr;
+            float m_used = -INFINITY, lsum = 0.f;
+            for (int i = tfirst; i < t1; i += step) {
+                if (!(ok = mbar_wait(bar_sfull(l), c_s & 1, s_abort, p.status))) break;
+                ++c_s;
                 if (warp_active) {
                     tc_fence_after();
-                    const uint32_t ts = tmem + buf * 128 + lane_addr;
-                    // visibility of the tile's 128 keys for this row: context keys below ctx, tree keys by the ancestor bits
-                    const bool is_tree = i == nct;
-                    const int kv = is_tree ? u.n : min(CB_KT, u.ctx - i * CB_KT);
-                    uint32_t vm[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
-                    // A context tile that lies wholly inside the context needs no masks.  Rows that do not exist take the fast
-                    // path too: whatever they compute stays in their own row.
-                    bool all_vis = !is_tree && kv == CB_KT;
+                    // Visibility of this thread's 64 keys: context keys below ctx, tree keys by the ancestor bits.  A context tile
+                    // that lies wholly inside the context needs no masks.  Rows that do not exist take the fast path too:
+                    // whatever they compute stays in their own row.
+                    const bool all_vis = i < nfull;
+                    uint32_t vm[2] = {0xFFFFFFFFu, 0xFFFFFFFFu}, vref = 0xFFFFFFFFu;
+                    auto below = [&](int lo) { return lo >= 32 ? 0xFFFFFFFFu : (lo <= 0 ? 0u : ((1u << lo) - 1u)); };
                     if (!all_vis) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int lo = kv - 32 * k;
-                            const uint32_t below = lo >= 32 ? 0xFFFFFFFFu : (lo <= 0 ? 0u : ((1u << lo) - 1u));
-                            vm[k] = row_valid ? (is_tree ? (mrow[k] & below) : below) : 0u;
-                        }
-                        all_vis = __all_sync(CB_FULL, !row_valid || (vm[0] & vm[1] & vm[2] & vm[3]) == 0xFFFFFFFFu);
+                        const bool is_tree = i == u->tiles - 1;
+                        const int kv = is_tree ? u->n : u->ctx - i * CB_KT;
+                        vm[0] = below(kv - 64 * hf); vm[1] = below(kv - 64 * hf - 32); vref = below(kv);
+                        if (is_tree) { vm[0] &= mlo; vm[1] &= mhi; vref &= mref; }
+                        if (!row_valid) vm[0] = vm[1] = vref = 0u;
                     }
-                    uint32_t sa[32], sb[32];
                     // Single pass, tried first on every tile: P against the reference maximum in use, held back in registers so
                     // that S is still whole if the tile has to be done again.  No row maximum is taken.  The reference exists
                     // to keep 2^(s - reference) and its sums inside fp32 (P is bf16, same exponent range), not for precision,
-                    // so the tile's row sum tells all that matters: while it stays below 2^20 no score is more than 20
-                    // above the reference and the tile stands; above that (or not finite) the two passes below run instead
-                    // and move the reference to the new maximum.  A share's first tile has no reference yet and takes the
-                    // largest of its first 32 scores.
-                    bool single = false;
-                    {
-                        uint32_t pk[64];
-                        CB_TMEM_LD32(sa, 0, ts);
-                        CB_TMEM_WAIT_LD32(sa);
-                        CB_TMEM_LD32(sb, 0, ts + 32);
+                    // so the half row's sum tells all that matters: while it stays below 2^20 no score is more than 20
+                    // above the reference and the tile stands; above that (or not finite) in either half, the two passes below
+                    // run instead in both and move the reference to the new maximum.  A share's first tile has no reference
+                    // yet and takes the largest of the row's first 32 scores (both threads of the row read them).
+                    if (i == tfirst) {
+                        uint32_t rf[32];
+                        CB_TMEM_LD32(rf, 0, ts);
+                        CB_TMEM_WAIT_LD32(rf);
                         if (!all_vis) {
 #pragma unroll
                             for (int jx = 0; jx < 32; ++jx)
-                                if (!((vm[0] >> jx) & 1u)) sa[jx] = 0xFF800000u;
+                                if (!((vref >> jx) & 1u)) rf[jx] = 0xFF800000u;
                         }
-                        if (i == u.t0) {
-                            float c0 = -INFINITY, c1 = -INFINITY, c2 = -INFINITY, c3 = -INFINITY;
+                        float c0 = -INFINITY, c1 = -INFINITY;
 #pragma unroll
-                            for (int jx = 0; jx < 32; jx += 4) {
-                                c0 = fmaxf(c0, __uint_as_float(sa[jx])); c1 = fmaxf(c1, __uint_as_float(sa[jx + 1]));
-                                c2 = fmaxf(c2, __uint_as_float(sa[jx + 2])); c3 = fmaxf(c3, __uint_as_float(sa[jx + 3]));
-                            }
-                            m_used = fmaxf(fmaxf(c0, c1), fmaxf(c2, c3)) * p.scale_log2;   // -inf if the row sees none of them
+                        for (int jx = 0; jx < 32; jx += 4) {
+                            c0 = fmax3(c0, __uint_as_float(rf[jx]), __uint_as_float(rf[jx + 1]));
+                            c1 = fmax3(c1, __uint_as_float(rf[jx + 2]), __uint_as_float(rf[jx + 3]));
                         }
-                        const float mu = (m_used == -INFINITY) ? 0.f : m_used;
+                        m_used = fmaxf(c0, c1) * p.scale_log2;   // -inf if the row sees none of them
+                    }
+                    uint32_t pk[32];
+                    // P of this thread's 64 scores (packed into pk) against reference mu; returns their sum.  16 scores at a time with
+                    // the next 16 in flight: a thread has 96 registers, and what does not fit them spills past an L1 that the
+                    // tiles leave 28 KB.
+                    auto make_p = [&](float mu) {
                         const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2), negmu2 = f2_pack(-mu, -mu);
                         uint64_t lsa = f2_pack(0.f, 0.f), lsb = f2_pack(0.f, 0.f);
+                        uint32_t sa[16], sb[16];
+                        CB_TMEM_LD16(sa, tsh);
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
                             uint32_t* cur = (c & 1) ? sb : sa;
                             uint32_t* nxt = (c & 1) ? sa : sb;
-                            if (c > 0) {
-                                CB_TMEM_WAIT_LD32(cur);
-                                if (c < 3) CB_TMEM_LD32(nxt, 0, ts + 32 * (c + 1));
-                                if (!all_vis) {
+                            CB_TMEM_WAIT_LD16(cur);
+                            if (c < 3) CB_TMEM_LD16(nxt, tsh + 16 * (c + 1));
+                            if (!all_vis) {
 #pragma unroll
-                                    for (int jx = 0; jx < 32; ++jx)
-                                        if (!((vm[c] >> jx) & 1u)) cur[jx] = 0xFF800000u;
-                                }
+                                for (int jx = 0; jx < 16; ++jx)
+                                    if (!((vm[c >> 1] >> ((c & 1) * 16 + jx)) & 1u)) cur[jx] = 0xFF800000u;
                             }
 #pragma unroll
-                            for (int jx = 0; jx < 32; jx += 4) {
-                                float p0, p1, p2, p3;
-                                f2_unpack(f2_fma(f2_pack(__uint_as_float(cur[jx]), __uint_as_float(cur[jx + 1])), scale2, negmu2), p0, p1);
-                                f2_unpack(f2_fma(f2_pack(__uint_as_float(cur[jx + 2]), __uint_as_float(cur[jx + 3])), scale2, negmu2), p2, p3);
-                                p0 = ex2(p0); p1 = ex2(p1); p2 = ex2(p2); p3 = ex2(p3);
-                                lsa = f2_add(lsa, f2_pack(p0, p1));
-                                lsb = f2_add(lsb, f2_pack(p2, p3));
-                                pk[c * 16 + (jx >> 1)] = pack_bf16(p0, p1);
-                                pk[c * 16 + (jx >> 1) + 1] = pack_bf16(p2, p3);
+                            for (int q = 0; q < 8; ++q) {
+                                const uint64_t x = f2_fma(f2_pack(__uint_as_float(cur[2 * q]), __uint_as_float(cur[2 * q + 1])), scale2, negmu2);
+                                float p0, p1;
+                                if (q % 4 == kFmaExpPhase) {
+                                    ex2_pair_fma(x, p0, p1);
+                                } else {
+                                    f2_unpack(x, p0, p1);
+                                    p0 = ex2(p0); p1 = ex2(p1);
+                                }
+                                if (q & 1) lsb = f2_add(lsb, f2_pack(p0, p1));
+                                else lsa = f2_add(lsa, f2_pack(p0, p1));
+                                pk[c * 8 + q] = pack_bf16(p0, p1);
                             }
                         }
                         float l0, l1, l2, l3;
                         f2_unpack(lsa, l0, l1);
                         f2_unpack(lsb, l2, l3);
-                        const float lt = (l0 + l1) + (l2 + l3);
-                        if (!__any_sync(CB_FULL, row_valid && !(lt <= kRowSumLimit))) {   // rows that do not exist hold anything: they never ask
-                            CB_TMEM_ST16(pk, 0, ts);
-                            CB_TMEM_ST16(pk, 16, ts + 16);
-                            CB_TMEM_ST16(pk, 32, ts + 32);
-                            CB_TMEM_ST16(pk, 48, ts + 48);
-                            l += lt;
-                            tmem_wait_st();
-                            single = true;
-                        }
-                    }
-                    if (!single) {
-                    // pass 1: row maximum of the visible scores, 32 columns at a time with the next 32 in flight
-                    CB_TMEM_LD32(sa, 0, ts);
-                    float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t* cur = (c & 1) ? sb : sa;
-                        uint32_t* nxt = (c & 1) ? sa : sb;
-                        CB_TMEM_WAIT_LD32(cur);
-                        if (c < 3) CB_TMEM_LD32(nxt, 0, ts + 32 * (c + 1));
-                        if (all_vis) {
-#pragma unroll
-                            for (int jx = 0; jx < 32; jx += 4) {
-                                m0 = fmaxf(m0, __uint_as_float(cur[jx])); m1 = fmaxf(m1, __uint_as_float(cur[jx + 1]));
-                                m2 = fmaxf(m2, __uint_as_float(cur[jx + 2])); m3 = fmaxf(m3, __uint_as_float(cur[jx + 3]));
-                            }
-                        } else {
-#pragma unroll
-                            for (int jx = 0; jx < 32; ++jx) m0 = fmaxf(m0, ((vm[c] >> jx) & 1u) ? __uint_as_float(cur[jx]) : -INFINITY);
-                        }
-                    }
-                    float mloc = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
-                    CB_TMEM_LD32(sa, 0, ts);                     // first columns of pass 2, in flight during the bookkeeping below
-                    mloc *= p.scale_log2;
-                    // lazy rescaling: keep the reference maximum until the running maximum exceeds it by 2^8 (a tile that
-                    // comes here from the single pass holds a score at least 2^13 above it)
-                    const bool need = mloc > m_used + 8.0f;
-                    const float alpha = need ? ex2(m_used - mloc) : 1.0f;
-                    if (need) m_used = mloc;
-                    if (i > u.t0 && __any_sync(CB_FULL, need)) {
-                        // O must be complete up to the previous tile before it is rescaled
-                        if (!(ok = wait_pv(i - 1))) break;
-                        tc_fence_after();
-#pragma unroll
-                        for (int c = 0; c < D / 32; ++c) {
-                            uint32_t o[32];
-                            CB_TMEM_LD32(o, 0, tm_O + c * 32);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int jx = 0; jx < 32; ++jx) o[jx] = __float_as_uint(__uint_as_float(o[jx]) * alpha);
-                            CB_TMEM_ST32(o, 0, tm_O + c * 32);
-                        }
-                    }
-                    l *= alpha;
-                    const float mu = (m_used == -INFINITY) ? 0.f : m_used;
-                    // pass 2: P = 2^(s * scale - m), written back over S as packed bf16 (64 scores -> 32 columns)
-                    const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2), negmu2 = f2_pack(-mu, -mu);
-                    uint64_t lsa = f2_pack(0.f, 0.f), lsb = f2_pack(0.f, 0.f);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t pk[16];
-                        uint32_t* cur = (c & 1) ? sb : sa;
-                        uint32_t* nxt = (c & 1) ? sa : sb;
-                        CB_TMEM_WAIT_LD32(cur);
-                        if (c < 3) CB_TMEM_LD32(nxt, 0, ts + 32 * (c + 1));
+                        return (l0 + l1) + (l2 + l3);
+                    };
+                    float lt = make_p(m_used == -INFINITY ? 0.f : m_used);
+                    if (pair_sync(row_valid && !(lt <= kRowSumLimit))) {          // rows that do not exist hold anything: they never ask
+                        // pass 1: the row's maximum over all its visible scores (both threads of the row take it)
+                        uint32_t va[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
                         if (!all_vis) {
+                            const bool is_tree = i == u->tiles - 1;
+                            const int kv = is_tree ? u->n : u->ctx - i * CB_KT;
+                            const uint32_t* mp = p.tree_mask + ((size_t)u->b * p.T + (row_valid ? node : 0)) * p.W;
 #pragma unroll
-                            for (int jx = 0; jx < 32; ++jx)
-                                if (!((vm[c] >> jx) & 1u)) cur[jx] = 0xFF800000u;
+                            for (int k = 0; k < 4; ++k) {
+                                const uint32_t bl = below(kv - 32 * k);
+                                va[k] = !row_valid ? 0u : (!is_tree ? bl : (k < p.W ? bl & mp[k] : 0u));
+                            }
                         }
+                        float mx = -INFINITY;
+#pragma unroll 1
+                        for (int c = 0; c < 4; ++c) {
+                            uint32_t rf[32];
+                            CB_TMEM_LD32(rf, 0, ts + 32 * c);
+                            CB_TMEM_WAIT_LD32(rf);
 #pragma unroll
-                        for (int jx = 0; jx < 32; jx += 4) {
-                            float p0, p1, p2, p3;
-                            f2_unpack(f2_fma(f2_pack(__uint_as_float(cur[jx]), __uint_as_float(cur[jx + 1])), scale2, negmu2), p0, p1);
-                            f2_unpack(f2_fma(f2_pack(__uint_as_float(cur[jx + 2]), __uint_as_float(cur[jx + 3])), scale2, negmu2), p2, p3);
-                            p0 = ex2(p0); p1 = ex2(p1); p2 = ex2(p2); p3 = ex2(p3);
-                            lsa = f2_add(lsa, f2_pack(p0, p1));
-                            lsb = f2_add(lsb, f2_pack(p2, p3));
-                            pk[jx >> 1] = pack_bf16(p0, p1);
-                            pk[(jx >> 1) + 1] = pack_bf16(p2, p3);
+                            for (int jx = 0; jx < 32; ++jx) mx = fmaxf(mx, ((va[c] >> jx) & 1u) ? __uint_as_float(rf[jx]) : -INFINITY);
                         }
-                        CB_TMEM_ST16(pk, 0, ts + c * 16);             // the 32 scores just read become 16 columns of packed P
+                        pair_sync(false);                                         // both have read S: either may write P over it now
+                        const float mloc = mx * p.scale_log2;
+                        // lazy rescaling: keep the reference maximum until the running maximum exceeds it by 2^8 (a tile that
+                        // comes here from the single pass holds a score at least 2^13 above it)
+                        const bool need = mloc > m_used + 8.0f;
+                        const float alpha = need ? ex2(m_used - mloc) : 1.0f;
+                        if (need) m_used = mloc;
+                        if (i > tfirst && __any_sync(CB_FULL, need)) {
+                            // O is complete up to the chain's previous tile: that product came before this S in the issue order.
+                            // Each of the two threads rescales half of the columns.
+#pragma unroll 1
+                            for (int c = 0; c < 2; ++c) {
+                                uint32_t o[CW];
+                                const uint32_t ta = tm_O + hf * (D / 2) + c * CW;
+                                tmem_ld_w<CW>(o, ta);
+#pragma unroll
+                                for (int jx = 0; jx < CW; ++jx) o[jx] = __float_as_uint(__uint_as_float(o[jx]) * alpha);
+                                tmem_st_w<CW>(o, ta);
+                            }
+                            tmem_wait_st();
+                        }
+                        lsum *= alpha;
+                        // pass 2: P = 2^(s * scale - m)
+                        lt = make_p(m_used == -INFINITY ? 0.f : m_used);
                     }
-                    float l0, l1, l2, l3;
-                    f2_unpack(lsa, l0, l1);
-                    f2_unpack(lsb, l2, l3);
-                    l += (l0 + l1) + (l2 + l3);
+                    CB_TMEM_ST32(pk, 0, tsh);                 // the 64 scores become 32 columns of packed P at their start
+                    lsum += lt;
                     tmem_wait_st();
-                    }
                 }
                 tc_fence_before();
-                mbar_arrive_n(bar_pready(buf), two ? 2u : 1u);   // 256 arrivals per phase: the other half is the watching warpgroup's
+                mbar_arrive(bar_pready(l));
             }
             if (!ok) break;
-            have = fetch_next();
-            // ---- epilogue of this unit's share: O is complete once its last PV has finished
-            if (!(ok = wait_pv(u.t1 - 1))) break;
+            // ---- epilogue of this unit's share
+            const int ub = u->b, t0 = u->t0, h = u->kh * p.G + row % p.G;
+            const bool whole = t0 == 0 && t1 == u->tiles;
+            // this thread's columns of the output row: with two row tiles half a row in two steps, with one a quarter in one
+            int ncol, c0;
+            if (two) {
+                s_x[(l * 2 + hf) * CB_MT + row] = lsum;
+                pair_sync(false);
+                x_l = lsum + s_x[(l * 2 + 1 - hf) * CB_MT + row];
+                x_m = m_used; x_w0 = x_w1 = 1.f;
+                ncol = 2; c0 = hf * 2 * CW;
+                if (!(ok = mbar_wait(bar_odone(l), c_od & 1, s_abort, p.status))) break;
+                ++c_od;
+            } else {
+                if (!(ok = mbar_wait(bar_odone_both, c_ob & 1, s_abort, p.status))) break;
+                ++c_ob;
+                s_x[(l * 2 + hf) * CB_MT + row] = lsum;
+                pair_sync(false);
+                const float lrow = lsum + s_x[(l * 2 + 1 - hf) * CB_MT + row];
+                pair_sync(false);
+                s_x[(l * 2 + hf) * CB_MT + row] = hf ? lrow : m_used;
+                mbar_arrive(bar_sums);
+                if (!(ok = mbar_wait(bar_sums, (c_ob - 1) & 1, s_abort, p.status))) break;
+                const float m0 = s_x[row], l0 = s_x[CB_MT + row], m1 = s_x[2 * CB_MT + row], l1 = s_x[3 * CB_MT + row];
+                x_m = fmaxf(m0, m1);
+                x_w0 = m0 == -INFINITY ? 0.f : ex2(m0 - x_m);
+                x_w1 = m1 == -INFINITY ? 0.f : ex2(m1 - x_m);
+                x_l = l0 * x_w0 + l1 * x_w1;
+                ncol = 1; c0 = (l * 2 + hf) * CW;
+            }
             tc_fence_after();
             if (p.cs > 0) {
-                c_m = m_used; c_l = l; c_share = true;         // O stays in TMEM until the exchange below
-            } else if (warp_active) {
-                const bool whole = u.t0 == 0 && u.t1 == u.tiles;
-                if (whole) {
-                    const float inv = l > 0.f ? 1.0f / l : 0.f;
+                c_share = true;                               // O stays in TMEM until the exchange below
+                x_w1 = t1 - t0 > 1 ? x_w1 : -1.f;             // a share of one tile has no second accumulator
+                break;                                        // a CTA of a cluster has one share
+            }
+            if (warp_active) {
+                const float inv = whole ? (x_l > 0.f ? 1.0f / x_l : 0.f) : 1.0f;
+                const float w0 = two ? inv : x_w0 * inv, w1 = x_w1 * inv;
+                const size_t slot = 2 * (size_t)cta + (t0 == 0 ? 1 : 0);
+                float* pp = p.part + ((slot * 2 + (two ? l : 0)) * CB_MT + row) * (D + 4);
+                __nv_bfloat16* op = p.out + (((size_t)ub * p.T + (row_valid ? node : 0)) * p.Hq + h) * D;
+#pragma unroll 1
+                for (int c = 0; c < ncol; ++c) {
+                    uint32_t o[CW];
+                    const int col = c0 + c * CW;
+                    if (two) {
+                        tmem_ld_w<CW>(o, tm_O + col);
 #pragma unroll
-                    for (int c = 0; c < D / 32; ++c) {
-                        uint32_t o[32];
-                        CB_TMEM_LD32(o, 0, tm_O + c * 32);
-                        tmem_wait_ld();
-                        if (row_valid) {
-                            __nv_bfloat16* op = p.out + (((size_t)u.b * p.T + node) * p.Hq + h) * D + c * 32;
-                            uint32_t w[16];
+                        for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * w0);
+                    } else {
+                        tmem_ld_w<CW>(o, tmem + C::O_COL + lane_addr + col);
 #pragma unroll
-                            for (int k2 = 0; k2 < 16; ++k2) w[k2] = pack_bf16(__uint_as_float(o[2 * k2]) * inv, __uint_as_float(o[2 * k2 + 1]) * inv);
-                            st_global_v8(op, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-                            st_global_v8(op + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+                        for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * w0);
+                        if (t1 - t0 > 1) {
+                            uint32_t o1[CW];
+                            tmem_ld_w<CW>(o1, tmem + C::O_COL + D + lane_addr + col);
+#pragma unroll
+                            for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) + __uint_as_float(o1[k]) * w1);
                         }
                     }
-                    if (row_valid && p.lse)
-                        p.lse[((size_t)u.b * p.Hq + h) * p.T + node] = l > 0.f ? (m_used + log2f(l)) * 0.6931471805599453f : 0.f;
-                } else {
-                    const size_t slot = 2 * (size_t)cta + (u.t0 == 0 ? 1 : 0);
-                    float* pp = p.part + ((slot * 2 + wg) * CB_MT + row) * (D + 4);
+                    if (!row_valid) continue;
+                    if (whole) {
+                        uint32_t w[CW / 2];
 #pragma unroll
-                    for (int c = 0; c < D / 32; ++c) {
-                        uint32_t o[32];
-                        CB_TMEM_LD32(o, 0, tm_O + c * 32);
-                        tmem_wait_ld();
-                        if (row_valid) {
-                            // partial rows are D + 4 floats long: 16-byte aligned only
+                        for (int k = 0; k < CW / 2; ++k) w[k] = pack_bf16(__uint_as_float(o[2 * k]), __uint_as_float(o[2 * k + 1]));
 #pragma unroll
-                            for (int v4 = 0; v4 < 8; ++v4)
-                                *reinterpret_cast<uint4*>(pp + c * 32 + v4 * 4) = make_uint4(o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
-                        }
+                        for (int k = 0; k < CW / 2; k += 8) st_global_v8(op + col + 2 * k, w[k], w[k + 1], w[k + 2], w[k + 3], w[k + 4], w[k + 5], w[k + 6], w[k + 7]);
+                    } else {
+                        // partial rows are D + 4 floats long: 16-byte aligned only
+#pragma unroll
+                        for (int v4 = 0; v4 < CW / 4; ++v4)
+                            *reinterpret_cast<uint4*>(pp + col + v4 * 4) = make_uint4(o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
                     }
-                    if (row_valid) { pp[D] = m_used; pp[D + 1] = l; }
+                }
+                if (row_valid && c0 == 0) {
+                    if (!whole) { pp[D] = x_m; pp[D + 1] = x_l; }
+                    else if (p.lse) p.lse[((size_t)ub * p.Hq + h) * p.T + node] = x_l > 0.f ? (x_m + log2f(x_l)) * 0.6931471805599453f : 0.f;
                 }
             }
             tc_fence_before();
-            mbar_arrive(bar_ofree(wg));
+            if (two) mbar_arrive_n(bar_ofree(l), 2u);          // 512 arrivals per unit either way
+            else { mbar_arrive(bar_ofree(0)); mbar_arrive(bar_ofree(1)); }
+        }
+        if (!ok) {
+            // The other warp of the pair may have entered a pair barrier that this one will not: answer for it until it has left too.
+            // Its own waits end as well, so this does; the loop is bounded all the same.
+            __syncwarp();
+            if (lane == 0) { __threadfence_block(); s_pair[sw] = -1; }
+            for (int k = 0; k < 1 << 16; ++k) {
+                const int other = __shfl_sync(CB_FULL, lane == 0 ? s_pair[sw ^ 4] : 0, 0);
+                if (other < 0) break;
+                if (other > entered) { ++entered; pair_arrive(pair_id); }
+                __nanosleep(200);
+            }
         }
         if (p.cs > 0 && s_sched->c_has) {
             // ------------------------------------------------------------------ cluster mode: combine the unit's shares
-            // Every CTA of the cluster holds the unnormalised rows of its share (O in TMEM, running maximum and sum in
-            // registers).  Row i is combined by CTA i % cs: each CTA writes its copy of the row into that CTA's shared memory,
-            // arrives on its data barrier, and the owner merges the cs contributions and writes the output row.  The rows are
+            // Every CTA of the cluster holds the unnormalised rows of its share (O0 and O1 in TMEM, their weights, the running
+            // maximum and the sum in registers).  Row i is combined by CTA i % cs: each CTA writes its copy of the row into that
+            // CTA's shared memory (four threads a row, D / 4 columns each), arrives on its data barrier, and the owner merges the
+            // cs contributions and writes the output row.  The rows are
             // received in the two query tiles when they fit (they are idle from a CTA's last S product on, which the query
             // loader reports), otherwise in the K/V ring (idle from the last P.V on, reported here).
             const int cs = p.cs, rank = cta % cs;
@@ -693,36 +598,41 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             constexpr uint32_t ROWB = (D + 4) * 4;
             const bool in_q = (uint32_t)(cs * Rv) * ROWB <= 2u * C::Q_BYTES;
             const uint32_t recv = sbase + (in_q ? C::OFF_Q : C::OFF_RING);     // [cs sources][Rv rows][D + 4] floats
-            if (ok && !in_q && wg == 0 && row == 0)
+            if (ok && !in_q && sw == 0 && lane == 0)
                 for (int r = 0; r < cs; ++r) mbar_arrive_remote(cluster_addr(bar_cready, (uint32_t)r));
             if (ok) ok = mbar_wait_cluster(bar_cready, 0, s_abort, p.status);
-            if (ok && wg == 0) {
+            if (ok) {
                 const int dest = row % cs, rl = row / cs;
                 const bool valid = row < RT && (row / p.G) < cn;
                 const uint32_t ra = cluster_addr(recv + (uint32_t)(rank * Rv + rl) * ROWB, (uint32_t)dest);
                 const bool act = (wq * 32) < RT && ((wq * 32) / p.G) < cn;     // row 0 of the warp is valid
+                const int col = (l * 2 + hf) * CW;
                 if (act && c_share) {
+                    uint32_t o[CW];
+                    tmem_ld_w<CW>(o, tmem + C::O_COL + lane_addr + col);
 #pragma unroll
-                    for (int c = 0; c < D / 32; ++c) {
-                        uint32_t o[32];
-                        CB_TMEM_LD32(o, 0, tm_O + c * 32);
-                        tmem_wait_ld();
-                        if (valid) {
+                    for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * x_w0);
+                    if (__any_sync(CB_FULL, x_w1 >= 0.f)) {
+                        uint32_t o1[CW];
+                        tmem_ld_w<CW>(o1, tmem + C::O_COL + D + lane_addr + col);
 #pragma unroll
-                            for (int v4 = 0; v4 < 8; ++v4)
-                                st_cluster_v4(ra + (uint32_t)(c * 32 + v4 * 4) * 4u, o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
-                        }
+                        for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) + __uint_as_float(o1[k]) * x_w1);
+                    }
+                    if (valid) {
+#pragma unroll
+                        for (int v4 = 0; v4 < CW / 4; ++v4)
+                            st_cluster_v4(ra + (uint32_t)(col + v4 * 4) * 4u, o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
                     }
                 }
-                if (valid) st_cluster_v4(ra + D * 4u, __float_as_uint(c_share ? c_m : -INFINITY), __float_as_uint(c_share ? c_l : 0.f), 0u, 0u);
+                if (valid && col == 0) st_cluster_v4(ra + D * 4u, __float_as_uint(c_share ? x_m : -INFINITY), __float_as_uint(c_share ? x_l : 0.f), 0u, 0u);
                 mbar_arrive_remote(cluster_addr(bar_cdata, (uint32_t)dest));
             }
             if (ok) ok = mbar_wait_cluster(bar_cdata, 0, s_abort, p.status);
             if (ok) {
-                // up to 256 threads: tpr threads per row, each a run of D / tpr >= 8 columns in groups of 8
-                int tpr = D / 8;                                 // a power of two
-                while (tpr * Rv > 256) tpr >>= 1;
-                const int t = wg * 128 + row, rl = t / tpr, sub = t % tpr;
+                // up to 512 threads: tpr threads per row, each a run of D / tpr >= 4 columns in groups of 4
+                int tpr = D / 4;                                 // a power of two
+                while (tpr * Rv > 512) tpr >>= 1;
+                const int t = sw * 32 + lane, rl = t / tpr, sub = t % tpr;
                 const int gr = rl * cs + rank, node = gr / p.G, h = ckh * p.G + gr % p.G;
                 if (rl < Rv && gr < RT && node < cn) {
                     float mx = -INFINITY;
@@ -739,25 +649,22 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     }
                     const float inv = wsum > 0.f ? 1.0f / wsum : 0.f;
                     const int cols = D / tpr;
-                    for (int g8 = 0; g8 < cols; g8 += 8) {
-                        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                    for (int g4 = 0; g4 < cols; g4 += 4) {
+                        float acc[4] = {0.f, 0.f, 0.f, 0.f};
                         for (int sidx = 0; sidx < cs; ++sidx) {
                             const uint32_t base = recv + (uint32_t)(sidx * Rv + rl) * ROWB;
                             float ms;
                             asm volatile("ld.shared.f32 %0, [%1];" : "=f"(ms) : "r"(base + D * 4u));
                             if (ms == -INFINITY) continue;      // that CTA had no tiles: its row was not written
                             const float w = ex2(ms - mx);
-                            float v[8];
+                            float v[4];
                             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
-                                         : "r"(base + (uint32_t)(sub * cols + g8) * 4u));
-                            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-                                         : "r"(base + (uint32_t)(sub * cols + g8 + 4) * 4u));
+                                         : "r"(base + (uint32_t)(sub * cols + g4) * 4u));
 #pragma unroll
-                            for (int k = 0; k < 8; ++k) acc[k] += w * v[k];
+                            for (int k = 0; k < 4; ++k) acc[k] += w * v[k];
                         }
-                        __nv_bfloat16* op = p.out + (((size_t)cb_ * p.T + node) * p.Hq + h) * D + sub * cols + g8;
-                        *reinterpret_cast<uint4*>(op) = make_uint4(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv),
-                                                                   pack_bf16(acc[4] * inv, acc[5] * inv), pack_bf16(acc[6] * inv, acc[7] * inv));
+                        __nv_bfloat16* op = p.out + (((size_t)cb_ * p.T + node) * p.Hq + h) * D + sub * cols + g4;
+                        *reinterpret_cast<uint2*>(op) = make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
                     }
                     if (sub == 0 && p.lse)
                         p.lse[((size_t)cb_ * p.Hq + h) * p.T + node] = wsum > 0.f ? (mx + log2f(wsum)) * 0.6931471805599453f : 0.f;
@@ -924,7 +831,7 @@ int pick_cluster_size(const CbAttnParams& p, int num_sms) {
         const long long in_cluster = (p.max_tiles + cs - 1) / cs, stream_k = units * (p.max_tiles + 2) / num_sms + 3;
         if (in_cluster >= stream_k) continue;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(units * cs)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = Cfg<D>::SMEM_ALLOC;
+        cfg.gridDim = dim3((unsigned)(units * cs)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = Cfg<D>::SMEM;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = (unsigned)cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -1002,7 +909,7 @@ cb_status launch(CbAttnParams p, const TcMaps& maps, cudaStream_t st, int num_sm
         std::lock_guard<std::mutex> lock(g_launch_mutex);
         const int di = device >= 0 && device < kMaxDevices ? device : -1;
         if (di < 0 || !g_attr_set[D == 128][di]) {
-            CB_CUDA(cudaFuncSetAttribute(cb_attn_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<D>::SMEM_ALLOC));
+            CB_CUDA(cudaFuncSetAttribute(cb_attn_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<D>::SMEM));
             if (di >= 0) g_attr_set[D == 128][di] = true;
         }
         // the choice depends on the shape only
@@ -1022,7 +929,7 @@ cb_status launch(CbAttnParams p, const TcMaps& maps, cudaStream_t st, int num_sm
     }
     if (p.cs > 0) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(p.B * p.Hkv * p.cs)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = Cfg<D>::SMEM_ALLOC; cfg.stream = st;
+        cfg.gridDim = dim3((unsigned)(p.B * p.Hkv * p.cs)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = Cfg<D>::SMEM; cfg.stream = st;
         cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = (unsigned)p.cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -1033,7 +940,7 @@ cb_status launch(CbAttnParams p, const TcMaps& maps, cudaStream_t st, int num_sm
         cb_count_launch(1);
         return CB_OK;
     }
-    CB_CUDA(cb_launch_pdl(cb_attn_tc_kernel<D>, dim3(p.nc), dim3(kThreads), Cfg<D>::SMEM_ALLOC, st, p, maps));
+    CB_CUDA(cb_launch_pdl(cb_attn_tc_kernel<D>, dim3(p.nc), dim3(kThreads), Cfg<D>::SMEM, st, p, maps));
     CB_CUDA(cb_launch_pdl(cb_attn_merge_kernel<D>, dim3(p.nc, 4), dim3(256), 0, st, p));
     cb_count_launch(2);
     CB_CUDA(cudaGetLastError());

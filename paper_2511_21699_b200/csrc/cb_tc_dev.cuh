@@ -11,7 +11,7 @@ namespace {
 constexpr long long kWaitCycles = 1ll << 32;     // bound of every wait, in SM clock cycles (about two seconds)
 constexpr uint32_t kSuspendNs = 20000;
 constexpr float kRowSumLimit = 1048576.f;        // a tile's row sum of P above which the row takes a new reference maximum
-constexpr int kThreads = 384;
+constexpr int kThreads = 640;
 constexpr uint32_t kTmemCols = 512;
 
 struct TcMaps { CUtensorMap k_pool, v_pool, k_tree, v_tree, q; };
@@ -146,6 +146,9 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
                  "%13, %14, %15}, [%16];" : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]),  \
                  "=r"(a[6]), "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), \
                  "=r"(a[14]), "=r"(a[15]) : "r"(taddr) : "memory")
+#define CB_TMEM_WAIT_LD16(a)                                                                                         \
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), \
+                 "+r"(a[7]), "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15]) :: "memory")
 #define CB_TMEM_ST16(a, o, taddr)                                                                                    \
     asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, " \
                  "%12, %13, %14, %15};" ::"r"(a[o + 0]), "r"(a[o + 1]), "r"(a[o + 2]), "r"(a[o + 3]), "r"(a[o + 4]),  \
@@ -181,6 +184,29 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
     uint64_t d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
+}
+// 2^x of a pair on the FMA and integer pipes, for the share of a tile's exponentials that the exponential unit (a warp instruction
+// every 8 cycles) would hold up: x = n + f with n the nearest whole number (added and taken off again as 1.5 * 2^23), 2^f on
+// [-0.5, 0.5] by the degree-5 polynomial of smallest relative error (Remez exchange: 7.5e-8, against 2^-22 of ex2.approx), n
+// added to the exponent.  x is clamped to [-126, 127]: below, 2^-126 stands for what would round to nothing beside the row's
+// sum; above, 2^127 sends the tile to the two-pass form like any sum over its limit.
+__device__ __forceinline__ void ex2_pair_fma(uint64_t x, float& a, float& b) {
+    float x0, x1;
+    f2_unpack(x, x0, x1);
+    x = f2_pack(fminf(fmaxf(x0, -126.f), 127.f), fminf(fmaxf(x1, -126.f), 127.f));
+    const uint64_t r = f2_add(x, f2_pack(12582912.f, 12582912.f));
+    const uint64_t f = f2_fma(f2_add(r, f2_pack(-12582912.f, -12582912.f)), f2_pack(-1.f, -1.f), x);
+    uint64_t y = f2_pack(1.3276472454890609e-3f, 1.3276472454890609e-3f);
+    y = f2_fma(y, f, f2_pack(9.675540961325169e-3f, 9.675540961325169e-3f));
+    y = f2_fma(y, f, f2_pack(5.550713092088699e-2f, 5.550713092088699e-2f));
+    y = f2_fma(y, f, f2_pack(2.4022120237350464e-1f, 2.4022120237350464e-1f));
+    y = f2_fma(y, f, f2_pack(6.931469440460205e-1f, 6.931469440460205e-1f));
+    y = f2_fma(y, f, f2_pack(1.f, 1.f));
+    float y0, y1, r0, r1;
+    f2_unpack(y, y0, y1);
+    f2_unpack(r, r0, r1);
+    a = __int_as_float(__float_as_int(y0) + (__float_as_int(r0) << 23));
+    b = __int_as_float(__float_as_int(y1) + (__float_as_int(r1) << 23));
 }
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
     float d;
@@ -243,6 +269,51 @@ __device__ __forceinline__ void mma_pv_block(uint32_t d_tmem, uint32_t p_tmem, u
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, pa;\n\t"
         CB_MMA_TS_STEP(1) CB_MMA_TS_STEP(2) CB_MMA_TS_STEP(3) CB_MMA_TS_STEP(4) CB_MMA_TS_STEP(5) CB_MMA_TS_STEP(6) CB_MMA_TS_STEP(7) "}"
         ::"r"(d_tmem), "r"(p_tmem), "r"(vlo), "r"(kDescHi), "r"(idesc), "r"(accum) : "memory");
+}
+
+// The same with P in two halves of 64 keys, the second one 64 columns after the first (each half overlays the scores it came from).
+#define CB_MMA_TSH_STEP(K)                                                                                           \
+    "add.u32 ra, %1, 8 * " #K " + 32 * (" #K " / 4);\n\tadd.u32 rb, %2, 128 * " #K ";\n\tmov.b64 db, {rb, %3};\n\t"  \
+    "tcgen05.mma.cta_group::1.kind::f16 [%0], [ra], db, %4, pt;\n\t"
+__device__ __forceinline__ void mma_pv_halves_block(uint32_t d_tmem, uint32_t p_tmem, uint32_t vlo, uint32_t idesc, uint32_t accum) {
+    asm volatile(
+        "{\n\t.reg .pred pt, pa;\n\t.reg .b64 db;\n\t.reg .b32 ra, rb;\n\t"
+        "setp.eq.u32 pt, %4, %4;\n\tsetp.ne.u32 pa, %5, 0;\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, pa;\n\t"
+        CB_MMA_TSH_STEP(1) CB_MMA_TSH_STEP(2) CB_MMA_TSH_STEP(3) CB_MMA_TSH_STEP(4) CB_MMA_TSH_STEP(5) CB_MMA_TSH_STEP(6) CB_MMA_TSH_STEP(7) "}"
+        ::"r"(d_tmem), "r"(p_tmem), "r"(vlo), "r"(kDescHi), "r"(idesc), "r"(accum) : "memory");
+}
+
+// One lane of a converged warp; the compiler knows that a single thread runs what the result guards (a tcgen05.mma issues every
+// 40 to 50 cycles that way and every 60 from `if (lane == 0)`, a commit takes 54 instead of 76).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0u;
+}
+// Barrier of the two warps that share 32 rows, with the OR of their predicates.
+__device__ __forceinline__ bool pair_or(int id, bool v) {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %2, 0;\n\tbar.red.or.pred q, %1, 64, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r) : "r"(id), "r"((uint32_t)v) : "memory");
+    return r != 0u;
+}
+__device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+// W consecutive columns of this thread's TMEM lane (W = 16 or 32), waited for.
+template <int W>
+__device__ __forceinline__ void tmem_ld_w(uint32_t* a, uint32_t taddr) {
+    if constexpr (W == 32) {
+        CB_TMEM_LD32(a, 0, taddr);
+        CB_TMEM_WAIT_LD32(a);
+    } else {
+        CB_TMEM_LD16(a, taddr);
+        CB_TMEM_WAIT_LD16(a);
+    }
+}
+template <int W>
+__device__ __forceinline__ void tmem_st_w(const uint32_t* a, uint32_t taddr) {
+    if constexpr (W == 32) { CB_TMEM_ST32(a, 0, taddr); } else { CB_TMEM_ST16(a, 0, taddr); }
 }
 
 template <int REGS> __device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS)); }

@@ -9,11 +9,14 @@
 // values (one (sequence, kv head), all its row groups) then lie a fixed fraction of the whole sequence apart, so that they
 // are worked on at the same time by different CTAs and the keys and values are fetched from HBM once and found in L2 by
 // the others; with the row group innermost one CTA would stream them again and again, each time after everything else
-// it holds has passed through L2.  Starting a unit costs about as much as two or
-// three tiles (query load, pipeline refill, epilogue), so every unit is preceded by that many padding positions in the
-// sequence: they carry no work, they only make a CTA that handles many short units receive fewer tiles.  A CTA therefore finishes whole
-// units, plus at most one unit it shares with earlier CTAs and one it shares with later CTAs; shared
-// units leave unnormalised partials that the merge pass combines.
+// it holds has passed through L2.  A key tile of a unit with two row tiles takes twice as long as one of a unit with one
+// (3.4 k against 1.8 k cycles: the two softmax chains share the latter's tiles), so a tile counts w2 = 2 or w1 = 1 positions of the
+// sequence (batch 13 of small trees, head_dim 64: with one position each the CTAs ended between 42 k and 92 k cycles).  Starting a
+// unit costs about as much as two or three tiles (query load, pipeline refill, epilogue), so every unit is preceded by that many
+// padding positions: they carry no work, they only make a CTA that handles many short units receive fewer tiles.  A tile
+// belongs to the CTA whose range holds its first position.  A CTA therefore finishes whole units, plus at most one unit it shares
+// with earlier CTAs and one it shares with later CTAs; the CTAs of a shared unit combine unnormalised partials (in the kernel, or
+// in the merge pass of the CTA-pair kernel, which counts one position per tile).
 #pragma once
 #include "cb_common.cuh"
 
@@ -32,11 +35,13 @@ struct CbAttnParams {
     const int32_t* n_nodes;
     __nv_bfloat16* out;
     float* lse;
-    float* part;          // [2 * nc slots][2 row tiles][128 rows][D + 4]: unnormalised O row, running max (log2 domain), sum
+    float* part;          // [2 * nc slots] of 2 * 128 * (D + 4) floats: unnormalised output columns, running max (log2 domain), sum
+    uint32_t* part_ticket; // [nc][16 softmax warps]: parts of a shared unit left in memory so far, zero between calls
     int B, T, W, Hq, Hkv, G, D, P, max_pages, num_pages;
     int NPT;              // tree nodes per row tile = 128 / G
     int MT;               // row tiles that T nodes need = ceil(T / NPT)
     int nc;               // persistent CTAs (= ranges of the global tile sequence)
+    int w1, w2;           // positions that a key tile of a unit with one or with two row tiles counts
     int max_tiles;        // host's upper bound on the key tiles of a unit (from max_ctx, else from the block table's width)
     int cs;               // > 0: cluster mode, one unit per cluster of cs CTAs (see cb_attn_tc.cu); 0: the stream-K split
     float scale_log2;     // softmax scale * log2(e)
@@ -46,10 +51,15 @@ struct CbAttnParams {
 // Per-sequence shape of the decomposition.
 struct CbSeqShape {
     int n, ctx, tiles, mtn, RG;
-    int ov;               // padding positions in front of each unit of this sequence
+    int w1, w2;
+    bool one;             // the launch has one row tile per unit throughout
     long long W;          // positions (padding + key tiles) of all units of this sequence
+    __device__ __forceinline__ bool two_rows(int rg) const { return !one && mtn - 2 * rg >= 2; }
+    __device__ __forceinline__ int wt(int rg) const { return two_rows(rg) ? w2 : w1; }              // positions per key tile
+    __device__ __forceinline__ int ov(int rg) const { return two_rows(rg) ? 3 * w2 : 2 * w1; }      // padding positions in front of a unit
+    __device__ __forceinline__ int unit(int rg) const { return tiles * wt(rg) + ov(rg); }           // positions of one unit
     // positions of this sequence's units of row group rg (all kv heads); 0 if the tree has no such row group
-    __device__ __forceinline__ long long w_of(int Hkv, int rg) const { return rg < RG ? (long long)Hkv * (tiles + ov) : 0ll; }
+    __device__ __forceinline__ long long w_of(int Hkv, int rg) const { return rg < RG ? (long long)Hkv * unit(rg) : 0ll; }
 };
 
 __device__ __forceinline__ CbSeqShape cb_seq_shape(const CbAttnParams& p, int b) {
@@ -58,15 +68,22 @@ __device__ __forceinline__ CbSeqShape cb_seq_shape(const CbAttnParams& p, int b)
     s.ctx = min(max(p.ctx_len[b], 0), p.max_pages * p.P);
     s.tiles = (s.ctx + CB_KT - 1) / CB_KT + 1;
     s.mtn = (s.n + p.NPT - 1) / p.NPT;
-    s.RG = p.MT == 1 ? (s.mtn > 0 ? 1 : 0) : (s.mtn + 1) / 2;
-    s.ov = s.mtn >= 2 ? 3 : 2;
-    s.W = (long long)p.Hkv * s.RG * (s.tiles + s.ov);
+    s.one = p.MT == 1;
+    s.RG = s.one ? (s.mtn > 0 ? 1 : 0) : (s.mtn + 1) / 2;
+    s.w1 = p.w1; s.w2 = p.w2;
+    // every row group but the last has two row tiles
+    s.W = s.RG > 0 ? (long long)p.Hkv * ((long long)(s.RG - 1) * s.unit(0) + s.unit(s.RG - 1)) : 0;
     return s;
 }
 
-__device__ __forceinline__ long long cb_range_start(long long total, int nc, int c) { return total * c / nc; }
+// a / b for a >= 0, b > 0: 32 bits wide where that does (the 64-bit division is some 100 instructions, four of them in a row at
+// the start of every CTA).
+__device__ __forceinline__ long long cb_div(long long a, long long b) {
+    return ((unsigned long long)a | (unsigned long long)b) >> 32 ? a / b : (long long)((uint32_t)a / (uint32_t)b);
+}
+__device__ __forceinline__ long long cb_range_start(long long total, int nc, int c) { return cb_div(total * c, nc); }
 // CTA whose range holds global tile x.
-__device__ __forceinline__ int cb_cta_of(long long total, int nc, long long x) { return (int)(((x + 1) * nc - 1) / total); }
+__device__ __forceinline__ int cb_cta_of(long long total, int nc, long long x) { return (int)cb_div((x + 1) * nc - 1, total); }
 
 // Row groups a launch can have per sequence (trees of max_nodes nodes).
 __device__ __forceinline__ int cb_max_row_groups(const CbAttnParams& p) { return p.MT == 1 ? 1 : (p.MT + 1) / 2; }
@@ -157,14 +174,14 @@ struct CbWalker {
                 w = s.w_of(p.Hkv, rg);
             }
             const long long off = g - pre;
-            const int vt = s.tiles + s.ov;                    // positions of one unit
-            const int kh = (int)(off / vt);
+            const int vt = s.unit(rg), wt = s.wt(rg), ov = s.ov(rg);
+            const int kh = (int)cb_div(off, vt);
             const int v0 = (int)(off - (long long)kh * vt);
             const int v1 = (int)min((long long)vt, (long long)v0 + (g1 - g));
             g += v1 - v0;
-            u->t0 = max(v0 - s.ov, 0);
-            u->t1 = max(v1 - s.ov, 0);
-            if (u->t1 <= u->t0) continue;                     // only padding of this unit falls into the range
+            u->t0 = (max(v0 - ov, 0) + wt - 1) / wt;
+            u->t1 = (max(v1 - ov, 0) + wt - 1) / wt;
+            if (u->t1 <= u->t0) continue;                     // no tile of this unit begins in the range
             u->b = b; u->kh = kh; u->rg = rg; u->tiles = s.tiles; u->n = s.n; u->ctx = s.ctx;
             u->nrt = p.MT == 1 ? 1 : min(2, s.mtn - 2 * rg);
             return true;

@@ -29,17 +29,20 @@
 //
 // Cluster mode.  When a launch has so few units that the split above would make every unit a shared one (batch 1), the
 // kernel is launched as thread-block clusters instead: cluster k works on unit k, its CTAs take equal parts of the unit's
-// key tiles, and at the end they combine their shares through distributed shared memory: row i of the 128 rows is
-// gathered in CTA i mod cs, which merges the contributions and writes the output.  No partials go to HBM and no merge pass runs.
+// key tiles, and at the end they combine their shares through distributed shared memory: every CTA gathers D / cs columns of
+// all rows, merges the contributions and writes the output.  No partials go to HBM.
 #include <cuda.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "cb_tc_dev.cuh"
 
 namespace {
 
-struct UnitDesc { int b, kh, rg, t0, t1, tiles, n, ctx, nrt, pad; };   // nrt = 0: no more units
+// A unit as the softmax warps see it (nrt = 0: no more units).  cf, np: the CTA that holds the unit's first key tile and the number of
+// CTAs that hold one; xpos: position of that tile where a CTA holds one tile at most, else -1.
+struct UnitDesc { int b, kh, rg, t0, t1, tiles, n, ctx, nrt, cf, np, xpos, wt, pad; };
 constexpr int kFmaExpPhase = 3;                              // of every four pairs of exponentials this one is taken by the FMA pipe
 constexpr int kUnitRing = 4;                                 // units published ahead of the slowest softmax thread: at most two
 
@@ -72,6 +75,22 @@ static_assert(sizeof(SchedSmem) <= 64, "the schedule block is followed by the tm
 
 namespace {
 
+// What a CTA of a cluster receives: from every source CTA the columns it owns, in groups of 4 (16 bytes), the rows of a group side
+// by side (one more than there are, so that reading along the groups meets no bank twice), then every row's reference and sum.
+struct CbExchange {
+    int rows;              // rows of the unit's tree, in whole warps
+    uint32_t bytes;        // room for them
+    __device__ __forceinline__ uint32_t expected(int cs, int D) const { return (uint32_t)(rows * (D * 4 + cs * 8)); }   // bytes that arrive
+    __device__ __forceinline__ uint32_t value(int src, int ch, int row, int nch) const { return (uint32_t)(((src * nch + ch) * (rows + 1) + row) * 16); }
+    __device__ __forceinline__ uint32_t sums(int src, int row, int cs, int nch) const { return (uint32_t)(cs * nch * (rows + 1) * 16 + (src * rows + row) * 8); }
+};
+__device__ __forceinline__ CbExchange cb_exchange(const CbAttnParams& p, int D, int n) {
+    CbExchange e;
+    e.rows = (min(p.NPT, n) * p.G + 31) & ~31;
+    e.bytes = (uint32_t)(D / 4 * (e.rows + 1) * 16 + p.cs * e.rows * 8);
+    return e;
+}
+
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
@@ -102,15 +121,15 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
     SchedSmem* s_sched = reinterpret_cast<SchedSmem*>(sgen + C::OFF_MISC);
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sgen + C::OFF_MISC + 64);
     volatile int* s_abort = reinterpret_cast<volatile int*>(sgen + C::OFF_MISC + 68);
-    volatile int* s_pair = reinterpret_cast<volatile int*>(sgen + C::OFF_MISC + 96);   // [16 softmax warps]: pair barriers entered, -1 = left
+    long long* s_tot = reinterpret_cast<long long*>(sgen + C::OFF_MISC + 72);   // positions of the global tile sequence
+    volatile int* s_pair = reinterpret_cast<volatile int*>(sgen + C::OFF_MISC + 96);   // [16 softmax warps]: last pair barrier entered, -1 = left
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cta = blockIdx.x;
     const int RT = p.NPT * p.G;                               // rows of a row tile that exist
     // Set-up that reads no input (TMEM allocation, barrier initialisation, descriptor prefetch) runs before the wait for the
-    // kernels earlier in the stream, so it overlaps their tail.  The merge pass (like the next kernel of a step) is launched as
-    // a programmatic dependent in turn: its blocks may take the SMs that this grid's CTAs leave and do their set-up there;
-    // they wait for this whole grid before they read any partial.
+    // kernels earlier in the stream, so it overlaps their tail.  The next kernel of a step is launched as a programmatic dependent in
+    // turn: its blocks may take the SMs that this grid's CTAs leave and do their set-up there.
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -124,7 +143,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             }
             mbar_init(bar_odone_both, 1); mbar_init(bar_sums, 512);
             for (int k = 0; k < kUnitRing; ++k) mbar_init(bar_ufull(k), 1);
-            mbar_init(bar_cready, p.cs > 0 ? (uint32_t)p.cs : 1u); mbar_init(bar_cdata, 512);
+            mbar_init(bar_cready, p.cs > 0 ? (uint32_t)p.cs : 1u); mbar_init(bar_cdata, 1);
             *s_abort = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             tma_prefetch_desc(&maps.k_pool); tma_prefetch_desc(&maps.v_pool); tma_prefetch_desc(&maps.q);
@@ -133,6 +152,13 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
         if (lane < 16) s_pair[lane] = 0;
     }
     CB_PDL_ENTRY();
+    if (warp == 3) {
+        // The block table into L2, a slice per CTA: the first copies' addresses come from it, and which part of it a CTA needs is
+        // known only after the schedule below (two memory round trips one after the other otherwise).
+        const long long lines = ((long long)p.B * p.max_pages * 4 + 127) / 128;
+        for (long long k = (long long)cta * 32 + lane, n = 0; k < lines && n < 4; k += (long long)gridDim.x * 32, ++n)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p.block_table) + k * 128));
+    }
 
     if (warp == 0 && p.cs > 0) {
         // Cluster mode: cluster k works on unit k = (sequence, kv head) and its CTAs take equal parts of the unit's key tiles.
@@ -153,18 +179,19 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
         int b0 = 0, rg0 = 0;
         long long pre0 = 0;
         if (g0 < g1) cb_sched_locate(p, g0, lane, &rg0, &b0, &pre0);
-        if (lane == 0) { s_sched->g0 = g0; s_sched->g1 = g1; s_sched->b0 = b0; s_sched->rg0 = rg0; s_sched->pre0 = pre0; }
+        if (lane == 0) { s_sched->g0 = g0; s_sched->g1 = g1; s_sched->b0 = b0; s_sched->rg0 = rg0; s_sched->pre0 = pre0; *s_tot = tot; }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
     constexpr uint32_t ns = (uint32_t)C::NSLOT;
-    if (p.cs > 0) {
-        // the peers' barriers must exist before anything arrives on them
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
+    // Cluster mode: the peers' barriers must exist before anything arrives on them.  Every thread reports here and waits where its
+    // role first reaches over, or at its end (a CTA must not leave before the others' report either).
+    if (p.cs > 0) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    auto cluster_wait = [&]() {
+        if (p.cs > 0) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    };
 
     if (warp < 4) {
         reg_dealloc<64>();
@@ -180,12 +207,14 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
         CbUnit u;
         if (warp == 0 || warp == 3) {
             // ------------------------------------------------------------------ K/V producers: warp 0 the K tiles, warp 3 the V tiles
-            // A tile is 8 * DB boxes of 16 keys x 64 dims, one copy instruction each, and the copies of one warp instruction
-            // are issued one after the other: two warps issue the two tiles of a key tile side by side.
+            // A page's 16 keys are one box, laid out in shared memory as groups of 8 keys with a group's 64-dim column blocks
+            // behind one another (which is why the products' descriptors step by 1024 * DB from group to group).  The copies of
+            // a warp instruction are issued one after the other, some 80 cycles each: eight a tile, and the two tiles of a key
+            // tile by a warp each.  The tree's own keys are boxes of 8 rows (max_nodes need not be a multiple of 16).
             const bool isV = warp == 3;
-            constexpr int NB = 8 * C::DB;                    // boxes per tile
-            const bool active = lane < NB;
-            const int j = lane % 8, dblk = (lane % NB) / 8;
+            constexpr uint32_t GROUP = 1024 * C::DB;         // bytes of 8 keys
+            const bool active = lane < 8;
+            const int j = lane % 8;
             uint32_t seq = isV ? 1u : 0u;                    // K and V tiles alternate in the ring
             bool ok = true;
             const uint64_t pol = l2_evict_first_policy();
@@ -211,10 +240,10 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     if (seq >= ns && !(ok = mbar_wait(bar_free(sl), (seq / ns - 1) & 1, s_abort, p.status))) break;
                     if (lane == 0) mbar_expect_tx(bar_full(sl), C::TILE_BYTES);
                     __syncwarp();
-                    if (active) {
-                        const uint32_t dst = slot_base(sl) + dblk * (CB_KT * 128) + j * 2048;
-                        if (i < nct) tma_load_4d_hint(dst, isV ? &maps.v_pool : &maps.k_pool, bar_full(sl), dblk * 64, u.kh, 0, page, pol);
-                        else tma_load_4d(dst, isV ? &maps.v_tree : &maps.k_tree, bar_full(sl), dblk * 64, u.kh, 16 * j, u.b);
+                    if (i < nct) {
+                        if (active) tma_load_5d_hint(slot_base(sl) + j * 2 * GROUP, isV ? &maps.v_pool : &maps.k_pool, bar_full(sl), 0, 0, 0, page * 2, u.kh, pol);
+                    } else if (lane < 16) {
+                        tma_load_5d(slot_base(sl) + lane * GROUP, isV ? &maps.v_tree : &maps.k_tree, bar_full(sl), 0, 8 * lane, 0, u.kh, u.b);
                     }
                     seq += 2;
                 }
@@ -241,7 +270,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                                 ++c_p[l];
                                 if (e < 4 && uq > 0 && !(ok = mbar_wait(bar_ofree(l), (uq - 1) & 1, s_abort, p.status))) break;
                                 tc_fence_after();
-                                mma_pv_halves_block(tmem + C::O_COL + l * D, tmem + l * 128, desc_lo(slot_base(vs), CB_KT * 128), idesc_o, e < 4 ? 0u : 1u);
+                                mma_pv_halves_block<D>(tmem + C::O_COL + l * D, tmem + l * 128, desc_lo(slot_base(vs), 1024), idesc_o, e < 4 ? 0u : 1u);
                                 if (!two || l == 1) tc_commit(bar_free(vs));
                                 if (two ? iv == nt - 1 : iv == nt - 1) tc_commit(two ? bar_odone(l) : bar_odone_both);
                             }
@@ -252,7 +281,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                                 if (!(ok = mbar_wait(bar_full(ks), (kseq / ns) & 1, s_abort, p.status))) break;
                                 tc_fence_after();
                             }
-                            mma_s_block<D>(tmem + l * 128, desc_lo(sbase + C::OFF_Q + (two ? l : 0) * C::Q_BYTES, 16), desc_lo(slot_base(ks), 16), idesc_s);
+                            mma_s_grouped_block<D>(tmem + l * 128, desc_lo(sbase + C::OFF_Q + (two ? l : 0) * C::Q_BYTES, 16), desc_lo(slot_base(ks), 16), idesc_s);
                             tc_commit(bar_sfull(l));
                             if (!two || l == 1) {
                                 tc_commit(bar_free(ks));
@@ -268,12 +297,25 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             }
         } else {
             // ------------------------------------------------------------------ units for the softmax warps, query tiles
+            uint32_t uq = 0;
             if (lane == 0) {
-                uint32_t uq = 0;
                 bool ok = true;
                 while (ok && wk.next(p, &u)) {
                     volatile UnitDesc* d = &s_units[uq % kUnitRing];
                     d->b = u.b; d->kh = u.kh; d->rg = u.rg; d->t0 = u.t0; d->t1 = u.t1; d->tiles = u.tiles; d->n = u.n; d->ctx = u.ctx; d->nrt = u.nrt;
+                    if (p.cs == 0 && !(u.t0 == 0 && u.t1 == u.tiles)) {
+                        // a unit shared with other CTAs: who holds its first tile, and how many of them there are
+                        // (ranges of at least one tile's positions: the CTAs from the first tile's to the last one's; shorter ranges
+                        // hold the beginning of one tile at most, so every tile has a CTA of its own)
+                        const int wt = wk.s.wt(u.rg);
+                        const long long tot = *s_tot, x0 = wk.pre + (long long)u.kh * wk.s.unit(u.rg) + wk.s.ov(u.rg);
+                        const int cf = cb_cta_of(tot, p.nc, x0);
+                        const bool wide = tot >= (long long)p.nc * wt;
+                        d->cf = cf;
+                        d->np = wide ? cb_cta_of(tot, p.nc, x0 + (long long)(u.tiles - 1) * wt) - cf + 1 : u.tiles;
+                        d->xpos = wide ? -1 : (int)x0;
+                        d->wt = wt;
+                    }
                     mbar_arrive(bar_ufull(uq % kUnitRing));
                     if (uq > 0 && !(ok = mbar_wait(bar_qfree, (uq - 1) & 1, s_abort, p.status))) break;
                     mbar_expect_tx(bar_qfull, (uint32_t)(u.nrt * C::DB * RT * 128));
@@ -287,11 +329,15 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     s_units[uq % kUnitRing].nrt = 0;
                     mbar_arrive(bar_ufull(uq % kUnitRing));
                 }
+            }
+            __syncwarp();
+            cluster_wait();
+            if (lane == 0) {
                 if (p.cs > 0 && s_sched->c_has) {
+                    mbar_expect_tx(bar_cdata, cb_exchange(p, D, s_sched->c_n).expected(p.cs, D));
                     // Cluster mode: the peers write their rows into this CTA's query tiles, so it reports itself ready to
                     // receive as soon as its last S product has released them (before its last P.V is done).
-                    const int Rv = (min(RT, p.T * p.G) + p.cs - 1) / p.cs;
-                    if ((uint32_t)(p.cs * Rv) * (uint32_t)((D + 4) * 4) <= 2u * C::Q_BYTES) {
+                    if (cb_exchange(p, D, s_sched->c_n).bytes <= 2u * C::Q_BYTES) {
                         if (uq == 0 || mbar_wait(bar_qfree, 0, s_abort, p.status))
                             for (int r = 0; r < p.cs; ++r) mbar_arrive_remote(cluster_addr(bar_cready, (uint32_t)r));
                     }
@@ -299,6 +345,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             }
         }
         __syncwarp();
+        if (warp != 2) cluster_wait();
     } else {
         // ---------------------------------------------------------------------- softmax / correction / epilogue
         reg_alloc<104>();
@@ -308,6 +355,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
         const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
         const int pair_id = 1 + l * 4 + wq;                   // named barrier of the two warps that share these rows
         constexpr int CW = D / 4;                             // accumulator columns handled at a time
+        const bool out32 = (reinterpret_cast<uintptr_t>(p.out) & 31u) == 0;   // output rows may be written 32 bytes at a time
         {
             // rows of padding nodes (node >= n_nodes) are written as zeros while the first tiles are on their way
             const int per_row = p.Hq * D / 8;                 // 16-byte chunks per node row
@@ -320,17 +368,16 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                 if (p.lse) for (int h = lane; h < p.Hq; h += 32) p.lse[((size_t)b * p.Hq + h) * p.T + nd] = 0.f;
             }
         }
-        int entered = 0;                                      // pair barriers entered
-        auto pair_sync = [&](bool v) {
-            ++entered;
-            if (lane == 0) s_pair[sw] = entered;
+        uint32_t c_s = 0, c_od = 0, c_ob = 0, uq = 0;                 // completions consumed: S of this chain, o_done of this chain, o_done_both
+        // The pair's barrier; k numbers the barriers between two tiles, so that what a warp notes before it waits only grows.
+        auto pair_sync = [&](bool v, uint32_t k) {
+            if (lane == 0) s_pair[sw] = (int)(4u * (c_s + uq) + k);
             return pair_or(pair_id, v);
         };
-        uint32_t c_s = 0, c_od = 0, c_ob = 0;                 // completions consumed: S of this chain, o_done of this chain, o_done_both
         bool ok = true;
         float x_m = -INFINITY, x_l = 0.f, x_w0 = 0.f, x_w1 = 0.f;   // one-row-tile unit: combined reference and sum, weights of O0 and O1
-        bool c_share = false;                                 // cluster mode: this CTA has a share of the unit
-        for (uint32_t uq = 0; ok; ++uq) {
+        bool c_share = false, x_two = false;                  // cluster mode: this CTA has a share of the unit, and of two tiles or more
+        for (; ok; ++uq) {
             if (!(ok = mbar_wait(bar_ufull(uq % kUnitRing), (uq / kUnitRing) & 1, s_abort, p.status))) break;
             const volatile UnitDesc* u = &s_units[uq % kUnitRing];   // read again where it is needed: registers are short
             if (u->nrt == 0) break;
@@ -393,21 +440,21 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                         m_used = fmaxf(c0, c1) * p.scale_log2;   // -inf if the row sees none of them
                     }
                     uint32_t pk[32];
-                    // P of this thread's 64 scores (packed into pk) against reference mu; returns their sum.  16 scores at a time with
-                    // the next 16 in flight: a thread has 96 registers, and what does not fit them spills past an L1 that the
-                    // tiles leave 28 KB.
-                    auto make_p = [&](float mu) {
+                    // P of this thread's 64 scores (packed into pk) against reference mu; returns their sum.  32 scores at a time:
+                    // a thread has 96 registers, and what does not fit them spills past an L1 that the tiles leave 28 KB (with all 64
+                    // scores in registers batch 32 took 256 us; with the next 16 in flight it takes what it takes without).
+                    // The form without masks is code of its own: a branch per 16 scores keeps the compiler from overlapping
+                    // one group's exponentials with the next one's (1,274 against 1,115 cycles a tile for this loop alone).
+                    auto make_p_of = [&](float mu, auto masked) {
+                        constexpr bool MASKED = decltype(masked)::value;
                         const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2), negmu2 = f2_pack(-mu, -mu);
                         uint64_t lsa = f2_pack(0.f, 0.f), lsb = f2_pack(0.f, 0.f);
-                        uint32_t sa[16], sb[16];
-                        CB_TMEM_LD16(sa, tsh);
+                        uint32_t sa[32];
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
-                            uint32_t* cur = (c & 1) ? sb : sa;
-                            uint32_t* nxt = (c & 1) ? sa : sb;
-                            CB_TMEM_WAIT_LD16(cur);
-                            if (c < 3) CB_TMEM_LD16(nxt, tsh + 16 * (c + 1));
-                            if (!all_vis) {
+                            uint32_t* cur = sa + 16 * (c & 1);
+                            if ((c & 1) == 0) { CB_TMEM_LD32(sa, 0, tsh + 16 * c); CB_TMEM_WAIT_LD32(sa); }
+                            if (MASKED) {
 #pragma unroll
                                 for (int jx = 0; jx < 16; ++jx)
                                     if (!((vm[c >> 1] >> ((c & 1) * 16 + jx)) & 1u)) cur[jx] = 0xFF800000u;
@@ -416,7 +463,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                             for (int q = 0; q < 8; ++q) {
                                 const uint64_t x = f2_fma(f2_pack(__uint_as_float(cur[2 * q]), __uint_as_float(cur[2 * q + 1])), scale2, negmu2);
                                 float p0, p1;
-                                if (q % 4 == kFmaExpPhase) {
+                                if (!MASKED && q % 4 == kFmaExpPhase) {
                                     ex2_pair_fma(x, p0, p1);
                                 } else {
                                     f2_unpack(x, p0, p1);
@@ -432,8 +479,11 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                         f2_unpack(lsb, l2, l3);
                         return (l0 + l1) + (l2 + l3);
                     };
+                    auto make_p = [&](float mu) {
+                        return all_vis ? make_p_of(mu, std::false_type{}) : make_p_of(mu, std::true_type{});
+                    };
                     float lt = make_p(m_used == -INFINITY ? 0.f : m_used);
-                    if (pair_sync(row_valid && !(lt <= kRowSumLimit))) {          // rows that do not exist hold anything: they never ask
+                    if (pair_sync(row_valid && !(lt <= kRowSumLimit), 0)) {          // rows that do not exist hold anything: they never ask
                         // pass 1: the row's maximum over all its visible scores (both threads of the row take it)
                         uint32_t va[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
                         if (!all_vis) {
@@ -455,7 +505,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
 #pragma unroll
                             for (int jx = 0; jx < 32; ++jx) mx = fmaxf(mx, ((va[c] >> jx) & 1u) ? __uint_as_float(rf[jx]) : -INFINITY);
                         }
-                        pair_sync(false);                                         // both have read S: either may write P over it now
+                        pair_sync(false, 1);                                      // both have read S: either may write P over it now
                         const float mloc = mx * p.scale_log2;
                         // lazy rescaling: keep the reference maximum until the running maximum exceeds it by 2^8 (a tile that
                         // comes here from the single pass holds a score at least 2^13 above it)
@@ -491,23 +541,29 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             // ---- epilogue of this unit's share
             const int ub = u->b, t0 = u->t0, h = u->kh * p.G + row % p.G;
             const bool whole = t0 == 0 && t1 == u->tiles;
-            // this thread's columns of the output row: with two row tiles half a row in two steps, with one a quarter in one
-            int ncol, c0;
+            // this thread's columns of the output row, 16 at a time: half a row with two row tiles, a quarter with one
+            int npc, c0;
+            // a shared unit: how many parts of it are in memory already (most often all the others, see below); the look is taken here,
+            // where it overlaps the wait for the last product
+            const int np = whole || p.cs > 0 ? 1 : u->np, cf = whole || p.cs > 0 ? 0 : u->cf;
+            uint32_t* const ticket = p.part_ticket + cf * 16 + sw;
+            uint32_t arrived = 0;
+            if (np > 1 && lane == 0) arrived = ld_acquire(ticket);
             if (two) {
                 s_x[(l * 2 + hf) * CB_MT + row] = lsum;
-                pair_sync(false);
+                pair_sync(false, 2);
                 x_l = lsum + s_x[(l * 2 + 1 - hf) * CB_MT + row];
                 x_m = m_used; x_w0 = x_w1 = 1.f;
-                ncol = 2; c0 = hf * 2 * CW;
+                npc = CW / 8; c0 = hf * 2 * CW;
                 if (!(ok = mbar_wait(bar_odone(l), c_od & 1, s_abort, p.status))) break;
                 ++c_od;
             } else {
                 if (!(ok = mbar_wait(bar_odone_both, c_ob & 1, s_abort, p.status))) break;
                 ++c_ob;
                 s_x[(l * 2 + hf) * CB_MT + row] = lsum;
-                pair_sync(false);
+                pair_sync(false, 2);
                 const float lrow = lsum + s_x[(l * 2 + 1 - hf) * CB_MT + row];
-                pair_sync(false);
+                pair_sync(false, 3);
                 s_x[(l * 2 + hf) * CB_MT + row] = hf ? lrow : m_used;
                 mbar_arrive(bar_sums);
                 if (!(ok = mbar_wait(bar_sums, (c_ob - 1) & 1, s_abort, p.status))) break;
@@ -516,56 +572,151 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                 x_w0 = m0 == -INFINITY ? 0.f : ex2(m0 - x_m);
                 x_w1 = m1 == -INFINITY ? 0.f : ex2(m1 - x_m);
                 x_l = l0 * x_w0 + l1 * x_w1;
-                ncol = 1; c0 = (l * 2 + hf) * CW;
+                npc = CW / 16; c0 = (l * 2 + hf) * CW;
             }
             tc_fence_after();
             if (p.cs > 0) {
                 c_share = true;                               // O stays in TMEM until the exchange below
-                x_w1 = t1 - t0 > 1 ? x_w1 : -1.f;             // a share of one tile has no second accumulator
+                x_two = t1 - t0 > 1;                          // a share of one tile has no second accumulator
                 break;                                        // a CTA of a cluster has one share
             }
             if (warp_active) {
-                const float inv = whole ? (x_l > 0.f ? 1.0f / x_l : 0.f) : 1.0f;
-                const float w0 = two ? inv : x_w0 * inv, w1 = x_w1 * inv;
-                const size_t slot = 2 * (size_t)cta + (t0 == 0 ? 1 : 0);
-                float* pp = p.part + ((slot * 2 + (two ? l : 0)) * CB_MT + row) * (D + 4);
                 __nv_bfloat16* op = p.out + (((size_t)ub * p.T + (row_valid ? node : 0)) * p.Hq + h) * D;
+                // 16 of this thread's accumulator columns, relative to reference x_m; with one row tile both accumulators put together
+                auto load_o = [&](float* o, int col) {
+                    uint32_t* r = reinterpret_cast<uint32_t*>(o);
+                    tmem_ld_w<16>(r, tmem + C::O_COL + (two ? l * D : 0) + lane_addr + col);
+                    if (two) return;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) o[k] *= x_w0;
+                    if (t1 - t0 > 1) {
+                        uint32_t o1[16];
+                        tmem_ld_w<16>(o1, tmem + C::O_COL + D + lane_addr + col);
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) o[k] = fmaf(__uint_as_float(o1[k]), x_w1, o[k]);
+                    }
+                };
+                auto store_out = [&](const float* o, int col, float inv) {
+                    if (!row_valid) return;
+                    uint32_t w[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) w[k] = pack_bf16(o[2 * k] * inv, o[2 * k + 1] * inv);
+                    if (out32) {
+                        st_global_v8(op + col, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+                    } else {
+                        *reinterpret_cast<uint4*>(op + col) = make_uint4(w[0], w[1], w[2], w[3]);
+                        *reinterpret_cast<uint4*>(op + col + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+                    }
+                };
+                auto store_lse = [&](float mx, float sum) {
+                    if (row_valid && c0 == 0 && p.lse) p.lse[((size_t)ub * p.Hq + h) * p.T + node] = sum > 0.f ? (mx + log2f(sum)) * 0.6931471805599453f : 0.f;
+                };
+                if (whole) {
+                    const float inv = x_l > 0.f ? 1.0f / x_l : 0.f;
 #pragma unroll 1
-                for (int c = 0; c < ncol; ++c) {
-                    uint32_t o[CW];
-                    const int col = c0 + c * CW;
-                    if (two) {
-                        tmem_ld_w<CW>(o, tm_O + col);
+                    for (int e = 0; e < npc; ++e) {
+                        float o[16];
+                        load_o(o, c0 + 16 * e);
+                        store_out(o, c0 + 16 * e, inv);
+                    }
+                    store_lse(x_m, x_l);
+                } else {
+                    // A unit shared with other CTAs.  The same warp of each of them has the same rows and columns, so the warps settle it
+                    // among themselves: all but the last to come leave their partial (unnormalised columns, reference and sum) in
+                    // memory and count themselves; the last one reads the others', in the order of the CTAs whoever is last, and
+                    // writes the output.  Nobody waits.  (A CTA's first unit is shared with the CTA before it, which comes to it
+                    // last, so most often the partial has long been there: the pass that merged both partials from memory after the
+                    // kernel cost 9 us a call at batch 32.)  A warp's partial is laid out by lane: 512 bytes per access.
+                    const int xpos = u->xpos;
+                    auto slot_of = [&](int cc, bool start) {
+                        return p.part + (size_t)(2 * cc + (start ? 1 : 0)) * (2 * CB_MT * (D + 4));
+                    };
+                    auto part_of = [&](int k) { return slot_of(xpos < 0 ? cf + k : cb_cta_of(*s_tot, p.nc, (long long)xpos + k * u->wt), k == 0); };
+                    const int wofs = sw * (2 * CW * 32) + lane * 4, mlofs = 2 * CB_MT * D + (sw * 32 + lane) * 2;
+                    float* const own = slot_of(cta, t0 == 0);
+                    auto load_part = [&](float4* v, const float* pp, int e) {
 #pragma unroll
-                        for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * w0);
-                    } else {
-                        tmem_ld_w<CW>(o, tmem + C::O_COL + lane_addr + col);
+                        for (int q = 0; q < 4; ++q) v[q] = __ldcg(reinterpret_cast<const float4*>(pp + wofs + (e * 4 + q) * 128));
+                    };
+                    auto load_ml = [&](const float* pp) { return __ldcg(reinterpret_cast<const float2*>(pp + mlofs)); };
+                    auto weight = [](float m, float mx) { return m == -INFINITY ? 0.f : ex2(m - mx); };
+                    bool last = __shfl_sync(CB_FULL, arrived, 0) == (uint32_t)(np - 1);
+                    if (!last) {
+#pragma unroll 1
+                        for (int e = 0; e < npc; ++e) {
+                            float o[16];
+                            load_o(o, c0 + 16 * e);
 #pragma unroll
-                        for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * w0);
-                        if (t1 - t0 > 1) {
-                            uint32_t o1[CW];
-                            tmem_ld_w<CW>(o1, tmem + C::O_COL + D + lane_addr + col);
-#pragma unroll
-                            for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) + __uint_as_float(o1[k]) * w1);
+                            for (int q = 0; q < 4; ++q)
+                                *reinterpret_cast<float4*>(own + wofs + (e * 4 + q) * 128) = make_float4(o[q * 4], o[q * 4 + 1], o[q * 4 + 2], o[q * 4 + 3]);
                         }
+                        *reinterpret_cast<float2*>(own + mlofs) = make_float2(x_m, x_l);
+                        __syncwarp();
+                        if (lane == 0) arrived = atom_add_acq_rel(ticket, 1u);   // releases the whole warp's stores
+                        last = __shfl_sync(CB_FULL, arrived, 0) == (uint32_t)(np - 1);
                     }
-                    if (!row_valid) continue;
-                    if (whole) {
-                        uint32_t w[CW / 2];
+                    if (last) {
+                        __syncwarp();
+                        if (lane == 0) *reinterpret_cast<volatile uint32_t*>(ticket) = 0u;   // for the next call
+                        float mx = -INFINITY, sum = 0.f;
+                        if (np == 2) {
+                            // the usual case: one other part, its columns fetched a group ahead
+                            const bool first = t0 == 0;
+                            const float* const po = part_of(first ? 1 : 0);
+                            float4 v[4], vn[4];
+                            load_part(v, po, 0);
+                            const float2 ml = load_ml(po);
+                            mx = fmaxf(x_m, ml.x);
+                            const float wo = weight(x_m, mx), wp = weight(ml.x, mx);
+                            sum = first ? fmaf(wp, ml.y, wo * x_l) : fmaf(wo, x_l, wp * ml.y);
+                            const float inv = sum > 0.f ? 1.0f / sum : 0.f;
+#pragma unroll 1
+                            for (int e = 0; e < npc; ++e) {
+                                float o[16];
+                                if (e + 1 < npc) load_part(vn, po, e + 1);
+                                load_o(o, c0 + 16 * e);
+                                const float* vf = reinterpret_cast<const float*>(v);
 #pragma unroll
-                        for (int k = 0; k < CW / 2; ++k) w[k] = pack_bf16(__uint_as_float(o[2 * k]), __uint_as_float(o[2 * k + 1]));
+                                for (int k = 0; k < 16; ++k) o[k] = first ? fmaf(wp, vf[k], wo * o[k]) : fmaf(wo, o[k], wp * vf[k]);
+                                store_out(o, c0 + 16 * e, inv);
 #pragma unroll
-                        for (int k = 0; k < CW / 2; k += 8) st_global_v8(op + col + 2 * k, w[k], w[k + 1], w[k + 2], w[k + 3], w[k + 4], w[k + 5], w[k + 6], w[k + 7]);
-                    } else {
-                        // partial rows are D + 4 floats long: 16-byte aligned only
+                                for (int q = 0; q < 4; ++q) v[q] = vn[q];
+                            }
+                        } else {
+                            for (int k = 0; k < np; ++k) {
+                                const float* pp = part_of(k);
+                                const float2 ml = pp == own ? make_float2(x_m, x_l) : load_ml(pp);
+                                const float mn = fmaxf(mx, ml.x);
+                                sum = fmaf(weight(ml.x, mn), ml.y, sum * weight(mx, mn));
+                                mx = mn;
+                            }
+                            const float inv = sum > 0.f ? 1.0f / sum : 0.f;
+#pragma unroll 1
+                            for (int e = 0; e < npc; ++e) {
+                                float acc[16];
 #pragma unroll
-                        for (int v4 = 0; v4 < CW / 4; ++v4)
-                            *reinterpret_cast<uint4*>(pp + col + v4 * 4) = make_uint4(o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
+                                for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+#pragma unroll 1
+                                for (int k = 0; k < np; ++k) {
+                                    const float* pp = part_of(k);
+                                    float4 v[4];
+                                    float mk = x_m;
+                                    if (pp == own) {
+                                        load_o(reinterpret_cast<float*>(v), c0 + 16 * e);
+                                    } else {
+                                        load_part(v, pp, e);
+                                        mk = load_ml(pp).x;
+                                    }
+                                    const float w = weight(mk, mx);
+                                    const float* vf = reinterpret_cast<const float*>(v);
+#pragma unroll
+                                    for (int q = 0; q < 16; ++q) acc[q] = fmaf(w, vf[q], acc[q]);
+                                }
+                                store_out(acc, c0 + 16 * e, inv);
+                            }
+                        }
+                        store_lse(mx, sum);
                     }
-                }
-                if (row_valid && c0 == 0) {
-                    if (!whole) { pp[D] = x_m; pp[D + 1] = x_l; }
-                    else if (p.lse) p.lse[((size_t)ub * p.Hq + h) * p.T + node] = x_l > 0.f ? (x_m + log2f(x_l)) * 0.6931471805599453f : 0.f;
                 }
             }
             tc_fence_before();
@@ -576,97 +727,84 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             // The other warp of the pair may have entered a pair barrier that this one will not: answer for it until it has left too.
             // Its own waits end as well, so this does; the loop is bounded all the same.
             __syncwarp();
+            int seen = __shfl_sync(CB_FULL, lane == 0 ? s_pair[sw] : 0, 0);
             if (lane == 0) { __threadfence_block(); s_pair[sw] = -1; }
             for (int k = 0; k < 1 << 16; ++k) {
                 const int other = __shfl_sync(CB_FULL, lane == 0 ? s_pair[sw ^ 4] : 0, 0);
                 if (other < 0) break;
-                if (other > entered) { ++entered; pair_arrive(pair_id); }
+                if (other > seen) { seen = other; pair_arrive(pair_id); }
                 __nanosleep(200);
             }
         }
+        __syncwarp();
+        cluster_wait();
         if (p.cs > 0 && s_sched->c_has) {
             // ------------------------------------------------------------------ cluster mode: combine the unit's shares
             // Every CTA of the cluster holds the unnormalised rows of its share (O0 and O1 in TMEM, their weights, the running
-            // maximum and the sum in registers).  Row i is combined by CTA i % cs: each CTA writes its copy of the row into that
-            // CTA's shared memory (four threads a row, D / 4 columns each), arrives on its data barrier, and the owner merges the
-            // cs contributions and writes the output row.  The rows are
-            // received in the two query tiles when they fit (they are idle from a CTA's last S product on, which the query
-            // loader reports), otherwise in the K/V ring (idle from the last P.V on, reported here).
+            // maximum and the sum in registers).  CTA r puts columns [r D / cs, (r + 1) D / cs) of all rows together: a thread's
+            // columns go to one CTA (two with cs = 8), 32 rows side by side, so that a warp writes 512 bytes in a run to shared memory
+            // over there (by rows, one CTA for every cs-th row, the same 64 KB took 4.2 k cycles).  They are received in
+            // the two query tiles when they fit (idle from a CTA's last S product on, which the query loader reports), otherwise
+            // in the K/V ring (idle from the last P.V on, reported here).  With them come every row's reference and sum.
             const int cs = p.cs, rank = cta % cs;
-            const int Rv = (min(RT, p.T * p.G) + cs - 1) / cs;   // rows that one CTA may own (rows beyond T nodes never exist)
             const int cb_ = s_sched->c_b, ckh = s_sched->c_kh, cn = s_sched->c_n;
-            constexpr uint32_t ROWB = (D + 4) * 4;
-            const bool in_q = (uint32_t)(cs * Rv) * ROWB <= 2u * C::Q_BYTES;
-            const uint32_t recv = sbase + (in_q ? C::OFF_Q : C::OFF_RING);     // [cs sources][Rv rows][D + 4] floats
-            if (ok && !in_q && sw == 0 && lane == 0)
+            const CbExchange ex = cb_exchange(p, D, cn);
+            const uint32_t recv = sbase + (ex.bytes <= 2u * C::Q_BYTES ? C::OFF_Q : C::OFF_RING);
+            if (ok && ex.bytes > 2u * C::Q_BYTES && sw == 0 && lane == 0)
                 for (int r = 0; r < cs; ++r) mbar_arrive_remote(cluster_addr(bar_cready, (uint32_t)r));
-            if (ok) ok = mbar_wait_cluster(bar_cready, 0, s_abort, p.status);
-            if (ok) {
-                const int dest = row % cs, rl = row / cs;
-                const bool valid = row < RT && (row / p.G) < cn;
-                const uint32_t ra = cluster_addr(recv + (uint32_t)(rank * Rv + rl) * ROWB, (uint32_t)dest);
-                const bool act = (wq * 32) < RT && ((wq * 32) / p.G) < cn;     // row 0 of the warp is valid
-                const int col = (l * 2 + hf) * CW;
-                if (act && c_share) {
-                    uint32_t o[CW];
-                    tmem_ld_w<CW>(o, tmem + C::O_COL + lane_addr + col);
+            // columns of one CTA, in groups of 4; powers of two
+            const int lc = 31 - __clz(D / cs), nch = 1 << (lc - 2);
+            const int col = (l * 2 + hf) * CW;
+            uint32_t o[CW];
 #pragma unroll
-                    for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * x_w0);
-                    if (__any_sync(CB_FULL, x_w1 >= 0.f)) {
-                        uint32_t o1[CW];
-                        tmem_ld_w<CW>(o1, tmem + C::O_COL + D + lane_addr + col);
+            for (int k = 0; k < CW; ++k) o[k] = 0u;             // what a CTA without tiles contributes
+            if (ok && c_share && row < ex.rows) {               // whole warps
+                tmem_ld_w<CW>(o, tmem + C::O_COL + lane_addr + col);
 #pragma unroll
-                        for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) + __uint_as_float(o1[k]) * x_w1);
-                    }
-                    if (valid) {
+                for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * x_w0);
+                if (x_two) {
+                    uint32_t o1[CW];
+                    tmem_ld_w<CW>(o1, tmem + C::O_COL + D + lane_addr + col);
 #pragma unroll
-                        for (int v4 = 0; v4 < CW / 4; ++v4)
-                            st_cluster_v4(ra + (uint32_t)(col + v4 * 4) * 4u, o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
-                    }
+                    for (int k = 0; k < CW; ++k) o[k] = __float_as_uint(fmaf(__uint_as_float(o1[k]), x_w1, __uint_as_float(o[k])));
                 }
-                if (valid && col == 0) st_cluster_v4(ra + D * 4u, __float_as_uint(c_share ? x_m : -INFINITY), __float_as_uint(c_share ? x_l : 0.f), 0u, 0u);
-                mbar_arrive_remote(cluster_addr(bar_cdata, (uint32_t)dest));
+            }
+            if (ok) ok = mbar_wait_cluster(bar_cready, 0, s_abort, p.status);
+            if (ok && row < ex.rows) {
+                // Stores that count themselves off the receiver's barrier: a release by an ordinary remote arrival waits for
+                // every store before it to come back.
+#pragma unroll
+                for (int v4 = 0; v4 < CW / 4; ++v4) {
+                    const int c = col + v4 * 4, d = c >> lc;
+                    st_async_v4(cluster_addr(recv + ex.value(rank, (c >> 2) & (nch - 1), row, nch), (uint32_t)d), cluster_addr(bar_cdata, (uint32_t)d),
+                                o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
+                }
+                for (int c = col; c < col + CW; c += 4)
+                    if ((c & (4 * nch - 1)) == 0)
+                        st_async_v2(cluster_addr(recv + ex.sums(rank, row, cs, nch), (uint32_t)(c >> lc)), cluster_addr(bar_cdata, (uint32_t)(c >> lc)),
+                                    __float_as_uint(c_share ? x_m : -INFINITY), __float_as_uint(c_share ? x_l : 0.f));
             }
             if (ok) ok = mbar_wait_cluster(bar_cdata, 0, s_abort, p.status);
             if (ok) {
-                // up to 512 threads: tpr threads per row, each a run of D / tpr >= 4 columns in groups of 4
-                int tpr = D / 4;                                 // a power of two
-                while (tpr * Rv > 512) tpr >>= 1;
-                const int t = sw * 32 + lane, rl = t / tpr, sub = t % tpr;
-                const int gr = rl * cs + rank, node = gr / p.G, h = ckh * p.G + gr % p.G;
-                if (rl < Rv && gr < RT && node < cn) {
+                const int nrow = min(RT, cn * p.G), cols = 4 * nch;
+                for (int t = sw * 32 + lane; t < nrow * nch; t += 512) {
+                    const int r = t >> (lc - 2), ch = t & (nch - 1);
                     float mx = -INFINITY;
-                    for (int sidx = 0; sidx < cs; ++sidx) {
-                        float ms;
-                        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(ms) : "r"(recv + (uint32_t)(sidx * Rv + rl) * ROWB + D * 4u));
-                        mx = fmaxf(mx, ms);
-                    }
-                    float wsum = 0.f;
-                    for (int sidx = 0; sidx < cs; ++sidx) {
-                        float ms, ls;
-                        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(ms), "=f"(ls) : "r"(recv + (uint32_t)(sidx * Rv + rl) * ROWB + D * 4u));
-                        wsum += (ms == -INFINITY) ? 0.f : ex2(ms - mx) * ls;
+                    for (int k = 0; k < cs; ++k) mx = fmaxf(mx, ld_shared_f2(recv + ex.sums(k, r, cs, nch)).x);
+                    float acc[4] = {0.f, 0.f, 0.f, 0.f}, wsum = 0.f;
+                    for (int k = 0; k < cs; ++k) {
+                        const float2 ml = ld_shared_f2(recv + ex.sums(k, r, cs, nch));
+                        if (ml.x == -INFINITY) continue;         // that CTA had no tiles: its rows were not written
+                        const float w = ex2(ml.x - mx);
+                        const float4 v = ld_shared_f4(recv + ex.value(k, ch, r, nch));
+                        wsum = fmaf(w, ml.y, wsum);
+                        acc[0] = fmaf(w, v.x, acc[0]); acc[1] = fmaf(w, v.y, acc[1]); acc[2] = fmaf(w, v.z, acc[2]); acc[3] = fmaf(w, v.w, acc[3]);
                     }
                     const float inv = wsum > 0.f ? 1.0f / wsum : 0.f;
-                    const int cols = D / tpr;
-                    for (int g4 = 0; g4 < cols; g4 += 4) {
-                        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-                        for (int sidx = 0; sidx < cs; ++sidx) {
-                            const uint32_t base = recv + (uint32_t)(sidx * Rv + rl) * ROWB;
-                            float ms;
-                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(ms) : "r"(base + D * 4u));
-                            if (ms == -INFINITY) continue;      // that CTA had no tiles: its row was not written
-                            const float w = ex2(ms - mx);
-                            float v[4];
-                            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
-                                         : "r"(base + (uint32_t)(sub * cols + g4) * 4u));
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) acc[k] += w * v[k];
-                        }
-                        __nv_bfloat16* op = p.out + (((size_t)cb_ * p.T + node) * p.Hq + h) * D + sub * cols + g4;
-                        *reinterpret_cast<uint2*>(op) = make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
-                    }
-                    if (sub == 0 && p.lse)
+                    const int node = r / p.G, h = ckh * p.G + r % p.G;
+                    __nv_bfloat16* op = p.out + (((size_t)cb_ * p.T + node) * p.Hq + h) * D + rank * cols + ch * 4;
+                    *reinterpret_cast<uint2*>(op) = make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
+                    if (rank == 0 && ch == 0 && p.lse)
                         p.lse[((size_t)cb_ * p.Hq + h) * p.T + node] = wsum > 0.f ? (mx + log2f(wsum)) * 0.6931471805599453f : 0.f;
                 }
             }
@@ -686,7 +824,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
     }
 }
 
-// Merge pass: block (c, *) looks at the unit that CTA c of the attention kernel started but did not finish,
+// Merge pass of the CTA-pair kernel (cb_attn_pair.cuh): block (c, *) looks at the unit that CTA c of the attention kernel started but did not finish,
 // and combines the partials that CTA c and the following CTAs left for it.  One warp per output row.
 // Every block waits for the attention grid before it leaves, also the ones that find nothing to merge: the next kernel
 // in the stream is ordered behind this grid only, so this grid must not end while the attention kernel still runs.
@@ -708,10 +846,10 @@ __global__ void __launch_bounds__(256) cb_attn_merge_kernel(const CbAttnParams p
         cb_sched_locate(p, g1 - 1, lane, &rg, &b, &pre);
         s = cb_seq_shape(p, b);
         const long long off = g1 - 1 - pre;
-        vt = s.tiles + s.ov;                                  // positions of one unit: padding, then its key tiles
+        vt = s.unit(rg);                                      // positions of one unit: padding, then its key tiles (one each)
         j = (int)(off / vt);
         ustart = pre + (long long)j * vt;
-        const long long first_tile = ustart + s.ov;
+        const long long first_tile = ustart + s.ov(rg);
         nothing = (int)(off - (long long)j * vt) == vt - 1    // the unit ends with this range
                   || first_tile < g0                          // started by an earlier CTA: that CTA's block merges it
                   || first_tile >= g1;                        // only padding so far: the next CTA starts the unit
@@ -818,6 +956,26 @@ bool encode_map(CUtensorMap* m, const void* base, int D, int heads, int rows, lo
     return r == CUDA_SUCCESS;
 }
 
+// 5-D view of a [blocks, rows, heads, D] bf16 tensor in the order (64 dims, row, 64-dim column block, ...): with `fold`, rows of all
+// blocks are counted in groups of 8 and the last two coordinates are (group, head), box = 8 rows x D dims x 2 groups; without,
+// they are (head, block), box = 8 rows x D dims.
+bool encode_grouped_map(CUtensorMap* m, const void* base, int D, int heads, int rows, long blocks, bool fold) {
+    EncodeTiledFn enc = get_encode();
+    if (!enc) { fprintf(stderr, "cacheback: cuTensorMapEncodeTiled entry point not found\n"); return false; }
+    const cuuint64_t row = (cuuint64_t)heads * D * 2;          // bytes
+    cuuint64_t dims[5] = {64, fold ? 8u : (cuuint64_t)rows, (cuuint64_t)(D / 64), fold ? (cuuint64_t)blocks * (rows / 8) : (cuuint64_t)heads,
+                          fold ? (cuuint64_t)heads : (cuuint64_t)blocks};
+    cuuint64_t strides[4] = {row, 128, fold ? 8 * row : (cuuint64_t)D * 2, fold ? (cuuint64_t)D * 2 : (cuuint64_t)rows * row};
+    cuuint32_t box[5] = {64, 8, (cuuint32_t)(D / 64), fold ? 2u : 1u, 1};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_128B, D >= 128 ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS)
+        fprintf(stderr, "cacheback: tensor map encode failed (%d): D=%d heads=%d rows=%d blocks=%ld base=%p\n", (int)r, D, heads, rows, blocks, base);
+    return r == CUDA_SUCCESS;
+}
+
 // Cluster mode is for launches with few units, where the stream-K split would make every unit a shared one: all trees fit
 // one row tile (so a unit is one (sequence, kv head)), units times a cluster size of 8, 4 or 2 does not exceed the SMs, that
 // many clusters can be resident at once, and a CTA's part of a unit (tiles / cs) is shorter than a CTA's range under the
@@ -886,7 +1044,7 @@ cb_status launch_pairs(CbAttnParams p, const TcMaps& maps, cudaStream_t st, int 
     // same time, so that one fetch from HBM serves all of them.
     const int row_groups = (p.MT + 1) / 2;
     if (npairs > row_groups) npairs -= npairs % row_groups;
-    p.nc = npairs; p.cs = 0;
+    p.nc = npairs; p.cs = 0; p.w1 = p.w2 = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * npairs)); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairCfg::SMEM_ALLOC; cfg.stream = st;
     cudaLaunchAttribute at[2];
@@ -941,8 +1099,7 @@ cb_status launch(CbAttnParams p, const TcMaps& maps, cudaStream_t st, int num_sm
         return CB_OK;
     }
     CB_CUDA(cb_launch_pdl(cb_attn_tc_kernel<D>, dim3(p.nc), dim3(kThreads), Cfg<D>::SMEM, st, p, maps));
-    CB_CUDA(cb_launch_pdl(cb_attn_merge_kernel<D>, dim3(p.nc, 4), dim3(256), 0, st, p));
-    cb_count_launch(2);
+    cb_count_launch(1);
     CB_CUDA(cudaGetLastError());
     return CB_OK;
 }
@@ -954,10 +1111,10 @@ cb_status launch(CbAttnParams p, const TcMaps& maps, cudaStream_t st, int num_sm
 namespace {
 struct MapKey {
     const void *q, *k_pool, *v_pool, *k_tree, *v_tree;
-    int D, Hq, Hkv, P, T, B, G, NPT, num_pages;
+    int D, Hq, Hkv, P, T, B, G, NPT, num_pages, pairs;
     bool operator==(const MapKey& o) const {
         return q == o.q && k_pool == o.k_pool && v_pool == o.v_pool && k_tree == o.k_tree && v_tree == o.v_tree && D == o.D && Hq == o.Hq &&
-               Hkv == o.Hkv && P == o.P && T == o.T && B == o.B && G == o.G && NPT == o.NPT && num_pages == o.num_pages;
+               Hkv == o.Hkv && P == o.P && T == o.T && B == o.B && G == o.G && NPT == o.NPT && num_pages == o.num_pages && pairs == o.pairs;
     }
 };
 constexpr int kMapCache = 16;
@@ -970,7 +1127,7 @@ std::mutex g_map_mutex;
 cb_status cb_attn_launch_tensor(cb_ctx* ctx, const CbAttnParams& p, cudaStream_t st) {
     if (p.P != 16) return CB_ERR_UNSUPPORTED;
     const bool pairs = p.D == 128 && p.MT > 1 && (ctx->cfg.flags & CB_FLAG_ATTN_CTA_PAIRS);
-    const MapKey key = {p.q, p.k_pool, p.v_pool, p.k_tree, p.v_tree, p.D, p.Hq, p.Hkv, p.P, p.T, p.B, p.G, p.NPT, p.num_pages};
+    const MapKey key = {p.q, p.k_pool, p.v_pool, p.k_tree, p.v_tree, p.D, p.Hq, p.Hkv, p.P, p.T, p.B, p.G, p.NPT, p.num_pages, pairs ? 1 : 0};
     TcMaps maps;
     bool hit = false;
     {
@@ -979,10 +1136,17 @@ cb_status cb_attn_launch_tensor(cb_ctx* ctx, const CbAttnParams& p, cudaStream_t
             if (g_map_keys[i] == key) { maps = g_map_vals[i]; hit = true; }
     }
     if (!hit) {
-        if (!encode_map(&maps.k_pool, p.k_pool, p.D, p.Hkv, p.P, p.num_pages, 1, 16)) return CB_ERR_CUDA;
-        if (!encode_map(&maps.v_pool, p.v_pool, p.D, p.Hkv, p.P, p.num_pages, 1, 16)) return CB_ERR_CUDA;
-        if (!encode_map(&maps.k_tree, p.k_tree, p.D, p.Hkv, p.T, p.B, 1, 16)) return CB_ERR_CUDA;
-        if (!encode_map(&maps.v_tree, p.v_tree, p.D, p.Hkv, p.T, p.B, 1, 16)) return CB_ERR_CUDA;
+        if (pairs) {
+            if (!encode_map(&maps.k_pool, p.k_pool, p.D, p.Hkv, p.P, p.num_pages, 1, 16)) return CB_ERR_CUDA;
+            if (!encode_map(&maps.v_pool, p.v_pool, p.D, p.Hkv, p.P, p.num_pages, 1, 16)) return CB_ERR_CUDA;
+            if (!encode_map(&maps.k_tree, p.k_tree, p.D, p.Hkv, p.T, p.B, 1, 16)) return CB_ERR_CUDA;
+            if (!encode_map(&maps.v_tree, p.v_tree, p.D, p.Hkv, p.T, p.B, 1, 16)) return CB_ERR_CUDA;
+        } else {
+            if (!encode_grouped_map(&maps.k_pool, p.k_pool, p.D, p.Hkv, p.P, p.num_pages, true)) return CB_ERR_CUDA;
+            if (!encode_grouped_map(&maps.v_pool, p.v_pool, p.D, p.Hkv, p.P, p.num_pages, true)) return CB_ERR_CUDA;
+            if (!encode_grouped_map(&maps.k_tree, p.k_tree, p.D, p.Hkv, p.T, p.B, false)) return CB_ERR_CUDA;
+            if (!encode_grouped_map(&maps.v_tree, p.v_tree, p.D, p.Hkv, p.T, p.B, false)) return CB_ERR_CUDA;
+        }
         if (!encode_map(&maps.q, p.q, p.D, p.Hq, p.T, p.B, p.G, p.NPT)) return CB_ERR_CUDA;
         std::lock_guard<std::mutex> lock(g_map_mutex);
         const int slot = g_map_used < kMapCache ? g_map_used++ : (g_map_next++ % kMapCache);

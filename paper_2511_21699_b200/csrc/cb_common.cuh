@@ -100,6 +100,7 @@ struct cb_ctx {
     size_t guard_off[CB_MAX_GUARDS];
     int n_guards;
     float* d_attn_part;     // partial outputs of units shared between CTAs
+    uint32_t* d_attn_ticket; // [CTAs][16] parts of a shared unit that are in memory, zero between calls
     size_t attn_part_floats;
     int attn_max_units;     // partial row tiles available
     int num_sms;
@@ -108,7 +109,7 @@ struct cb_ctx {
 struct CbLayout {
     uint32_t nslots, E;
     size_t off_hdr, off_index, off_lstamp, off_entries, off_status, off_counters, off_rowmax, off_ticket, off_bulk_plan,
-        off_attn_part, attn_part_floats, total;
+        off_attn_ticket, off_attn_part, attn_part_floats, total;
     int attn_max_units;
     size_t guard_off[CB_MAX_GUARDS];   // checking build: start of the guard area behind each region
     int n_guards;
@@ -126,6 +127,7 @@ cb_status cb_frozen_layout(const cb_frozen_config* cfg, CbFrozenLayout* L);
 CbTables cb_frozen_view(const cb_frozen_config* cfg, const CbFrozenLayout& L, void* dev_table);
 void cb_count_launch(int n);
 
+#define CB_ATTN_TICKETS (160 * 16)   // persistent CTAs x softmax warps
 #define CB_ATTN_MAX_UNITS 640   // partial row tiles (128 rows x (D + 4) floats): 2 shared units x 2 row tiles per persistent CTA, 160 CTAs
 
 // Programmatic dependent launch.  Every kernel of the step begins with CB_PDL_ENTRY: it waits until the kernels before

@@ -66,8 +66,24 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t local, uint32_t rank) 
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t remote_bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote_bar) : "memory");
 }
-__device__ __forceinline__ void st_cluster_v4(uint32_t raddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(raddr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+// Stores to another CTA's shared memory that take their bytes off the count a barrier there expects.
+__device__ __forceinline__ void st_async_v4(uint32_t raddr, uint32_t rbar, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];"
+                 ::"r"(raddr), "r"(rbar), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void st_async_v2(uint32_t raddr, uint32_t rbar, uint32_t a, uint32_t b) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%2, %3}, [%1];"
+                 ::"r"(raddr), "r"(rbar), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ float2 ld_shared_f2(uint32_t addr) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
 }
 __device__ __forceinline__ uint32_t mbar_try_cluster(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -108,6 +124,17 @@ __device__ __forceinline__ void tma_load_4d_hint(uint32_t dst, const CUtensorMap
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cta.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
         ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "l"(pol) : "memory");
+}
+
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3, int c4) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4) : "memory");
+}
+__device__ __forceinline__ void tma_load_5d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3, int c4, uint64_t pol) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cta.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "l"(pol) : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -228,7 +255,8 @@ __host__ __device__ constexpr uint32_t make_idesc(int M, int N, bool b_mn_major)
 // Low and high 32-bit words of a shared-memory matrix descriptor (128-byte swizzle, 1024-byte stride between
 // 8-row groups).  All operands live below 256 KB, so stepping the low word by (bytes >> 4) moves the start address.
 __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) { return ((saddr & 0x3FFFFu) >> 4) | ((lbo_bytes >> 4) << 16); }
-constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__host__ __device__ constexpr uint32_t desc_hi(uint32_t sbo_bytes) { return (sbo_bytes >> 4) | (1u << 14) | (2u << 29); }
+constexpr uint32_t kDescHi = desc_hi(1024u);
 
 // One MMA issuer thread feeds the tensor pipe, so the instructions between two MMAs are kept to a minimum: each
 // of the blocks below issues all MMAs of one 128 x 128 x D (or 128 x D x 128) product from a single asm statement.
@@ -271,10 +299,33 @@ __device__ __forceinline__ void mma_pv_block(uint32_t d_tmem, uint32_t p_tmem, u
         ::"r"(d_tmem), "r"(p_tmem), "r"(vlo), "r"(kDescHi), "r"(idesc), "r"(accum) : "memory");
 }
 
-// The same with P in two halves of 64 keys, the second one 64 columns after the first (each half overlays the scores it came from).
+// The products of the default kernel, whose K and V tiles are groups of 8 keys x D dims: a group's 64-dim column blocks are 1024
+// bytes apart and the groups D * 16 bytes.
+// S[tmem] = Q[smem, K-major, column blocks 128 rows long] * K[smem, K-major, grouped]^T over D.
+#define CB_MMA_SG_STEP(OA, OB)                                                                                       \
+    "add.u32 ra, %1, " #OA ";\n\tadd.u32 rb, %2, " #OB ";\n\tmov.b64 da, {ra, %3};\n\tmov.b64 db, {rb, %5};\n\t"    \
+    "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pt;\n\t"
+template <int D>
+__device__ __forceinline__ void mma_s_grouped_block(uint32_t d_tmem, uint32_t qlo, uint32_t klo, uint32_t idesc) {
+    if (D == 128) {
+        asm volatile(
+            "{\n\t.reg .pred pt, pf;\n\t.reg .b64 da, db;\n\t.reg .b32 ra, rb;\n\t"
+            "setp.eq.u32 pt, %4, %4;\n\tsetp.ne.u32 pf, %4, %4;\n\t"
+            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %5};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pf;\n\t"
+            CB_MMA_SG_STEP(2, 2) CB_MMA_SG_STEP(4, 4) CB_MMA_SG_STEP(6, 6) CB_MMA_SG_STEP(1024, 64) CB_MMA_SG_STEP(1026, 66)
+            CB_MMA_SG_STEP(1028, 68) CB_MMA_SG_STEP(1030, 70) "}"
+            ::"r"(d_tmem), "r"(qlo), "r"(klo), "r"(kDescHi), "r"(idesc), "r"(desc_hi(D * 16)) : "memory");
+    } else {
+        mma_s_block<D>(d_tmem, qlo, klo, idesc);              // one column block: the same layout
+    }
+}
+// O[tmem] (+)= P[tmem] * V[smem, MN-major, grouped] over the tile's 128 keys; P in two halves of 64 keys, the second one 64 columns after
+// the first (each half overlays the scores it came from).
 #define CB_MMA_TSH_STEP(K)                                                                                           \
-    "add.u32 ra, %1, 8 * " #K " + 32 * (" #K " / 4);\n\tadd.u32 rb, %2, 128 * " #K ";\n\tmov.b64 db, {rb, %3};\n\t"  \
+    "add.u32 ra, %1, 8 * " #K " + 32 * (" #K " / 4);\n\tmad.lo.u32 rb, %6, " #K ", %2;\n\tmov.b64 db, {rb, %3};\n\t"  \
     "tcgen05.mma.cta_group::1.kind::f16 [%0], [ra], db, %4, pt;\n\t"
+template <int D>
 __device__ __forceinline__ void mma_pv_halves_block(uint32_t d_tmem, uint32_t p_tmem, uint32_t vlo, uint32_t idesc, uint32_t accum) {
     asm volatile(
         "{\n\t.reg .pred pt, pa;\n\t.reg .b64 db;\n\t.reg .b32 ra, rb;\n\t"
@@ -282,7 +333,7 @@ __device__ __forceinline__ void mma_pv_halves_block(uint32_t d_tmem, uint32_t p_
         "mov.b64 db, {%2, %3};\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, pa;\n\t"
         CB_MMA_TSH_STEP(1) CB_MMA_TSH_STEP(2) CB_MMA_TSH_STEP(3) CB_MMA_TSH_STEP(4) CB_MMA_TSH_STEP(5) CB_MMA_TSH_STEP(6) CB_MMA_TSH_STEP(7) "}"
-        ::"r"(d_tmem), "r"(p_tmem), "r"(vlo), "r"(kDescHi), "r"(idesc), "r"(accum) : "memory");
+        ::"r"(d_tmem), "r"(p_tmem), "r"(vlo), "r"(desc_hi(D * 16)), "r"(idesc), "r"(accum), "n"(D * 2) : "memory");
 }
 
 // One lane of a converged warp; the compiler knows that a single thread runs what the result guards (a tcgen05.mma issues every
@@ -298,6 +349,16 @@ __device__ __forceinline__ bool pair_or(int id, bool v) {
     asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %2, 0;\n\tbar.red.or.pred q, %1, 64, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
                  : "=r"(r) : "r"(id), "r"((uint32_t)v) : "memory");
     return r != 0u;
+}
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t* p, uint32_t v) {
+    uint32_t r;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(r) : "l"(p), "r"(v) : "memory");
+    return r;
 }
 __device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
 // W consecutive columns of this thread's TMEM lane (W = 16 or 32), waited for.

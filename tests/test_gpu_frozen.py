@@ -196,3 +196,21 @@ def test_builder_edge_cases(oracle):
     ft = FrozenTable(1, 2, 8, 2)
     with pytest.raises(CachebackError):
         ft.cb_frozen_build(dev(np.array([1, 2, -1, 3, 4, 5], np.int32)))     # negative ids are rejected
+
+
+def _one_leader_with_ties(n):
+    """Leader 0 followed by n distinct pairs, once each, whose first tokens are three values in turn."""
+    i = np.arange(n)
+    return np.stack([np.zeros(n), 1 + i % 3, 10 + i], 1).reshape(-1).astype(np.int32)
+
+
+@pytest.mark.parametrize("LL,FL,LC,FC,corpus", [
+    (1, 3, 2, 4, np.random.default_rng(1).integers(0, 5, 40000)),      # the LC-th best count is above a histogram pass's exact bins
+    (1, 2, 4, 8, _one_leader_with_ties(700)),                          # more ties than candidates are ranked: cut by the second token
+    (1, 2, 4, 8, _one_leader_with_ties(3000)),                         # the same in a group that a large block takes
+    (1, 2, 4, 128, _one_leader_with_ties(1024)),
+    (2, 1, 33, 31, np.random.default_rng(2).integers(0, 40, 30000)),   # groups of 31 to 40 distinct followers
+    (1, 1, 1 << 12, 2, np.arange(5000) % 4100),                        # every leader's count is 1 or 2
+], ids=["counts", "ties", "ties-block", "ties-128", "groups", "singles"])
+def test_builder_selection_edges(oracle, LL, FL, LC, FC, corpus):
+    _build_and_compare(oracle, corpus.astype(np.int32), LL, FL, LC, FC)

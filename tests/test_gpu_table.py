@@ -235,3 +235,33 @@ def test_argument_errors():
     tree = cb.alloc_tree()
     with pytest.raises(CachebackError):
         cb.cb_accept(tree)                                          # neither logits nor ids
+
+
+@pytest.mark.parametrize("LL,FL,LC,FC,vocab", [(1, 2, 8, 2, 5),        # repeated leaders inside a run; the capacity is reached and evicts
+                                               (1, 1, 64, 40, 60),     # new leaders in one bucket of a small index, long follower lists
+                                               (2, 3, 512, 4, 30),     # stored and new leaders mixed
+                                               (3, 2, 40, 1, 9),       # the capacity falls inside a run
+                                               (4, 8, 4096, 4, 1000)])  # nearly every leader is new
+def test_update_draft_runs_of_windows(oracle, LL, FL, LC, FC, vocab):
+    """cb_update_draft_tree applies up to eight windows of a sequence side by side: runs around that number, against the oracle's
+    insertions one after the other (tables, recency, trees)."""
+    from paper_2511_21699_b200 import Cacheback
+    B, T, depth = 3, 20, 7
+    rng = np.random.default_rng(LL * 10 + FL)
+    toks = rng.integers(0, vocab, (B, 400)).astype(np.int32)
+    cb = Cacheback(B, LL, FL, LC, FC, T, 4, depth, 1000, 1, 1, 64)
+    otabs = [oracle.OracleTable(LL, FL, LC, FC) for _ in range(B)]
+    toks_d, pos, tree = dev(toks), np.zeros(B, np.int32), cb.alloc_tree()
+    for run in (LL + FL - 1, 1, 2, 7, 8, 9, 16, 17, 40, 0, 3, 64):
+        new = (pos + run + np.arange(B) % 2).astype(np.int32)
+        cb.cb_update_draft_tree(toks_d, dev(pos), dev(new), tree)
+        g = {k: v.cpu().numpy() for k, v in tree.items()}
+        for b in range(B):
+            otabs[b].update(toks[b], int(pos[b]), int(new[b]))
+            n, tok, par, dep, mask = otabs[b].draft_tree(toks[b], int(new[b]), T, 4, depth)
+            assert g["n_nodes"][b] == n and np.array_equal(g["tokens"][b], tok) and np.array_equal(g["parent"][b], par), (run, b)
+            assert np.array_equal(g["mask"][b].view(np.uint32), mask), (run, b)
+        pos = new
+    _assert_tables_equal(cb, otabs, range(B))
+    st, cnt = cb.cb_poll_status()
+    assert st == 0 and cnt["inserts"] == sum(int(p) - LL - FL + 1 for p in pos)

@@ -184,7 +184,7 @@ def attn_flops(cfg, ctx, n_nodes, pairs):
 
 
 def attn_roofline(cfg, ctx, n_nodes, pairs, ms, pk):
-    """Roofline record of one cb_tree_attn launch (attention kernel plus its merge pass): the slower of bytes over the
+    """Roofline record of one cb_tree_attn launch: the slower of bytes over the
     measured copy bandwidth and flops over the measured bf16 matmul rate."""
     a_bytes, fl = attn_bytes(cfg, ctx, n_nodes), attn_flops(cfg, ctx, n_nodes, pairs)
     t_mem, t_cmp = a_bytes / (pk["hbm_gbs"] * 1e9), fl / (pk["tflops"] * 1e12)
@@ -649,7 +649,7 @@ def measure(args, cfg_name, rank, world, device, headline):
     elif ATTN_TRAFFIC["sources_sha1"] == attn_sources_sha1() and cfg_name in ATTN_TRAFFIC["scaled"]:
         traffic, traffic_source = ATTN_TRAFFIC["scaled"][cfg_name]
     roof_full.update({"traffic": traffic, "traffic_source": traffic_source,
-                      "kernel": "cb_tree_attn (attention kernel, plus its merge pass where the launch is not in cluster mode)"})
+                      "kernel": "cb_tree_attn (one launch)"})
     acc_bytes_full, acc_bytes_dr = float(B * T) * cfg.vocab * 4, float(np.sum(nn_mean)) * cfg.vocab * 4
     accept = {"gbs": acc_bytes_full / (per_call["cb_accept"] * 1e-3) / 1e9, "algorithmic_bytes": acc_bytes_full,
               "ms_per_launch": per_call["cb_accept"],

@@ -220,3 +220,42 @@ def test_attn_cta_pair_kernel(oracle, case):
         _run(W.get_config("c3_8b_gqa"), oracle, True, _sampled(3, 3, 6), flags=_lib.CB_FLAG_ATTN_CTA_PAIRS)
     else:
         _jumps(oracle, SMALL_GQA, [300, 300, 300, 257, 140], flags=_lib.CB_FLAG_ATTN_CTA_PAIRS)
+
+
+def _few_heads(name, hq, hkv, d, t):
+    return W.CbConfig(name, 1, 2, 2, 64, 2, t, 6, 0, hq, hkv, d, (1, 20000), 100, 1.1, 0.3, (4, 8), 64)
+
+
+@pytest.mark.parametrize("cfg,ctx", [
+    (_few_heads("shared_wide", 8, 1, 128, 40), 20000),       # units of 158 tiles over some 70 CTAs each; two and one row tiles
+    (_few_heads("shared_narrow", 8, 1, 128, 40), 6000),      # fewer positions than two per CTA: a CTA holds one tile at most
+    (_few_heads("shared_tiny", 16, 2, 64, 20), 300),         # fewer positions than CTAs
+    (_few_heads("shared_d64", 16, 1, 64, 17), 9001),
+], ids=lambda x: getattr(x, "name", x))
+def test_attn_units_shared_by_many_ctas(oracle, cfg, ctx):
+    """Units whose parts lie in many CTAs, combined by the last of them to come: three times with the same context (the tickets are
+    back at zero, the result does not depend on who comes last), output rows that are aligned to 16 bytes and not to 32."""
+    from paper_2511_21699_b200 import Cacheback
+    prob = Problem(cfg)
+    prob.ctx = np.array([ctx], np.int32)
+    prob.bt, prob.num_pages = W.make_block_table(cfg, prob.ctx)
+    T = cfg.max_nodes
+    _, _, mask, n = synthetic_trees(cfg, full=True)
+    d = device_attn_inputs(cfg, prob)
+    cb = Cacheback.from_config(cfg)
+    outs = []
+    for _ in range(3):
+        lse = torch.full((1, cfg.n_q_heads, T), 7.0, dtype=torch.float32, device="cuda")
+        flat = torch.full((T * cfg.n_q_heads * cfg.head_dim + 8,), 3.0, dtype=torch.bfloat16, device="cuda")
+        out = flat[8:].view(1, T, cfg.n_q_heads, cfg.head_dim)
+        cb.cb_tree_attn(d["q"], d["k_pool"], d["v_pool"], d["block_table"], d["ctx_len"], d["k_tree"], d["v_tree"], dev(mask.view(np.int32)), dev(n),
+                        out=out, lse=lse, max_ctx=ctx)
+        torch.cuda.synchronize()
+        assert cb.cb_poll_status()[0] == 0 and (flat[:8] == 3.0).all()
+        outs.append((out, lse))
+    assert all(torch.equal(outs[0][0], o) and torch.equal(outs[0][1], l) for o, l in outs[1:])
+    rows = [(h, i) for h in (0, cfg.n_q_heads - 1) for i in (0, T // 2, T - 1)]
+    ref, ref_lse = oracle_attn_rows(oracle, cfg, prob, mask, 0, rows)
+    hh = torch.tensor([r[0] for r in rows], device="cuda")
+    ii = torch.tensor([r[1] for r in rows], device="cuda")
+    _check_rows(bf16_to_f64(outs[0][0][0, ii, hh]), outs[0][1][0, hh, ii].cpu().numpy().astype(np.float64), ref, ref_lse, (cfg.name, ctx))

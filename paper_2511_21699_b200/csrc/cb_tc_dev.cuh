@@ -120,12 +120,6 @@ __device__ __forceinline__ uint64_t l2_evict_first_policy() {
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     return pol;
 }
-__device__ __forceinline__ void tma_load_4d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3, uint64_t pol) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cta.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
-        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "l"(pol) : "memory");
-}
-
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3, int c4) {
     asm volatile(
         "cp.async.bulk.tensor.5d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
@@ -263,42 +257,6 @@ constexpr uint32_t kDescHi = desc_hi(1024u);
 #define CB_MMA_SS_STEP(OFF)                                                                                          \
     "add.u32 ra, %1, " #OFF ";\n\tadd.u32 rb, %2, " #OFF ";\n\tmov.b64 da, {ra, %3};\n\tmov.b64 db, {rb, %3};\n\t"  \
     "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pt;\n\t"
-// S[tmem] = Q[smem, K-major] * K[smem, K-major]^T over D.  qlo / klo: low descriptor words of the first 16-wide slice.
-template <int D>
-__device__ __forceinline__ void mma_s_block(uint32_t d_tmem, uint32_t qlo, uint32_t klo, uint32_t idesc) {
-    if (D == 128) {
-        asm volatile(
-            "{\n\t.reg .pred pt, pf;\n\t.reg .b64 da, db;\n\t.reg .b32 ra, rb;\n\t"
-            "setp.eq.u32 pt, %4, %4;\n\tsetp.ne.u32 pf, %4, %4;\n\t"
-            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pf;\n\t"
-            CB_MMA_SS_STEP(2) CB_MMA_SS_STEP(4) CB_MMA_SS_STEP(6) CB_MMA_SS_STEP(1024) CB_MMA_SS_STEP(1026) CB_MMA_SS_STEP(1028)
-            CB_MMA_SS_STEP(1030) "}"
-            ::"r"(d_tmem), "r"(qlo), "r"(klo), "r"(kDescHi), "r"(idesc) : "memory");
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred pt, pf;\n\t.reg .b64 da, db;\n\t.reg .b32 ra, rb;\n\t"
-            "setp.eq.u32 pt, %4, %4;\n\tsetp.ne.u32 pf, %4, %4;\n\t"
-            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pf;\n\t"
-            CB_MMA_SS_STEP(2) CB_MMA_SS_STEP(4) CB_MMA_SS_STEP(6) "}"
-            ::"r"(d_tmem), "r"(qlo), "r"(klo), "r"(kDescHi), "r"(idesc) : "memory");
-    }
-}
-#define CB_MMA_TS_STEP(K)                                                                                            \
-    "add.u32 ra, %1, 8 * " #K ";\n\tadd.u32 rb, %2, 128 * " #K ";\n\tmov.b64 db, {rb, %3};\n\t"                     \
-    "tcgen05.mma.cta_group::1.kind::f16 [%0], [ra], db, %4, pt;\n\t"
-// O[tmem] (+)= P[tmem, packed bf16] * V[smem, MN-major] over the tile's 128 keys.  vlo: low descriptor word of the V tile.
-__device__ __forceinline__ void mma_pv_block(uint32_t d_tmem, uint32_t p_tmem, uint32_t vlo, uint32_t idesc, uint32_t accum) {
-    asm volatile(
-        "{\n\t.reg .pred pt, pa;\n\t.reg .b64 db;\n\t.reg .b32 ra, rb;\n\t"
-        "setp.eq.u32 pt, %4, %4;\n\tsetp.ne.u32 pa, %5, 0;\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, pa;\n\t"
-        CB_MMA_TS_STEP(1) CB_MMA_TS_STEP(2) CB_MMA_TS_STEP(3) CB_MMA_TS_STEP(4) CB_MMA_TS_STEP(5) CB_MMA_TS_STEP(6) CB_MMA_TS_STEP(7) "}"
-        ::"r"(d_tmem), "r"(p_tmem), "r"(vlo), "r"(kDescHi), "r"(idesc), "r"(accum) : "memory");
-}
-
 // The products of the default kernel, whose K and V tiles are groups of 8 keys x D dims: a group's 64-dim column blocks are 1024
 // bytes apart and the groups D * 16 bytes.
 // S[tmem] = Q[smem, K-major, column blocks 128 rows long] * K[smem, K-major, grouped]^T over D.
@@ -317,7 +275,14 @@ __device__ __forceinline__ void mma_s_grouped_block(uint32_t d_tmem, uint32_t ql
             CB_MMA_SG_STEP(1028, 68) CB_MMA_SG_STEP(1030, 70) "}"
             ::"r"(d_tmem), "r"(qlo), "r"(klo), "r"(kDescHi), "r"(idesc), "r"(desc_hi(D * 16)) : "memory");
     } else {
-        mma_s_block<D>(d_tmem, qlo, klo, idesc);              // one column block: the same layout
+        // one column block: K's groups lie like Q's
+        asm volatile(
+            "{\n\t.reg .pred pt, pf;\n\t.reg .b64 da, db;\n\t.reg .b32 ra, rb;\n\t"
+            "setp.eq.u32 pt, %4, %4;\n\tsetp.ne.u32 pf, %4, %4;\n\t"
+            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pf;\n\t"
+            CB_MMA_SS_STEP(2) CB_MMA_SS_STEP(4) CB_MMA_SS_STEP(6) "}"
+            ::"r"(d_tmem), "r"(qlo), "r"(klo), "r"(kDescHi), "r"(idesc) : "memory");
     }
 }
 // O[tmem] (+)= P[tmem] * V[smem, MN-major, grouped] over the tile's 128 keys; P in two halves of 64 keys, the second one 64 columns after

@@ -132,8 +132,9 @@ struct Appender {
         if (m && lane == 0) k = atomicAdd(&n, (uint32_t)__popc(m));
         k = __shfl_sync(CB_FULL, k, 0) + __popc(m & ((1u << lane) - 1u));
         if (has) item[k] = x;
-        __syncthreads();
-        if (n > kCap - 256u) flush(list, counter);
+        // The block decides as one: every warp reads the count before it arrives at the barrier (the last to add sees all of it), and
+        // nobody adds again before all have.  Read after a barrier, the count could already hold the next call's additions.
+        if (__syncthreads_or(n > kCap - 256u)) flush(list, counter);
     }
     __device__ __forceinline__ void flush(uint32_t* list, uint32_t* counter) {
         __syncthreads();

@@ -214,3 +214,37 @@ def _one_leader_with_ties(n):
 ], ids=["counts", "ties", "ties-block", "ties-128", "groups", "singles"])
 def test_builder_selection_edges(oracle, LL, FL, LC, FC, corpus):
     _build_and_compare(oracle, corpus.astype(np.int32), LL, FL, LC, FC)
+
+
+def _bigram_table(corpus, LC, FC):
+    """frozen_build for LL = FL = 1 by sorting (the oracle's dictionaries take half a minute on millions of distinct tokens)."""
+    lead, follow = corpus[:-1], corpus[1:]
+    tok, cnt = np.unique(lead, return_counts=True)
+    top = tok[np.lexsort((tok, -cnt))][:LC]
+    pair, pc = np.unique(lead.astype(np.int64) << 32 | follow, return_counts=True)
+    pl, pf = (pair >> 32).astype(np.int32), (pair & 0xFFFFFFFF).astype(np.int32)
+    order = np.lexsort((pf, -pc, pl))
+    pl, pf = pl[order], pf[order]
+    first = np.searchsorted(pl, top)
+    nf = np.minimum(np.searchsorted(pl, top, side="right") - first, FC).astype(np.int32)
+    k = np.arange(FC)
+    F = np.where(k < nf[:, None], pf[np.minimum(first[:, None] + k, len(pf) - 1)], -1).astype(np.int32)
+    return top[:, None], nf, F[:, :, None]
+
+
+def test_builder_with_more_new_leaders_than_a_block_gathers(oracle):
+    """2.2 M distinct tokens: every block of the leader count makes some 1,850 new leaders, more than it gathers in shared memory
+    (1,536 less one round of 256), so the list is written out between rounds as well as at the end.  The same for the leaders that tie
+    with the LC-th best, which are all that occur once.  A list entry lost or written twice changes the table."""
+    from paper_2511_21699_b200 import FrozenTable
+    small = (np.random.default_rng(4).zipf(1.2, 5000) % 700).astype(np.int32)
+    assert all(np.array_equal(a, b) for a, b in zip(_bigram_table(small, 64, 3), oracle.frozen_build(small, 1, 1, 64, 3)))
+    rng = np.random.default_rng(9)
+    corpus = np.concatenate([rng.permutation(2_200_000), rng.permutation(300_000) * 7]).astype(np.int32)
+    ft = FrozenTable(1, 1, 1 << 20, 2)
+    exp = _bigram_table(corpus, 1 << 20, 2)
+    d = dev(corpus)
+    for _ in range(3):
+        ft.cb_frozen_build(d)
+        for a, b in zip(ft.cb_frozen_dump(), exp):
+            assert np.array_equal(a, b)

@@ -268,7 +268,10 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                                 if ((!two || l == 0) && !(ok = mbar_wait(bar_full(vs), (vseq / ns) & 1, s_abort, p.status))) break;
                                 if (!(ok = mbar_wait(bar_pready(l), c_p[l] & 1, s_abort, p.status))) break;
                                 ++c_p[l];
+                                // the unit before is done with this chain's accumulator; a chain without a tile of this unit takes its turn
+                                // on the barrier here too: it is done with its row sums before odone_both lets it write the next ones
                                 if (e < 4 && uq > 0 && !(ok = mbar_wait(bar_ofree(l), (uq - 1) & 1, s_abort, p.status))) break;
+                                if (nev < 2 && uq > 0 && !(ok = mbar_wait(bar_ofree(1), (uq - 1) & 1, s_abort, p.status))) break;
                                 tc_fence_after();
                                 mma_pv_halves_block<D>(tmem + C::O_COL + l * D, tmem + l * 128, desc_lo(slot_base(vs), 1024), idesc_o, e < 4 ? 0u : 1u);
                                 if (!two || l == 1) tc_commit(bar_free(vs));
@@ -289,8 +292,6 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                             }
                         }
                     }
-                    // a chain without a tile in this unit still takes its turn on the accumulator's barrier
-                    if (ok && nev < 2 && uq > 0 && !(ok = mbar_wait(bar_ofree(1), (uq - 1) & 1, s_abort, p.status))) break;
                     seq0 += 2u * (uint32_t)nt;
                     ++uq;
                 }
@@ -550,13 +551,15 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             uint32_t arrived = 0;
             if (np > 1 && lane == 0) arrived = ld_acquire(ticket);
             if (two) {
+                // The wait comes before s_x is written: the unit's first product follows the other chain's end of the unit before
+                // (bar_ofree), and if that one had one row tile, the other chain read this chain's row sums there.
+                if (!(ok = mbar_wait(bar_odone(l), c_od & 1, s_abort, p.status))) break;
+                ++c_od;
                 s_x[(l * 2 + hf) * CB_MT + row] = lsum;
                 pair_sync(false, 2);
                 x_l = lsum + s_x[(l * 2 + 1 - hf) * CB_MT + row];
                 x_m = m_used; x_w0 = x_w1 = 1.f;
                 npc = CW / 8; c0 = hf * 2 * CW;
-                if (!(ok = mbar_wait(bar_odone(l), c_od & 1, s_abort, p.status))) break;
-                ++c_od;
             } else {
                 if (!(ok = mbar_wait(bar_odone_both, c_ob & 1, s_abort, p.status))) break;
                 ++c_ob;

@@ -6,7 +6,8 @@ import pytest
 import torch
 
 import workloads as W
-from tests.harness import tree_mask_from_parents, Problem, dev, device_attn_inputs, synthetic_trees, oracle_attn_rows, bf16_to_f64
+from tests.harness import (tree_mask_from_parents, Problem, dev, device_attn_inputs, synthetic_trees, oracle_attn_rows, oracle_attn_rows_by_head,
+                           stream_k_shares, bf16_to_f64)
 
 pytestmark = pytest.mark.gpu
 
@@ -259,3 +260,46 @@ def test_attn_units_shared_by_many_ctas(oracle, cfg, ctx):
     hh = torch.tensor([r[0] for r in rows], device="cuda")
     ii = torch.tensor([r[1] for r in rows], device="cuda")
     _check_rows(bf16_to_f64(outs[0][0][0, ii, hh]), outs[0][1][0, hh, ii].cpu().numpy().astype(np.float64), ref, ref_lse, (cfg.name, ctx))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_attn_one_tile_shares_between_units_of_one_and_two_row_tiles(oracle, d):
+    """A unit of one row tile is put together by both softmax chains from row sums that they exchange in shared memory; the unit after
+    it may be a share of a single key tile (a context of none, or the end of a CTA's range), whose sums go to the same places.  Every row
+    of the units on both sides of such a change, the same bits in every one of 20 calls."""
+    from paper_2511_21699_b200 import Cacheback
+    B, T = 256, 40
+    cfg = W.CbConfig("one_tile_shares", B, 2, 2, 64, 2, T, 6, 0, 4, 1, d, (0, 600), 100, 1.1, 0.3, (4, 8), 64)
+    prob = Problem(cfg)
+    rng = np.random.default_rng(12)
+    prob.ctx = rng.choice([0, 0, 0, 130, 600], B).astype(np.int32)
+    prob.bt, prob.num_pages = W.make_block_table(cfg, np.maximum(prob.ctx, 1))
+    par, dep, mask, n = synthetic_trees(cfg, full=False)
+    n[:] = np.where(np.arange(B) % 2, rng.choice([33, 40], B), rng.choice([5, 31], B))     # a row tile holds 32 nodes
+    for b in range(B):
+        par[b], dep[b] = W.random_tree(cfg.seed, b, int(n[b]), cfg.max_depth, T)
+        mask[b] = tree_mask_from_parents(par[b], int(n[b]), (T + 31) // 32)
+    units, one_two, two_one = set(), 0, 0
+    ctas = stream_k_shares(cfg, prob.ctx, n, min(torch.cuda.get_device_properties(0).multi_processor_count, 160))
+    for shares in ctas:
+        for a, b in zip(shares, shares[1:]):
+            if a[3] != b[3] and b[6] - b[5] == 1:
+                units |= {a[:4], b[:4]}
+                one_two += b[3] == 2
+                two_one += b[3] == 1
+    assert one_two >= 16 and two_one >= 16, (one_two, two_one)
+    d_in = device_attn_inputs(cfg, prob)
+    cb = Cacheback.from_config(cfg)
+    mask_d, n_d = dev(mask.view(np.int32)), dev(n)
+    outs = []
+    for _ in range(20):
+        lse = torch.full((B, cfg.n_q_heads, T), 7.0, dtype=torch.float32, device="cuda")
+        outs.append((cb.cb_tree_attn(d_in["q"], d_in["k_pool"], d_in["v_pool"], d_in["block_table"], d_in["ctx_len"], d_in["k_tree"], d_in["v_tree"],
+                                     mask_d, n_d, lse=lse, max_ctx=int(prob.ctx.max())), lse))
+    assert cb.cb_poll_status()[0] == 0
+    assert all(torch.equal(outs[0][0], o) and torch.equal(outs[0][1], l) for o, l in outs[1:])
+    rows = np.array([(b, kh * cfg.gqa + g, i) for b, kh, rg, nrt in sorted(units) for g in range(cfg.gqa)
+                     for i in range(rg * 64, min(rg * 64 + 32 * nrt, int(n[b])))], np.int64)
+    ref, ref_lse = oracle_attn_rows_by_head(oracle, cfg, prob, mask, rows)
+    bb, hh, ii = (torch.from_numpy(rows[:, k]).cuda() for k in range(3))
+    _check_rows(bf16_to_f64(outs[0][0][bb, ii, hh]), outs[0][1][bb, hh, ii].cpu().numpy().astype(np.float64), ref, ref_lse, (cfg.name, d))

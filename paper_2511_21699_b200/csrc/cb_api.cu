@@ -45,10 +45,10 @@ cb_status cb_compute_layout(const cb_config* c, CbLayout* L) {
     L->off_index = region(B * ns * 4);
     L->off_lstamp = region(B * (size_t)c->LC * 4);
     L->off_entries = region(B * (size_t)c->LC * L->E * 4);
-    L->off_status = region(4 * 4);
+    L->off_status = region(16 * 4);                          // status words; from word 8 on, what tree attention's launches hand on
     L->off_counters = region(CB_NUM_COUNTERS * 8);
     L->off_rowmax = region(B * (size_t)c->max_nodes * 8);
-    L->off_ticket = region(align_up(B * 4, 256) + CB_ATTN_TICKETS * 4);      // acceptance's counters, then tree attention's
+    L->off_ticket = region(align_up(B * 4, 256) + 2 * CB_ATTN_TICKETS * 4);  // acceptance's counters, then tree attention's
     L->off_attn_ticket = L->off_ticket + align_up(B * 4, 256);
     L->off_bulk_plan = region(B * 16);
     L->attn_max_units = CB_ATTN_MAX_UNITS;
@@ -99,6 +99,7 @@ extern "C" cb_status cb_create(const cb_config* cfg, void* dev_workspace, size_t
     c->d_ticket = (uint32_t*)(c->ws + L.off_ticket);
     c->d_bulk_plan = (uint32_t*)(c->ws + L.off_bulk_plan);
     c->d_attn_ticket = (uint32_t*)(c->ws + L.off_attn_ticket);
+    c->d_attn_turn = c->d_status + 8;
     c->d_attn_part = (float*)(c->ws + L.off_attn_part);
     c->attn_part_floats = L.attn_part_floats;
     c->attn_max_units = L.attn_max_units;
@@ -227,8 +228,6 @@ extern "C" cb_status cb_poll_status(cb_ctx* ctx, cb_status* device_status, uint6
     }
     if (device_status) *device_status = (cb_status)st[0];
     if (st[0] != 0) CB_CUDA(cudaMemset(ctx->d_status, 0, sizeof(st)));
-    // an attention launch that gave up may have left its counts of shared units half way
-    if (st[0] == (uint32_t)CB_ERR_TIMEOUT) CB_CUDA(cudaMemset(ctx->d_attn_ticket, 0, CB_ATTN_TICKETS * 4));
     if (counters) CB_CUDA(cudaMemcpy(counters, ctx->d_counters, CB_NUM_COUNTERS * 8, cudaMemcpyDeviceToHost));
     return CB_OK;
 }

@@ -133,7 +133,7 @@ extern "C" cb_status cb_tree_attn(cb_ctx* ctx, const cb_attn_args* a, void* stre
     p.block_table = a->block_table; p.ctx_len = a->ctx_len;
     p.k_tree = (const __nv_bfloat16*)a->k_tree; p.v_tree = (const __nv_bfloat16*)a->v_tree;
     p.tree_mask = a->tree_mask; p.n_nodes = a->n_nodes;
-    p.out = (__nv_bfloat16*)a->out; p.lse = a->lse; p.part = ctx->d_attn_part; p.part_ticket = ctx->d_attn_ticket;
+    p.out = (__nv_bfloat16*)a->out; p.lse = a->lse; p.part = ctx->d_attn_part; p.part_ticket = ctx->d_attn_ticket; p.part_turn = ctx->d_attn_turn;
     p.B = c.batch; p.T = c.max_nodes; p.W = (c.max_nodes + 31) / 32; p.Hq = c.n_q_heads; p.Hkv = c.n_kv_heads;
     p.G = c.n_q_heads / c.n_kv_heads; p.D = c.head_dim; p.P = c.page_size;
     p.max_pages = a->max_pages; p.num_pages = a->num_pages;

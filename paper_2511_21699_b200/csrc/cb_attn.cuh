@@ -36,7 +36,8 @@ struct CbAttnParams {
     __nv_bfloat16* out;
     float* lse;
     float* part;          // [2 * nc slots] of 2 * 128 * (D + 4) floats: unnormalised output columns, running max (log2 domain), sum
-    uint32_t* part_ticket; // [nc][16 softmax warps]: parts of a shared unit left in memory so far, zero between calls
+    uint32_t* part_ticket; // [2 sets][CB_ATTN_MAX_CTAS][16 softmax warps]: parts of a shared unit left in memory so far
+    uint32_t* part_turn;  // [0] launches of the context so far: the lowest bit names the set in use; [1] CTAs of this one that have left
     int B, T, W, Hq, Hkv, G, D, P, max_pages, num_pages;
     int NPT;              // tree nodes per row tile = 128 / G
     int MT;               // row tiles that T nodes need = ceil(T / NPT)

@@ -41,8 +41,8 @@
 namespace {
 
 // A unit as the softmax warps see it (nrt = 0: no more units).  cf, np: the CTA that holds the unit's first key tile and the number of
-// CTAs that hold one; xpos: position of that tile where a CTA holds one tile at most, else -1.
-struct UnitDesc { int b, kh, rg, t0, t1, tiles, n, ctx, nrt, cf, np, xpos, wt, pad; };
+// CTAs that hold one; ticket: where its parts are counted; xpos: position of that tile where a CTA holds one tile at most, else -1.
+struct UnitDesc { int b, kh, rg, t0, t1, tiles, n, ctx, nrt, cf, np, xpos, wt, ticket; };
 constexpr int kFmaExpPhase = 3;                              // of every four pairs of exponentials this one is taken by the FMA pipe
 constexpr int kUnitRing = 4;                                 // units published ahead of the slowest softmax thread: at most two
 
@@ -152,6 +152,13 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
         if (lane < 16) s_pair[lane] = 0;
     }
     CB_PDL_ENTRY();
+    // The set of tickets that this launch counts in.  The other one is cleared for the next launch, so that it finds zeros even
+    // where the launch before this one gave up on a wait and left counts half way, whatever the status word says.
+    int ticket_set = 0;
+    if (warp == 2 && p.cs == 0) {
+        ticket_set = (int)(*reinterpret_cast<volatile uint32_t*>(p.part_turn) & 1u) * CB_ATTN_TICKETS;
+        if (lane < 16) p.part_ticket[CB_ATTN_TICKETS - ticket_set + cta * 16 + lane] = 0u;
+    }
     if (warp == 3) {
         // The block table into L2, a slice per CTA: the first copies' addresses come from it, and which part of it a CTA needs is
         // known only after the schedule below (two memory round trips one after the other otherwise).
@@ -316,6 +323,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                         d->np = wide ? cb_cta_of(tot, p.nc, x0 + (long long)(u.tiles - 1) * wt) - cf + 1 : u.tiles;
                         d->xpos = wide ? -1 : (int)x0;
                         d->wt = wt;
+                        d->ticket = ticket_set + cf * 16;
                     }
                     mbar_arrive(bar_ufull(uq % kUnitRing));
                     if (uq > 0 && !(ok = mbar_wait(bar_qfree, (uq - 1) & 1, s_abort, p.status))) break;
@@ -546,8 +554,8 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             int npc, c0;
             // a shared unit: how many parts of it are in memory already (most often all the others, see below); the look is taken here,
             // where it overlaps the wait for the last product
-            const int np = whole || p.cs > 0 ? 1 : u->np, cf = whole || p.cs > 0 ? 0 : u->cf;
-            uint32_t* const ticket = p.part_ticket + cf * 16 + sw;
+            const int np = whole || p.cs > 0 ? 1 : u->np;
+            uint32_t* const ticket = p.part_ticket + (np > 1 ? u->ticket : 0) + sw;
             uint32_t arrived = 0;
             if (np > 1 && lane == 0) arrived = ld_acquire(ticket);
             if (two) {
@@ -630,7 +638,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     // writes the output.  Nobody waits.  (A CTA's first unit is shared with the CTA before it, which comes to it
                     // last, so most often the partial has long been there: the pass that merged both partials from memory after the
                     // kernel cost 9 us a call at batch 32.)  A warp's partial is laid out by lane: 512 bytes per access.
-                    const int xpos = u->xpos;
+                    const int xpos = u->xpos, cf = u->cf;
                     auto slot_of = [&](int cc, bool start) {
                         return p.part + (size_t)(2 * cc + (start ? 1 : 0)) * (2 * CB_MT * (D + 4));
                     };
@@ -660,7 +668,6 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     }
                     if (last) {
                         __syncwarp();
-                        if (lane == 0) *reinterpret_cast<volatile uint32_t*>(ticket) = 0u;   // for the next call
                         float mx = -INFINITY, sum = 0.f;
                         if (np == 2) {
                             // the usual case: one other part, its columns fetched a group ahead
@@ -824,6 +831,8 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+        // the last CTA to leave hands the turn on: nobody looks at this launch's tickets any more
+        if (p.cs == 0 && elect_one() && atomicInc(&p.part_turn[1], gridDim.x - 1u) == gridDim.x - 1u) atomicAdd(&p.part_turn[0], 1u);
     }
 }
 

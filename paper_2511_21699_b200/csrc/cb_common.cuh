@@ -90,7 +90,7 @@ struct cb_ctx {
     CbTables tables;
     CbTables frozen;        // the read-only table of cb_frozen_attach (one "sequence", shared by the batch)
     bool has_frozen;
-    uint32_t* d_status;     // [4]
+    uint32_t* d_status;     // [4], the head of a block of 16 words
     unsigned long long* d_counters;  // [CB_NUM_COUNTERS]
     unsigned long long* d_rowmax;    // [batch * max_nodes] packed (value, index) maxima, zero between calls
     uint32_t* d_ticket;     // [batch] CTAs-finished counters, zero between calls
@@ -100,7 +100,8 @@ struct cb_ctx {
     size_t guard_off[CB_MAX_GUARDS];
     int n_guards;
     float* d_attn_part;     // partial outputs of units shared between CTAs
-    uint32_t* d_attn_ticket; // [CTAs][16] parts of a shared unit that are in memory, zero between calls
+    uint32_t* d_attn_ticket; // [2][CTAs][16] parts of a shared unit that are in memory; an attention launch counts in one set and clears the other
+    uint32_t* d_attn_turn;   // [0] attention launches so far, its lowest bit names the set; [1] CTAs of the running one that have left
     size_t attn_part_floats;
     int attn_max_units;     // partial row tiles available
     int num_sms;

@@ -234,8 +234,8 @@ def _few_heads(name, hq, hkv, d, t):
     (_few_heads("shared_d64", 16, 1, 64, 17), 9001),
 ], ids=lambda x: getattr(x, "name", x))
 def test_attn_units_shared_by_many_ctas(oracle, cfg, ctx):
-    """Units whose parts lie in many CTAs, combined by the last of them to come: three times with the same context (the tickets are
-    back at zero, the result does not depend on who comes last), output rows that are aligned to 16 bytes and not to 32."""
+    """Units whose parts lie in many CTAs, combined by the last of them to come: three times with the same context (each time the tickets count
+    from zero, the result does not depend on who comes last), output rows that are aligned to 16 bytes and not to 32."""
     from paper_2511_21699_b200 import Cacheback
     prob = Problem(cfg)
     prob.ctx = np.array([ctx], np.int32)
@@ -303,3 +303,43 @@ def test_attn_one_tile_shares_between_units_of_one_and_two_row_tiles(oracle, d):
     ref, ref_lse = oracle_attn_rows_by_head(oracle, cfg, prob, mask, rows)
     bb, hh, ii = (torch.from_numpy(rows[:, k]).cuda() for k in range(3))
     _check_rows(bf16_to_f64(outs[0][0][bb, ii, hh]), outs[0][1][bb, hh, ii].cpu().numpy().astype(np.float64), ref, ref_lse, (cfg.name, d))
+
+
+@pytest.mark.parametrize("poll", [True, False])
+def test_attn_after_a_launch_that_left_its_tickets_half_way(oracle, poll):
+    """A launch that gives up on a wait leaves counts of shared units behind, and its status may go unseen behind an earlier one.  The
+    state is planted from the host: counts of one everywhere in the set that the last launch used, a status of another call's, other
+    partials in memory.  The next calls are right, polled or not."""
+    import ctypes as C
+    from paper_2511_21699_b200 import Cacheback, _lib
+    cfg = W.CbConfig("left_tickets", 9, 2, 2, 64, 2, 64, 6, 0, 32, 8, 128, (1000, 1000), 100, 1.1, 0.3, (4, 8), 64)   # two or three CTAs a unit
+    prob = Problem(cfg)
+    B, T = cfg.batch, cfg.max_nodes
+    _, _, mask, n = synthetic_trees(cfg, full=True)
+    d = device_attn_inputs(cfg, prob)
+    cb = Cacheback.from_config(cfg)
+    call = lambda q, lse: cb.cb_tree_attn(q, d["k_pool"], d["v_pool"], d["block_table"], d["ctx_len"], d["k_tree"], d["v_tree"],
+                                          dev(mask.view(np.int32)), dev(n), lse=lse, max_ctx=1000)
+    # the workspace from its end: partial outputs, the bulk update's plans (16 bytes a sequence), two sets of 160 x 16 ticket words
+    up = lambda x: (x + 255) // 256 * 256
+    nbytes = C.c_size_t(0)
+    assert cb.lib.cb_workspace_bytes(C.byref(cb.cfg), C.byref(nbytes)) == 0
+    base = up(cb.workspace.data_ptr()) - cb.workspace.data_ptr()
+    tickets_at = base + nbytes.value - up(640 * 128 * (cfg.head_dim + 4) * 4) - up(16 * cfg.batch) - 2 * 160 * 16 * 4
+    tickets = cb.workspace[tickets_at:tickets_at + 2 * 160 * 16 * 4].view(torch.int32).view(2, 160, 16)
+    call(-d["q"], None)                                    # other partials
+    used = (tickets != 0).flatten(1).any(1)
+    assert bool(used[0]) and not bool(used[1]), "the ticket words are not where this test looks for them"
+    tickets[0] = 1
+    none = torch.zeros(B, dtype=torch.int32, device="cuda")          # a commit that finds the sequences' pages full
+    cb.cb_kv_commit(d["k_pool"], d["v_pool"], d["block_table"], none + prob.bt.shape[1] * cfg.page_size, d["k_tree"], d["v_tree"], none,
+                    none.view(B, 1).expand(B, cfg.max_depth).contiguous())
+    if poll:
+        assert cb.cb_poll_status()[0] == _lib.CB_ERR_KV_FULL
+    rows = np.array([(b, h, i) for b in range(B) for h in range(0, cfg.n_q_heads, 4) for i in (0, 40)], np.int64)     # every unit, both row tiles
+    ref, ref_lse = oracle_attn_rows_by_head(oracle, cfg, prob, mask, rows)
+    bb, hh, ii = (torch.from_numpy(rows[:, k]).cuda() for k in range(3))
+    for _ in range(3):
+        lse = torch.full((B, cfg.n_q_heads, T), 7.0, dtype=torch.float32, device="cuda")
+        out = call(d["q"], lse)
+        _check_rows(bf16_to_f64(out[bb, ii, hh]), lse[bb, hh, ii].cpu().numpy().astype(np.float64), ref, ref_lse, cfg.name)

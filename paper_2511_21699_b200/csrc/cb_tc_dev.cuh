@@ -206,15 +206,26 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ float clamp_keep_nan(float x, float lo, float hi) {
+    asm("max.NaN.f32 %0, %0, %1;\n\tmin.NaN.f32 %0, %0, %2;" : "+f"(x) : "f"(lo), "f"(hi));
+    return x;
+}
 // 2^x of a pair on the FMA and integer pipes, for the share of a tile's exponentials that the exponential unit (a warp instruction
 // every 8 cycles) would hold up: x = n + f with n the nearest whole number (added and taken off again as 1.5 * 2^23), 2^f on
-// [-0.5, 0.5] by the degree-5 polynomial of smallest relative error (Remez exchange: 7.5e-8, against 2^-22 of ex2.approx), n
-// added to the exponent.  x is clamped to [-126, 127]: below, 2^-126 stands for what would round to nothing beside the row's
-// sum; above, 2^127 sends the tile to the two-pass form like any sum over its limit.
+// [-0.5, 0.5] by the degree-5 polynomial of smallest relative error (Remez exchange: 7.5e-8, against 2^-22 of ex2.approx), and
+// 2^n put together in the exponent's place.  x is clamped to [-127, 127]: 2^-127 is put together as zero, which is what
+// ex2.approx.ftz makes of everything below -126; above, 2^127 sends the tile to the two-pass form like any sum over its limit.
+// NaN stays NaN (a broken key shows in its rows whichever place of the tile it has), hence the clamp that keeps it and a product
+// by 2^n where adding n to the exponent's bits would make a number of it.
 __device__ __forceinline__ void ex2_pair_fma(uint64_t x, float& a, float& b) {
     float x0, x1;
     f2_unpack(x, x0, x1);
-    x = f2_pack(fminf(fmaxf(x0, -126.f), 127.f), fminf(fmaxf(x1, -126.f), 127.f));
+    x = f2_pack(clamp_keep_nan(x0, -127.f, 127.f), clamp_keep_nan(x1, -127.f, 127.f));
     const uint64_t r = f2_add(x, f2_pack(12582912.f, 12582912.f));
     const uint64_t f = f2_fma(f2_add(r, f2_pack(-12582912.f, -12582912.f)), f2_pack(-1.f, -1.f), x);
     uint64_t y = f2_pack(1.3276472454890609e-3f, 1.3276472454890609e-3f);
@@ -223,11 +234,9 @@ __device__ __forceinline__ void ex2_pair_fma(uint64_t x, float& a, float& b) {
     y = f2_fma(y, f, f2_pack(2.4022120237350464e-1f, 2.4022120237350464e-1f));
     y = f2_fma(y, f, f2_pack(6.931469440460205e-1f, 6.931469440460205e-1f));
     y = f2_fma(y, f, f2_pack(1.f, 1.f));
-    float y0, y1, r0, r1;
-    f2_unpack(y, y0, y1);
+    float r0, r1;
     f2_unpack(r, r0, r1);
-    a = __int_as_float(__float_as_int(y0) + (__float_as_int(r0) << 23));
-    b = __int_as_float(__float_as_int(y1) + (__float_as_int(r1) << 23));
+    f2_unpack(f2_mul(y, f2_pack(__int_as_float((__float_as_int(r0) << 23) + 0x3F800000), __int_as_float((__float_as_int(r1) << 23) + 0x3F800000))), a, b);
 }
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
     float d;

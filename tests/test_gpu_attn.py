@@ -343,3 +343,25 @@ def test_attn_after_a_launch_that_left_its_tickets_half_way(oracle, poll):
         lse = torch.full((B, cfg.n_q_heads, T), 7.0, dtype=torch.float32, device="cuda")
         out = call(d["q"], lse)
         _check_rows(bf16_to_f64(out[bb, ii, hh]), lse[bb, hh, ii].cpu().numpy().astype(np.float64), ref, ref_lse, cfg.name)
+
+
+@pytest.mark.parametrize("cfg", [W.CbConfig("nan_two_rows", 8, 2, 2, 64, 2, 40, 6, 0, 8, 2, 128, (300, 300), 100, 1.1, 0.3, (4, 8), 64),
+                                 W.CbConfig("nan_one_row", 8, 2, 2, 64, 2, 24, 6, 0, 8, 2, 64, (300, 300), 100, 1.1, 0.3, (4, 8), 64)],
+                         ids=lambda c: c.name)
+def test_attn_nan_key_reaches_its_rows(cfg):
+    """A key that is NaN makes every row of its sequence and kv head NaN, whichever of the softmax's two forms of the exponential its
+    place in the tile gets (a place in eight per sequence, in a tile that needs no masks); the other kv head's rows stay finite."""
+    from paper_2511_21699_b200 import Cacheback
+    prob = Problem(cfg)
+    B, T = cfg.batch, cfg.max_nodes
+    _, _, mask, n = synthetic_trees(cfg, full=True)
+    d = device_attn_inputs(cfg, prob)
+    for b in range(B):
+        pos = 128 + 40 + b
+        d["k_pool"][int(prob.bt[b, pos // 16]), pos % 16, 0] = float("nan")
+    out = Cacheback.from_config(cfg).cb_tree_attn(d["q"], d["k_pool"], d["v_pool"], d["block_table"], d["ctx_len"], d["k_tree"], d["v_tree"],
+                                                  dev(mask.view(np.int32)), dev(n), max_ctx=300)
+    G = cfg.gqa
+    bad = torch.isnan(out[:, :, :G].float()).flatten(1).all(1)
+    assert bad.all(), bad.tolist()
+    assert torch.isfinite(out[:, :, G:].float()).all()

@@ -217,7 +217,8 @@ __device__ __forceinline__ float clamp_keep_nan(float x, float lo, float hi) {
 }
 // 2^x of a pair on the FMA and integer pipes, for the share of a tile's exponentials that the exponential unit (a warp instruction
 // every 8 cycles) would hold up: x = n + f with n the nearest whole number (added and taken off again as 1.5 * 2^23), 2^f on
-// [-0.5, 0.5] by the degree-5 polynomial of smallest relative error (Remez exchange: 7.5e-8, against 2^-22 of ex2.approx), and
+// [-0.5, 0.5] by the degree-5 polynomial with constant term 1 of smallest relative error (coefficients rounded one after the other, the
+// rest fitted again: 9.4e-8; 1.5e-7 evaluated in fp32, by microbench/exp2_error.cu, against 2^-22 = 2.4e-7 of ex2.approx), and
 // 2^n put together in the exponent's place.  x is clamped to [-127, 127]: 2^-127 is put together as zero, which is what
 // ex2.approx.ftz makes of everything below -126; above, 2^127 sends the tile to the two-pass form like any sum over its limit.
 // NaN stays NaN (a broken key shows in its rows whichever place of the tile it has), hence the clamp that keeps it and a product
@@ -228,11 +229,11 @@ __device__ __forceinline__ void ex2_pair_fma(uint64_t x, float& a, float& b) {
     x = f2_pack(clamp_keep_nan(x0, -127.f, 127.f), clamp_keep_nan(x1, -127.f, 127.f));
     const uint64_t r = f2_add(x, f2_pack(12582912.f, 12582912.f));
     const uint64_t f = f2_fma(f2_add(r, f2_pack(-12582912.f, -12582912.f)), f2_pack(-1.f, -1.f), x);
-    uint64_t y = f2_pack(1.3276472454890609e-3f, 1.3276472454890609e-3f);
-    y = f2_fma(y, f, f2_pack(9.675540961325169e-3f, 9.675540961325169e-3f));
-    y = f2_fma(y, f, f2_pack(5.550713092088699e-2f, 5.550713092088699e-2f));
-    y = f2_fma(y, f, f2_pack(2.4022120237350464e-1f, 2.4022120237350464e-1f));
-    y = f2_fma(y, f, f2_pack(6.931469440460205e-1f, 6.931469440460205e-1f));
+    uint64_t y = f2_pack(1.3268813490867615e-3f, 1.3268813490867615e-3f);
+    y = f2_fma(y, f, f2_pack(9.67121496796608e-3f, 9.67121496796608e-3f));
+    y = f2_fma(y, f, f2_pack(5.5507123470306396e-2f, 5.5507123470306396e-2f));
+    y = f2_fma(y, f, f2_pack(2.402224838733673e-1f, 2.402224838733673e-1f));
+    y = f2_fma(y, f, f2_pack(6.931470036506653e-1f, 6.931470036506653e-1f));
     y = f2_fma(y, f, f2_pack(1.f, 1.f));
     float r0, r1;
     f2_unpack(r, r0, r1);

@@ -365,3 +365,25 @@ def test_attn_nan_key_reaches_its_rows(cfg):
     bad = torch.isnan(out[:, :, :G].float()).flatten(1).all(1)
     assert bad.all(), bad.tolist()
     assert torch.isfinite(out[:, :, G:].float()).all()
+
+
+def test_exponential_of_the_fma_pipe(tmp_path):
+    """The softmax's own 2^x against exp2 in double over [-126, 127], both ends, beyond them, infinities and NaN.  Bound: 9.4e-8 of the
+    polynomial, 2^-24 of the last rounding and a sixth of that for the product before it."""
+    import os
+    import subprocess
+    from paper_2511_21699_b200 import build as b
+    exe = str(tmp_path / "exp2_error")
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")] + b.NVCC_FLAGS + ["-diag-suppress", "177", "-o", exe,
+                          os.path.join(b.HERE, "microbench", "exp2_error.cu")])
+    lines = [l.split() for l in subprocess.run([exe], check=True, capture_output=True, text=True, timeout=60).stdout.splitlines()]
+    fig = {l[0]: float(l[1]) for l in lines if l[0] != "edge"}
+    assert fig["values"] > 1e6 and fig["fma_max_rel"] <= 9.42e-8 + 2.0 ** -24 * 7 / 6 and abs(fig["fma_mean_rel"]) <= 3e-8, fig
+    edge = {l[1]: (float(l[2]), float(l[3])) for l in lines if l[0] == "edge"}
+    for x in ("-inf", "-1e+30", "-300", "-127.5", "-127"):
+        assert edge[x] == (0.0, 0.0), (x, edge[x])
+    assert 0.0 <= edge["-126.5"][0] < 2.0 ** -126              # ex2.approx.ftz: 0
+    for x in ("127.01", "300", "inf"):                         # stands for "over the row sum's limit"
+        assert edge[x][0] == 2.0 ** 127, (x, edge[x])
+    assert edge["0"] == (1.0, 1.0) and edge["127"] == (2.0 ** 127, 2.0 ** 127)
+    assert np.isnan(edge["nan"][0]) and np.isnan(edge["nan"][1])

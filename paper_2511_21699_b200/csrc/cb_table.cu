@@ -899,8 +899,13 @@ struct AcceptArgs {
     int32_t* n_accept; int32_t* accept_nodes; int32_t* out_tokens; int32_t* target_out;
 };
 
-template <int FETCH, bool BF16>
-__global__ void __launch_bounds__(256) cb_accept_draft_kernel(AcceptArgs a, CbTables t, CbTables tf, int T, int crt, int max_depth, int NL, int KF,
+// CTAS: CTAs that an SM has registers for.  The drafting code takes 96 registers and up, room for two.  A grid that is not resident at
+// once that way streams the logits with a third less in flight than with three CTAs of 75 (batch 32, fp32 logits over 128 k tokens: 287
+// against 216 us; batch 2 over 32 k: 16.9 against 16.0); one that is gains nothing from the bound and pays for it in the chain behind
+// the logits (batch 1 over 32 k: 13.9 against 14.2 us, a whole step 45.1 against 46.3).  With more than 32 followers a leader the code
+// takes 116 registers and stays at two.
+template <int FETCH, bool BF16, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) cb_accept_draft_kernel(AcceptArgs a, CbTables t, CbTables tf, int T, int crt, int max_depth, int NL, int KF,
                                                               int32_t* tokens, int64_t row_stride, int32_t* seq_len,
                                                               int32_t* o_tok, int32_t* o_par, int32_t* o_dep, uint32_t* o_mask, int32_t* o_n,
                                                               uint32_t* status, unsigned long long* counters) {
@@ -1087,13 +1092,15 @@ extern "C" cb_status cb_accept_update_draft_tree(cb_ctx* ctx, const cb_accept_dr
     const size_t smem = sizeof(int32_t) * ((size_t)3 * T + (size_t)11 * NL + (size_t)NL * c.FL * KF);
     if (smem > 200 * 1024) return CB_ERR_UNSUPPORTED;
     const bool bf = a->logits_dtype == CB_DTYPE_BF16;
-    auto kernel = FCmax <= 32 ? (bf ? cb_accept_draft_kernel<1, true> : cb_accept_draft_kernel<1, false>)
-                              : (bf ? cb_accept_draft_kernel<2, true> : cb_accept_draft_kernel<2, false>);
+    const bool resident = (long long)cpr * T * c.batch <= 2ll * ctx->num_sms;
+    auto kernel = FCmax > 32  ? (bf ? cb_accept_draft_kernel<2, true, 2> : cb_accept_draft_kernel<2, false, 2>)
+                  : resident  ? (bf ? cb_accept_draft_kernel<1, true, 2> : cb_accept_draft_kernel<1, false, 2>)
+                              : (bf ? cb_accept_draft_kernel<1, true, 3> : cb_accept_draft_kernel<1, false, 3>);
     if (smem > 48 * 1024) {
         static std::mutex mu;
-        static size_t opted[64][4] = {};                       // largest size opted into so far, per device and kernel
+        static size_t opted[64][6] = {};                       // largest size opted into so far, per device and kernel
         std::lock_guard<std::mutex> lock(mu);
-        const int d = ctx->device & 63, k = (FCmax <= 32 ? 0 : 2) + (bf ? 1 : 0);
+        const int d = ctx->device & 63, k = (FCmax > 32 ? 0 : resident ? 2 : 4) + (bf ? 1 : 0);
         if (opted[d][k] < smem) {
             CB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             opted[d][k] = smem;

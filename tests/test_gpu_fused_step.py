@@ -18,8 +18,18 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("name,dtype,steps", [("c1_tiny", "f32", 8), ("c1_tiny", "bf16", 8), ("c2_7b", "f32", 6), ("c4_13b_turns", "f32", 4),
                                               ("p_tuned", "f32", 5)])
 def test_accept_update_draft_in_one_launch(oracle, name, dtype, steps):
+    _loop(oracle, W.get_config(name), dtype, steps)
+
+
+@pytest.mark.parametrize("batch,dtype", [(1, "f32"), (2, "f32"), (2, "bf16"), (3, "bf16")])
+def test_grids_on_both_sides_of_two_ctas_a_sm(oracle, batch, dtype):
+    """64 nodes x 32 k tokens in four (two) chunks a row: 256 CTAs run at once two to an SM, 384 and 512 take the form for three."""
+    from dataclasses import replace
+    _loop(oracle, replace(W.get_config("c2_7b"), name="c2_small_batch", batch=batch, max_nodes=64), dtype, 3)
+
+
+def _loop(oracle, cfg, dtype, steps):
     from paper_2511_21699_b200 import Cacheback
-    cfg = W.get_config(name)
     prob = Problem(cfg)
     B, T, V = cfg.batch, cfg.max_nodes, cfg.vocab
     cb = Cacheback.from_config(cfg)
@@ -90,7 +100,7 @@ def test_accept_update_draft_in_one_launch(oracle, name, dtype, steps):
     _assert_tables_equal(cb, otabs, check)
     assert cb.cb_poll_status()[0] == 0
     assert emitted >= steps * len(check)
-    if name in ("c1_tiny", "p_tuned"):
+    if cfg.name in ("c1_tiny", "p_tuned"):
         assert emitted > steps * len(check)                   # draft tokens were accepted, not only bonus tokens
 
 

@@ -282,7 +282,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                                 tc_fence_after();
                                 mma_pv_halves_block<D>(tmem + C::O_COL + l * D, tmem + l * 128, desc_lo(slot_base(vs), 1024), idesc_o, e < 4 ? 0u : 1u);
                                 if (!two || l == 1) tc_commit(bar_free(vs));
-                                if (two ? iv == nt - 1 : iv == nt - 1) tc_commit(two ? bar_odone(l) : bar_odone_both);
+                                if (iv == nt - 1) tc_commit(two ? bar_odone(l) : bar_odone_both);
                             }
                         }
                         if (ik < nt) {

@@ -1,10 +1,11 @@
-// Microbenchmark behind the figures the design doc quotes for the tensor-core side of tree attention.
+// Microbenchmark behind the figures quoted for the tensor-core side of tree attention.
 //
 //   nvcc -gencode arch=compute_100a,code=sm_100a -O3 -o mma_issue mma_issue.cu && ./mma_issue
 //
 // Throughput of tcgen05.mma blocks as the attention kernels issue them: time to issue n MMAs (128x128x16 per SM, bf16) and
 // time until their commit completes, for cta_group::1 and for a pair of CTAs with cta_group::2; also 128xNx16 with N = 64
-// and N = 256 (cta_group::1, both operands from shared memory).  Operands are whatever
+// (A from shared memory or from TMEM) and N = 256 (cta_group::1).  The attention kernel issues from an elected lane (elect.sync, the
+// compiler knows that one thread runs the code); the form guarded by `lane == 0` is timed beside it.  Operands are whatever
 // shared memory holds (zeroed); only timing matters.
 #include <cstdio>
 #include <cstdint>
@@ -37,7 +38,13 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint32_t blo
 }
 
 // res[0..]: per repetition (issue cycles, cycles until the commit's barrier completed)
-template <int CG, int TS, int NN = 128>
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0u;
+}
+
+template <int CG, int TS, int NN = 128, bool ELECT = true>
 __global__ void __launch_bounds__(128, 1) k(long long* res, int n_mma, int reps) {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) unsigned long long bar;
@@ -66,7 +73,7 @@ __global__ void __launch_bounds__(128, 1) k(long long* res, int n_mma, int reps)
     if (CG == 2) { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s_tmem;
-    if (warp == 1 && lane == 0 && rank == 0) {
+    if (warp == 1 && rank == 0 && (ELECT ? elect_one() : lane == 0)) {
         const uint32_t idesc = TS ? make_idesc(128 * CG, NN, true) : make_idesc(128 * CG, NN, false);
         const uint32_t alo = desc_lo(sbase, 16), blo = desc_lo(sbase + 32768, TS ? 16384 : 16);
         const uint32_t b = smem_u32(&bar);
@@ -98,17 +105,17 @@ __global__ void __launch_bounds__(128, 1) k(long long* res, int n_mma, int reps)
     }
 }
 
-template <int CG, int TS, int NN = 128>
+template <int CG, int TS, int NN = 128, bool ELECT = true>
 int run(long long* res, const char* name) {
     const int smem = (NN > 128 ? 112 : 64) * 1024 + 1024 + 1024;   // B of N = 256: two 32 KB blocks from offset 32 KB and 48 KB
-    CHK(cudaFuncSetAttribute(k<CG, TS, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CHK(cudaFuncSetAttribute(k<CG, TS, NN, ELECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     for (int n : {1, 8, 16, 64}) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(CG); cfg.blockDim = dim3(128); cfg.dynamicSmemBytes = smem;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = CG; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
         cfg.attrs = at; cfg.numAttrs = 1;
-        CHK(cudaLaunchKernelEx(&cfg, k<CG, TS, NN>, res, n, 4));
+        CHK(cudaLaunchKernelEx(&cfg, k<CG, TS, NN, ELECT>, res, n, 4));
         CHK(cudaDeviceSynchronize());
         long long h[12]; CHK(cudaMemcpy(h, res, sizeof(h), cudaMemcpyDeviceToHost));
         printf("%-28s n=%2d  issue %lld  commit %lld  until complete %lld cycles  (last of 4 repetitions; %.1f cycles per MMA)\n", name, n, h[9], h[10], h[11],
@@ -121,7 +128,10 @@ int main() {
     long long* res; CHK(cudaMalloc(&res, 64 * 8));
     if (run<1, 0>(res, "cta_group::1 SS (Q K^T)")) return 1;
     if (run<1, 1>(res, "cta_group::1 TS (P V)")) return 1;
+    if (run<1, 0, 128, false>(res, "cta_group::1 SS, lane == 0")) return 1;
+    if (run<1, 1, 128, false>(res, "cta_group::1 TS, lane == 0")) return 1;
     if (run<1, 0, 64>(res, "cta_group::1 SS, N = 64")) return 1;
+    if (run<1, 1, 64>(res, "cta_group::1 TS, N = 64")) return 1;
     if (run<1, 0, 256>(res, "cta_group::1 SS, N = 256")) return 1;
     if (run<2, 0>(res, "cta_group::2 SS (Q K^T)")) return 1;
     if (run<2, 1>(res, "cta_group::2 TS (P V)")) return 1;

@@ -1,4 +1,4 @@
-// Pipe-rate microbenchmark behind the figures the design doc quotes for the softmax loop of tree attention (one block on one SM):
+// Pipe-rate microbenchmark behind the figures quoted for the softmax loop of tree attention (one block on one SM):
 // cycles per warp instruction for the instructions that loop is made of (ex2, packed fp32 FMA and ADD, bf16x2 conversion,
 // three-input max), alone and mixed, with one warp (32 threads), one warp per SM sub-partition (128) and two (256); and the
 // wake-up latency of an mbarrier wait, suspended (try_wait) or spinning (test_wait).

@@ -179,46 +179,16 @@ def stream_k_shares(cfg, ctx, n, n_ctas):
 
 
 def shared_unit_rows(cfg, ctx, n, n_ctas, seed=11):
-    """One (b, h, i) row in every unit of tree attention that two persistent CTAs (or CTA pairs) share.
-
-    Restates the decomposition the attention kernel documents: work is counted in 128-key tiles; sequence b has
-    ceil(ctx_b / 128) + 1 of them (the last holds the tree's own keys); a row tile packs 128 / G nodes with the G query
-    heads of a kv head; a unit is one (sequence, kv head, row group), a row group being a pair of row tiles (one when the
-    whole tree cap fits one); every unit is preceded by 3 padding positions when its sequence has two or more row tiles,
-    else 2; all units laid end to end in (row group, sequence, kv head) order, row group outermost, are cut into n_ctas
-    equal ranges, range c = [total * c // n_ctas, total * (c + 1) // n_ctas)."""
-    G, Hkv, T = cfg.gqa, cfg.n_kv_heads, cfg.max_nodes
-    npt = 128 // G
-    MT = -(-T // npt)
+    """One (b, h, i) row in every unit of tree attention that two or more persistent CTAs share (stream_k_shares)."""
+    npt = 128 // cfg.gqa
     rng = np.random.default_rng(seed)
-    shapes = []
-    for b in range(cfg.batch):
-        nb = int(min(max(n[b], 0), T))
-        tiles = -(-int(ctx[b]) // 128) + 1
-        mtn = -(-nb // npt)
-        RG = (1 if mtn > 0 else 0) if MT == 1 else (mtn + 1) // 2
-        shapes.append((tiles, mtn, RG, 3 if mtn >= 2 else 2))
-    units = []                                             # (first position, padding, tiles, b, kh, rg, row tiles)
-    pos = 0
-    for rg in range(1 if MT == 1 else (MT + 1) // 2):
-        for b in range(cfg.batch):
-            tiles, mtn, RG, ov = shapes[b]
-            if rg >= RG:
-                continue
-            for kh in range(Hkv):
-                nrt = 1 if MT == 1 else min(2, mtn - 2 * rg)
-                units.append((pos, ov, tiles, b, kh, rg, nrt))
-                pos += ov + tiles
-    total = pos
-    starts = sorted({total * c // n_ctas for c in range(1, n_ctas)})
-    rows, k = [], 0
-    for g in starts:
-        while k + 1 < len(units) and units[k + 1][0] <= g:
-            k += 1
-        p0, ov, tiles, b, kh, rg, nrt = units[k]
-        first, end = p0 + ov, p0 + ov + tiles
-        if first < g < end:                                # key tiles on both sides of the cut
+    parts = {}
+    for shares in stream_k_shares(cfg, ctx, n, n_ctas):
+        for unit in shares:
+            parts[unit[:4]] = parts.get(unit[:4], 0) + 1
+    rows = []
+    for (b, kh, rg, nrt), k in parts.items():
+        if k > 1:
             rt = rg * 2 + int(rng.integers(0, nrt))
-            lo, hi = rt * npt, min((rt + 1) * npt, int(n[b]))
-            rows.append((b, kh * G + int(rng.integers(0, G)), int(rng.integers(lo, hi))))
+            rows.append((b, kh * cfg.gqa + int(rng.integers(0, cfg.gqa)), int(rng.integers(rt * npt, min((rt + 1) * npt, int(n[b]))))))
     return rows

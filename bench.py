@@ -58,7 +58,7 @@ def parse(argv=None):
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one cb_attn_tc_kernel launch with full trees, from the ncu
 # captures summarised under profiles/.  Reported only while the kernel sources still hash to the captured ones; after any
 # change to them the figure is stale and `traffic` is null until the capture is redone.
-ATTN_TRAFFIC = {"sources_sha1": "622be013b2c75fd8d537b7c5a4791cdfe61d0b72",
+ATTN_TRAFFIC = {"sources_sha1": "65ab3ff363cc67507ad703ad0bb7a5d541e9990a",
                 "bytes_per_launch": {"c2_7b": 70.0e6, "c3_8b_gqa": 555.1e6, "c4_13b_turns": 2763.9e6},
                 "source": {k: "profiles/cb_attn_tc_kernel_c2_c3_c4_c5b8.md" for k in ("c2_7b", "c3_8b_gqa", "c4_13b_turns")},
                 # config 5 holds 25 GB and runs 20 ms per launch: too large to capture.  The same shape at batch 8 was captured

@@ -9,8 +9,8 @@
 // values (one (sequence, kv head), all its row groups) then lie a fixed fraction of the whole sequence apart, so that they
 // are worked on at the same time by different CTAs and the keys and values are fetched from HBM once and found in L2 by
 // the others; with the row group innermost one CTA would stream them again and again, each time after everything else
-// it holds has passed through L2.  A key tile of a unit with two row tiles takes twice as long as one of a unit with one
-// (3.4 k against 1.8 k cycles: the two softmax chains share the latter's tiles), so a tile counts w2 = 2 or w1 = 1 positions of the
+// it holds has passed through L2.  A key tile of a unit with two row tiles takes about twice as long as one of a unit with one
+// (the two softmax chains share the latter's tiles; 3.1 k cycles at the 70B shape), so a tile counts w2 = 2 or w1 = 1 positions of the
 // sequence (batch 13 of small trees, head_dim 64: with one position each the CTAs ended between 42 k and 92 k cycles).  Starting a
 // unit costs about as much as two or three tiles (query load, pipeline refill, epilogue), so every unit is preceded by that many
 // padding positions: they carry no work, they only make a CTA that handles many short units receive fewer tiles.  A tile

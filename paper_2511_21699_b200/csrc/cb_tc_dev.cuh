@@ -312,7 +312,8 @@ __device__ __forceinline__ void mma_pv_halves_block(uint32_t d_tmem, uint32_t p_
 }
 
 // One lane of a converged warp; the compiler knows that a single thread runs what the result guards (a tcgen05.mma issues every
-// 40 to 50 cycles that way and every 60 from `if (lane == 0)`, a commit takes 54 instead of 76).
+// 15 to 20 cycles that way until the pipe's queue is full, and every 71 to 78 from `if (lane == 0)`, which is slower than the pipe's
+// 64; a commit takes 48 instead of 76: microbench/mma_issue.cu).
 __device__ __forceinline__ bool elect_one() {
     uint32_t e;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));

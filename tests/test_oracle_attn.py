@@ -178,20 +178,24 @@ def test_shared_unit_rows_lie_in_units_cut_by_a_range_boundary():
     n = np.full(cfg.batch, cfg.max_nodes, np.int32)
     rows = shared_unit_rows(cfg, ctx, n, 148)
     assert 74 <= len(rows) <= 147
-    # brute force: label every position of the global sequence with its unit and whether it is a key tile
+    # brute force: label every position of the global sequence with its unit and with whether a key tile begins there; a tile of a
+    # unit with two row tiles has two positions, and three tiles' worth of them are padding in front of the unit
     G, npt = cfg.gqa, 128 // cfg.gqa
     label = []
     for b in range(cfg.batch):                             # 64 nodes x 4 heads = two row tiles = one row group
         tiles = -(-int(ctx[b]) // 128) + 1
         for kh in range(cfg.n_kv_heads):
-            label += [(b, kh, False)] * 3 + [(b, kh, True)] * tiles
-    total = len(label)
-    cut_units = set()
-    for c in range(1, 148):
-        g = total * c // 148
-        if label[g - 1][:2] == label[g][:2] and label[g - 1][2] and label[g][2]:
-            cut_units.add(label[g][:2])
-    assert {(b, h // G) for b, h, i in rows} == cut_units
+            label += [(b, kh, False)] * 6 + [(b, kh, True), (b, kh, False)] * tiles
+
+    def cut(label, ranges):
+        holders = {}                                           # unit -> ranges in which a tile of it begins
+        for c in range(ranges):
+            for *unit, begins in label[len(label) * c // ranges:len(label) * (c + 1) // ranges]:
+                if begins:
+                    holders.setdefault(tuple(unit), set()).add(c)
+        return {u for u, cs in holders.items() if len(cs) > 1}
+
+    assert {(b, h // G) for b, h, i in rows} == cut(label, 148)
     assert all(0 <= i < cfg.max_nodes for _, _, i in rows)
     # several row groups (128 nodes x 8 heads = 8 row tiles = 4 row groups): the row group is the outermost index
     cfg = W.get_config("c5_70b_long")
@@ -203,12 +207,6 @@ def test_shared_unit_rows_lie_in_units_cut_by_a_range_boundary():
         for b in range(cfg.batch):
             tiles = -(-int(ctx[b]) // 128) + 1
             for kh in range(cfg.n_kv_heads):
-                label += [(b, kh, rg, False)] * 3 + [(b, kh, rg, True)] * tiles
-    total = len(label)
-    cut_units = set()
-    for c in range(1, 74):
-        g = total * c // 74
-        if label[g - 1][:3] == label[g][:3] and label[g - 1][3] and label[g][3]:
-            cut_units.add(label[g][:3])
+                label += [(b, kh, rg, False)] * 6 + [(b, kh, rg, True), (b, kh, rg, False)] * tiles
     npt = 128 // cfg.gqa
-    assert {(b, h // cfg.gqa, i // (2 * npt)) for b, h, i in rows} == cut_units
+    assert {(b, h // cfg.gqa, i // (2 * npt)) for b, h, i in rows} == cut(label, 74)

@@ -118,19 +118,21 @@ cb_status cb_update(cb_ctx* ctx, const int32_t* tokens, int64_t row_stride, cons
  * cb_update for long runs of new tokens (Section 3.3: the dynamic table is initialised with a sliding window over the
  * prompt).  Same arguments, same resulting tables, clocks and counters as cb_update; the work of one sequence is spread
  * over many warps where that cannot change the result (no leader can be evicted during the run: leaders stored + windows
- * <= LC, and at least 64 windows), and done by one warp in order otherwise.  Two launches (seven with scratch attached,
- * see below).  CB_CNT_FOLLOWER_EVICTIONS counts the followers this call displaced from the lists; on the order-free path
- * a follower that the run itself would have stored and displaced again is never stored and so is not counted.
+ * <= LC, and at least 64 windows), and done by one warp in order otherwise.  Runs of up to 8,192 windows take one launch,
+ * whose blocks reduce a run in shared memory without regard to its order (batches of up to 1,024 sequences, under the reading
+ * that re-inserting a stored follower refreshes it); where row_stride has room for longer ones two more follow (seven with
+ * scratch attached, see below).  CB_CNT_FOLLOWER_EVICTIONS counts the followers this call displaced from the lists; where a
+ * run is reduced, a follower that the run itself would have stored and displaced again is never stored and so is not counted.
  */
 cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t row_stride, const int32_t* n_old,
                          const int32_t* n_new, void* stream);
 
 /*
- * Scratch memory for the order-free path of cb_update_bulk.  After a run in which no leader can be evicted, and under the
+ * Scratch memory for the order-free reduction of longer runs by cb_update_bulk.  After a run in which no leader can be evicted, and under the
  * reading that re-inserting a stored follower refreshes it (the default), a leader's stamp is that of its last window and its
  * followers are the FC distinct ones touched last (Section 3.1: both lists are least-recently-used lists), whatever the
- * order of the windows.  With scratch attached, the sequences of a call whose runs qualify (as above) and fit the scratch,
- * taken in batch order, are reduced that way: one thread per window, then one warp per distinct leader.  The resulting
+ * order of the windows.  With scratch attached, the sequences of a call whose runs qualify (as above), have more than 8,192
+ * windows and fit the scratch, taken in batch order, are reduced in it: one thread per window, then one warp per distinct leader.  The resulting
  * tables and clocks are those of cb_update; which place a follower or an entry takes inside the table may differ, which no
  * call reports.
  *   cb_bulk_scratch_bytes    HOST out: bytes for calls whose qualifying runs hold up to max_windows windows in total

@@ -120,6 +120,7 @@ extern "C" void cb_destroy(cb_ctx* ctx) { delete ctx; }
 extern "C" int cb_debug_build(void) { return CB_DEBUG_BUILD; }
 
 __global__ void cb_reset_kernel(CbTables t, const int32_t* __restrict__ mask) {
+    CB_PDL_ENTRY();
     const int b = blockIdx.y;
     if (mask && mask[b] == 0) return;
     CbSeq s = cb_seq(t, b);
@@ -130,9 +131,8 @@ __global__ void cb_reset_kernel(CbTables t, const int32_t* __restrict__ mask) {
 extern "C" cb_status cb_reset(cb_ctx* ctx, const int32_t* dev_seq_mask, void* stream) {
     CB_CHECK_ARG(ctx);
     uint32_t gx = std::min<uint32_t>(64, (ctx->tables.nslots + 255) / 256);
-    cb_reset_kernel<<<dim3(gx, ctx->cfg.batch), 256, 0, (cudaStream_t)stream>>>(ctx->tables, dev_seq_mask);
+    CB_CUDA(cb_launch_pdl(cb_reset_kernel, dim3(gx, ctx->cfg.batch), dim3(256), 0, (cudaStream_t)stream, ctx->tables, dev_seq_mask));
     cb_count_launch(1);
-    CB_CUDA(cudaGetLastError());
     return CB_OK;
 }
 

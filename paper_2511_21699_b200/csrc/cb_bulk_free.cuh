@@ -1,5 +1,5 @@
-// Order-free form of the bulk update (prompt initialisation, Section 3.3), used by cb_update_bulk when the caller has
-// attached scratch memory (cb_bulk_scratch_attach).  Included by cb_table.cu after the table helpers.
+// Order-free form of the bulk update (prompt initialisation, Section 3.3) for runs that are too long for a block's shared memory
+// (cb_bulk_block.cuh), used by cb_update_bulk when the caller has attached scratch memory (cb_bulk_scratch_attach).  Included by cb_table.cu after the table helpers.
 //
 // When no leader can be evicted during a run of insertions and a stored follower is refreshed by re-insertion, the state
 // after the run does not depend on the order of the windows (Section 3.1: both lists are least-recently-used lists, and the
@@ -86,7 +86,7 @@ constexpr int kBulkFreeMaxBatch = 4096;      // the plan kernel keeps one word p
 // where their windows start in the global numbering.  One block.
 __global__ void __launch_bounds__(1024) cb_bulk_free_plan_kernel(CbTables t, int B, const int32_t* __restrict__ n_old,
                                                                 const int32_t* __restrict__ n_new, BulkPlan* plan, BulkFreeView v,
-                                                                unsigned long long* counters) {
+                                                                unsigned long long* counters, int done) {
     CB_PDL_ENTRY();
     __shared__ uint32_t s_nwin[kBulkFreeMaxBatch];
     const int w = t.LL + t.FL;
@@ -99,9 +99,10 @@ __global__ void __launch_bounds__(1024) cb_bulk_free_plan_kernel(CbTables t, int
         p.first = (uint32_t)first;
         p.nwin = (uint32_t)nwin;
         p.parallel = (nwin >= 64 && (unsigned long long)s.hdr[1] + (unsigned long long)nwin <= (unsigned long long)t.LC) ? 1u : 0u;
-        if (p.parallel) s.hdr[0] = p.clock0 + (uint32_t)nwin;
+        if (nwin <= done) p.parallel = 2u;
+        if (p.parallel == 1u) s.hdr[0] = p.clock0 + (uint32_t)nwin;
         plan[b] = p;
-        s_nwin[b] = (p.parallel && t.refresh) ? (uint32_t)nwin : 0u;
+        s_nwin[b] = (p.parallel == 1u && t.refresh) ? (uint32_t)nwin : 0u;
     }
     __syncthreads();
     if (threadIdx.x == 0) {

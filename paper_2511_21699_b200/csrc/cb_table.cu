@@ -377,10 +377,11 @@ __global__ void __launch_bounds__(128) cb_update_kernel(CbTables t, int B, const
 // (atomicAdd hands out entry ids) and the index, whose slots are claimed with atomicCAS; an entry is complete before its
 // index word is published.  A plan kernel takes that decision once per sequence, before any warp changes the table;
 // sequences that do not qualify (short runs, possible eviction) are done by their first warp alone, in order.
-struct BulkPlan { uint32_t parallel, clock0, first, nwin; };   // parallel: 0 one warp in order, 1 warps by leader, 2 order-free path (cb_bulk_free.cuh)
+struct BulkPlan { uint32_t parallel, clock0, first, nwin; };   // parallel: 0 one warp in order, 1 warps by leader, 2 elsewhere (cb_bulk_block.cuh, cb_bulk_free.cuh)
 
+// done: runs of up to that many windows have been dealt with by the block kernel (cb_bulk_block.cuh)
 __global__ void cb_bulk_plan_kernel(CbTables t, int B, const int32_t* __restrict__ n_old, const int32_t* __restrict__ n_new,
-                                    BulkPlan* plan) {
+                                    BulkPlan* plan, int done) {
     CB_PDL_ENTRY();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
@@ -393,7 +394,8 @@ __global__ void cb_bulk_plan_kernel(CbTables t, int B, const int32_t* __restrict
     p.first = (uint32_t)first;
     p.nwin = (uint32_t)nwin;
     p.parallel = (nwin >= 64 && (unsigned long long)s.hdr[1] + (unsigned long long)nwin <= (unsigned long long)t.LC) ? 1u : 0u;
-    if (p.parallel) s.hdr[0] = p.clock0 + (uint32_t)nwin;      // the clock after the run; the warps take stamps from positions
+    if (nwin <= done) p.parallel = 2u;
+    if (p.parallel == 1u) s.hdr[0] = p.clock0 + (uint32_t)nwin;   // the clock after the run; the warps take stamps from positions
     plan[b] = p;
 }
 
@@ -467,7 +469,7 @@ __global__ void __launch_bounds__(256) cb_update_bulk_kernel(CbTables t, int B, 
     if (b >= B) return;
     const CbSeq s = cb_seq(t, b);
     const BulkPlan pl = plan[b];
-    if (pl.parallel == 2u) return;                              // done by the order-free kernels
+    if (pl.parallel == 2u) return;                              // done by the block kernel or the order-free ones
     const int32_t* row = tokens + (size_t)b * row_stride;
     TblCounters cnt = {0, 0, 0, 0};
     if (!pl.parallel) {
@@ -556,6 +558,7 @@ __global__ void __launch_bounds__(256) cb_update_bulk_kernel(CbTables t, int B, 
 }  // namespace
 
 #include "cb_bulk_free.cuh"
+#include "cb_bulk_block.cuh"
 
 namespace {
 
@@ -950,6 +953,32 @@ extern "C" cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t 
                                     const int32_t* n_new, void* stream) {
     CB_CHECK_ARG(ctx && tokens && n_old && n_new && row_stride >= 1);
     const int B = ctx->cfg.batch;
+    int done = -1;
+    if (ctx->tables.refresh && B <= kBlkMaxBatch) {
+        // Runs of up to kBlkRun windows by blocks that hold them in shared memory.  A row that has no room for more needs nothing else.
+        using Kernel = void (*)(CbTables, int, const int32_t*, int64_t, const int32_t*, const int32_t*, uint32_t*, unsigned long long*);
+        static const Kernel kernels[CB_MAX_LL][2] = {{cb_update_bulk_block_kernel<1, 4>, cb_update_bulk_block_kernel<1, 8>},
+                                                     {cb_update_bulk_block_kernel<2, 4>, cb_update_bulk_block_kernel<2, 8>},
+                                                     {cb_update_bulk_block_kernel<3, 4>, cb_update_bulk_block_kernel<3, 8>},
+                                                     {cb_update_bulk_block_kernel<4, 4>, cb_update_bulk_block_kernel<4, 8>}};
+        const int l = ctx->tables.LL - 1, f = ctx->tables.FL <= 4 ? 0 : 1;
+        const Kernel kernel = kernels[l][f];
+        static std::mutex mu;
+        static bool opted[64][CB_MAX_LL][2] = {};              // per device
+        {
+            std::lock_guard<std::mutex> lock(mu);
+            bool& done_here = opted[ctx->device & 63][l][f];
+            if (!done_here) {
+                CB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlkSmem)));
+                done_here = true;
+            }
+        }
+        CB_CUDA(cb_launch_pdl(kernel, dim3((unsigned)ctx->num_sms), dim3(kBlkThreads), sizeof(BlkSmem), (cudaStream_t)stream, ctx->tables, B, tokens,
+                              row_stride, n_old, n_new, ctx->d_status, ctx->d_counters));
+        cb_count_launch(1);
+        done = kBlkRun;
+        if (row_stride - (ctx->tables.LL + ctx->tables.FL) + 1 <= (int64_t)kBlkRun) return CB_OK;
+    }
     // enough warps per sequence to fill the GPU at small batch, fewer at large batch
     int wps = 1;
     while (wps < 256 && (long long)B * wps * 2 <= (long long)ctx->num_sms * 64) wps *= 2;
@@ -961,7 +990,7 @@ extern "C" cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t 
         const cudaStream_t st = (cudaStream_t)stream;
         const unsigned blocks = (unsigned)std::min<long long>((long long)v.S / 256, (long long)ctx->num_sms * 8);
         const unsigned wide = (unsigned)std::min<long long>((long long)v.S / 256, (long long)ctx->num_sms * 32);   // one item per thread, or a few
-        CB_CUDA(cb_launch_pdl(cb_bulk_free_plan_kernel, dim3(1), dim3(1024), 0, st, ctx->tables, B, n_old, n_new, plan, v, ctx->d_counters));
+        CB_CUDA(cb_launch_pdl(cb_bulk_free_plan_kernel, dim3(1), dim3(1024), 0, st, ctx->tables, B, n_old, n_new, plan, v, ctx->d_counters, done));
         CB_CUDA(cb_launch_pdl(cb_bulk_free_clear_kernel, dim3(wide), dim3(256), 0, st, v));
         CB_CUDA(cb_launch_pdl(cb_bulk_free_reduce_kernel, dim3(wide), dim3(256), 0, st, ctx->tables, B, tokens, row_stride, (const BulkPlan*)plan, v,
                               ctx->d_status));
@@ -971,7 +1000,7 @@ extern "C" cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t 
                               ctx->d_status, ctx->d_counters));
         cb_count_launch(6);
     } else {
-        CB_CUDA(cb_launch_pdl(cb_bulk_plan_kernel, dim3((B + 127) / 128), dim3(128), 0, (cudaStream_t)stream, ctx->tables, B, n_old, n_new, plan));
+        CB_CUDA(cb_launch_pdl(cb_bulk_plan_kernel, dim3((B + 127) / 128), dim3(128), 0, (cudaStream_t)stream, ctx->tables, B, n_old, n_new, plan, done));
         cb_count_launch(1);
     }
     const long long warps = (long long)B * wps;

@@ -5,7 +5,7 @@
 
 namespace {
 
-template <bool BF16>
+template <bool BF16, int UN>
 __global__ void __launch_bounds__(256) cb_accept_logits_kernel(
     int T, int V, int Dmax, int chunk, int chunks_per_row, const void* __restrict__ logits, int64_t row_stride,
     const int32_t* __restrict__ tok, const int32_t* __restrict__ par, const int32_t* __restrict__ dep,
@@ -13,8 +13,8 @@ __global__ void __launch_bounds__(256) cb_accept_logits_kernel(
     int32_t* __restrict__ n_accept, int32_t* __restrict__ accept_nodes, int32_t* __restrict__ out_tokens,
     int32_t* __restrict__ target_out) {
     CB_PDL_ENTRY();
-    accept_rows<BF16>(T, V, Dmax, chunk, chunks_per_row, logits, row_stride, tok, par, dep, n_nodes, rowmax, ticket, n_accept, accept_nodes,
-                      out_tokens, target_out);
+    accept_rows<BF16, UN>(T, V, Dmax, chunk, chunks_per_row, logits, row_stride, tok, par, dep, n_nodes, rowmax, ticket, n_accept, accept_nodes,
+                          out_tokens, target_out, [](int) {});
 }
 
 __global__ void __launch_bounds__(128) cb_accept_ids_kernel(int B, int T, int Dmax, const int32_t* __restrict__ target_in,
@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(128) cb_accept_ids_kernel(int B, int T, int Dm
                                                             int32_t* __restrict__ out_tokens, int32_t* __restrict__ target_out) {
     CB_PDL_ENTRY();
     __shared__ int32_t s_target[4][CB_MAX_T];
+    __shared__ WalkSmem s_walk[4];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int b = blockIdx.x * 4 + w;
     if (b >= B) return;
@@ -34,7 +35,7 @@ __global__ void __launch_bounds__(128) cb_accept_ids_kernel(int B, int T, int Dm
         if (target_out) target_out[(size_t)b * T + k] = tg;
     }
     __syncwarp();
-    accept_walk(b, Dmax, tok + (size_t)b * T, par + (size_t)b * T, dep + (size_t)b * T, n, s_target[w], n_accept, accept_nodes, out_tokens, lane);
+    accept_walk(b, Dmax, tok + (size_t)b * T, par + (size_t)b * T, dep + (size_t)b * T, n, s_target[w], s_walk[w], n_accept, accept_nodes, out_tokens, lane);
 }
 
 }  // namespace
@@ -66,14 +67,11 @@ extern "C" cb_status cb_accept(cb_ctx* ctx, const int32_t* tree_tokens, const in
         cpr = (c.vocab + chunk - 1) / chunk;
         dim3 grid(cpr, T, c.batch);
         if (c.batch > 65535) return CB_ERR_UNSUPPORTED;
-        if (logits_dtype == CB_DTYPE_F32)
-            CB_CUDA(cb_launch_pdl(cb_accept_logits_kernel<false>, grid, dim3(256), 0, st, T, c.vocab, Dmax, chunk, cpr, logits, logits_row_stride,
-                                  tree_tokens, tree_parent, tree_depth, n_nodes, ctx->d_rowmax, ctx->d_ticket, n_accept, accept_nodes,
-                                  out_tokens, target_ids_out));
-        else
-            CB_CUDA(cb_launch_pdl(cb_accept_logits_kernel<true>, grid, dim3(256), 0, st, T, c.vocab, Dmax, chunk, cpr, logits, logits_row_stride,
-                                  tree_tokens, tree_parent, tree_depth, n_nodes, ctx->d_rowmax, ctx->d_ticket, n_accept, accept_nodes,
-                                  out_tokens, target_ids_out));
+        const bool wide = (long long)cpr * T * c.batch <= 4ll * ctx->num_sms, f32 = logits_dtype == CB_DTYPE_F32;
+        auto kernel = f32 ? (wide ? cb_accept_logits_kernel<false, 8> : cb_accept_logits_kernel<false, 4>)
+                          : (wide ? cb_accept_logits_kernel<true, 8> : cb_accept_logits_kernel<true, 4>);
+        CB_CUDA(cb_launch_pdl(kernel, grid, dim3(256), 0, st, T, c.vocab, Dmax, chunk, cpr, logits, logits_row_stride, tree_tokens, tree_parent,
+                              tree_depth, n_nodes, ctx->d_rowmax, ctx->d_ticket, n_accept, accept_nodes, out_tokens, target_ids_out));
     }
     cb_count_launch(1);
     return CB_OK;
@@ -147,11 +145,11 @@ extern "C" cb_status cb_accept_static(int32_t batch, int32_t max_nodes, int32_t 
     cpr = (vocab + chunk - 1) / chunk;
     dim3 grid(cpr, max_nodes, batch);
     if (logits_dtype == CB_DTYPE_F32)
-        cb_accept_logits_kernel<false><<<grid, 256, 0, st>>>(max_nodes, vocab, max_depth, chunk, cpr, logits, logits_row_stride,
+        cb_accept_logits_kernel<false, 4><<<grid, 256, 0, st>>>(max_nodes, vocab, max_depth, chunk, cpr, logits, logits_row_stride,
                                                              tree_tokens, tree_parent, tree_depth, n_nodes, su.rowmax, su.ticket,
                                                              n_accept, accept_nodes, out_tokens, target_ids_out);
     else
-        cb_accept_logits_kernel<true><<<grid, 256, 0, st>>>(max_nodes, vocab, max_depth, chunk, cpr, logits, logits_row_stride,
+        cb_accept_logits_kernel<true, 4><<<grid, 256, 0, st>>>(max_nodes, vocab, max_depth, chunk, cpr, logits, logits_row_stride,
                                                             tree_tokens, tree_parent, tree_depth, n_nodes, su.rowmax, su.ticket,
                                                             n_accept, accept_nodes, out_tokens, target_ids_out);
     cb_count_launch(1);

@@ -37,60 +37,102 @@ __device__ __forceinline__ uint4 ldg_stream4u(const void* p, uint64_t pol) {
     return v;
 }
 
+// An atomic add that orders this thread's writes before it and the block's reads behind it (with the barrier that follows).
+__device__ __forceinline__ uint32_t add_acq_rel(uint32_t* p, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
+
+// What the walk needs beside the tree, in shared memory: a word per node, and the winner's path from its end to the root.
+struct WalkSmem { uint16_t up[CB_MAX_T]; uint16_t path[CB_MAX_T]; };
+
 // Walk of one sequence by one warp (n <= 128 nodes, parents precede children).
-// tk, pa, de: the sequence's own tree rows (shared or global memory).
-__device__ void accept_walk(int b, int Dmax, const int32_t* tk, const int32_t* pa, const int32_t* de, int n,
-                            const int32_t* target_s /*shared, [T]*/,
+// tk, pa, de: the sequence's own tree rows (shared or global memory).  emit: if not null, the first 256 emitted tokens (m accepted
+// ones, then the target's next) are left there too; *have: how many tokens are emitted.
+// A node is verified if it and all its ancestors but the root match their parents' targets.  Every node knows its own match; a word
+// holds "some node on the way to here does not match" and the ancestor that the way has reached, and doubles its reach with
+// every round: 3 to 4 rounds for the usual depths.  Climbing node by node, with the path written from one lane, the walk took
+// 4.4 k of the 13.7 k cycles of one sequence's acceptance over 32 k tokens.
+__device__ __noinline__ void accept_walk(int b, int Dmax, const int32_t* tk, const int32_t* pa, const int32_t* de, int n,
+                            const int32_t* target_s /*shared, [T]*/, WalkSmem& ws,
                             int32_t* __restrict__ n_accept, int32_t* __restrict__ accept_nodes,
-                            int32_t* __restrict__ out_tokens, int lane) {
+                            int32_t* __restrict__ out_tokens, int lane, int32_t* emit = nullptr, int* have = nullptr) {
+    constexpr int PER = CB_MAX_T / 32;
+    constexpr uint32_t kBad = 0x100u;
+    uint32_t up[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const int i = q * 32 + lane;
+        up[q] = 0u;
+        if (i > 0 && i < n) {
+            const int p = pa[i];
+            if (p < 0 || p >= i) up[q] = kBad;                  // malformed tree: treat as unverified
+            else up[q] = (uint32_t)p | (tk[i] == target_s[p] ? 0u : kBad);
+        }
+        if (i < n) ws.up[i] = (uint16_t)up[q];
+    }
+    for (int round = 0; round < 8; ++round) {
+        bool more = false;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) more = more || (up[q] & 0xFFu) != 0u;
+        if (!__any_sync(CB_FULL, more)) break;
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+            if ((up[q] & 0xFFu) != 0u) { const uint32_t a = ws.up[up[q] & 0xFFu]; up[q] = (a & 0xFFu) | ((a | up[q]) & kBad); }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < PER; ++q) if (q * 32 + lane < n) ws.up[q * 32 + lane] = (uint16_t)up[q];
+    }
     // key = (depth << 8) | (255 - index) for verified nodes: max = deepest, lowest index among ties
     uint32_t best = 0;
-    for (int i = lane; i < n; i += 32) {
-        bool good = true;
-        int c = i;
-        for (int guard = 0; guard < CB_MAX_T && c > 0; ++guard) {
-            const int p = pa[c];
-            if (p < 0 || p >= c) { good = false; break; }      // malformed tree: treat as unverified
-            good = good && (tk[c] == target_s[p]);
-            c = p;
-        }
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const int i = q * 32 + lane;
+        if (i >= n) break;
         // a depth outside [0, Dmax] cannot come from the drafter (malformed input): such a node counts as unverified, so the
         // winner's depth always fits the output rows
         const int d = de[i];
-        if (good && d >= 0 && d <= Dmax) best = max(best, ((uint32_t)d << 8) | (uint32_t)(255 - i));
+        if (!(up[q] & kBad) && d >= 0 && d <= Dmax) best = max(best, ((uint32_t)d << 8) | (uint32_t)(255 - i));
     }
     best = __reduce_max_sync(CB_FULL, best);
     int node = n > 0 ? 255 - (int)(best & 255u) : 0;
     int m = n > 0 ? (int)(best >> 8) : 0;
     if (node >= n) { node = 0; m = 0; }                        // nothing verified, not even the root (malformed input)
-    for (int k = lane; k < Dmax; k += 32) accept_nodes[(size_t)b * Dmax + k] = -1;
-    for (int k = lane; k <= Dmax; k += 32) out_tokens[(size_t)b * (Dmax + 1) + k] = -1;
+    int hops = 0;
+    if (lane == 0)
+        for (int c = node; hops < m && c > 0; c = pa[c]) ws.path[hops++] = (uint16_t)c;
+    hops = __shfl_sync(CB_FULL, hops, 0);
     __syncwarp();
+    const int32_t bonus = n > 0 ? target_s[node] : -1;
+    for (int k = lane; k <= Dmax; k += 32) {
+        const int j = m - 1 - k;                                // position on the path, counted from its end
+        const int c = j >= 0 && j < hops ? (int)ws.path[j] : -1;
+        const int32_t t = c >= 0 ? tk[c] : (k == m ? bonus : -1);
+        if (k < Dmax) accept_nodes[(size_t)b * Dmax + k] = c;
+        out_tokens[(size_t)b * (Dmax + 1) + k] = t;
+        if (emit && k < 256) emit[k] = t;
+    }
     if (lane == 0) {
         n_accept[b] = m;
-        if (n > 0) {
-            out_tokens[(size_t)b * (Dmax + 1) + m] = target_s[node];
-            int c = node;
-            for (int k = m - 1; k >= 0 && c > 0; --k) {
-                accept_nodes[(size_t)b * Dmax + k] = c;
-                out_tokens[(size_t)b * (Dmax + 1) + k] = tk[c];
-                c = pa[c];
-            }
-        }
+        if (have) *have = n > 0 ? m + 1 : 0;
     }
 }
 
 // The work of one CTA of the acceptance grid (row chunk ck = blockIdx.x, node i = blockIdx.y, sequence b = blockIdx.z): its
 // chunk of the node's logits row is reduced into the row's packed maximum; the last CTA of the sequence to arrive turns the
 // maxima into the target's tokens, walks the tree and writes the result.  Returns true in that CTA (all its threads), after
-// the result has been written; false in all others.
-template <bool BF16>
+// the result has been written; false in all others.  beside(k): what the threads from 128 on (k = 0 ...) of that CTA do meanwhile.
+// UN: 16-byte loads in flight per thread.  A grid that is resident at once is as long as its chain of round trips and takes all of
+// its 32 KB chunk (8 loads a thread) at once; a larger one has enough in flight with 4 and needs the registers for more CTAs.
+template <bool BF16, int UN, typename Beside>
 __device__ __forceinline__ bool accept_rows(
     int T, int V, int Dmax, int chunk, int chunks_per_row, const void* __restrict__ logits, int64_t row_stride,
     const int32_t* __restrict__ tok, const int32_t* __restrict__ par, const int32_t* __restrict__ dep,
     const int32_t* __restrict__ n_nodes, unsigned long long* rowmax, uint32_t* ticket,
     int32_t* __restrict__ n_accept, int32_t* __restrict__ accept_nodes, int32_t* __restrict__ out_tokens,
-    int32_t* __restrict__ target_out) {
+    int32_t* __restrict__ target_out, Beside&& beside, int32_t* emit = nullptr, int* have = nullptr) {
     const int b = blockIdx.z, i = blockIdx.y, ck = blockIdx.x, tid = threadIdx.x;
     const int n = min(max(n_nodes[b], 0), T);
     // Rows past the tree have nothing to add and do not queue for the ticket either (hundreds of atomics on one word at
@@ -98,6 +140,7 @@ __device__ __forceinline__ bool accept_rows(
     if (i >= max(n, 1)) return false;
     __shared__ unsigned long long s_red[8];
     __shared__ int32_t s_target[CB_MAX_T], s_tok[CB_MAX_T], s_par[CB_MAX_T], s_dep[CB_MAX_T];
+    __shared__ WalkSmem s_walk;
     __shared__ int s_last;
     if (i < n) {
         const int v0 = ck * chunk, v1 = min(V, v0 + chunk);
@@ -114,13 +157,13 @@ __device__ __forceinline__ bool accept_rows(
             v += head;
             const int nvec = (v1 - v) >> 2;
             const float* base = rowp + v;
-            for (int k = tid; k < nvec; k += blockDim.x * 4) {
-                float4 x[4];
-                int kk[4];
+            for (int k = tid; k < nvec; k += blockDim.x * UN) {
+                float4 x[UN];
+                int kk[UN];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) { kk[u] = k + u * blockDim.x; if (kk[u] < nvec) x[u] = ldg_stream4(base + 4 * (size_t)kk[u], pol); }
+                for (int u = 0; u < UN; ++u) { kk[u] = k + u * blockDim.x; if (kk[u] < nvec) x[u] = ldg_stream4(base + 4 * (size_t)kk[u], pol); }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) if (kk[u] < nvec) {
+                for (int u = 0; u < UN; ++u) if (kk[u] < nvec) {
                     const uint32_t id = (uint32_t)(v + 4 * kk[u]);
                     best = umax64(best, pack(x[u].x, id));
                     best = umax64(best, pack(x[u].y, id + 1));
@@ -140,13 +183,13 @@ __device__ __forceinline__ bool accept_rows(
             v += head;
             const int nvec = (v1 - v) >> 3;
             const __nv_bfloat16* base = rowp + v;
-            for (int k = tid; k < nvec; k += blockDim.x * 4) {
-                uint4 x[4];
-                int kk[4];
+            for (int k = tid; k < nvec; k += blockDim.x * UN) {
+                uint4 x[UN];
+                int kk[UN];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) { kk[u] = k + u * blockDim.x; if (kk[u] < nvec) x[u] = ldg_stream4u(base + 8 * (size_t)kk[u], pol); }
+                for (int u = 0; u < UN; ++u) { kk[u] = k + u * blockDim.x; if (kk[u] < nvec) x[u] = ldg_stream4u(base + 8 * (size_t)kk[u], pol); }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) if (kk[u] < nvec) {
+                for (int u = 0; u < UN; ++u) if (kk[u] < nvec) {
                     const uint32_t id = (uint32_t)(v + 8 * kk[u]);
                     const uint32_t wds[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
 #pragma unroll
@@ -170,29 +213,29 @@ __device__ __forceinline__ bool accept_rows(
     }
     // The last CTA of this sequence to arrive owns the walk (and re-zeroes the scratch for the next call).
     if (tid == 0) {
-        __threadfence();
         const uint32_t total = gridDim.x * (uint32_t)max(n, 1);
-        s_last = (atomicAdd(&ticket[b], 1u) == total - 1u) ? 1 : 0;
+        s_last = (add_acq_rel(&ticket[b], 1u) == total - 1u) ? 1 : 0;
     }
     __syncthreads();
     if (!s_last) return false;
-    __threadfence();
-    for (int k = tid; k < T; k += blockDim.x) {
-        int32_t tg = -1;
-        if (k < n) {
-            const unsigned long long r = atomicExch(&rowmax[(size_t)b * T + k], 0ull);
+    static_assert(CB_MAX_T <= 128, "the first 128 threads have a node each, the others do what goes beside");
+    if (tid >= 128) {
+        beside(tid - 128);
+    } else if (tid < T) {
+        // the tree's rows come along, so that the walk below reads shared memory
+        int32_t tg = -1, tk = -1, pa = -1, de = -1;
+        if (tid < n) {
+            const size_t at = (size_t)b * T + tid;
+            tk = tok[at]; pa = par[at]; de = dep[at];
+            const unsigned long long r = atomicExch(&rowmax[at], 0ull);
             tg = (int32_t)(0xFFFFFFFFu - (uint32_t)(r & 0xFFFFFFFFull));
         }
-        s_target[k] = tg;
-        if (target_out) target_out[(size_t)b * T + k] = tg;
-        // the tree's rows come along, so that the climb from each node to the root below reads shared memory
-        s_tok[k] = k < n ? tok[(size_t)b * T + k] : -1;
-        s_par[k] = k < n ? par[(size_t)b * T + k] : -1;
-        s_dep[k] = k < n ? dep[(size_t)b * T + k] : -1;
+        s_target[tid] = tg; s_tok[tid] = tk; s_par[tid] = pa; s_dep[tid] = de;
+        if (target_out) target_out[(size_t)b * T + tid] = tg;
     }
     if (tid == 0) ticket[b] = 0u;
     __syncthreads();
-    if (tid < 32) accept_walk(b, Dmax, s_tok, s_par, s_dep, n, s_target, n_accept, accept_nodes, out_tokens, tid);
+    if (tid < 32) accept_walk(b, Dmax, s_tok, s_par, s_dep, n, s_target, s_walk, n_accept, accept_nodes, out_tokens, tid, emit, have);
     return true;
 }
 

@@ -914,8 +914,9 @@ __global__ void __launch_bounds__(256, CTAS) cb_accept_draft_kernel(AcceptArgs a
                                                               uint32_t* status, unsigned long long* counters) {
     CB_PDL_ENTRY();
     extern __shared__ int32_t smem[];
-    if (!accept_rows<BF16>(T, a.V, a.Dmax, a.chunk, a.chunks_per_row, a.logits, a.logits_row_stride, a.tok, a.par, a.dep, a.n_nodes, a.rowmax,
-                           a.ticket, a.n_accept, a.accept_nodes, a.out_tokens, a.target_out))
+    if (!accept_rows<BF16, CTAS == 2 && FETCH == 1 ? 8 : 4>(T, a.V, a.Dmax, a.chunk, a.chunks_per_row, a.logits, a.logits_row_stride, a.tok, a.par, a.dep,
+                                                            a.n_nodes, a.rowmax, a.ticket, a.n_accept, a.accept_nodes, a.out_tokens, a.target_out,
+                                                            [](int) {}))
         return;
     __threadfence_block();
     __syncthreads();                                            // the walk (first warp) has written the sequence's result

@@ -151,21 +151,30 @@ template <bool PRE = false>
 __device__ __forceinline__ void tbl_put_follower(const CbTables& t, uint32_t* e, int32_t myfol, uint32_t c, int lane, TblCounters& cnt,
                                                  const EntryRegs* er = nullptr) {
     // Lane l looks after followers l, l + 32, ...: one pass finds a stored copy of the follower, the lowest free place
-    // and the least recently inserted follower.  PRE: the stamps came with the lookup.
+    // and the least recently inserted follower.  PRE: the stamps came with the lookup; the first tokens of all of the lane's
+    // followers are then read at once, and the others only of those that match so far (read follower by follower and token by
+    // token they were a chain of 12 memory round trips with FC = 128, FL = 3).
+    constexpr int CH = CB_MAX_FC / 32;
+    const int32_t f0 = __shfl_sync(CB_FULL, myfol, 0);
+    int32_t t0[CH];
+#pragma unroll
+    for (int ch = 0; ch < CH; ++ch) t0[ch] = PRE && er->fs4[ch] != 0u ? (int32_t)e[t.LL + t.FC + (ch * 32 + lane) * t.FL] : 0;
     int match_f = -1, free_f = -1, lru_f = -1;
     uint32_t lru_stamp = 0xFFFFFFFFu;
 #pragma unroll
-    for (int ch = 0; ch < CB_MAX_FC / 32; ++ch) {
+    for (int ch = 0; ch < CH; ++ch) {
         const int base = ch * 32;
         if (base >= t.FC || match_f >= 0) break;
         const int f = base + lane;
         const bool mine = f < t.FC;
         const uint32_t fs = PRE ? er->fs4[ch] : (mine ? e[t.LL + f] : 0u);
         bool match = mine && fs != 0u;
-        for (int j = 0; j < t.FL; ++j) {
-            const int32_t fj = __shfl_sync(CB_FULL, myfol, j);
-            if (match) match = ((int32_t)e[t.LL + t.FC + f * t.FL + j] == fj);
-        }
+        if (PRE) match = match && t0[ch] == f0;
+        if (!PRE || __any_sync(CB_FULL, match))
+            for (int j = PRE ? 1 : 0; j < t.FL; ++j) {
+                const int32_t fj = __shfl_sync(CB_FULL, myfol, j);
+                if (match) match = ((int32_t)e[t.LL + t.FC + f * t.FL + j] == fj);
+            }
         const uint32_t mm = __ballot_sync(CB_FULL, match);
         if (mm) { match_f = base + __ffs(mm) - 1; break; }
         const uint32_t freem = __ballot_sync(CB_FULL, mine && fs == 0u);
@@ -270,18 +279,21 @@ __device__ __forceinline__ void update_seq(const CbTables& t, int b, const int32
 // a window whose leader an earlier window of the eight has, a new leader whose slot lies in the same bucket as an earlier new
 // one's, a failed lookup.  When the eight could overflow the leader capacity, all of them do (an eviction looks at the stamps of
 // the windows before it only).
+// Meanwhile a warp without a window does idle(): it looks the tree's root up, so that the draft that follows finds the root's bucket and
+// entry in L1 (a write by this CTA goes through that L1, so what it finds there is current; no other CTA writes this sequence's table).
 constexpr int kUpdWarps = 8;
-template <int FETCH>
-__device__ __forceinline__ void update_seq_cta(const CbTables& t, int b, const int32_t* tokens, int64_t row_stride, int n0, int n1,
-                                               int warp, int lane, uint32_t* status, unsigned long long* counters) {
+template <int FETCH, typename Tokens, typename Idle>
+__device__ __forceinline__ void update_seq_cta(const CbTables& t, int b, const Tokens& row, int n0, int n1,
+                                               int warp, int lane, uint32_t* status, unsigned long long* counters, Idle&& idle) {
     __shared__ unsigned long long sh_h[kUpdWarps];
     __shared__ uint32_t sh_state[kUpdWarps], sh_bucket[kUpdWarps], sh_count[2];
     const CbSeq s = cb_seq(t, b);
     const int w = t.LL + t.FL;
-    const int32_t* row = tokens + (size_t)b * row_stride;
     uint32_t clock = s.hdr[0], count = s.hdr[1];
     TblCounters cnt = {0, 0, 0, 0};
     int flip = 0;
+    const int n_all = n1 - w + 1 - max(0, n0 - w + 1);
+    if (n_all > 0 && n_all < kUpdWarps && warp == kUpdWarps - 1) idle();
     for (int i0 = max(0, n0 - w + 1); i0 + w <= n1; i0 += kUpdWarps) {
         const int nb = min(kUpdWarps, n1 - w + 1 - i0), i = i0 + warp;
         const bool mine = warp < nb, together = count + (uint32_t)nb <= (uint32_t)t.LC;
@@ -292,8 +304,8 @@ __device__ __forceinline__ void update_seq_cta(const CbTables& t, int b, const i
             EntryRegs er;
             Probe pr = {};
             if (mine) {
-                if (lane < t.LL) mykey = row[i + lane];
-                if (lane < t.FL) myfol = row[i + t.LL + lane];
+                if (lane < t.LL) mykey = row(i + lane);
+                if (lane < t.FL) myfol = row(i + t.LL + lane);
                 h = warp_hash(t, mykey);
                 pr = tbl_find<false, FETCH>(t, s, mykey, h, lane, &er);
                 if (lane == 0) {
@@ -329,8 +341,8 @@ __device__ __forceinline__ void update_seq_cta(const CbTables& t, int b, const i
                 uint32_t n = count;
                 for (uint32_t m = later; m; m &= m - 1u) {
                     const int k = __ffs(m) - 1;
-                    const int32_t mykey = lane < t.LL ? row[i0 + k + lane] : 0;
-                    const int32_t myfol = lane < t.FL ? row[i0 + k + t.LL + lane] : 0;
+                    const int32_t mykey = lane < t.LL ? row(i0 + k + lane) : 0;
+                    const int32_t myfol = lane < t.FL ? row(i0 + k + t.LL + lane) : 0;
                     uint32_t c = clock + (uint32_t)k;
                     tbl_insert<FETCH>(t, s, mykey, myfol, c, n, lane, status, cnt);
                 }
@@ -343,7 +355,7 @@ __device__ __forceinline__ void update_seq_cta(const CbTables& t, int b, const i
         clock += (uint32_t)nb;
     }
     if (lane == 0) {
-        const int nw = max(0, n1 - w + 1 - max(0, n0 - w + 1));
+        const int nw = max(0, n_all);
         if (warp == 0) {
             s.hdr[0] = clock; s.hdr[1] = count;
             if (nw) atomicAdd(&counters[CB_CNT_INSERTS], (unsigned long long)nw);
@@ -572,9 +584,13 @@ namespace {
 // With a frozen table attached (Section 3.3) a second pass follows while the tree is below the size cap: its first
 // frontier is every node that was a frontier leaf of the first pass, in creation order, and its lookups go to the
 // frozen table, which is shared by all sequences and only read (no clock tick, no stamp).
+// A node goes to the output arrays when it is attached, its mask row being its leaf's plus a run of bits.  A level of one leaf (the
+// first one always is) is looked up, planned and filled in by one warp without a barrier.
 constexpr int kSerialLeaves = 16;
+// x / d = x * kInverse[d] >> 16 for d <= CB_MAX_FL and the x that occur here (below 1,024): a division is a chain of 100 cycles
+__constant__ uint32_t kInverse[CB_MAX_FL + 1] = {0u, 65537u, 32769u, 21846u, 16385u, 13108u, 10923u, 9363u, 8193u};
 struct DraftSmem {
-    int32_t* tok; int32_t* par; int32_t* dep;
+    int32_t* tok; int32_t* par; int32_t* dep; uint32_t* mask;
     int32_t* front; int32_t* next; int32_t* pts;
     int32_t* r_eid; int32_t* r_nf; int32_t* r_ok; uint32_t* r_stamp;
     int32_t* r_n0; int32_t* r_cl; int32_t* r_tot; int32_t* r_nn0;     // plan of a leaf's attachment: first node, chain length, nodes, first frontier place
@@ -582,18 +598,19 @@ struct DraftSmem {
 };
 
 // The work of the CTA that drafts sequence b, whose history holds L tokens.  upd_n_old >= 0: the windows that the tokens
-// from upd_n_old on complete are inserted first (cb_update_draft_tree and the call that follows an acceptance).  The
-// history may have been extended by this CTA just before (no read-only path to it).
-template <int FETCH>
+// from upd_n_old on complete are inserted first (cb_update_draft_tree and the call that follows an acceptance).  row(i): token i of
+// the history (which this CTA may have extended just before).
+template <int FETCH, typename Tokens>
 __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf, int T, int crt, int max_depth, int NL, int KF,
-                                           const int32_t* tokens, int64_t row_stride, int b, int L, int upd_n_old,
+                                           const Tokens& row, int b, int L, int upd_n_old,
                                            int32_t* __restrict__ o_tok, int32_t* __restrict__ o_par,
                                            int32_t* __restrict__ o_dep, uint32_t* __restrict__ o_mask,
                                            int32_t* __restrict__ o_n, uint32_t* status,
                                            unsigned long long* counters, int32_t* smem) {
     DraftSmem S;
-    S.tok = smem; S.par = S.tok + T; S.dep = S.par + T;
-    S.front = S.dep + T; S.next = S.front + NL; S.pts = S.next + NL;
+    const int W = (T + 31) >> 5;
+    S.tok = smem; S.par = S.tok + T; S.dep = S.par + T; S.mask = (uint32_t*)(S.dep + T);
+    S.front = (int32_t*)(S.mask + T * W); S.next = S.front + NL; S.pts = S.next + NL;
     S.r_eid = S.pts + NL; S.r_nf = S.r_eid + NL; S.r_ok = S.r_nf + NL; S.r_stamp = (uint32_t*)(S.r_ok + NL);
     S.r_n0 = (int32_t*)(S.r_stamp + NL); S.r_cl = S.r_n0 + NL; S.r_tot = S.r_cl + NL; S.r_nn0 = S.r_tot + NL;
     S.fol = S.r_nn0 + NL;
@@ -601,25 +618,58 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const CbSeq s = cb_seq(t, b);
-    const int32_t* row = tokens + (size_t)b * row_stride;
     if (upd_n_old >= 0) {
         // cb_update_draft_tree: the sequence's new windows go into the table first, then the CTA drafts from the updated table.
-        update_seq_cta<FETCH>(t, b, tokens, row_stride, upd_n_old, L, warp, lane, status, counters);
+        update_seq_cta<FETCH>(t, b, row, upd_n_old, L, warp, lane, status, counters, [&] {
+            if (L < t.LL) return;
+            const int32_t mykey = lane < t.LL ? row(L - t.LL + lane) : 0;
+            EntryRegs er;
+            const Probe pr = tbl_find<false, FETCH>(t, s, mykey, warp_hash(t, mykey), lane, &er);
+            if (pr.eid < 0) return;                              // nothing but the bucket was read
+            if (FETCH == 1) {
+                asm volatile("" ::"r"(er.fs));
+#pragma unroll
+                for (int j = 0; j < CB_MAX_FL; ++j) asm volatile("" ::"r"(er.tok[j]));
+            } else {
+#pragma unroll
+                for (int c = 0; c < CB_MAX_FC / 32; ++c) asm volatile("" ::"r"(er.fs4[c]));
+            }
+        });
         __threadfence_block();
         __syncthreads();
     }
-    const int W = (T + 31) >> 5;
     const int FLFC = t.FL * KF;                               // staged followers per leaf: the KF best
     const uint32_t clock0 = s.hdr[0];
     const bool has_frozen = tf.index != nullptr;
 
-    for (int i = tid; i < T; i += blockDim.x) { S.tok[i] = -1; S.par[i] = -1; S.dep[i] = -1; }
+    // Nodes [0, tot) of leaf `leaf` (depth d), numbered from n0 on, by one warp: node x is token x % cl of follower x / cl.
+    auto attach = [&](int leaf, int d, int n0, int cl, int tot, const int32_t* fol) {
+        const uint32_t inv = kInverse[cl];
+        for (int x = lane; x < tot; x += 32) {
+            const int f = (int)(((uint32_t)x * inv) >> 16), j = x - f * cl, node = n0 + x;
+            const int tk = fol[f * t.FL + j], pa = j == 0 ? leaf : node - 1, de = d + j + 1;
+            S.tok[node] = tk; S.par[node] = pa; S.dep[node] = de;
+            const size_t at = (size_t)b * T + node;
+            o_tok[at] = tk; o_par[at] = pa; o_dep[at] = de;
+            for (int k = 0; k < W; ++k) {
+                uint32_t m = S.mask[leaf * W + k];
+                const int lo = max(node - j - 32 * k, 0), hi = min(node - 32 * k, 31);   // the chain so far: nodes node - j ... node
+                if (lo <= hi) m |= (0xFFFFFFFFu >> (31 - hi)) & (0xFFFFFFFFu << lo);
+                S.mask[node * W + k] = m;
+                o_mask[at * W + k] = m;
+            }
+        }
+    };
     if (tid == 0) {
-        sh_n = 0; sh_nfront = 0; sh_npts = 0; sh_q = 0; sh_hits = 0; sh_fq = 0; sh_fhits = 0;
-    }
-    __syncthreads();
-    if (tid == 0 && L >= 1) {
-        S.tok[0] = row[L - 1]; S.dep[0] = 0; sh_n = 1; S.front[0] = 0; sh_nfront = 1; S.pts[0] = 0; sh_npts = 1;
+        const bool root = L >= 1;
+        sh_n = root ? 1 : 0; sh_nfront = root ? 1 : 0; sh_npts = root ? 1 : 0; sh_q = 0; sh_hits = 0; sh_fq = 0; sh_fhits = 0;
+        if (root) {
+            const int tk = row(L - 1);
+            S.tok[0] = tk; S.par[0] = -1; S.dep[0] = 0; S.front[0] = 0; S.pts[0] = 0;
+            const size_t at = (size_t)b * T;
+            o_tok[at] = tk; o_par[at] = -1; o_dep[at] = 0;
+            for (int k = 0; k < W; ++k) { S.mask[k] = k == 0 ? 1u : 0u; o_mask[at * W + k] = k == 0 ? 1u : 0u; }
+        }
     }
     __syncthreads();
 
@@ -635,8 +685,8 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
             __syncthreads();
         }
         while (true) {
-            const int nfront = sh_nfront;
-            if (nfront == 0 || sh_n >= T) break;
+            const int nfront = sh_nfront, n_top = sh_n;
+            if (nfront == 0 || n_top >= T) break;
             if (pass == 0 && S.dep[S.front[0]] >= max_depth) break;   // a level's leaves lie at one depth: none may be queried
             for (int li = tid; li < nfront; li += blockDim.x) S.r_stamp[li] = 0u;
             if (tid == 0) sh_nnext = 0;
@@ -645,7 +695,7 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
             // level ends as soon as the tree is full (the first leaves of a level then usually take all the room).
             const int BS = tt.FC > 32 ? nwarps : nfront;          // short follower lists: the whole frontier at once
             for (int base = 0; base < nfront; base += BS) {
-                const int n_now = sh_n;
+                const int n_now = base == 0 ? n_top : sh_n;       // (the warp of a single leaf changes sh_n while others come by here)
                 if (n_now >= T) break;
                 // (1) parallel lookups, one warp per leaf
                 for (int li = base + warp; li < min(nfront, base + BS); li += nwarps) {
@@ -666,7 +716,7 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                             mykey = S.tok[c];
                         } else {
                             const int pos = L - 1 - (back - d);
-                            mykey = pos >= 0 ? row[pos] : -1;
+                            mykey = pos >= 0 ? row(pos) : -1;
                         }
                     }
                     ok = ok && __all_sync(CB_FULL, mykey >= 0);
@@ -690,6 +740,18 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                                 else if (FETCH == 2) fs[c] = er.fs4[c];            // the stamps came with the lookup
                                 else fs[c] = (c * 32 + lane) < tt.FC ? e[tt.LL + c * 32 + lane] : 0u;
                                 nf += __popc(__ballot_sync(CB_FULL, fs[c] != 0u));
+                            }
+                            // The followers' tokens.  FC > 32: on their way while the followers are picked below (of all of them: the
+                            // round trip costs more than the bytes).
+                            int32_t ft[CB_MAX_FC / 32][CB_MAX_FL];
+#pragma unroll
+                            for (int c = 0; c < CB_MAX_FC / 32; ++c) {
+                                const int f = c * 32 + lane;
+#pragma unroll
+                                for (int j = 0; j < CB_MAX_FL; ++j) {
+                                    if (FETCH == 1) ft[c][j] = c == 0 ? er.tok[j] : -1;
+                                    else ft[c][j] = fs[c] != 0u && j < tt.FL ? (int32_t)e[tt.LL + tt.FC + f * tt.FL + j] : -1;
+                                }
                             }
                             // no more than the tree has room for chains of this length
                             const int cl = min(tt.FL, max_depth - d), room = (leaf == 0 ? max(1, T - crt) : T) - n_now;
@@ -726,18 +788,7 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                                 for (int c = 0; c < CB_MAX_FC / 32; ++c)
                                     if (fs[c] != 0u && cntr[c] < nf) rank[c] = cntr[c];
                             }
-                            // every lane copies the tokens of its picked followers (all loads before the first store, so that their
-                            // round trips overlap)
-                            int32_t ft[CB_MAX_FC / 32][CB_MAX_FL];
-#pragma unroll
-                            for (int c = 0; c < CB_MAX_FC / 32; ++c) {
-                                const int f = c * 32 + lane;
-#pragma unroll
-                                for (int j = 0; j < CB_MAX_FL; ++j) {
-                                    if (FETCH == 1) ft[c][j] = c == 0 ? er.tok[j] : -1;
-                                    else ft[c][j] = rank[c] >= 0 && j < tt.FL ? (int32_t)e[tt.LL + tt.FC + f * tt.FL + j] : -1;
-                                }
-                            }
+                            // every lane stages its picked followers
 #pragma unroll
                             for (int c = 0; c < CB_MAX_FC / 32; ++c) {
                                 if (rank[c] < 0) continue;
@@ -747,9 +798,32 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                             }
                         }
                     }
-                    if (lane == 0) { S.r_eid[li] = eid; S.r_nf[li] = nf; S.r_ok[li] = ok ? 1 : 0; }
+                    if (nfront > 1) {
+                        if (lane == 0) { S.r_eid[li] = eid; S.r_nf[li] = nf; S.r_ok[li] = ok ? 1 : 0; }
+                    } else {
+                        // the only leaf of its level: what (2) and (3) do, in place
+                        const int cap = leaf == 0 ? max(1, T - crt) : T;
+                        if (ok && n_now < cap) {
+                            const int cl = min(t.FL, max_depth - d), tot = eid >= 0 ? min(max(nf, 0) * cl, cap - n_now) : 0;
+                            const int ends = cl == t.FL ? (int)(((uint32_t)tot * kInverse[cl]) >> 16) : 0;
+                            __syncwarp();
+                            attach(leaf, d, n_now, cl, tot, S.fol + li * FLFC);
+                            for (int c = lane; c < ends; c += 32) S.next[c] = n_now + c * t.FL + t.FL - 1;
+                            if (lane == 0) {
+                                sh_n = n_now + tot; sh_nnext = ends;
+                                if (pass == 0) {
+                                    ++sh_q;
+                                    if (eid >= 0) { ++sh_hits; atomicMax(&s.lstamp[eid], clock0 + (uint32_t)sh_q); }
+                                } else {
+                                    ++sh_fq;
+                                    if (eid >= 0) ++sh_fhits;
+                                }
+                            }
+                        }
+                    }
                 }
                 __syncthreads();
+                if (nfront == 1) break;
                 // (2) the sequential breadth-first order, planned by one thread or warp and filled in by all.  A query at the root (the only
                 // leaf of level 1, the first one of the frozen pass) is issued, and its followers attached, while the tree has fewer
                 // than max(1, T - crt) nodes; any other while fewer than T.  Below a leaf of depth d every follower is a chain of
@@ -776,7 +850,7 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                             const int tot = min(max(S.r_nf[l2], 0) * cl, cap - n);
                             S.r_n0[l2] = n; S.r_cl[l2] = cl; S.r_tot[l2] = tot; S.r_nn0[l2] = nn;
                             n += tot;
-                            if (cl == t.FL) nn += tot / t.FL;
+                            if (cl == t.FL) nn += (int)(((uint32_t)tot * kInverse[cl]) >> 16);
                         }
                         sh_n = n; sh_nnext = nn;
                         if (pass == 0) { sh_q += q; sh_hits += hits; } else { sh_fq += q; sh_fhits += hits; }
@@ -807,7 +881,7 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                         const int tot = issued ? min(want, T - start) : 0;
                         const uint32_t mi = __ballot_sync(CB_FULL, issued);
                         hits += __popc(__ballot_sync(CB_FULL, issued && hit));
-                        const int leaves = cl == t.FL ? tot / t.FL : 0;
+                        const int leaves = cl == t.FL ? (int)(((uint32_t)tot * kInverse[cl]) >> 16) : 0;
                         int lincl = leaves;
 #pragma unroll
                         for (int o = 1; o < 32; o <<= 1) {
@@ -831,19 +905,14 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                 for (int l2 = base + warp; l2 < lend; l2 += nwarps) {
                     const int tot = S.r_tot[l2];
                     if (tot == 0) continue;
-                    const int leaf = S.front[l2], n0 = S.r_n0[l2], cl = S.r_cl[l2], d = S.dep[leaf];
-                    for (int x = lane; x < tot; x += 32) {
-                        const int f = x / cl, j = x - f * cl;
-                        S.tok[n0 + x] = S.fol[l2 * FLFC + f * t.FL + j];
-                        S.par[n0 + x] = j == 0 ? leaf : n0 + x - 1;
-                        S.dep[n0 + x] = d + j + 1;
-                    }
+                    const int leaf = S.front[l2], n0 = S.r_n0[l2], cl = S.r_cl[l2];
+                    attach(leaf, S.dep[leaf], n0, cl, tot, S.fol + l2 * FLFC);
                     if (cl == t.FL)
-                        for (int c = lane; c < tot / t.FL; c += 32) S.next[S.r_nn0[l2] + c] = n0 + c * t.FL + t.FL - 1;
+                        for (int c = lane; c < (int)(((uint32_t)tot * kInverse[cl]) >> 16); c += 32) S.next[S.r_nn0[l2] + c] = n0 + c * t.FL + t.FL - 1;
                 }
             }
             // (3) stamp the leaders the sequential order reached; publish the next frontier
-            if (pass == 0)
+            if (pass == 0 && nfront > 1)
                 for (int li = tid; li < nfront; li += blockDim.x)
                     if (S.r_stamp[li] != 0u) atomicMax(&s.lstamp[S.r_eid[li]], S.r_stamp[li]);
             const int nn = sh_nnext, np = sh_npts;
@@ -866,13 +935,10 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
         if (sh_fq) atomicAdd(&counters[CB_CNT_FROZEN_QUERIES], (unsigned long long)sh_fq);
         if (sh_fhits) atomicAdd(&counters[CB_CNT_FROZEN_HITS], (unsigned long long)sh_fhits);
     }
-    for (int i = tid; i < T; i += blockDim.x) {
-        o_tok[(size_t)b * T + i] = S.tok[i];
-        o_par[(size_t)b * T + i] = S.par[i];
-        o_dep[(size_t)b * T + i] = S.dep[i];
-        uint32_t m[4] = {0u, 0u, 0u, 0u};
-        if (i < n) for (int c = i; c >= 0; c = S.par[c]) m[c >> 5] |= 1u << (c & 31);
-        for (int k = 0; k < W; ++k) o_mask[((size_t)b * T + i) * W + k] = m[k];
+    for (int i = n + tid; i < T; i += blockDim.x) {              // places without a node
+        const size_t at = (size_t)b * T + i;
+        o_tok[at] = -1; o_par[at] = -1; o_dep[at] = -1;
+        for (int k = 0; k < W; ++k) o_mask[at * W + k] = 0u;
     }
 }
 
@@ -887,8 +953,9 @@ __global__ void __launch_bounds__(256) cb_draft_kernel(CbTables t, CbTables tf, 
     CB_PDL_ENTRY();
     extern __shared__ int32_t smem[];
     const int b = blockIdx.x;
-    draft_body<FETCH>(t, tf, T, crt, max_depth, NL, KF, tokens, row_stride, b, seq_len[b], upd_n_old ? upd_n_old[b] : -1, o_tok, o_par, o_dep,
-                      o_mask, o_n, status, counters, smem);
+    const int32_t* history = tokens + (size_t)b * row_stride;
+    draft_body<FETCH>(t, tf, T, crt, max_depth, NL, KF, [=](int i) { return history[i]; }, b, seq_len[b], upd_n_old ? upd_n_old[b] : -1, o_tok, o_par,
+                      o_dep, o_mask, o_n, status, counters, smem);
 }
 
 // Acceptance of one step and update + draft of the next in one launch (the three are a chain per sequence: Fig. 2).  The
@@ -914,28 +981,38 @@ __global__ void __launch_bounds__(256, CTAS) cb_accept_draft_kernel(AcceptArgs a
                                                               uint32_t* status, unsigned long long* counters) {
     CB_PDL_ENTRY();
     extern __shared__ int32_t smem[];
+    // The end of the history, from the first token of the first new window on, with the emitted tokens behind it: what the update and
+    // the root's key need, without going through memory.
+    __shared__ int32_t s_tail[CB_MAX_LL + CB_MAX_FL + 256], s_emit[256];
+    __shared__ int s_have, s_len;
+    const int b = blockIdx.z, tid = threadIdx.x, w = t.LL + t.FL;
+    int32_t* const history = tokens + (size_t)b * row_stride;
+    auto beside = [&](int k) {
+        if (k >= 32) return;
+        const int L = seq_len[b], tail0 = max(0, L - w + 1);
+        if (k < L - tail0 && L <= row_stride) s_tail[k] = history[tail0 + k];
+        if (k == 0) s_len = L;
+    };
     if (!accept_rows<BF16, CTAS == 2 && FETCH == 1 ? 8 : 4>(T, a.V, a.Dmax, a.chunk, a.chunks_per_row, a.logits, a.logits_row_stride, a.tok, a.par, a.dep,
-                                                            a.n_nodes, a.rowmax, a.ticket, a.n_accept, a.accept_nodes, a.out_tokens, a.target_out,
-                                                            [](int) {}))
+                                                            a.n_nodes, a.rowmax, a.ticket, a.n_accept, a.accept_nodes, a.out_tokens, a.target_out, beside,
+                                                            s_emit, &s_have))
         return;
-    __threadfence_block();
     __syncthreads();                                            // the walk (first warp) has written the sequence's result
-    const int b = blockIdx.z, tid = threadIdx.x;
-    const int m = __ldcg(&a.n_accept[b]);
-    const int have = min(max(__ldcg(&a.n_nodes[b]), 0), T) > 0 ? m + 1 : 0;   // tokens emitted (an empty tree emits none)
-    const int L = seq_len[b];
+    const int have = s_have;                                    // tokens emitted (an empty tree emits none)
+    const int L = s_len, tail0 = max(0, L - w + 1);
     int L1 = L + have;
     if (L1 > row_stride) {
         // no room in the history: nothing is appended and the step is reported; the draft below continues from what is there
         if (tid == 0) atomicCAS(status, 0u, (uint32_t)CB_ERR_INVALID_ARG);
         L1 = L;
     } else if (tid < have) {
-        tokens[(size_t)b * row_stride + L + tid] = __ldcg(&a.out_tokens[(size_t)b * (a.Dmax + 1) + tid]);
+        history[L + tid] = s_emit[tid];
+        s_tail[L - tail0 + tid] = s_emit[tid];
     }
-    __threadfence_block();
     __syncthreads();
     if (tid == 0) seq_len[b] = L1;
-    draft_body<FETCH>(t, tf, T, crt, max_depth, NL, KF, tokens, row_stride, b, L1, L, o_tok, o_par, o_dep, o_mask, o_n, status, counters, smem);
+    draft_body<FETCH>(t, tf, T, crt, max_depth, NL, KF, [&](int i) { return i >= tail0 && L <= row_stride ? s_tail[i - tail0] : history[i]; }, b, L1, L,
+                      o_tok, o_par, o_dep, o_mask, o_n, status, counters, smem);
 }
 
 }  // namespace
@@ -1058,7 +1135,7 @@ static cb_status draft_launch(cb_ctx* ctx, const int32_t* tokens, int64_t row_st
     // A leaf can receive at most T - 1 followers (each adds a node), so no more than that many are staged per lookup.
     const int FCmax = ctx->has_frozen ? max(c.FC, ctx->frozen.FC) : c.FC;
     const int KF = max(1, min(FCmax, T - 1));
-    const size_t smem = sizeof(int32_t) * ((size_t)3 * T + (size_t)11 * NL + (size_t)NL * c.FL * KF);
+    const size_t smem = sizeof(int32_t) * ((size_t)(3 + (T + 31) / 32) * T + (size_t)11 * NL + (size_t)NL * c.FL * KF);
     if (smem > 200 * 1024) return CB_ERR_UNSUPPORTED;
     if (smem > 48 * 1024) {
         static size_t opted[64] = {0};                         // largest size opted into so far, per device
@@ -1119,7 +1196,7 @@ extern "C" cb_status cb_accept_update_draft_tree(cb_ctx* ctx, const cb_accept_dr
     const int NL = min(T, (T - 1) / c.FL + 1);
     const int FCmax = ctx->has_frozen ? max(c.FC, ctx->frozen.FC) : c.FC;
     const int KF = max(1, min(FCmax, T - 1));
-    const size_t smem = sizeof(int32_t) * ((size_t)3 * T + (size_t)11 * NL + (size_t)NL * c.FL * KF);
+    const size_t smem = sizeof(int32_t) * ((size_t)(3 + (T + 31) / 32) * T + (size_t)11 * NL + (size_t)NL * c.FL * KF);
     if (smem > 200 * 1024) return CB_ERR_UNSUPPORTED;
     const bool bf = a->logits_dtype == CB_DTYPE_BF16;
     const bool resident = (long long)cpr * T * c.batch <= 2ll * ctx->num_sms;

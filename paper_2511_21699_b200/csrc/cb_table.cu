@@ -969,11 +969,11 @@ struct AcceptArgs {
     int32_t* n_accept; int32_t* accept_nodes; int32_t* out_tokens; int32_t* target_out;
 };
 
-// CTAS: CTAs that an SM has registers for.  The drafting code takes 96 registers and up, room for two.  A grid that is not resident at
-// once that way streams the logits with a third less in flight than with three CTAs of 75 (batch 32, fp32 logits over 128 k tokens: 287
-// against 216 us; batch 2 over 32 k: 16.9 against 16.0); one that is gains nothing from the bound and pays for it in the chain behind
-// the logits (batch 1 over 32 k: 13.9 against 14.2 us, a whole step 45.1 against 46.3).  With more than 32 followers a leader the code
-// takes 116 registers and stays at two.
+// CTAS: CTAs that an SM has registers for.  The drafting code takes 106 registers, room for two.  A grid that is not resident at
+// once that way streams the logits with half in flight of what four CTAs of 59 have (a step of batch 6 with trees of 96: 86.6 us with three
+// of 72, 82.9 with four; batch 4 of 64: 61.3 and 59.6); one that is gains nothing from the bound and pays for it in the chain behind
+// the logits, and takes all of a thread's chunk at once instead.  With more than 32 followers a leader the code takes 109 registers and
+// stays at two.
 template <int FETCH, bool BF16, int CTAS>
 __global__ void __launch_bounds__(256, CTAS) cb_accept_draft_kernel(AcceptArgs a, CbTables t, CbTables tf, int T, int crt, int max_depth, int NL, int KF,
                                                               int32_t* tokens, int64_t row_stride, int32_t* seq_len,
@@ -1202,7 +1202,7 @@ extern "C" cb_status cb_accept_update_draft_tree(cb_ctx* ctx, const cb_accept_dr
     const bool resident = (long long)cpr * T * c.batch <= 2ll * ctx->num_sms;
     auto kernel = FCmax > 32  ? (bf ? cb_accept_draft_kernel<2, true, 2> : cb_accept_draft_kernel<2, false, 2>)
                   : resident  ? (bf ? cb_accept_draft_kernel<1, true, 2> : cb_accept_draft_kernel<1, false, 2>)
-                              : (bf ? cb_accept_draft_kernel<1, true, 3> : cb_accept_draft_kernel<1, false, 3>);
+                              : (bf ? cb_accept_draft_kernel<1, true, 4> : cb_accept_draft_kernel<1, false, 4>);
     if (smem > 48 * 1024) {
         static std::mutex mu;
         static size_t opted[64][6] = {};                       // largest size opted into so far, per device and kernel

@@ -124,13 +124,14 @@ __global__ void cb_reset_kernel(CbTables t, const int32_t* __restrict__ mask) {
     const int b = blockIdx.y;
     if (mask && mask[b] == 0) return;
     CbSeq s = cb_seq(t, b);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < t.nslots; i += gridDim.x * blockDim.x) s.index[i] = 0;
+    uint4* const index = reinterpret_cast<uint4*>(s.index);     // buckets of 32 words, 256-byte aligned as a region
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < t.nslots / 4; i += gridDim.x * blockDim.x) index[i] = make_uint4(0u, 0u, 0u, 0u);
     if (blockIdx.x == 0 && threadIdx.x < 4) s.hdr[threadIdx.x] = 0;
 }
 
 extern "C" cb_status cb_reset(cb_ctx* ctx, const int32_t* dev_seq_mask, void* stream) {
     CB_CHECK_ARG(ctx);
-    uint32_t gx = std::min<uint32_t>(64, (ctx->tables.nslots + 255) / 256);
+    uint32_t gx = std::min<uint32_t>(64, (ctx->tables.nslots / 4 + 255) / 256);
     CB_CUDA(cb_launch_pdl(cb_reset_kernel, dim3(gx, ctx->cfg.batch), dim3(256), 0, (cudaStream_t)stream, ctx->tables, dev_seq_mask));
     cb_count_launch(1);
     return CB_OK;

@@ -339,14 +339,15 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                 uint32_t* e = s.entries + (size_t)eid * t.E;
                 if (team == 0u) s.lstamp[eid] = clock0 + (lw & 0xFFFFu);
                 // key, stamps (0: free), tokens of the followers that there are; zeros behind them up to 16 bytes
-                const uint32_t end = (uint32_t)(LL + t.FC) + n * (uint32_t)t.FL;
+                // (most leaders have one follower, which is looked up once)
+                const uint32_t end = (uint32_t)(LL + t.FC) + n * (uint32_t)t.FL, pw0 = S.pair[S.group[g]];
                 for (uint32_t q0 = 4u * team; q0 < end; q0 += 4u << lg) {
                     uint32_t v[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const int q = (int)q0 + j, f = q - LL, x = f - t.FC;
                         const uint32_t fi = x < 0 ? (uint32_t)max(f, 0) : ((uint32_t)x * fl_inv) >> 16;
-                        const uint32_t pw = fi < n ? S.pair[S.group[g + fi]] : 0u;
+                        const uint32_t pw = fi == 0u ? pw0 : (fi < n ? S.pair[S.group[g + fi]] : 0u);
                         v[j] = pw ? clock0 + (pw & 0xFFFFu) : 0u;
                         if (f < 0 || (x >= 0 && pw)) v[j] = (uint32_t)S.tok[f < 0 ? kpos + q : (pw >> 16) - 1u + (uint32_t)(LL + x) - fi * (uint32_t)t.FL];
                     }

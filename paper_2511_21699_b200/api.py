@@ -1,7 +1,8 @@
 """Thin Python binding of the C-ABI library: argument marshalling only.
 
 Tensors are torch CUDA tensors (device memory and streams are torch's); every step of the path runs in
-the library's kernels.  Method names mirror the C entry points.
+the library's kernels.  Method names mirror the C entry points.  The calls of a decoding loop are marshalled by the compiled
+module _binding (csrc/cb_binding.cpp), the others by ctypes here.
 """
 import ctypes as C
 
@@ -9,7 +10,7 @@ import numpy as np
 import torch
 
 from . import _lib
-from ._lib import CbConfigC, CbAttnArgsC, CbKvCommitArgsC, CbFrozenConfigC
+from ._lib import CbConfigC, CbFrozenConfigC
 
 
 class CachebackError(RuntimeError):
@@ -33,6 +34,26 @@ def _ptr(t, dtype=None):
 
 def _stream(stream):
     return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
+
+
+_BOUND = ("cb_reset", "cb_update", "cb_update_bulk", "cb_draft_tree", "cb_update_draft_tree", "cb_tree_attn", "cb_accept",
+          "cb_accept_update_draft_tree", "cb_kv_commit", "cb_status_str")
+_host_module = None
+
+
+def _host():
+    """The module _binding, calling the build of the library that _lib.load() chose."""
+    global _host_module
+    if _host_module is None:
+        lib = _lib.load()
+        try:
+            from . import _binding
+        except ImportError as e:
+            raise RuntimeError("_binding.so is not built or does not fit this torch (%s). Run `python -m paper_2511_21699_b200.build` "
+                               "or __graft_entry__.build(); there is no fallback path." % e) from e
+        _binding.set_library(CachebackError, {n: C.cast(getattr(lib, n), C.c_void_p).value for n in _BOUND})
+        _host_module = _binding
+    return _host_module
 
 
 def cb_accept_static(tree, logits, max_depth, res=None, stream=None):
@@ -128,6 +149,7 @@ class Cacheback:
         self.lib = _lib.load()
         if not torch.cuda.is_available():
             raise CachebackError("no CUDA device: the library has no CPU path")
+        self._host = _host()
         self.device = torch.device(device)
         self.cfg = CbConfigC(batch, LL, FL, LC, FC, max_nodes, crt, max_depth, vocab, n_q_heads, n_kv_heads, head_dim,
                              page_size, flags)
@@ -161,15 +183,13 @@ class Cacheback:
 
     # ---- the four step calls -----------------------------------------------------------------------
     def cb_reset(self, seq_mask=None, stream=None):
-        _check(self.lib.cb_reset(self._h, _ptr(seq_mask, torch.int32), _stream(stream)), "cb_reset")
+        self._host.reset(self._h, seq_mask, stream)
 
     def cb_update(self, tokens, n_old, n_new, stream=None):
-        _check(self.lib.cb_update(self._h, _ptr(tokens, torch.int32), tokens.stride(0), _ptr(n_old, torch.int32),
-                                  _ptr(n_new, torch.int32), _stream(stream)), "cb_update")
+        self._host.update(self._h, tokens, n_old, n_new, stream)
 
     def cb_update_bulk(self, tokens, n_old, n_new, stream=None):
-        _check(self.lib.cb_update_bulk(self._h, _ptr(tokens, torch.int32), tokens.stride(0), _ptr(n_old, torch.int32),
-                                       _ptr(n_new, torch.int32), _stream(stream)), "cb_update_bulk")
+        self._host.update_bulk(self._h, tokens, n_old, n_new, stream)
 
     def cb_bulk_scratch_attach(self, max_windows):
         """Allocates and attaches scratch for the order-free path of cb_update_bulk (runs of up to max_windows windows in
@@ -195,20 +215,13 @@ class Cacheback:
 
     def cb_draft_tree(self, tokens, seq_len, tree=None, stream=None):
         tree = tree if tree is not None else self.alloc_tree()
-        _check(self.lib.cb_draft_tree(self._h, _ptr(tokens, torch.int32), tokens.stride(0), _ptr(seq_len, torch.int32),
-                                      _ptr(tree["tokens"], torch.int32), _ptr(tree["parent"], torch.int32),
-                                      _ptr(tree["depth"], torch.int32), _ptr(tree["mask"], torch.int32),
-                                      _ptr(tree["n_nodes"], torch.int32), _stream(stream)), "cb_draft_tree")
+        self._host.draft_tree(self._h, tokens, seq_len, tree, stream)
         return tree
 
     def cb_update_draft_tree(self, tokens, n_old, n_new, tree=None, stream=None):
         """cb_update(tokens, n_old, n_new) and cb_draft_tree(tokens, n_new) in one launch."""
         tree = tree if tree is not None else self.alloc_tree()
-        _check(self.lib.cb_update_draft_tree(self._h, _ptr(tokens, torch.int32), tokens.stride(0), _ptr(n_old, torch.int32),
-                                             _ptr(n_new, torch.int32),
-                                             _ptr(tree["tokens"], torch.int32), _ptr(tree["parent"], torch.int32),
-                                             _ptr(tree["depth"], torch.int32), _ptr(tree["mask"], torch.int32),
-                                             _ptr(tree["n_nodes"], torch.int32), _stream(stream)), "cb_update_draft_tree")
+        self._host.update_draft_tree(self._h, tokens, n_old, n_new, tree, stream)
         return tree
 
     def cb_tree_add_branches(self, tree, branches, branch_len, stream=None):
@@ -224,19 +237,12 @@ class Cacheback:
                      lse=None, max_ctx=0, scale=0.0, stream=None):
         if out is None:
             out = torch.empty_like(q)
-        a = CbAttnArgsC(_ptr(q, torch.bfloat16), _ptr(k_pool, torch.bfloat16), _ptr(v_pool, torch.bfloat16),
-                        _ptr(block_table, torch.int32), _ptr(ctx_len, torch.int32), _ptr(k_tree, torch.bfloat16),
-                        _ptr(v_tree, torch.bfloat16), _ptr(tree_mask, torch.int32), _ptr(n_nodes, torch.int32),
-                        _ptr(out, torch.bfloat16), _ptr(lse, torch.float32), block_table.shape[1], k_pool.shape[0],
-                        int(max_ctx), float(scale))
-        _check(self.lib.cb_tree_attn(self._h, C.byref(a), _stream(stream)), "cb_tree_attn")
+        self._host.tree_attn(self._h, q, k_pool, v_pool, block_table, ctx_len, k_tree, v_tree, tree_mask, n_nodes, out, lse, int(max_ctx),
+                             float(scale), stream)
         return out
 
     def cb_kv_commit(self, k_pool, v_pool, block_table, ctx_len, k_tree, v_tree, n_accept, accept_nodes, stream=None):
-        a = CbKvCommitArgsC(_ptr(k_pool, torch.bfloat16), _ptr(v_pool, torch.bfloat16), _ptr(block_table, torch.int32),
-                            _ptr(ctx_len, torch.int32), _ptr(k_tree, torch.bfloat16), _ptr(v_tree, torch.bfloat16),
-                            _ptr(n_accept, torch.int32), _ptr(accept_nodes, torch.int32), block_table.shape[1], k_pool.shape[0])
-        _check(self.lib.cb_kv_commit(self._h, C.byref(a), _stream(stream)), "cb_kv_commit")
+        self._host.kv_commit(self._h, k_pool, v_pool, block_table, ctx_len, k_tree, v_tree, n_accept, accept_nodes, stream)
 
     def alloc_accept(self):
         B, Dm = self.cfg.batch, self.cfg.max_depth
@@ -246,23 +252,7 @@ class Cacheback:
 
     def cb_accept(self, tree, logits=None, target_ids=None, res=None, stream=None):
         res = res if res is not None else self.alloc_accept()
-        dtype, stride, lp = 0, 0, None
-        if logits is not None:
-            if logits.dtype == torch.float32:
-                dtype = _lib.CB_DTYPE_F32
-            elif logits.dtype == torch.bfloat16:
-                dtype = _lib.CB_DTYPE_BF16
-            else:
-                raise CachebackError("logits must be float32 or bfloat16")
-            if not (logits.is_cuda and logits.dim() == 3 and logits.stride(2) == 1 and
-                    logits.stride(0) == logits.shape[1] * logits.stride(1)):
-                raise CachebackError("logits must be [batch, max_nodes, vocab] with a uniform row stride")
-            stride, lp = logits.stride(1), logits.data_ptr()
-        _check(self.lib.cb_accept(self._h, _ptr(tree["tokens"], torch.int32), _ptr(tree["parent"], torch.int32),
-                                  _ptr(tree["depth"], torch.int32), _ptr(tree["n_nodes"], torch.int32), lp, dtype, stride,
-                                  _ptr(target_ids, torch.int32), _ptr(res["n_accept"], torch.int32),
-                                  _ptr(res["accept_nodes"], torch.int32), _ptr(res["out_tokens"], torch.int32),
-                                  _ptr(res["target_ids"], torch.int32), _stream(stream)), "cb_accept")
+        self._host.accept(self._h, tree, logits, target_ids, res, stream)
         return res
 
     def cb_accept_update_draft_tree(self, tree, logits, tokens, seq_len, next_tree=None, res=None, stream=None):
@@ -270,23 +260,7 @@ class Cacheback:
         and cb_draft_tree into next_tree (default: the same arrays as `tree`), in one launch."""
         res = res if res is not None else self.alloc_accept()
         next_tree = next_tree if next_tree is not None else tree
-        if logits.dtype == torch.float32:
-            dtype = _lib.CB_DTYPE_F32
-        elif logits.dtype == torch.bfloat16:
-            dtype = _lib.CB_DTYPE_BF16
-        else:
-            raise CachebackError("logits must be float32 or bfloat16")
-        if not (logits.is_cuda and logits.dim() == 3 and logits.stride(2) == 1 and logits.stride(0) == logits.shape[1] * logits.stride(1)):
-            raise CachebackError("logits must be [batch, max_nodes, vocab] with a uniform row stride")
-        a = _lib.CbAcceptDraftArgsC(logits.data_ptr(), dtype, logits.stride(1), _ptr(tree["tokens"], torch.int32),
-                                    _ptr(tree["parent"], torch.int32), _ptr(tree["depth"], torch.int32), _ptr(tree["n_nodes"], torch.int32),
-                                    _ptr(res["n_accept"], torch.int32), _ptr(res["accept_nodes"], torch.int32),
-                                    _ptr(res["out_tokens"], torch.int32), _ptr(res["target_ids"], torch.int32),
-                                    _ptr(tokens, torch.int32), tokens.stride(0), _ptr(seq_len, torch.int32),
-                                    _ptr(next_tree["tokens"], torch.int32), _ptr(next_tree["parent"], torch.int32),
-                                    _ptr(next_tree["depth"], torch.int32), _ptr(next_tree["mask"], torch.int32),
-                                    _ptr(next_tree["n_nodes"], torch.int32))
-        _check(self.lib.cb_accept_update_draft_tree(self._h, C.byref(a), _stream(stream)), "cb_accept_update_draft_tree")
+        self._host.accept_update_draft_tree(self._h, tree, logits, tokens, seq_len, next_tree, res, stream)
         return res
 
     # ---- helpers ------------------------------------------------------------------------------------

@@ -40,6 +40,7 @@ struct CbAttnParams {
     uint32_t* part_turn;  // [0] launches of the context so far: the lowest bit names the set in use; [1] CTAs of this one that have left
     int B, T, W, Hq, Hkv, G, D, P, max_pages, num_pages;
     int NPT;              // tree nodes per row tile = 128 / G
+    uint32_t npt_inv;     // x / NPT = x * npt_inv >> 16 for x < 256
     int MT;               // row tiles that T nodes need = ceil(T / NPT)
     int nc;               // persistent CTAs (= ranges of the global tile sequence)
     int w1, w2;           // positions that a key tile of a unit with one or with two row tiles counts
@@ -68,7 +69,7 @@ __device__ __forceinline__ CbSeqShape cb_seq_shape(const CbAttnParams& p, int b)
     s.n = min(max(p.n_nodes[b], 0), p.T);
     s.ctx = min(max(p.ctx_len[b], 0), p.max_pages * p.P);
     s.tiles = (s.ctx + CB_KT - 1) / CB_KT + 1;
-    s.mtn = (s.n + p.NPT - 1) / p.NPT;
+    s.mtn = (int)(((uint32_t)(s.n + p.NPT - 1) * p.npt_inv) >> 16);
     s.one = p.MT == 1;
     s.RG = s.one ? (s.mtn > 0 ? 1 : 0) : (s.mtn + 1) / 2;
     s.w1 = p.w1; s.w2 = p.w2;
@@ -82,9 +83,24 @@ __device__ __forceinline__ CbSeqShape cb_seq_shape(const CbAttnParams& p, int b)
 __device__ __forceinline__ long long cb_div(long long a, long long b) {
     return ((unsigned long long)a | (unsigned long long)b) >> 32 ? a / b : (long long)((uint32_t)a / (uint32_t)b);
 }
-__device__ __forceinline__ long long cb_range_start(long long total, int nc, int c) { return cb_div(total * c, nc); }
+// a / b for a >= 0 and 0 < b < 2^22.  A division is a chain of some 200 cycles, and the first copy of a launch waited for five of
+// them (batch 13, head_dim 64: 2.3 k cycles from the schedule to the block table's entry); small numbers are divided in fp32, exactly.
+__device__ __forceinline__ long long cb_quot(long long a, int b) {
+    if (a < (1ll << 22)) {
+        const int x = (int)a;
+        int q = (int)__fdividef((float)x, (float)b);
+        const int r = x - q * b;
+        q += r < 0 ? -1 : (r >= b ? 1 : 0);
+        return q;
+    }
+    return cb_div(a, b);
+}
+__device__ __forceinline__ long long cb_range_start(long long total, int nc, int c) { return cb_quot(total * c, nc); }
 // CTA whose range holds global tile x.
-__device__ __forceinline__ int cb_cta_of(long long total, int nc, long long x) { return (int)cb_div((x + 1) * nc - 1, total); }
+__device__ __forceinline__ int cb_cta_of(long long total, int nc, long long x) {
+    const long long at = (x + 1) * nc - 1;
+    return (int)(total < (1ll << 22) ? cb_quot(at, (int)total) : cb_div(at, total));
+}
 
 // Row groups a launch can have per sequence (trees of max_nodes nodes).
 __device__ __forceinline__ int cb_max_row_groups(const CbAttnParams& p) { return p.MT == 1 ? 1 : (p.MT + 1) / 2; }
@@ -176,12 +192,12 @@ struct CbWalker {
             }
             const long long off = g - pre;
             const int vt = s.unit(rg), wt = s.wt(rg), ov = s.ov(rg);
-            const int kh = (int)cb_div(off, vt);
+            const int kh = (int)cb_quot(off, vt);
             const int v0 = (int)(off - (long long)kh * vt);
             const int v1 = (int)min((long long)vt, (long long)v0 + (g1 - g));
             g += v1 - v0;
-            u->t0 = (max(v0 - ov, 0) + wt - 1) / wt;
-            u->t1 = (max(v1 - ov, 0) + wt - 1) / wt;
+            u->t0 = (max(v0 - ov, 0) + wt - 1) >> (wt - 1);  // wt is 1 or 2
+            u->t1 = (max(v1 - ov, 0) + wt - 1) >> (wt - 1);
             if (u->t1 <= u->t0) continue;                     // no tile of this unit begins in the range
             u->b = b; u->kh = kh; u->rg = rg; u->tiles = s.tiles; u->n = s.n; u->ctx = s.ctx;
             u->nrt = p.MT == 1 ? 1 : min(2, s.mtn - 2 * rg);

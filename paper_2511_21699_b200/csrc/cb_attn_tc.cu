@@ -195,7 +195,9 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
     constexpr uint32_t ns = (uint32_t)C::NSLOT;
     // Cluster mode: the peers' barriers must exist before anything arrives on them.  Every thread reports here and waits where its
     // role first reaches over, or at its end (a CTA must not leave before the others' report either).
-    if (p.cs > 0) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    // What they must see of this CTA, its initialised barriers, went out with the fence behind the initialisation, so the report itself
+    // releases nothing (a releasing one waits for every access before it: 0.9 k of the cycles before batch 1's first copy).
+    if (p.cs > 0) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     auto cluster_wait = [&]() {
         if (p.cs > 0) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     };
@@ -226,7 +228,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             bool ok = true;
             const uint64_t pol = l2_evict_first_policy();
             while (ok && wk.next(p, &u)) {
-                const int npages = (u.ctx + p.P - 1) / p.P, nct = u.tiles - 1;
+                const int npages = (u.ctx + 15) / 16, nct = u.tiles - 1;   // pages of 16 tokens (checked by the launcher)
                 const int32_t* bt = p.block_table + (size_t)u.b * p.max_pages;
                 // The page number of a lane's box comes from the block table: a memory round trip that the copy depends on.
                 // It is fetched one tile ahead, so that it is under way while this tile's copies are issued and waited for.

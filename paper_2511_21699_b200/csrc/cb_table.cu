@@ -317,14 +317,19 @@ __device__ __forceinline__ void update_seq_cta(const CbTables& t, int b, const T
             __syncthreads();
             // lane j looks at window j: every warp comes to the same masks (all lanes take part in every vote)
             const bool there = lane < nb;
-            const uint32_t state = there ? sh_state[lane] : 2u, below = (1u << lane) - 1u;
+            const uint32_t state = there ? sh_state[lane] : 2u;
             const unsigned long long hj = there ? sh_h[lane] : 0ull;
-            const uint32_t same = __match_any_sync(CB_FULL, hj) & ((1u << nb) - 1u) & below;
-            const bool seq = there && (same != 0u || state == 2u);
+            // (seven comparisons each: __match_any_sync took 500 cycles for either of the two)
+            bool same = false;
+#pragma unroll
+            for (int k = 0; k < kUpdWarps - 1; ++k) same = same || (k < lane && k < nb && sh_h[k] == hj);
+            const bool seq = there && (same || state == 2u);
             const bool fresh = there && state == 1u && !seq;
             const uint32_t bj = fresh ? sh_bucket[lane] : 0x80000000u | (uint32_t)lane;
-            const uint32_t beside = __match_any_sync(CB_FULL, bj) & below;
-            const bool clash = fresh && beside != 0u;
+            bool beside = false;
+#pragma unroll
+            for (int k = 0; k < kUpdWarps - 1; ++k) beside = (__shfl_sync(CB_FULL, bj, k) == bj && k < lane) || beside;
+            const bool clash = fresh && beside;
             later = __ballot_sync(CB_FULL, seq || clash);
             const uint32_t newm = __ballot_sync(CB_FULL, fresh && !clash);
             if (mine && !((later >> warp) & 1u)) {

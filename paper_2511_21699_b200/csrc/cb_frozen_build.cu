@@ -9,16 +9,19 @@
 //   2. the LC best leaders under the order (count falling, tokens rising) are found by a most-significant-digit-first
 //      radix select over the distinct leaders (one histogram pass per 12 bits of the composite key; the block that comes
 //      last picks the digit), then written into the frozen table's entries and hashed into its index;
-//   3. follower counts: windows whose leader was selected insert-or-increment the whole window in a second table; a distinct
-//      window takes its ordinal among its leader's when it is created, every leader takes a range of the group array, and
-//      position and count of the distinct windows go there, grouped by leader;
-//   4. a warp per leader (a block for those with more than 32 distinct windows) picks the FC best of its group under
-//      (count falling, follower tokens rising): a threshold by bisection on the count, then on the tokens of the windows that
-//      tie with it where those are many, and ranks what is left.
-// What bounds it is random access to the two hash tables (8 bytes a slot, 2 to 4 slots a window) and the counting of frequent
-// keys; a block gathers its counts of repeated slots in shared memory, so that a key that makes up a tenth of the corpus costs
-// an atomic per block and not one per occurrence.  4 M tokens, LL = 2, LC = 65,536, FC = 8: 3.1 ms with a scan of the whole group per
-// distinct window (1.57 ms of it), 37 launches and a one-block scan, 0.75 ms with this form; 8 M tokens, LL = 1, FC = 128: 26.9 and 2.8 ms.
+//   3. the windows of the selected leaders go into the leaders' ranges of one array (a counting sort: the leader counts are known
+//      from step 1), all but those of the few leaders with more than kBigGroup windows: these insert-or-increment the whole window in
+//      a second hash table, and the distinct ones are grouped by leader afterwards;
+//   4. a leader's windows are told apart, counted and the FC best picked under (count falling, follower tokens rising) by a warp
+//      (up to 32 windows: the lanes match their tokens against one another) or by a block with a table in shared memory; of a
+//      big leader's distinct windows a block picks the FC best from memory.  The pick: a threshold by bisection on the count, then on
+//      the tokens of the windows that tie with it where those are many; what is left is ranked.
+// What bounds it is random access: to the leader table (8 bytes a slot, 2 to 4 slots a window) and to the leaders' ranges.  The frequent
+// keys' counts and the lists are gathered per block in shared memory, so that a key that makes up a tenth of the corpus costs
+// an atomic per block and not one per occurrence.  Counting every selected window in a second hash table took 212 us of a build from 4 M
+// tokens (LL = 2, LC = 65,536, FC = 8: 167 MB of tables at random, more than the L2 holds), grouping its slots 49 us, ranking 187 us.
+// The whole call with the draft that follows it: 763 us that way, 547 us this way (60,000 tokens: 220 and 164; 8 launches of the selection
+// are one, which is most of it there).
 // Which occurrence represents a key, and which entry id a leader gets, depends on timing; the table's content (and
 // cb_frozen_dump's output) does not.
 #include <algorithm>
@@ -31,39 +34,47 @@ constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 constexpr unsigned long long kEmptySlot = 0x00000000FFFFFFFFull;   // low word: position, high word: count
 constexpr int kMaxWords = 1 + CB_MAX_LL;      // composite selection key: count (complemented), then the leader's tokens
 constexpr int kDigitBits = 12, kBins = 1 << kDigitBits;
-constexpr uint32_t kMidGroup = 1024;          // distinct windows of one leader up to which a block of 128 threads does the selection
-constexpr int kCand = 512;                    // candidates ranked against one another (at least FC)
+constexpr int kMaxPasses = 1 + 3 * kMaxWords;  // leader counts below 4,095, then three digits for each word of the key
+constexpr uint32_t kWarpGroup = 128;          // windows of one leader that a warp takes (up to 32: a lane each)
+constexpr uint32_t kMidGroup = 512;           // windows of one leader that a block of 128 threads takes
+constexpr uint32_t kBigGroup = 4096;          // windows of one leader that a block of 512 threads takes; above: the second hash table
+constexpr int kCand = 256;                    // candidates ranked against one another (at least FC)
 static_assert(kCand >= 2 * CB_MAX_FC, "the FC best and as many ties fit");
 
 struct BuildState {                           // head of the scratch buffer
-    uint32_t status;
+    uint32_t status;                          // (the state is cleared before the first launch)
     uint32_t n_uniq;                          // distinct leaders
     uint32_t n_sel;                           // entry ids handed out
-    uint32_t n_mid, n_big;                    // leaders with groups of more than 32, of more than kMidGroup windows
+    uint32_t n_warp, n_mid, n_large, n_big;   // leaders with more than 32, kWarpGroup, kMidGroup, kBigGroup windows
     uint32_t n_ties;                          // leaders whose count is exactly that of the LC-th best
-    uint32_t count_known;                     // word 0 of the prefix is resolved
-    uint32_t k_rem;                           // radix select: rank still to be resolved inside the current prefix
-    uint32_t cursor;                          // next free place of the group array
-    uint32_t arrived;                         // blocks of the running histogram pass that are done
-    uint32_t max_token;                       // largest token of a leader
-    uint32_t prefix[kMaxWords];               // composite key of the LC-th best leader, resolved digit by digit
-    uint32_t hist[kBins];
+    uint32_t cursor, big_cursor;              // next free place of the window array, of the group array (the big leaders' windows)
+    uint32_t arrived;                         // blocks of the selection that have come to its barriers so far
+    uint32_t max_token;                       // largest token of the corpus
+    uint32_t has_neg;                         // some token is negative
+    alignas(16) uint32_t hist[kMaxPasses][kBins];   // one histogram per pass of the selection (read 16 bytes at a time)
 };
+
+static_assert(offsetof(BuildState, hist) % 16 == 0, "histograms are read 16 bytes at a time");
 
 struct BuildView {
     BuildState* st;
-    unsigned long long* h1; int32_t* h1_eid;                      // [S] leaders: position and count; entry id or -1
-    unsigned long long* h2; uint32_t* h2_ord;                     // [S] windows of selected leaders; ordinal in the leader's group
+    unsigned long long* h1;                                       // [S] leaders: position and count; a selected one: kTaken | entry id in the count's place
+    unsigned long long* h2; uint32_t* h2_ord;                     // [S] windows of big leaders (big_slots in use); ordinal in the leader's group
     uint32_t* lslot;                                              // [M] leader slot of every window (kEmpty: left out)
-    uint2* group;                                                 // [S] distinct windows grouped by leader: position, count
-    uint32_t* uniq; uint32_t* ties;                               // [M] slots of the distinct leaders, of those that tie with the LC-th best
+    uint2* group;                                                 // [M] distinct windows of the big leaders, grouped by leader: position, count
+    uint32_t* uniq; uint2* ties;                                  // [M] slots of the distinct leaders; slot and position of those that tie with the LC-th best
                                                                   // (both share group's memory: dead before that is filled)
-    uint32_t* grp_n; uint32_t* grp_off; uint32_t* listed;         // [LC] group size, start; leaders with middling groups from the front, large from the back
+    uint32_t* wpos;                                               // [M] windows of the other selected leaders, grouped by leader
+    uint32_t* grp_n; uint32_t* grp_off;                           // [LC] windows placed (big: distinct ones); start, kBigFlag: of group, else of wpos
+    uint32_t* listed; uint32_t* listed_big;                       // [LC] each: middling leaders from the front, large ones from the back; big ones
+                                                                  // from the front, those that a warp takes from the back
     uint32_t S;                                                   // slots of each hash table (a power of two)
     const int32_t* corpus;
-    uint32_t M;
+    uint32_t M, n_tokens;
     int LL, FL, LC, FC;
 };
+
+constexpr uint32_t kTaken = 0x80000000u, kBigFlag = 0x80000000u;   // counts and positions stay below 2^30
 
 __device__ __forceinline__ uint64_t hash_tokens(const int32_t* p, int n) {
     uint64_t h = 0x9E3779B97F4A7C15ull ^ (uint64_t)n;
@@ -75,11 +86,10 @@ __device__ __forceinline__ bool same_tokens(const int32_t* a, const int32_t* b, 
     for (int j = 0; j < n; ++j) if (a[j] != b[j]) return false;
     return true;
 }
-// Finds or creates the slot of the n-token key at corpus position i.  Returns the slot, or kEmpty when every slot was
+// Finds or creates the slot of the n-token key at corpus position i, from slot s on.  Returns the slot, or kEmpty when every slot was
 // visited (cannot happen at the load factor the tables are sized for; reported as CB_ERR_PROBE_LIMIT).  A slot's position never
 // changes once it is set, so an ordinary load will do; one that still shows an empty slot is put right by the compare-and-swap.
-__device__ __forceinline__ uint32_t find_or_claim(unsigned long long* slots, uint32_t S, const int32_t* corpus, uint32_t i, int n, bool* created) {
-    uint32_t s = (uint32_t)(hash_tokens(corpus + i, n) >> 20) & (S - 1);
+__device__ __forceinline__ uint32_t find_or_claim(unsigned long long* slots, uint32_t S, uint32_t s, const int32_t* corpus, uint32_t i, int n, bool* created) {
     *created = false;
     for (uint32_t p = 0; p < S; ++p) {
         uint32_t pos = *reinterpret_cast<const uint32_t*>(&slots[s]);
@@ -92,6 +102,13 @@ __device__ __forceinline__ uint32_t find_or_claim(unsigned long long* slots, uin
         s = (s + 1) & (S - 1);
     }
     return kEmpty;
+}
+__device__ __forceinline__ uint32_t home_slot(const int32_t* key, int n, uint32_t S) { return (uint32_t)(hash_tokens(key, n) >> 20) & (S - 1); }
+// Slots of the second table that this corpus needs: a power of two, at least twice the windows that go there.
+__device__ __forceinline__ uint32_t big_slots(const BuildView& v) {
+    uint32_t s = 1024;
+    while (s < 2u * __ldcg(&v.st->big_cursor) && s < v.S) s <<= 1;
+    return s;
 }
 __device__ __forceinline__ uint32_t* count_of(unsigned long long* slots, uint32_t s) { return reinterpret_cast<uint32_t*>(&slots[s]) + 1; }
 
@@ -121,22 +138,35 @@ struct CountCache {
 
 // Items that threads of a block append to a list in memory: gathered in shared memory, so that the list's counter takes an atomic
 // per thousand or so (one address takes one atomic in about 2 ns: an atomic per warp was 260 of 310 us of the leader count).
+template <typename T>
 struct Appender {
-    static constexpr uint32_t kCap = 1536;
-    uint32_t item[kCap], n, at;
+    static constexpr uint32_t kCap = 2048;
+    T item[kCap];
+    uint32_t n, at;
     __device__ __forceinline__ void clear() { if (threadIdx.x == 0) n = 0u; __syncthreads(); }
-    // all threads of the block together
-    __device__ __forceinline__ void add(bool has, uint32_t x, uint32_t* list, uint32_t* counter) {
-        const uint32_t m = __ballot_sync(CB_FULL, has), lane = threadIdx.x & 31;
-        uint32_t k = 0;
-        if (m && lane == 0) k = atomicAdd(&n, (uint32_t)__popc(m));
-        k = __shfl_sync(CB_FULL, k, 0) + __popc(m & ((1u << lane) - 1u));
-        if (has) item[k] = x;
+    // All threads of the block together, U items each at most; true (in all of them) if there may be no room for as many again.
+    template <int U>
+    __device__ __forceinline__ bool gather(const bool (&has)[U], const T (&x)[U]) {
+        const uint32_t lane = threadIdx.x & 31;
+        uint32_t m[U], k = 0, total = 0;
+#pragma unroll
+        for (int q = 0; q < U; ++q) { m[q] = __ballot_sync(CB_FULL, has[q]); total += (uint32_t)__popc(m[q]); }
+        if (total && lane == 0) k = atomicAdd(&n, total);
+        k = __shfl_sync(CB_FULL, k, 0);
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            if (has[q]) item[k + __popc(m[q] & ((1u << lane) - 1u))] = x[q];
+            k += (uint32_t)__popc(m[q]);
+        }
         // The block decides as one: every warp reads the count before it arrives at the barrier (the last to add sees all of it), and
         // nobody adds again before all have.  Read after a barrier, the count could already hold the next call's additions.
-        if (__syncthreads_or(n > kCap - 256u)) flush(list, counter);
+        return __syncthreads_or(n > kCap - blockDim.x * U) != 0;
     }
-    __device__ __forceinline__ void flush(uint32_t* list, uint32_t* counter) {
+    template <int U>
+    __device__ __forceinline__ void add(const bool (&has)[U], const T (&x)[U], T* list, uint32_t* counter) {
+        if (gather(has, x)) flush(list, counter);
+    }
+    __device__ __forceinline__ void flush(T* list, uint32_t* counter) {
         __syncthreads();
         if (threadIdx.x == 0) at = n ? atomicAdd(counter, n) : 0u;
         __syncthreads();
@@ -147,185 +177,201 @@ struct Appender {
     }
 };
 
-__global__ void fb_init_kernel(BuildView v, CbTables t) {
+__global__ void __launch_bounds__(256) fb_init_kernel(BuildView v, CbTables t) {
+    CB_PDL_ENTRY();
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
-    ulonglong2* a = reinterpret_cast<ulonglong2*>(v.h1);
-    ulonglong2* b = reinterpret_cast<ulonglong2*>(v.h2);
-    for (size_t i = g; i < v.S / 2; i += stride) { a[i] = make_ulonglong2(kEmptySlot, kEmptySlot); b[i] = make_ulonglong2(kEmptySlot, kEmptySlot); }
     for (size_t i = g; i < (size_t)v.LC; i += stride) { v.grp_n[i] = 0u; t.lstamp[i] = 0u; }
     for (size_t i = g; i < t.nslots; i += stride) t.index[i] = CB_IDX_EMPTY;
-    for (size_t i = g; i < (size_t)v.LC * t.E; i += stride) t.entries[i] = 0u;
-    for (size_t i = g; i < sizeof(BuildState) / 4; i += stride) reinterpret_cast<uint32_t*>(v.st)[i] = 0u;
+    uint4* const e = reinterpret_cast<uint4*>(t.entries);      // E is a multiple of four words
+    for (size_t i = g; i < (size_t)v.LC * t.E / 4; i += stride) e[i] = make_uint4(0u, 0u, 0u, 0u);
     if (g < 4) t.hdr[g] = 0u;
+    // what the passes want to know of the corpus (the state was cleared before this launch)
+    int32_t lo = 0, hi = 0;
+    for (size_t i = g; i < v.n_tokens; i += stride) { const int32_t x = v.corpus[i]; lo = min(lo, x); hi = max(hi, x); }
+    const bool neg = __syncthreads_or(lo < 0) != 0;
+    hi = __reduce_max_sync(CB_FULL, hi);
+    __shared__ int32_t s_hi[8];
+    if ((threadIdx.x & 31) == 0) s_hi[threadIdx.x >> 5] = hi;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) hi = max(hi, s_hi[k]);
+        atomicMax(&v.st->max_token, (uint32_t)hi);
+        if (neg) { v.st->has_neg = 1u; if (v.M > 0) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_INVALID_ARG); }
+    }
+    // last, so that as much of it as possible is in L2 when the leaders are counted
+    ulonglong2* a = reinterpret_cast<ulonglong2*>(v.h1);
+    for (size_t i = g; i < v.S / 2; i += stride) a[i] = make_ulonglong2(kEmptySlot, kEmptySlot);
 }
 
-// 1. leader counts
+// 1. leader counts.  Four windows a thread, so that their chains (slot, tokens of the slot's occurrence) overlap; what the first look
+// does not settle is looked up slot by slot.
+template <int LL>
 __global__ void __launch_bounds__(256) fb_count_leaders_kernel(BuildView v) {
+    CB_PDL_ENTRY();
     __shared__ CountCache cache;
-    __shared__ Appender made;
+    __shared__ Appender<uint32_t> made;
     cache.clear();
     made.clear();
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    uint32_t mx = 0;
-    for (size_t i0 = (size_t)blockIdx.x * blockDim.x; i0 < v.M; i0 += stride) {
-        const size_t i = i0 + threadIdx.x;
-        uint32_t s = kEmpty;
-        bool created = false;
-        if (i < v.M) {
-            bool neg = false;
-            for (int j = 0; j < v.LL + v.FL; ++j) neg |= v.corpus[i + j] < 0;
-            if (neg) {
-                atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_INVALID_ARG);
-            } else {
-                for (int j = 0; j < v.LL; ++j) mx = max(mx, (uint32_t)v.corpus[i + j]);
-                s = find_or_claim(v.h1, v.S, v.corpus, (uint32_t)i, v.LL, &created);
-                if (s == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
-                else if (!created) cache.add(v.h1, s);
+    constexpr int U = 4;
+    const size_t stride = (size_t)gridDim.x * 256 * U;
+    const bool has_neg = v.st->has_neg != 0u;
+    for (size_t i0 = (size_t)blockIdx.x * 256 * U; i0 < v.M; i0 += stride) {
+        uint32_t s[U], pos[U];
+        bool ok[U], created[U];
+        int32_t key[U][LL], rep[U][LL];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const size_t i = i0 + q * 256 + threadIdx.x;
+            ok[q] = i < v.M;
+            created[q] = false;
+#pragma unroll
+            for (int j = 0; j < LL; ++j) key[q][j] = ok[q] ? v.corpus[i + j] : 0;
+        }
+        if (has_neg) {                                          // the windows with a negative token are left out
+#pragma unroll 1
+            for (int q = 0; q < U; ++q)
+                for (int j = 0; j < LL + v.FL && ok[q]; ++j) ok[q] = v.corpus[i0 + q * 256 + threadIdx.x + j] >= 0;
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            s[q] = home_slot(key[q], LL, v.S);
+            pos[q] = ok[q] ? *reinterpret_cast<const uint32_t*>(&v.h1[s[q]]) : kEmpty;
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q)
+#pragma unroll
+            for (int j = 0; j < LL; ++j) rep[q][j] = pos[q] != kEmpty ? v.corpus[pos[q] + j] : -1;
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const size_t i = i0 + q * 256 + threadIdx.x;
+            if (ok[q]) {
+                int32_t diff = 0;
+#pragma unroll
+                for (int j = 0; j < LL; ++j) diff |= rep[q][j] ^ key[q][j];
+                if (diff != 0)                                  // an empty slot or another key's
+                    s[q] = find_or_claim(v.h1, v.S, pos[q] == kEmpty ? s[q] : (s[q] + 1) & (v.S - 1), v.corpus, (uint32_t)i, LL, &created[q]);
+                if (s[q] == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
+                else if (!created[q]) cache.add(v.h1, s[q]);
             }
-            v.lslot[i] = s;
+            if (i < v.M) v.lslot[i] = ok[q] ? s[q] : kEmpty;
         }
         made.add(created, s, v.uniq, &v.st->n_uniq);
     }
     made.flush(v.uniq, &v.st->n_uniq);
-    mx = __reduce_max_sync(CB_FULL, mx);
-    if ((threadIdx.x & 31) == 0) atomicMax(&v.st->max_token, mx);
     cache.flush(v.h1);
 }
 
-// Word w of a leader's composite key: the count so that more comes first (counts are at most M < 2^cbits), then its tokens.
-__device__ __forceinline__ uint32_t sel_word(const BuildView& v, unsigned long long slot, int w, uint32_t cmask) {
-    return w == 0 ? cmask - (uint32_t)(slot >> 32) : (uint32_t)v.corpus[(uint32_t)slot + (w - 1)];
-}
+// ---------------------------------------------------------------------------------------------------
+// 2. Selection of the LC best leaders and what follows from it, as one cooperative launch: its steps are a few microseconds each
+// and every one needs the result of the one before (13 launches otherwise, for 60,000 tokens most of the build's time).
+constexpr int kSelThreads = 1024;
+struct SelSmem {
+    uint32_t bins[kBins], part[32], pick[2], last, cnt[33], start;
+    Appender<uint2> tied;
+};
 
-// The last block of a histogram pass picks the bin in which the k-th smallest key lies and clears the histogram.  Every thread of
-// the block gets the bin; *rest is the rank inside it.
-__device__ __forceinline__ uint32_t pick_bin(const BuildView& v, uint32_t k, uint32_t* s_part, uint32_t* s_pick, uint32_t* rest) {
-    constexpr int PER = kBins / 256;
-    uint32_t c[PER], sum = 0;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) { c[j] = __ldcg(&v.st->hist[threadIdx.x * PER + j]); sum += c[j]; v.st->hist[threadIdx.x * PER + j] = 0u; }
-    s_part[threadIdx.x] = sum;
-    __syncthreads();
-    for (int o = 1; o < 256; o <<= 1) {
-        const uint32_t add = (int)threadIdx.x >= o ? s_part[threadIdx.x - o] : 0u;
-        __syncthreads();
-        s_part[threadIdx.x] += add;
-        __syncthreads();
-    }
-    uint32_t cum = s_part[threadIdx.x] - sum;
-    if (cum < k && k <= cum + sum) {
-#pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            if (cum < k && k <= cum + c[j]) { s_pick[0] = (uint32_t)(threadIdx.x * PER + j); s_pick[1] = k - cum; }
-            cum += c[j];
-        }
-    }
-    __syncthreads();
-    *rest = s_pick[1];
-    return s_pick[0];
-}
-// All threads of a block: true in the block that comes last to this point of a launch.
-__device__ __forceinline__ bool last_block(const BuildView& v, uint32_t* s_last) {
-    __threadfence();
+// All blocks of the launch; false after a wait that ran out (recorded as CB_ERR_TIMEOUT; the others run out too).
+__device__ __forceinline__ bool grid_barrier(const BuildView& v, uint32_t* round, uint32_t* s_flag) {
     __syncthreads();
     if (threadIdx.x == 0) {
-        *s_last = atomicAdd(&v.st->arrived, 1u) == gridDim.x - 1u ? 1u : 0u;
-        if (*s_last) v.st->arrived = 0u;
+        *round += gridDim.x;
+        __threadfence();
+        atomicAdd(&v.st->arrived, 1u);
+        uint32_t ok = 0u;
+        for (uint32_t k = 0; k < (1u << 24) && !ok; ++k) {
+            uint32_t x;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(&v.st->arrived) : "memory");
+            ok = x >= *round ? 1u : 0u;
+        }
+        if (!ok) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_TIMEOUT);
+        *s_flag = ok;
     }
     __syncthreads();
-    __threadfence();
-    return *s_last != 0u;
+    return *s_flag != 0u;
 }
-// one shared atomic per warp and bin (most counts are 1); kEmpty: none
+__device__ __forceinline__ uint32_t sel_scan(uint32_t x, uint32_t* part, uint32_t* total) {   // exclusive, over the block
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(CB_FULL, incl, o);
+        if (lane >= o) incl += up;
+    }
+    __syncthreads();
+    if (lane == 31) part[warp] = incl;
+    __syncthreads();
+    uint32_t y = part[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(CB_FULL, y, o);
+        if (lane >= o) y += up;
+    }
+    *total = __shfl_sync(CB_FULL, y, 31);
+    const uint32_t before = __shfl_sync(CB_FULL, y, warp > 0 ? warp - 1 : 0);
+    return incl - x + (warp > 0 ? before : 0u);
+}
+// The bin of a finished histogram in which the k-th smallest key lies; *rest: its rank inside the bin.  Every block for itself.
+__device__ __forceinline__ uint32_t pick_bin(const uint32_t* hist, uint32_t k, SelSmem& S, uint32_t* rest) {
+    const uint4 c = __ldcg(reinterpret_cast<const uint4*>(hist) + threadIdx.x);      // four bins a thread
+    const uint32_t cs[4] = {c.x, c.y, c.z, c.w};
+    uint32_t total;
+    uint32_t cum = sel_scan(cs[0] + cs[1] + cs[2] + cs[3], S.part, &total);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (cum < k && k <= cum + cs[j]) { S.pick[0] = threadIdx.x * 4 + j; S.pick[1] = k - cum; }
+        cum += cs[j];
+    }
+    __syncthreads();
+    const uint32_t bin = S.pick[0];
+    *rest = S.pick[1];
+    __syncthreads();
+    return bin;
+}
+static_assert(kBins == 4 * kSelThreads, "four bins a thread");
+// Most counts are the same: the lanes with the first one's bin take one shared atomic, the others one each (__match_any_sync, for one
+// per bin, takes some 500 cycles).  kEmpty: none.
 __device__ __forceinline__ void add_bin(uint32_t* sh, uint32_t bin) {
-    const uint32_t peers = __match_any_sync(CB_FULL, bin);
-    if (bin != kEmpty && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&sh[bin], (uint32_t)__popc(peers));
+    const uint32_t some = __ballot_sync(CB_FULL, bin != kEmpty);
+    if (some == 0u) return;
+    const int head = __ffs(some) - 1;
+    const uint32_t with = __ballot_sync(CB_FULL, bin == __shfl_sync(CB_FULL, bin, head));
+    if ((int)(threadIdx.x & 31) == head) atomicAdd(&sh[bin], (uint32_t)__popc(with));
+    else if (bin != kEmpty && !((with >> (threadIdx.x & 31)) & 1u)) atomicAdd(&sh[bin], 1u);
 }
-
-// 2a. The count of the LC-th best leader, one pass where it is below 4,095: a bin per count, the last one for all above.
-__global__ void __launch_bounds__(256) fb_select_count_kernel(BuildView v, uint32_t cmask) {
-    __shared__ uint32_t sh[kBins];
-    __shared__ uint32_t s_last, s_part[256], s_pick[2];
-    const uint32_t n = v.st->n_uniq;
-    if (n <= (uint32_t)v.LC) return;          // all of them are taken
-    for (int i = threadIdx.x; i < kBins; i += 256) sh[i] = 0u;
+// Histogram of bin_of(i) over items [0, n) into hist; blocks without an item have nothing to clear and to add.
+template <typename F>
+__device__ __forceinline__ void sel_histogram(uint32_t n, uint32_t* hist, SelSmem& S, F&& bin_of) {
+    if (blockIdx.x * (uint32_t)kSelThreads >= n) return;
+    for (int i = threadIdx.x; i < kBins; i += kSelThreads) S.bins[i] = 0u;
     __syncthreads();
-    for (size_t i0 = (size_t)blockIdx.x * 256; i0 < n; i0 += (size_t)gridDim.x * 256) {
-        const size_t i = i0 + threadIdx.x;
-        add_bin(sh, i < n ? kBins - 1 - min((uint32_t)(v.h1[v.uniq[i]] >> 32), (uint32_t)(kBins - 1)) : kEmpty);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kBins; i += 256)
-        if (sh[i]) atomicAdd(&v.st->hist[i], sh[i]);
-    if (!last_block(v, &s_last)) return;
-    uint32_t rest;
-    const uint32_t bin = pick_bin(v, (uint32_t)v.LC, s_part, s_pick, &rest);
-    if (threadIdx.x == 0) {
-        v.st->k_rem = bin > 0u ? rest : (uint32_t)v.LC;
-        v.st->count_known = bin > 0u ? 1u : 0u;
-        v.st->prefix[0] = bin > 0u ? cmask - (kBins - 1 - bin) : 0u;
-    }
-}
-
-// 2b. Histogram of the digit at `shift` of word `w` over the leaders that match the prefix resolved so far; the last
-// block to finish picks the digit in which the k-th smallest composite key lies.  Word 0 goes over all leaders and only where
-// the pass above did not settle it, the tokens over the leaders that tie with its count; leading digits that are zero in
-// every token are passed over.
-__global__ void __launch_bounds__(256) fb_select_kernel(BuildView v, int w, int shift, uint32_t cmask) {
-    __shared__ uint32_t sh[kBins];
-    __shared__ uint32_t s_last, s_part[256], s_pick[2];
-    if (v.st->n_uniq <= (uint32_t)v.LC) return;
-    if (w == 0 && v.st->count_known) return;
-    if (w > 0 && shift > 0 && (v.st->max_token >> shift) == 0u) return;
-    const uint32_t n = w == 0 ? v.st->n_uniq : v.st->n_ties;
-    const uint32_t* const list = w == 0 ? v.uniq : v.ties;
-    for (int i = threadIdx.x; i < kBins; i += 256) sh[i] = 0u;
-    __syncthreads();
-    const uint32_t hi_mask = shift + kDigitBits >= 32 ? 0u : (0xFFFFFFFFu << (shift + kDigitBits));
-    uint32_t prefix[kMaxWords];
+    constexpr int U = 4;                                        // items of a thread whose look-ups overlap
+    const uint32_t step = gridDim.x * kSelThreads;
+    for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n; i0 += U * step) {
+        uint32_t bin[U];
 #pragma unroll
-    for (int k = 0; k < kMaxWords; ++k) prefix[k] = v.st->prefix[k];
-    for (size_t i0 = (size_t)blockIdx.x * 256; i0 < n; i0 += (size_t)gridDim.x * 256) {
-        const size_t i = i0 + threadIdx.x;
-        uint32_t bin = kEmpty;
-        if (i < n) {
-            const unsigned long long slot = v.h1[list[i]];
-            bool ok = true;
-            for (int k = 1; k < w && ok; ++k) ok = sel_word(v, slot, k, cmask) == prefix[k];
-            if (ok) {
-                const uint32_t x = sel_word(v, slot, w, cmask);
-                if ((x & hi_mask) == (prefix[w] & hi_mask)) bin = (x >> shift) & (kBins - 1);
-            }
+        for (int q = 0; q < U; ++q) {
+            const uint32_t i = i0 + q * step + threadIdx.x;
+            bin[q] = i < n ? bin_of(i) : kEmpty;
         }
-        add_bin(sh, bin);
+#pragma unroll
+        for (int q = 0; q < U; ++q) if (i0 + q * step < n) add_bin(S.bins, bin[q]);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kBins; i += 256)
-        if (sh[i]) atomicAdd(&v.st->hist[i], sh[i]);
-    if (!last_block(v, &s_last)) return;
-    uint32_t rest;
-    const uint32_t bin = pick_bin(v, v.st->k_rem, s_part, s_pick, &rest);
-    if (threadIdx.x == 0) { v.st->k_rem = rest; v.st->prefix[w] |= bin << shift; }
+    for (int i = threadIdx.x; i < kBins; i += kSelThreads)
+        if (S.bins[i]) atomicAdd(&hist[i], S.bins[i]);
 }
 
 // The leader in slot `at` of the first table gets the next entry (take; all threads of a block together, one atomic for all of
 // them); its key goes into the frozen table's index.
-__device__ __forceinline__ void place_leader(const BuildView& v, const CbTables& t, bool take, uint32_t at, unsigned long long slot, uint32_t* s_cnt /* [9] */) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t m = __ballot_sync(CB_FULL, take);
-    __syncthreads();
-    if (lane == 0) s_cnt[warp] = (uint32_t)__popc(m);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t total = 0;
-        for (int k = 0; k < 8; ++k) { const uint32_t c = s_cnt[k]; s_cnt[k] = total; total += c; }
-        s_cnt[8] = total ? atomicAdd(&v.st->n_sel, total) : 0u;
-    }
+__device__ __forceinline__ void place_leader(const BuildView& v, const CbTables& t, bool take, uint32_t at, unsigned long long slot, SelSmem& S) {
+    uint32_t total;
+    const uint32_t mine = sel_scan(take ? 1u : 0u, S.part, &total);
+    if (threadIdx.x == 0) S.start = total ? atomicAdd(&v.st->n_sel, total) : 0u;
     __syncthreads();
     if (!take) return;
-    const uint32_t eid = s_cnt[8] + s_cnt[warp] + __popc(m & ((1u << lane) - 1u));
-    if (eid >= (uint32_t)v.LC) { atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT); v.h1_eid[at] = -1; return; }
-    v.h1_eid[at] = (int32_t)eid;
+    const uint32_t eid = S.start + mine;
+    if (eid >= (uint32_t)v.LC) { atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT); return; }
+    *count_of(v.h1, at) = kTaken | eid;
     const int32_t* key = v.corpus + (uint32_t)slot;
     uint32_t* e = t.entries + (size_t)eid * t.E;
     int32_t k4[4] = {0, 0, 0, 0};
@@ -350,123 +396,216 @@ __device__ __forceinline__ void place_leader(const BuildView& v, const CbTables&
     atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
 }
 
-// 2c. the leaders with a larger count than the LC-th best are placed, those with the same count listed
-__global__ void __launch_bounds__(256) fb_place_leaders_kernel(BuildView v, CbTables t, uint32_t cmask) {
-    const uint32_t n = v.st->n_uniq;
-    const bool all = n <= (uint32_t)v.LC;
-    const uint32_t cut = cmask - v.st->prefix[0];
-    __shared__ uint32_t s_cnt[9];
-    __shared__ Appender tied;
-    tied.clear();
-    for (size_t i0 = (size_t)blockIdx.x * 256; i0 < n; i0 += (size_t)gridDim.x * 256) {
-        const size_t i = i0 + threadIdx.x;
-        bool take = false, tie = false;
-        uint32_t at = 0;
-        unsigned long long slot = 0;
-        if (i < n) {
-            at = v.uniq[i];
-            slot = v.h1[at];
-            take = all || (uint32_t)(slot >> 32) > cut;
-            tie = !take && (uint32_t)(slot >> 32) == cut;
-            if (!take) v.h1_eid[at] = -1;
-        }
-        tied.add(tie, at, v.ties, &v.st->n_ties);
-        place_leader(v, t, take, at, slot, s_cnt);
-    }
-    tied.flush(v.ties, &v.st->n_ties);
-    if (blockIdx.x == 0 && threadIdx.x == 0) t.hdr[1] = min(n, (uint32_t)v.LC);
-}
-// 2d. of the tied leaders those whose tokens come no later than the LC-th best's
-__global__ void __launch_bounds__(256) fb_place_ties_kernel(BuildView v, CbTables t, uint32_t cmask) {
-    const uint32_t n = v.st->n_ties;
-    __shared__ uint32_t s_cnt[9];
-    for (size_t i0 = (size_t)blockIdx.x * 256; i0 < n; i0 += (size_t)gridDim.x * 256) {
-        const size_t i = i0 + threadIdx.x;
-        bool take = i < n;
-        uint32_t at = 0;
-        unsigned long long slot = 0;
-        if (take) {
-            at = v.ties[i];
-            slot = v.h1[at];
-            for (int k = 1; k <= v.LL; ++k) {
-                const uint32_t x = sel_word(v, slot, k, cmask), y = v.st->prefix[k];
-                if (x != y) { take = x < y; break; }
+
+__global__ void __launch_bounds__(kSelThreads, 1) fb_select_kernel(BuildView v, CbTables t, int cbits) {
+    extern __shared__ __align__(16) unsigned char sel_smem[];
+    SelSmem& S = *reinterpret_cast<SelSmem*>(sel_smem);
+    const uint32_t n = v.st->n_uniq, LC = (uint32_t)v.LC, cmask = (1u << cbits) - 1u;
+    const bool all = n <= LC;                                   // all of them are taken
+    uint32_t round = 0, pass = 0, cut = 0, k = LC;
+    if (!all) {
+        // 2a. the count of the LC-th best leader: a bin per count below 4,095 (most comes first), the last one for all above
+        sel_histogram(n, v.st->hist[pass], S, [&](uint32_t i) { return kBins - 1 - min((uint32_t)(v.h1[v.uniq[i]] >> 32), (uint32_t)(kBins - 1)); });
+        if (!grid_barrier(v, &round, &S.last)) return;
+        uint32_t rest, bin = pick_bin(v.st->hist[pass++], k, S, &rest);
+        if (bin > 0u) {
+            cut = kBins - 1 - bin;
+            k = rest;
+        } else {
+            // 4,095 or more: digit by digit over the complemented count
+            uint32_t prefix = 0;
+            for (int shift = (cbits - 1) / kDigitBits * kDigitBits; shift >= 0; shift -= kDigitBits) {
+                const uint32_t hi_mask = shift + kDigitBits >= 32 ? 0u : (0xFFFFFFFFu << (shift + kDigitBits));
+                sel_histogram(n, v.st->hist[pass], S, [&](uint32_t i) {
+                    const uint32_t x = cmask - (uint32_t)(v.h1[v.uniq[i]] >> 32);
+                    return (x & hi_mask) == (prefix & hi_mask) ? (x >> shift) & (kBins - 1) : kEmpty;
+                });
+                if (!grid_barrier(v, &round, &S.last)) return;
+                bin = pick_bin(v.st->hist[pass++], k, S, &k);
+                prefix |= bin << shift;
             }
+            cut = cmask - prefix;
         }
-        place_leader(v, t, take, at, slot, s_cnt);
     }
+    // 2b. the leaders with a larger count are placed, those with the same count listed
+    S.tied.clear();
+    const uint32_t step = gridDim.x * kSelThreads;
+    for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n; i0 += 4 * step) {
+        uint32_t at[4];
+        unsigned long long slot[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) at[q] = i0 + q * step + threadIdx.x < n ? v.uniq[i0 + q * step + threadIdx.x] : 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) slot[q] = i0 + q * step + threadIdx.x < n ? v.h1[at[q]] : 0ull;
+#pragma unroll 1
+        for (int q = 0; q < 4 && i0 + q * step < n; ++q) {
+            const bool in = i0 + q * step + threadIdx.x < n;
+            const uint32_t a = q == 0 ? at[0] : q == 1 ? at[1] : q == 2 ? at[2] : at[3];
+            const unsigned long long x = q == 0 ? slot[0] : q == 1 ? slot[1] : q == 2 ? slot[2] : slot[3];
+            const bool take = in && (all || (uint32_t)(x >> 32) > cut);
+            const bool tie[1] = {in && !take && (uint32_t)(x >> 32) == cut};
+            const uint2 item[1] = {make_uint2(a, (uint32_t)x)};
+            S.tied.add(tie, item, v.ties, &v.st->n_ties);
+            place_leader(v, t, take, a, x, S);
+        }
+    }
+    S.tied.flush(v.ties, &v.st->n_ties);
+    if (blockIdx.x == 0 && threadIdx.x == 0) t.hdr[1] = min(n, LC);
+    if (!grid_barrier(v, &round, &S.last)) return;
+    if (!all) {
+        // 2c. of those the k first by tokens, digit by digit; leading digits that are zero in every token are passed over
+        const uint32_t n_ties = __ldcg(&v.st->n_ties);
+        uint32_t prefix[CB_MAX_LL] = {0u, 0u, 0u, 0u};
+        auto before_or_in = [&](uint32_t pos, int words) {      // -1, 0, 1: the leader's first words against the prefix
+            for (int j = 0; j < words; ++j) {
+                const uint32_t x = (uint32_t)v.corpus[pos + j];
+                if (x != prefix[j]) return x < prefix[j] ? -1 : 1;
+            }
+            return 0;
+        };
+        for (int w = 0; w < v.LL; ++w)
+            for (int shift = 24; shift >= 0; shift -= kDigitBits) {
+                if (shift > 0 && (v.st->max_token >> shift) == 0u) continue;
+                const uint32_t hi_mask = shift + kDigitBits >= 32 ? 0u : (0xFFFFFFFFu << (shift + kDigitBits));
+                sel_histogram(n_ties, v.st->hist[pass], S, [&](uint32_t i) {
+                    const uint32_t pos = __ldcg(&v.ties[i]).y;
+                    if (before_or_in(pos, w) != 0) return kEmpty;
+                    const uint32_t x = (uint32_t)v.corpus[pos + w];
+                    return (x & hi_mask) == (prefix[w] & hi_mask) ? (x >> shift) & (kBins - 1) : kEmpty;
+                });
+                if (!grid_barrier(v, &round, &S.last)) return;
+                const uint32_t bin = pick_bin(v.st->hist[pass++], k, S, &k);
+                prefix[w] |= bin << shift;
+            }
+        // 2d. placed like the others
+        for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n_ties; i0 += gridDim.x * kSelThreads) {
+            const uint32_t i = i0 + threadIdx.x;
+            const uint2 x = i < n_ties ? __ldcg(&v.ties[i]) : make_uint2(0u, 0u);
+            const bool take = i < n_ties && before_or_in(x.y, v.LL) <= 0;
+            place_leader(v, t, take, x.x, ((unsigned long long)cut << 32) | x.y, S);
+        }
+        if (!grid_barrier(v, &round, &S.last)) return;
+    }
+    // 3a. every selected leader takes a range (an atomic per block and 1,024 of them: their ranges lie side by side); those with more than
+    // 32 windows are listed by size
+    const uint32_t n_sel = min(__ldcg(&v.st->n_sel), LC);
+    for (uint32_t e0 = blockIdx.x * kSelThreads; e0 < n_sel; e0 += gridDim.x * kSelThreads) {
+        const uint32_t e = e0 + threadIdx.x, windows = e < n_sel ? __ldcg(&t.lstamp[e]) : 0u;
+        const bool big = windows > kBigGroup;
+        const uint32_t c = big ? 0u : windows;
+        uint32_t total;
+        const uint32_t before = sel_scan(c, S.part, &total);
+        if (threadIdx.x == 0) S.start = total ? atomicAdd(&v.st->cursor, total) : 0u;
+        // the most frequent of the listed kinds: an atomic per warp
+        const int lane = threadIdx.x & 31;
+        const bool by_warp = c > 32u && c <= kWarpGroup;
+        const uint32_t m = __ballot_sync(CB_FULL, by_warp);
+        uint32_t k2 = 0;
+        if (m && lane == 0) k2 = atomicAdd(&v.st->n_warp, (uint32_t)__popc(m));
+        k2 = __shfl_sync(CB_FULL, k2, 0) + __popc(m & ((1u << lane) - 1u));
+        if (by_warp) v.listed_big[v.LC - 1 - k2] = e;
+        __syncthreads();
+        if (big) {
+            v.grp_off[e] = kBigFlag | atomicAdd(&v.st->big_cursor, windows);   // no more distinct windows than windows
+            v.listed_big[atomicAdd(&v.st->n_big, 1u)] = e;
+        } else if (e < n_sel) {
+            v.grp_off[e] = S.start + before;
+            if (c > kMidGroup) v.listed[v.LC - 1 - atomicAdd(&v.st->n_large, 1u)] = e;
+            else if (c > kWarpGroup) v.listed[atomicAdd(&v.st->n_mid, 1u)] = e;
+        }
+    }
+    // 3b. the part of the second table that the big leaders' windows need
+    if (!grid_barrier(v, &round, &S.last)) return;
+    if (__ldcg(&v.st->n_big) == 0u) return;
+    const uint32_t S2 = big_slots(v);
+    ulonglong2* a = reinterpret_cast<ulonglong2*>(v.h2);
+    for (size_t i = (size_t)blockIdx.x * kSelThreads + threadIdx.x; i < S2 / 2; i += (size_t)gridDim.x * kSelThreads) a[i] = make_ulonglong2(kEmptySlot, kEmptySlot);
 }
 
-// 3a. follower counts of the selected leaders; a new window takes its ordinal in its leader's group
-__global__ void __launch_bounds__(256) fb_count_followers_kernel(BuildView v) {
+// 3c. every window of a selected leader goes into its leader's range; a big leader's window is counted in the second table, where a
+// new one takes its ordinal in its leader's group.  Four windows a thread, whose chains (leader slot, leader, place) overlap.
+__global__ void __launch_bounds__(256) fb_windows_kernel(BuildView v) {
+    CB_PDL_ENTRY();
     __shared__ CountCache cache;
-    cache.clear();
+    constexpr int U = 4;
+    const bool any_big = v.st->n_big != 0u;
+    const uint32_t S2 = any_big ? big_slots(v) : 0u;
+    if (any_big) cache.clear();
+    __shared__ Appender<uint2> big;
+    big.clear();
     const int lane = threadIdx.x & 31;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i0 = (size_t)blockIdx.x * blockDim.x; i0 < v.M; i0 += stride) {
-        const size_t i = i0 + threadIdx.x;
-        bool created = false;
-        uint32_t s = kEmpty;
-        int32_t eid = -1;
-        if (i < v.M) {
-            const uint32_t ls = v.lslot[i];
-            if (ls != kEmpty) eid = v.h1_eid[ls];
-            if (eid >= 0) {
-                s = find_or_claim(v.h2, v.S, v.corpus, (uint32_t)i, v.LL + v.FL, &created);
+    auto count_big = [&] {                                      // all threads of the block together
+        const uint32_t n = big.n;
+        for (uint32_t j0 = 0; j0 < n; j0 += blockDim.x) {
+            const uint32_t j = j0 + threadIdx.x;
+            const uint2 x = j < n ? big.item[j] : make_uint2(0u, 0u);
+            bool created = false;
+            uint32_t s = kEmpty;
+            if (j < n) {
+                s = find_or_claim(v.h2, S2, home_slot(v.corpus + x.x, v.LL + v.FL, S2), v.corpus, x.x, v.LL + v.FL, &created);
                 if (s == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
                 else if (!created) cache.add(v.h2, s);
             }
+            // the new windows of one leader in a warp take their ordinals with one atomic
+            if (__any_sync(CB_FULL, created)) {
+                const uint32_t peers = __match_any_sync(CB_FULL, created ? (int)x.y : -1 - lane);
+                const int head = __ffs(peers) - 1;
+                uint32_t o = 0;
+                if (created && lane == head) o = atomicAdd(&v.grp_n[x.y], (uint32_t)__popc(peers));
+                o = __shfl_sync(CB_FULL, o, head) + __popc(peers & ((1u << lane) - 1u));
+                if (created) v.h2_ord[s] = o;
+            }
         }
-        // the new windows of one leader in a warp take their ordinals with one atomic
-        if (__any_sync(CB_FULL, created)) {
-            const uint32_t peers = __match_any_sync(CB_FULL, created ? eid : -1 - lane);
-            const int head = __ffs(peers) - 1;
-            uint32_t at = 0;
-            if (created && lane == head) at = atomicAdd(&v.grp_n[eid], (uint32_t)__popc(peers));
-            at = __shfl_sync(CB_FULL, at, head) + __popc(peers & ((1u << lane) - 1u));
-            if (created) v.h2_ord[s] = at;
-        }
-    }
-    cache.flush(v.h2);
-}
-// 3b. every leader takes a range of the group array (an atomic per block of 256: their ranges lie side by side); the leaders with
-// more than 32 distinct windows are listed
-__global__ void __launch_bounds__(256) fb_group_ranges_kernel(BuildView v) {
-    const uint32_t n = min(v.st->n_sel, (uint32_t)v.LC);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __shared__ uint32_t s_tot[8], s_start;
-    for (uint32_t e0 = blockIdx.x * 256u; e0 < n; e0 += gridDim.x * 256u) {
-        const uint32_t e = e0 + threadIdx.x, c = e < n ? v.grp_n[e] : 0u;
-        uint32_t incl = c;
+        __syncthreads();
+        if (threadIdx.x == 0) big.n = 0u;
+        __syncthreads();
+    };
+    const size_t stride = (size_t)gridDim.x * blockDim.x * U;
+    for (size_t i0 = (size_t)blockIdx.x * blockDim.x * U; i0 < v.M; i0 += stride) {
+        uint32_t at[U], off[U];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t up = __shfl_up_sync(CB_FULL, incl, o);
-            if (lane >= o) incl += up;
+        for (int q = 0; q < U; ++q) {
+            const size_t i = i0 + (size_t)q * blockDim.x + threadIdx.x;
+            at[q] = i < v.M ? v.lslot[i] : kEmpty;
         }
-        if (lane == 31) s_tot[warp] = incl;
+#pragma unroll
+        for (int q = 0; q < U; ++q) at[q] = at[q] != kEmpty ? *count_of(v.h1, at[q]) : 0u;    // kTaken | entry id, or a count
+#pragma unroll
+        for (int q = 0; q < U; ++q) off[q] = (at[q] & kTaken) ? v.grp_off[at[q] & ~kTaken] : 0u;
+        uint32_t place[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) place[q] = (at[q] & kTaken) && !(off[q] & kBigFlag) ? atomicAdd(&v.grp_n[at[q] & ~kTaken], 1u) : 0u;
+#pragma unroll
+        for (int q = 0; q < U; ++q)
+            if ((at[q] & kTaken) && !(off[q] & kBigFlag)) v.wpos[off[q] + place[q]] = (uint32_t)(i0 + (size_t)q * blockDim.x + threadIdx.x);
+        if (!any_big) continue;
+        // The big leaders' windows are gathered and counted with full warps: they are a seventh of the windows here, some in every warp.
+        bool is_big[U];
+        uint2 item[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            is_big[q] = (at[q] & kTaken) && (off[q] & kBigFlag);
+            item[q] = make_uint2((uint32_t)(i0 + (size_t)q * blockDim.x + threadIdx.x), at[q] & ~kTaken);
+        }
+        if (big.gather(is_big, item)) count_big();
+    }
+    if (any_big) {
         __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t total = 0;
-            for (int k = 0; k < 8; ++k) { const uint32_t x = s_tot[k]; s_tot[k] = total; total += x; }
-            s_start = total ? atomicAdd(&v.st->cursor, total) : 0u;
-        }
-        __syncthreads();
-        if (e < n) {
-            v.grp_off[e] = s_start + s_tot[warp] + incl - c;
-            if (c > kMidGroup) v.listed[v.LC - 1 - atomicAdd(&v.st->n_big, 1u)] = e;
-            else if (c > 32) v.listed[atomicAdd(&v.st->n_mid, 1u)] = e;
-        }
-        __syncthreads();                                         // the shared words are rewritten by the next round
+        count_big();
+        cache.flush(v.h2);
     }
 }
-// 3c. the distinct windows, grouped by leader: position and count
+// 3d. the distinct windows of the big leaders, grouped by leader: position and count
 __global__ void __launch_bounds__(256) fb_group_scatter_kernel(BuildView v) {
+    CB_PDL_ENTRY();
+    if (v.st->n_big == 0u) return;
+    const uint32_t S2 = big_slots(v);
     const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x; s < v.S; s += stride) {
+    for (size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x; s < S2; s += stride) {
         const unsigned long long x = v.h2[s];
         if ((uint32_t)x == kEmpty) continue;
-        const int32_t eid = v.h1_eid[v.lslot[(uint32_t)x]];
-        v.group[v.grp_off[eid] + v.h2_ord[s]] = make_uint2((uint32_t)x, (uint32_t)(x >> 32));
+        const uint32_t eid = *count_of(v.h1, v.lslot[(uint32_t)x]) & ~kTaken;
+        v.group[(v.grp_off[eid] & ~kBigFlag) + v.h2_ord[s]] = make_uint2((uint32_t)x, (uint32_t)(x >> 32));
     }
 }
 
@@ -497,10 +636,23 @@ struct Candidates {
     }
 };
 
-template <int NT>
-__device__ void pick_followers(const BuildView& v, const CbTables& t, uint32_t eid, Candidates& cand, const Crew<NT>& crew) {
-    const uint32_t n = v.grp_n[eid];
-    const uint2* g = v.group + v.grp_off[eid];
+// The distinct windows of a leader: in memory (big leaders), or in shared memory (index of one occurrence + 1 and count in a word, the
+// occurrences' follower tokens).
+struct MemoryGroup {
+    const uint2* g; const int32_t* corpus; int LL;
+    __device__ __forceinline__ uint32_t count(uint32_t k) const { return g[k].y; }
+    __device__ __forceinline__ const int32_t* tokens(uint32_t k) const { return corpus + g[k].x + LL; }
+};
+struct SharedGroup {
+    const uint32_t* d; const int32_t* tok; int FL;
+    __device__ __forceinline__ uint32_t count(uint32_t k) const { return d[k] & 0xFFFFu; }
+    __device__ __forceinline__ const int32_t* tokens(uint32_t k) const { return tok + ((d[k] >> 16) - 1u) * FL; }
+};
+
+template <int NT, typename Group>
+__device__ void pick_followers(const BuildView& v, const CbTables& t, uint32_t eid, const Group& g, uint32_t n, Candidates& cand, const Crew<NT>& crew) {
+    // Ties are left in while ranking everything against everything is cheap: FC places and as many windows again, or 64.
+    const uint32_t few = (uint32_t)::max(2 * v.FC, 64);
     const int me = (int)threadIdx.x;
     uint32_t cmin = 1;                        // candidates have at least this count
     uint32_t ties = 0;                        // resolved tokens: candidates with exactly cmin come no later than lim[0 .. ties)
@@ -509,43 +661,43 @@ __device__ void pick_followers(const BuildView& v, const CbTables& t, uint32_t e
     if (n > (uint32_t)v.FC) {
         // the largest count that FC windows reach
         uint32_t top = 0;
-        for (uint32_t k = me; k < n; k += NT) top = ::max(top, g[k].y);
+        for (uint32_t k = me; k < n; k += NT) top = ::max(top, g.count(k));
         uint32_t lo = 1, hi = crew.max(top);
         have = n;
         while (lo < hi) {
             const uint32_t mid = lo + (hi - lo + 1u) / 2u;
             uint32_t c = 0;
-            for (uint32_t k = me; k < n; k += NT) c += g[k].y >= mid ? 1u : 0u;
+            for (uint32_t k = me; k < n; k += NT) c += g.count(k) >= mid ? 1u : 0u;
             c = crew.sum(c);
             if (c >= (uint32_t)v.FC) { lo = mid; have = c; } else hi = mid - 1u;
         }
         cmin = lo;
     }
-    if (have > (uint32_t)kCand) {
+    if (have > few) {
         // too many windows tie at that count: of those only the first by tokens, token by token, until the rest fits
         uint32_t above = 0;
-        for (uint32_t k = me; k < n; k += NT) above += g[k].y > cmin ? 1u : 0u;
+        for (uint32_t k = me; k < n; k += NT) above += g.count(k) > cmin ? 1u : 0u;
         uint32_t need = (uint32_t)v.FC - crew.sum(above);       // ties to be taken, at least one
-        for (int lev = 0; lev < v.FL && have > (uint32_t)kCand; ++lev) {
-            auto token = [&](const uint2& x, uint32_t* tok) {    // this level's token of a tie that matches the limits so far
-                if (x.y != cmin) return false;
-                const int32_t* f = v.corpus + x.x + v.LL;
+        for (int lev = 0; lev < v.FL && have > few; ++lev) {
+            auto token = [&](uint32_t k, uint32_t* tok) {         // this level's token of a tie that matches the limits so far
+                if (g.count(k) != cmin) return false;
+                const int32_t* f = g.tokens(k);
                 for (int j = 0; j < lev; ++j) if ((uint32_t)f[j] != lim[j]) return false;
                 *tok = (uint32_t)f[lev];
                 return true;
             };
             uint32_t top = 0, tok = 0;
-            for (uint32_t k = me; k < n; k += NT) if (token(g[k], &tok)) top = ::max(top, tok);
+            for (uint32_t k = me; k < n; k += NT) if (token(k, &tok)) top = ::max(top, tok);
             uint32_t lo = 0, hi = crew.max(top);                // the smallest token that `need` of them do not exceed
             while (lo < hi) {
                 const uint32_t mid = lo + (hi - lo) / 2u;
                 uint32_t c = 0;
-                for (uint32_t k = me; k < n; k += NT) c += token(g[k], &tok) && tok <= mid ? 1u : 0u;
+                for (uint32_t k = me; k < n; k += NT) c += token(k, &tok) && tok <= mid ? 1u : 0u;
                 if (crew.sum(c) >= need) hi = mid; else lo = mid + 1u;
             }
             uint32_t below = 0, equal = 0;
             for (uint32_t k = me; k < n; k += NT)
-                if (token(g[k], &tok)) { below += tok < lo ? 1u : 0u; equal += tok == lo ? 1u : 0u; }
+                if (token(k, &tok)) { below += tok < lo ? 1u : 0u; equal += tok == lo ? 1u : 0u; }
             lim[lev] = lo;
             ties = lev + 1;
             need -= crew.sum(below);
@@ -556,19 +708,19 @@ __device__ void pick_followers(const BuildView& v, const CbTables& t, uint32_t e
     if (me == 0) cand.n = 0u;
     __syncthreads();
     for (uint32_t k = me; k < n; k += NT) {
-        const uint2 x = g[k];
-        bool in = x.y > cmin;
-        if (x.y == cmin) {
+        const uint32_t c = g.count(k);
+        const int32_t* const f = g.tokens(k);
+        bool in = c > cmin;
+        if (c == cmin) {
             in = true;
-            const int32_t* f = v.corpus + x.x + v.LL;
             for (uint32_t j = 0; j < ties; ++j)
                 if ((uint32_t)f[j] != lim[j]) { in = (uint32_t)f[j] < lim[j]; break; }
         }
         if (in) {
             const uint32_t at = atomicAdd(&cand.n, 1u);
             if (at < (uint32_t)kCand) {
-                cand.cnt[at] = x.y;
-                for (int j = 0; j < v.FL; ++j) cand.tok[at * v.FL + j] = v.corpus[x.x + v.LL + j];
+                cand.cnt[at] = c;
+                for (int j = 0; j < v.FL; ++j) cand.tok[at * v.FL + j] = f[j];
             }
         }
     }
@@ -585,61 +737,316 @@ __device__ void pick_followers(const BuildView& v, const CbTables& t, uint32_t e
     __syncthreads();                                             // the candidates are overwritten by the next leader
 }
 
-// the common case, up to 32 distinct windows: a warp per leader; the next leader's group is looked up while this one is ranked
+// The five kernels of step 4 touch different leaders and depend on nothing but step 3, which is over when the first of them lets
+// the others start: so each of them starts as SMs become free and waits for the one before it only at its end (the stream's next
+// kernel is ordered behind the last of them only).
+__device__ __forceinline__ void fb_rank_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void fb_rank_end() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// the big leaders, a block each
+__global__ void __launch_bounds__(1024) fb_rank_big_kernel(BuildView v, CbTables t) {
+    CB_PDL_ENTRY();
+    __shared__ Candidates cand;
+    __shared__ uint32_t red[32];
+    const Crew<1024> crew = {red};
+    const uint32_t n = v.st->n_big;
+    for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
+        const uint32_t eid = v.listed_big[k];
+        const MemoryGroup g = {v.group + (v.grp_off[eid] & ~kBigFlag), v.corpus, v.LL};
+        pick_followers<1024>(v, t, eid, g, v.grp_n[eid], cand, crew);
+    }
+}
+
+// A block per leader with up to CAP windows: their follower tokens come into shared memory, the distinct ones and their counts are found
+// through a table there (a word per slot: index of the first claimant + 1, count).
+template <int NT, int CAP>
+__global__ void __launch_bounds__(NT) fb_rank_block_kernel(BuildView v, CbTables t, uint32_t n_leaders_at) {
+    fb_rank_begin();
+    extern __shared__ uint32_t fb_smem[];
+    uint32_t* const tab = fb_smem;                               // [2 CAP]
+    uint32_t* const dist = tab + 2 * CAP;                        // [CAP] distinct windows
+    int32_t* const tok = reinterpret_cast<int32_t*>(dist + CAP); // [CAP][FL]
+    __shared__ Candidates cand;
+    __shared__ uint32_t red[NT / 32], n_dist;
+    const Crew<NT> crew = {red};
+    const int me = (int)threadIdx.x, lane = me & 31;
+    const uint32_t n = n_leaders_at ? v.st->n_large : v.st->n_mid;
+    for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
+        const uint32_t eid = v.listed[n_leaders_at ? (uint32_t)v.LC - 1 - k : k], nw = v.grp_n[eid];
+        const uint32_t* const wp = v.wpos + v.grp_off[eid];
+        uint32_t slots = 64;                                     // a power of two, at least twice the windows
+        while (slots < 2u * nw) slots <<= 1;
+        for (uint32_t i = me; i < slots; i += NT) tab[i] = 0u;
+        if (me == 0) n_dist = 0u;
+        for (uint32_t i = me; i < nw; i += NT) {
+            const int32_t* f = v.corpus + wp[i] + v.LL;
+#pragma unroll
+            for (int j = 0; j < CB_MAX_FL; ++j) if (j < v.FL) tok[i * v.FL + j] = f[j];
+        }
+        __syncthreads();
+        for (uint32_t i = me; i < nw; i += NT) {
+            const int32_t* const f = tok + i * v.FL;
+            uint32_t x = 0x9E3779B9u;
+            for (int j = 0; j < v.FL; ++j) { x = (x ^ (uint32_t)f[j]) * 0x85EBCA77u; x ^= x >> 15; }
+            for (uint32_t p = 0, s = x & (slots - 1); p < slots; ++p, s = (s + 1) & (slots - 1)) {
+                uint32_t y = *reinterpret_cast<volatile uint32_t*>(&tab[s]);
+                if (y == 0u) {
+                    y = atomicCAS(&tab[s], 0u, ((i + 1u) << 16) | 1u);
+                    if (y == 0u) break;
+                }
+                const int32_t* const o = tok + ((y >> 16) - 1u) * v.FL;
+                int32_t diff = 0;
+                for (int j = 0; j < v.FL; ++j) diff |= o[j] ^ f[j];
+                if (diff == 0) { atomicAdd(&tab[s], 1u); break; }
+            }
+        }
+        __syncthreads();
+        for (uint32_t i0 = 0; i0 < slots; i0 += NT) {
+            const uint32_t i = i0 + me, y = i < slots ? tab[i] : 0u, m = __ballot_sync(CB_FULL, y != 0u);
+            uint32_t at = 0;
+            if (m && lane == 0) at = atomicAdd(&n_dist, (uint32_t)__popc(m));
+            at = __shfl_sync(CB_FULL, at, 0) + __popc(m & ((1u << lane) - 1u));
+            if (y) dist[at] = y;
+        }
+        __syncthreads();
+        const SharedGroup g = {dist, tok, v.FL};
+        pick_followers<NT>(v, t, eid, g, n_dist, cand, crew);    // ends with a barrier
+    }
+    fb_rank_end();
+}
+
+// Up to kWarpGroup windows, a warp per leader, four windows a lane: the same as the block kernel does with barriers, the warp's own
+// table in shared memory and the counts in registers.  A block of 128 threads took 12 us a leader.
+constexpr int kRankWarps = 8;
+__global__ void __launch_bounds__(32 * kRankWarps) fb_rank_warp_kernel(BuildView v, CbTables t) {
+    fb_rank_begin();
+    constexpr int PER = kWarpGroup / 32;
+    extern __shared__ uint32_t fb_smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t* const tab = fb_smem + warp * (kWarpGroup * (2 + v.FL));      // [2 kWarpGroup]: index of the first claimant + 1, count
+    int32_t* const tok = reinterpret_cast<int32_t*>(tab + 2 * kWarpGroup); // [kWarpGroup][FL]
+    const uint32_t n = v.st->n_warp, below = (1u << lane) - 1u;
+    for (uint32_t k = blockIdx.x * kRankWarps + warp; k < n; k += gridDim.x * kRankWarps) {
+        const uint32_t eid = v.listed_big[(uint32_t)v.LC - 1 - k], nw = v.grp_n[eid];
+        const uint32_t* const wp = v.wpos + v.grp_off[eid];
+        uint32_t pos[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) pos[q] = q * 32 + lane < nw ? wp[q * 32 + lane] : 0u;
+#pragma unroll
+        for (int q = 0; q < 2 * PER; ++q) tab[q * 32 + lane] = 0u;
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+            if (q * 32 + lane < nw) {
+                const int32_t* f = v.corpus + pos[q] + v.LL;
+#pragma unroll
+                for (int j = 0; j < CB_MAX_FL; ++j) if (j < v.FL) tok[(q * 32 + lane) * v.FL + j] = f[j];
+            }
+        __syncwarp();
+#pragma unroll 1
+        for (uint32_t i = lane; i < nw; i += 32) {
+            const int32_t* const f = tok + i * v.FL;
+            uint32_t x = 0x9E3779B9u;
+            for (int j = 0; j < v.FL; ++j) { x = (x ^ (uint32_t)f[j]) * 0x85EBCA77u; x ^= x >> 15; }
+            for (uint32_t p = 0, s = x & (2 * kWarpGroup - 1); p < 2 * kWarpGroup; ++p, s = (s + 1) & (2 * kWarpGroup - 1)) {
+                uint32_t y = *reinterpret_cast<volatile uint32_t*>(&tab[s]);
+                if (y == 0u) {
+                    y = atomicCAS(&tab[s], 0u, ((i + 1u) << 16) | 1u);
+                    if (y == 0u) break;
+                }
+                const int32_t* const o = tok + ((y >> 16) - 1u) * v.FL;
+                int32_t diff = 0;
+                for (int j = 0; j < v.FL; ++j) diff |= o[j] ^ f[j];
+                if (diff == 0) { atomicAdd(&tab[s], 1u); break; }
+            }
+        }
+        __syncwarp();
+        // the distinct ones to the front of the table (a slot is read before its group of 32 or an earlier one is written)
+        uint32_t nd = 0;
+#pragma unroll
+        for (int q = 0; q < 2 * PER; ++q) {
+            const uint32_t y = tab[q * 32 + lane], m = __ballot_sync(CB_FULL, y != 0u);
+            __syncwarp();
+            if (y) tab[nd + __popc(m & below)] = y;
+            nd += (uint32_t)__popc(m);
+            __syncwarp();
+        }
+        uint32_t cnt[PER];
+        const int32_t* f[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const uint32_t y = q * 32 + lane < nd ? tab[q * 32 + lane] : 0u;
+            cnt[q] = y & 0xFFFFu;
+            f[q] = tok + (y ? (y >> 16) - 1u : 0u) * v.FL;
+        }
+        // in[q]: among the FC best.  First the largest count that FC of them reach, then the ties at it token by token.
+        bool in[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) in[q] = cnt[q] > 0u;
+        if (nd > (uint32_t)v.FC) {
+            auto sum = [&](auto&& has) {
+                uint32_t c = 0;
+#pragma unroll
+                for (int q = 0; q < PER; ++q) c += (uint32_t)__popc(__ballot_sync(CB_FULL, has(q)));
+                return c;
+            };
+            uint32_t top = 0;
+#pragma unroll
+            for (int q = 0; q < PER; ++q) top = max(top, cnt[q]);
+            uint32_t lo = 1, hi = __reduce_max_sync(CB_FULL, top);
+            while (lo < hi) {
+                const uint32_t mid = lo + (hi - lo + 1u) / 2u;
+                if (sum([&](int q) { return cnt[q] >= mid; }) >= (uint32_t)v.FC) lo = mid; else hi = mid - 1u;
+            }
+            uint32_t need = (uint32_t)v.FC - sum([&](int q) { return cnt[q] > lo; });   // ties to be taken, at least one
+            bool tie[PER];
+#pragma unroll
+            for (int q = 0; q < PER; ++q) { in[q] = cnt[q] > lo; tie[q] = cnt[q] == lo; }
+            // the ties with the smallest first token, then the next ones; where one token has too many, those by their next token
+            for (int lev = 0; lev < v.FL && sum([&](int q) { return tie[q]; }) > need; ++lev) {
+                uint32_t x[PER], least = 0u, many = 0u;
+#pragma unroll
+                for (int q = 0; q < PER; ++q) x[q] = tie[q] ? (uint32_t)f[q][lev] : 0xFFFFFFFFu;
+                for (uint32_t got = 0u;;) {                      // at most FC rounds: each takes one tie or more
+                    uint32_t mn = 0xFFFFFFFFu;
+#pragma unroll
+                    for (int q = 0; q < PER; ++q) mn = min(mn, x[q]);
+                    least = __reduce_min_sync(CB_FULL, mn);
+                    many = sum([&](int q) { return x[q] == least; });
+                    if (got + many >= need) { need -= got; break; }
+                    got += many;
+#pragma unroll
+                    for (int q = 0; q < PER; ++q) if (x[q] == least) { in[q] = true; x[q] = 0xFFFFFFFFu; }
+                }
+#pragma unroll
+                for (int q = 0; q < PER; ++q) tie[q] = x[q] == least;
+            }
+#pragma unroll
+            for (int q = 0; q < PER; ++q) in[q] = in[q] || tie[q];
+        }
+        // those that are in, side by side at the front of the table, and each one's rank among them
+        __syncwarp();
+        uint32_t ni = 0;
+        uint32_t keep[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) keep[q] = q * 32 + lane < nd ? tab[q * 32 + lane] : 0u;
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const uint32_t m = __ballot_sync(CB_FULL, in[q]);
+            if (in[q]) tab[ni + __popc(m & below)] = keep[q];
+            ni += (uint32_t)__popc(m);
+        }
+        __syncwarp();
+        uint32_t* e = t.entries + (size_t)eid * t.E;
+        for (uint32_t i = lane; i < ni; i += 32) {
+            const uint32_t y = tab[i];
+            const int32_t* const g = tok + ((y >> 16) - 1u) * v.FL;
+            uint32_t rank = 0;
+            for (uint32_t o = 0; o < ni; ++o) {
+                const uint32_t z = tab[o];
+                bool before = (z & 0xFFFFu) > (y & 0xFFFFu);
+                if ((z & 0xFFFFu) == (y & 0xFFFFu)) {
+                    const int32_t* const h = tok + ((z >> 16) - 1u) * v.FL;
+                    for (int j = 0; j < v.FL; ++j)
+                        if (h[j] != g[j]) { before = h[j] < g[j]; break; }
+                }
+                rank += before ? 1u : 0u;
+            }
+            for (int j = 0; j < v.FL; ++j) e[v.LL + v.FC + rank * v.FL + j] = (uint32_t)g[j];
+            e[v.LL + rank] = (uint32_t)v.FC - rank;
+        }
+        __syncwarp();                                           // the table is overwritten by the next leader
+    }
+    fb_rank_end();
+}
+
+// the common case, up to 32 windows: a warp per leader, a lane per window; the next leader's range is looked up while this one is ranked
 __global__ void __launch_bounds__(256) fb_rank_kernel(BuildView v, CbTables t) {
+    fb_rank_begin();
     const int lane = threadIdx.x & 31;
     const uint32_t n = min(v.st->n_sel, (uint32_t)v.LC), nw = gridDim.x * 8;
+    const bool short_tokens = v.st->max_token < (1u << 26);
     uint32_t eid = blockIdx.x * 8 + (threadIdx.x >> 5);
-    uint32_t ng_next = eid < n ? v.grp_n[eid] : 0u, off_next = eid < n ? v.grp_off[eid] : 0u;
+    // windows of leader e for this warp (0: another kernel's) and this lane's position
+    auto range_of = [&](uint32_t e, uint32_t* pos) {
+        const uint32_t c = e < n ? t.lstamp[e] : 0u, off = e < n ? v.grp_off[e] : 0u;
+        *pos = 0u;
+        if (c == 0u || c > 32u) return 0u;
+        if ((uint32_t)lane < c) *pos = v.wpos[off + lane];
+        return c;
+    };
+    uint32_t pos_next, ng_next = range_of(eid, &pos_next);
     for (; eid < n; eid += nw) {
-        const uint32_t ng = ng_next, off = off_next;
-        if (eid + nw < n) { ng_next = v.grp_n[eid + nw]; off_next = v.grp_off[eid + nw]; }
-        if (ng > 32) continue;
-        // a lane per window, ranked against one another by shuffles
-        uint2 x = make_uint2(0u, 0u);
+        const uint32_t ng = ng_next, pos = pos_next;
+        const bool mine = (uint32_t)lane < ng;
         int32_t f[CB_MAX_FL];
 #pragma unroll
-        for (int j = 0; j < CB_MAX_FL; ++j) f[j] = 0;
-        if ((uint32_t)lane < ng) {
-            x = v.group[off + lane];
+        for (int j = 0; j < CB_MAX_FL; ++j) f[j] = mine && j < v.FL ? v.corpus[pos + v.LL + j] : -1 - lane;
+        ng_next = range_of(eid + nw, &pos_next);
+        if (ng == 0u) continue;
+        // the lanes with the same follower: its count; the first of them stands for it.  Compared by a hash, the hash by the tokens
+        // (__match_any_sync on each token instead held every warp of an SM up for some 500 cycles a call).
+        uint32_t x = 0x9E3779B9u;
 #pragma unroll
-            for (int j = 0; j < CB_MAX_FL; ++j) if (j < v.FL) f[j] = v.corpus[x.x + v.LL + j];
-        }
-        int rank = 0;
-        for (uint32_t k = 0; k < ng; ++k) {
-            const uint32_t oc = __shfl_sync(CB_FULL, x.y, k);
-            int cmp = oc > x.y ? -1 : (oc < x.y ? 1 : 0);        // -1: the other one comes before
+        for (int j = 0; j < CB_MAX_FL; ++j) { if (j >= v.FL) break; x = (x ^ (uint32_t)f[j]) * 0x85EBCA77u; x ^= x >> 15; }
+        uint32_t same = 0u;
+        for (uint32_t k = 0; k < ng; ++k) same |= (__shfl_sync(CB_FULL, x, k) == x ? 1u : 0u) << k;
+        const int rep = mine ? __ffs(same) - 1 : lane;
+        bool differ = false;
 #pragma unroll
-            for (int j = 0; j < CB_MAX_FL; ++j) {
-                if (j >= v.FL) break;
-                const int32_t o = __shfl_sync(CB_FULL, f[j], k);
-                if (cmp == 0 && o != f[j]) cmp = o < f[j] ? -1 : 1;
+        for (int j = 0; j < CB_MAX_FL; ++j) { if (j >= v.FL) break; differ = __shfl_sync(CB_FULL, f[j], rep) != f[j] || differ; }
+        if (__any_sync(CB_FULL, differ)) {                      // two followers with one hash: token by token
+            same = 0u;
+            for (uint32_t k = 0; k < ng; ++k) {
+                bool eq = true;
+#pragma unroll
+                for (int j = 0; j < CB_MAX_FL; ++j) { if (j >= v.FL) break; eq = __shfl_sync(CB_FULL, f[j], k) == f[j] && eq; }
+                same |= (eq ? 1u : 0u) << k;
             }
-            rank += cmp < 0 ? 1 : 0;
         }
-        if ((uint32_t)lane < ng && rank < v.FC) {
+        const uint32_t cnt = (uint32_t)__popc(same);
+        const bool stands = mine && (same & ((1u << lane) - 1u)) == 0u;
+        const uint32_t standing = __ballot_sync(CB_FULL, stands);
+        // Count and first token in one word (smaller comes first): four instructions for each of the others where the loop below, for two
+        // followers with the same word, takes twenty.
+        const uint32_t key = (32u - cnt) << 26 | (uint32_t)f[0];
+        int rank = 0, alike = 0;
+        if (short_tokens)
+            for (uint32_t m = standing; m; m &= m - 1u) {
+                const uint32_t o = __shfl_sync(CB_FULL, key, __ffs(m) - 1);
+                rank += o < key ? 1 : 0;
+                alike += o == key ? 1 : 0;
+            }
+        if (!short_tokens || __any_sync(CB_FULL, stands && alike > 1)) {
+            rank = 0;
+            for (uint32_t m = standing; m; m &= m - 1u) {
+                const int k = __ffs(m) - 1;
+                const uint32_t oc = __shfl_sync(CB_FULL, cnt, k);
+                int cmp = oc > cnt ? -1 : (oc < cnt ? 1 : 0);    // -1: the other one comes before
+#pragma unroll
+                for (int j = 0; j < CB_MAX_FL; ++j) {
+                    if (j >= v.FL) break;
+                    const int32_t o = __shfl_sync(CB_FULL, f[j], k);
+                    if (cmp == 0 && o != f[j]) cmp = o < f[j] ? -1 : 1;
+                }
+                rank += cmp < 0 ? 1 : 0;
+            }
+        }
+        if (stands && rank < v.FC) {
             uint32_t* e = t.entries + (size_t)eid * t.E;
 #pragma unroll
             for (int j = 0; j < CB_MAX_FL; ++j) if (j < v.FL) e[v.LL + v.FC + rank * v.FL + j] = (uint32_t)f[j];
             e[v.LL + rank] = (uint32_t)(v.FC - rank);
         }
     }
-}
-// the others, a block per leader: NT = 128 up to kMidGroup distinct windows, 1,024 above
-template <int NT>
-__global__ void __launch_bounds__(NT) fb_rank_listed_kernel(BuildView v, CbTables t) {
-    __shared__ Candidates cand;
-    __shared__ uint32_t red[NT / 32];
-    const Crew<NT> crew = {red};
-    const uint32_t n = NT == 1024 ? v.st->n_big : v.st->n_mid;
-    for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) pick_followers<NT>(v, t, v.listed[NT == 1024 ? (uint32_t)v.LC - 1 - k : k], cand, crew);
+    fb_rank_end();
 }
 
 size_t fb_align(size_t x) { return (x + 255) / 256 * 256; }
 
 struct BuildLayout {
     uint32_t S;
-    size_t off_h1, off_h1_eid, off_h2, off_h2_ord, off_lslot, off_group, off_grp, total;
+    size_t off_h1, off_h2, off_h2_ord, off_lslot, off_group, off_grp, total;
 };
 
 cb_status fb_layout(const cb_frozen_config* c, int64_t n_tokens, BuildLayout* B) {
@@ -650,12 +1057,11 @@ cb_status fb_layout(const cb_frozen_config* c, int64_t n_tokens, BuildLayout* B)
     B->S = (uint32_t)S;
     size_t o = fb_align(sizeof(BuildState));
     B->off_h1 = o;      o = fb_align(o + S * 8);
-    B->off_h1_eid = o;  o = fb_align(o + S * 4);
     B->off_h2 = o;      o = fb_align(o + S * 8);
     B->off_h2_ord = o;  o = fb_align(o + S * 4);
     B->off_lslot = o;   o = fb_align(o + (size_t)(M > 0 ? M : 1) * 4);
-    B->off_group = o;   o = fb_align(o + S * 8);
-    B->off_grp = o;     o = fb_align(o + (size_t)c->LC * 4 * 3);
+    B->off_group = o;   o = fb_align(o + S * 6);   // M x 8 bytes, then M x 4
+    B->off_grp = o;     o = fb_align(o + (size_t)c->LC * 4 * 4);
     B->total = o;
     return CB_OK;
 }
@@ -690,46 +1096,59 @@ extern "C" cb_status cb_frozen_build(const cb_frozen_config* cfg, const int32_t*
     char* base = (char*)dev_scratch;
     BuildView v;
     v.st = (BuildState*)base;
-    v.h1 = (unsigned long long*)(base + B.off_h1); v.h1_eid = (int32_t*)(base + B.off_h1_eid);
+    v.h1 = (unsigned long long*)(base + B.off_h1);
     v.h2 = (unsigned long long*)(base + B.off_h2); v.h2_ord = (uint32_t*)(base + B.off_h2_ord);
     v.lslot = (uint32_t*)(base + B.off_lslot);
-    v.group = (uint2*)(base + B.off_group); v.uniq = (uint32_t*)(base + B.off_group); v.ties = v.uniq + B.S / 2;   // M <= S / 2
+    v.group = (uint2*)(base + B.off_group); v.uniq = (uint32_t*)(base + B.off_group); v.ties = (uint2*)(v.uniq + B.S / 2);   // M <= S / 2
+    v.wpos = (uint32_t*)(v.group + B.S / 2);                      // behind group's M places
     v.grp_n = (uint32_t*)(base + B.off_grp); v.grp_off = v.grp_n + cfg->LC; v.listed = v.grp_off + cfg->LC;
+    v.listed_big = v.listed + cfg->LC;
     v.S = B.S;
     v.corpus = dev_corpus;
     const int64_t M = n_tokens - cfg->LL - cfg->FL + 1;
     v.M = (uint32_t)(M > 0 ? M : 0);
+    v.n_tokens = (uint32_t)n_tokens;
     v.LL = cfg->LL; v.FL = cfg->FL; v.LC = cfg->LC; v.FC = cfg->FC;
     int dev = 0, sms = 0;
     CB_CUDA(cudaGetDevice(&dev));
     CB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const dim3 grid((unsigned)(sms * 8)), block(256);
-    fb_init_kernel<<<grid, block, 0, st>>>(v, t);
+    CB_CUDA(cudaMemsetAsync(v.st, 0, sizeof(BuildState), st));
+    CB_CUDA(cb_launch_pdl(fb_init_kernel, grid, block, 0, st, v, t));
     if (v.M > 0) {
+        // shared memory of step 4's blocks: table, distinct windows, follower tokens
+        auto block_smem = [&](uint32_t cap) { return (size_t)(3 + cfg->FL) * cap * 4; };
+        auto* const mid = fb_rank_block_kernel<128, kMidGroup>;
+        auto* const large = fb_rank_block_kernel<512, kBigGroup>;
+        CB_CUDA(cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(3 + CB_MAX_FL) * kBigGroup * 4));
         int cbits = 1;                                        // counts are at most M
         while (cbits < 31 && (v.M >> cbits) != 0) ++cbits;
-        const uint32_t cmask = (1u << cbits) - 1u;
-        int passes = 0;
-        auto select = [&](int w, int bits) {
-            for (int shift = (bits - 1) / kDigitBits * kDigitBits; shift >= 0; shift -= kDigitBits, ++passes)
-                fb_select_kernel<<<grid, block, 0, st>>>(v, w, shift, cmask);
-        };
-        fb_count_leaders_kernel<<<grid, block, 0, st>>>(v);
-        fb_select_count_kernel<<<grid, block, 0, st>>>(v, cmask);
-        if (cbits > kDigitBits) select(0, cbits);             // counts of 4,095 and more can occur
-        fb_place_leaders_kernel<<<grid, block, 0, st>>>(v, t, cmask);
-        for (int w = 1; w <= cfg->LL; ++w) select(w, 31);
-        fb_place_ties_kernel<<<grid, block, 0, st>>>(v, t, cmask);
-        fb_count_followers_kernel<<<grid, block, 0, st>>>(v);
-        fb_group_ranges_kernel<<<dim3((unsigned)std::min(4 * sms, (cfg->LC + 255) / 256)), block, 0, st>>>(v);
-        fb_group_scatter_kernel<<<grid, block, 0, st>>>(v);
-        fb_rank_kernel<<<grid, block, 0, st>>>(v, t);
-        fb_rank_listed_kernel<128><<<dim3((unsigned)(sms * 8)), dim3(128), 0, st>>>(v, t);
-        fb_rank_listed_kernel<1024><<<dim3((unsigned)sms), dim3(1024), 0, st>>>(v, t);
-        cb_count_launch(10 + passes);
+        CB_CUDA(cudaFuncSetAttribute(fb_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SelSmem)));
+        static_assert(CB_MAX_LL == 4, "a leader count for every leader length");
+        auto* const count = cfg->LL == 1 ? fb_count_leaders_kernel<1> : cfg->LL == 2 ? fb_count_leaders_kernel<2>
+                            : cfg->LL == 3 ? fb_count_leaders_kernel<3> : fb_count_leaders_kernel<4>;
+        CB_CUDA(cb_launch_pdl(count, grid, block, 0, st, v));
+        {
+            // a block per SM, all resident at once: they wait for one another
+            cudaLaunchConfig_t lc = {};
+            lc.gridDim = dim3((unsigned)sms); lc.blockDim = dim3(kSelThreads); lc.dynamicSmemBytes = sizeof(SelSmem); lc.stream = st;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeCooperative;
+            at[0].val.cooperative = 1;
+            lc.attrs = at; lc.numAttrs = 1;
+            CB_CUDA(cudaLaunchKernelEx(&lc, fb_select_kernel, v, t, cbits));
+        }
+        CB_CUDA(cb_launch_pdl(fb_windows_kernel, grid, block, 0, st, v));
+        CB_CUDA(cb_launch_pdl(fb_group_scatter_kernel, grid, block, 0, st, v));
+        CB_CUDA(cb_launch_pdl(fb_rank_big_kernel, dim3((unsigned)sms), dim3(1024), 0, st, v, t));
+        CB_CUDA(cb_launch_pdl(large, dim3((unsigned)sms), dim3(512), block_smem(kBigGroup), st, v, t, 1u));
+        CB_CUDA(cb_launch_pdl(mid, dim3((unsigned)(sms * 8)), dim3(128), block_smem(kMidGroup), st, v, t, 0u));
+        const size_t warp_smem = (size_t)kRankWarps * kWarpGroup * (2 + cfg->FL) * 4;
+        CB_CUDA(cb_launch_pdl(fb_rank_warp_kernel, dim3((unsigned)(sms * 8)), dim3(32 * kRankWarps), warp_smem, st, v, t));
+        CB_CUDA(cb_launch_pdl(fb_rank_kernel, grid, block, 0, st, v, t));
+        cb_count_launch(9);
     }
     cb_count_launch(1);
-    CB_CUDA(cudaGetLastError());
     uint32_t status = 0;
     CB_CUDA(cudaMemcpyAsync(&status, &v.st->status, 4, cudaMemcpyDeviceToHost, st));
     CB_CUDA(cudaStreamSynchronize(st));

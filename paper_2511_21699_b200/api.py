@@ -39,18 +39,23 @@ def _stream(stream):
 _BOUND = ("cb_reset", "cb_update", "cb_update_bulk", "cb_draft_tree", "cb_update_draft_tree", "cb_tree_attn", "cb_accept",
           "cb_accept_update_draft_tree", "cb_kv_commit", "cb_status_str")
 _host_module = None
+try:                                     # loaded with the package (some 40 ms), not by the first context; not there yet while it is built
+    from . import _binding
+except ImportError:
+    _binding = None
 
 
 def _host():
     """The module _binding, calling the build of the library that _lib.load() chose."""
-    global _host_module
+    global _host_module, _binding
     if _host_module is None:
         lib = _lib.load()
-        try:
-            from . import _binding
-        except ImportError as e:
-            raise RuntimeError("_binding.so is not built or does not fit this torch (%s). Run `python -m paper_2511_21699_b200.build` "
-                               "or __graft_entry__.build(); there is no fallback path." % e) from e
+        if _binding is None:
+            try:
+                from . import _binding
+            except ImportError as e:
+                raise RuntimeError("_binding.so is not built or does not fit this torch (%s). Run `python -m paper_2511_21699_b200.build` "
+                                   "or __graft_entry__.build(); there is no fallback path." % e) from e
         _binding.set_library(CachebackError, {n: C.cast(getattr(lib, n), C.c_void_p).value for n in _BOUND})
         _host_module = _binding
     return _host_module

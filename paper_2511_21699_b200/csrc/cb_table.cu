@@ -582,25 +582,26 @@ namespace {
 // ---------------------------------------------------------------------------------------------------
 // Draft-tree expansion: one CTA per sequence, one warp per frontier leaf ("branch") for the lookups.
 // Each level: (1) warps look up the keys of all frontier leaves in parallel and stage the followers,
-// most recent first, in shared memory; (2) one thread replays the sequential breadth-first order over
+// most recent first, in shared memory; (2) one warp plans the sequential breadth-first order over
 // the staged results, which fixes node indices, the point where the size cap ends the level and the
-// ordinal of every query that the sequential order would have issued; (3) the leaders of those queries
-// get their new recency stamp with an atomic max (two leaves of one level may share a leader).
+// ordinal of every query that the sequential order would have issued, and gives the leaders of those queries
+// their new recency stamp with an atomic max (two leaves of one level may share a leader); (3) warps attach the nodes.
 // With a frozen table attached (Section 3.3) a second pass follows while the tree is below the size cap: its first
 // frontier is every node that was a frontier leaf of the first pass, in creation order, and its lookups go to the
 // frozen table, which is shared by all sequences and only read (no clock tick, no stamp).
 // A node goes to the output arrays when it is attached, its mask row being its leaf's plus a run of bits.  A level of one leaf (the
 // first one always is) is looked up, planned and filled in by one warp without a barrier.
-constexpr int kSerialLeaves = 16;
 // x / d = x * kInverse[d] >> 16 for d <= CB_MAX_FL and the x that occur here (below 1,024): a division is a chain of 100 cycles
 __constant__ uint32_t kInverse[CB_MAX_FL + 1] = {0u, 65537u, 32769u, 21846u, 16385u, 13108u, 10923u, 9363u, 8193u};
 struct DraftSmem {
     int32_t* tok; int32_t* par; int32_t* dep; uint32_t* mask;
     int32_t* front; int32_t* next; int32_t* pts;
-    int32_t* r_eid; int32_t* r_nf; int32_t* r_ok; uint32_t* r_stamp;
-    int32_t* r_n0; int32_t* r_cl; int32_t* r_tot; int32_t* r_nn0;     // plan of a leaf's attachment: first node, chain length, nodes, first frontier place
+    int32_t* r_eid;        // [NL each, by place in the frontier] the leader's entry
+    uint32_t* r_want;      // nodes that the leaf's followers would take | queried << 12 | found << 13 | nodes per follower << 16
+    uint32_t* r_plan;      // first node | nodes << 8 | first place in the next frontier << 16 | nodes per follower << 24
     int32_t* fol;
 };
+constexpr int kDraftArrays = 6;                               // of NL words
 
 // The work of the CTA that drafts sequence b, whose history holds L tokens.  upd_n_old >= 0: the windows that the tokens
 // from upd_n_old on complete are inserted first (cb_update_draft_tree and the call that follows an acceptance).  row(i): token i of
@@ -616,10 +617,12 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
     const int W = (T + 31) >> 5;
     S.tok = smem; S.par = S.tok + T; S.dep = S.par + T; S.mask = (uint32_t*)(S.dep + T);
     S.front = (int32_t*)(S.mask + T * W); S.next = S.front + NL; S.pts = S.next + NL;
-    S.r_eid = S.pts + NL; S.r_nf = S.r_eid + NL; S.r_ok = S.r_nf + NL; S.r_stamp = (uint32_t*)(S.r_ok + NL);
-    S.r_n0 = (int32_t*)(S.r_stamp + NL); S.r_cl = S.r_n0 + NL; S.r_tot = S.r_cl + NL; S.r_nn0 = S.r_tot + NL;
-    S.fol = S.r_nn0 + NL;
-    __shared__ int sh_n, sh_nfront, sh_nnext, sh_npts, sh_q, sh_hits, sh_fq, sh_fhits;
+    S.r_eid = S.pts + NL; S.r_want = (uint32_t*)(S.r_eid + NL); S.r_plan = S.r_want + NL;
+    S.fol = (int32_t*)(S.r_plan + NL);
+    // Nodes, leaves of the level's frontier, leaves listed for the frozen pass: a level reads one set and leaves the other for the next
+    // level, so that a barrier at its end is all that lies between two levels.
+    __shared__ int sh_n[2], sh_nfront[2], sh_npts[2];
+    int q = 0, hits = 0, fq = 0, fhits = 0;                   // kept by warp 0, which plans every level
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const CbSeq s = cb_seq(t, b);
@@ -667,7 +670,7 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
     };
     if (tid == 0) {
         const bool root = L >= 1;
-        sh_n = root ? 1 : 0; sh_nfront = root ? 1 : 0; sh_npts = root ? 1 : 0; sh_q = 0; sh_hits = 0; sh_fq = 0; sh_fhits = 0;
+        sh_n[0] = sh_nfront[0] = sh_npts[0] = root ? 1 : 0;
         if (root) {
             const int tk = row(L - 1);
             S.tok[0] = tk; S.par[0] = -1; S.dep[0] = 0; S.front[0] = 0; S.pts[0] = 0;
@@ -678,36 +681,32 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
     }
     __syncthreads();
 
+    int cur = 0;
     for (int pass = 0; pass < (has_frozen ? 2 : 1); ++pass) {
         const CbTables& tt = pass ? tf : t;
         const CbSeq ss = pass ? cb_seq(tf, 0) : s;
-        if (pass == 1) {
-            // the frozen pass starts from every frontier leaf the dynamic pass had
-            const int np = sh_npts;
-            __syncthreads();
-            for (int i = tid; i < np; i += blockDim.x) S.front[i] = S.pts[i];
-            if (tid == 0) sh_nfront = np;
-            __syncthreads();
-        }
+        // the frozen pass starts from every frontier leaf the dynamic pass had
+        bool listed = pass == 1;
+        if (listed) { S.next = S.front; S.front = S.pts; }
         while (true) {
-            const int nfront = sh_nfront, n_top = sh_n;
+            const int nfront = listed ? sh_npts[cur] : sh_nfront[cur], n_top = sh_n[cur], npts = sh_npts[cur];
             if (nfront == 0 || n_top >= T) break;
             if (pass == 0 && S.dep[S.front[0]] >= max_depth) break;   // a level's leaves lie at one depth: none may be queried
-            for (int li = tid; li < nfront; li += blockDim.x) S.r_stamp[li] = 0u;
-            if (tid == 0) sh_nnext = 0;
-            __syncthreads();
+            listed = false;
+            cur ^= 1;
+            if (tid == 0) { sh_n[cur] = n_top; sh_nfront[cur] = 0; sh_npts[cur] = npts; }
             // With long follower lists the frontier is worked off in batches of one leaf per warp, lookups then replay, so that a
             // level ends as soon as the tree is full (the first leaves of a level then usually take all the room).
             const int BS = tt.FC > 32 ? nwarps : nfront;          // short follower lists: the whole frontier at once
             for (int base = 0; base < nfront; base += BS) {
-                const int n_now = base == 0 ? n_top : sh_n;       // (the warp of a single leaf changes sh_n while others come by here)
+                const int n_now = base == 0 ? n_top : sh_n[cur];
                 if (n_now >= T) break;
                 // (1) parallel lookups, one warp per leaf
                 for (int li = base + warp; li < min(nfront, base + BS); li += nwarps) {
                     const int leaf = S.front[li];
                     const int d = S.dep[leaf];
                     if (d >= max_depth) {                     // nothing may hang below it: not queried
-                        if (lane == 0) { S.r_eid[li] = -1; S.r_nf[li] = 0; S.r_ok[li] = 0; }
+                        if (lane == 0) S.r_want[li] = 0u;
                         continue;
                     }
                     // key = last LL tokens of (row[0 .. L-1) ++ root->leaf path); lane j < LL holds key[j]
@@ -738,64 +737,63 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                             // (most recently inserted first in the dynamic table, most frequent first in the frozen one),
                             // and only as many as the tree still has room for: they are picked one by one with a warp-wide
                             // maximum (stamps are unique) and staged in that order.
-                            uint32_t fs[CB_MAX_FC / 32];
+                            constexpr int CH = FETCH == 1 ? 1 : CB_MAX_FC / 32;    // followers per lane
+                            uint32_t fs[CH];
 #pragma unroll
-                            for (int c = 0; c < CB_MAX_FC / 32; ++c) {
-                                if (FETCH == 1) fs[c] = c == 0 ? er.fs : 0u;       // FC <= 32: stamp and tokens came with the lookup
-                                else if (FETCH == 2) fs[c] = er.fs4[c];            // the stamps came with the lookup
-                                else fs[c] = (c * 32 + lane) < tt.FC ? e[tt.LL + c * 32 + lane] : 0u;
+                            for (int c = 0; c < CH; ++c) {
+                                fs[c] = FETCH == 1 ? er.fs : er.fs4[c];            // came with the lookup (FC <= 32: the tokens too)
                                 nf += __popc(__ballot_sync(CB_FULL, fs[c] != 0u));
                             }
                             // The followers' tokens.  FC > 32: on their way while the followers are picked below (of all of them: the
                             // round trip costs more than the bytes).
-                            int32_t ft[CB_MAX_FC / 32][CB_MAX_FL];
+                            int32_t ft[CH][CB_MAX_FL];
 #pragma unroll
-                            for (int c = 0; c < CB_MAX_FC / 32; ++c) {
+                            for (int c = 0; c < CH; ++c) {
                                 const int f = c * 32 + lane;
 #pragma unroll
                                 for (int j = 0; j < CB_MAX_FL; ++j) {
-                                    if (FETCH == 1) ft[c][j] = c == 0 ? er.tok[j] : -1;
+                                    if (FETCH == 1) ft[c][j] = er.tok[j];
                                     else ft[c][j] = fs[c] != 0u && j < tt.FL ? (int32_t)e[tt.LL + tt.FC + f * tt.FL + j] : -1;
                                 }
                             }
                             // no more than the tree has room for chains of this length
                             const int cl = min(tt.FL, max_depth - d), room = (leaf == 0 ? max(1, T - crt) : T) - n_now;
                             nf = min(nf, min(KF, (max(room, 0) + cl - 1) / cl));
-                            int rank[CB_MAX_FC / 32];
+                            int rank[CH];
 #pragma unroll
-                            for (int c = 0; c < CB_MAX_FC / 32; ++c) rank[c] = -1;
-                            if (nf <= 40) {                   // about where a maximum each costs what the counting below does
+                            for (int c = 0; c < CH; ++c) rank[c] = -1;
+                            if (FETCH == 1 || nf <= 40) {     // about where a maximum each costs what the counting below does
                                 for (int r = 0; r < nf; ++r) {
                                     uint32_t m = fs[0];
 #pragma unroll
-                                    for (int c = 1; c < CB_MAX_FC / 32; ++c) m = max(m, fs[c]);
+                                    for (int c = 1; c < CH; ++c) m = max(m, fs[c]);
                                     const uint32_t g = __reduce_max_sync(CB_FULL, m);
 #pragma unroll
-                                    for (int c = 0; c < CB_MAX_FC / 32; ++c)
+                                    for (int c = 0; c < CH; ++c)
                                         if (fs[c] == g) { rank[c] = r; fs[c] = 0u; }
                                 }
                             } else {
                                 // many are wanted: rank every follower by counting the larger stamps (independent shuffles,
                                 // where the repeated maximum is a chain of reductions)
-                                int cntr[CB_MAX_FC / 32];
+                                int cntr[CH];
 #pragma unroll
-                                for (int c = 0; c < CB_MAX_FC / 32; ++c) cntr[c] = 0;
+                                for (int c = 0; c < CH; ++c) cntr[c] = 0;
 #pragma unroll
-                                for (int c2 = 0; c2 < CB_MAX_FC / 32; ++c2) {
+                                for (int c2 = 0; c2 < CH; ++c2) {
                                     if (c2 * 32 >= tt.FC) break;
                                     for (int l = 0; l < 32; ++l) {
                                         const uint32_t o = __shfl_sync(CB_FULL, fs[c2], l);
 #pragma unroll
-                                        for (int c = 0; c < CB_MAX_FC / 32; ++c) cntr[c] += (o > fs[c]) ? 1 : 0;
+                                        for (int c = 0; c < CH; ++c) cntr[c] += (o > fs[c]) ? 1 : 0;
                                     }
                                 }
 #pragma unroll
-                                for (int c = 0; c < CB_MAX_FC / 32; ++c)
+                                for (int c = 0; c < CH; ++c)
                                     if (fs[c] != 0u && cntr[c] < nf) rank[c] = cntr[c];
                             }
                             // every lane stages its picked followers
 #pragma unroll
-                            for (int c = 0; c < CB_MAX_FC / 32; ++c) {
+                            for (int c = 0; c < CH; ++c) {
                                 if (rank[c] < 0) continue;
 #pragma unroll
                                 for (int j = 0; j < CB_MAX_FL; ++j)
@@ -803,74 +801,54 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                             }
                         }
                     }
+                    const int cl = min(t.FL, max_depth - d);
                     if (nfront > 1) {
-                        if (lane == 0) { S.r_eid[li] = eid; S.r_nf[li] = nf; S.r_ok[li] = ok ? 1 : 0; }
+                        if (lane == 0) {
+                            S.r_eid[li] = eid;
+                            S.r_want[li] = (uint32_t)(max(nf, 0) * cl) | (ok ? 1u << 12 : 0u) | (eid >= 0 ? 1u << 13 : 0u) | (uint32_t)cl << 16;
+                        }
                     } else {
-                        // the only leaf of its level: what (2) and (3) do, in place
+                        // the only leaf of its level (this is warp 0): what (2) and (3) do, in place
                         const int cap = leaf == 0 ? max(1, T - crt) : T;
                         if (ok && n_now < cap) {
-                            const int cl = min(t.FL, max_depth - d), tot = eid >= 0 ? min(max(nf, 0) * cl, cap - n_now) : 0;
+                            const int tot = eid >= 0 ? min(max(nf, 0) * cl, cap - n_now) : 0;
                             const int ends = cl == t.FL ? (int)(((uint32_t)tot * kInverse[cl]) >> 16) : 0;
+                            if (pass == 0) { ++q; hits += eid >= 0 ? 1 : 0; } else { ++fq; fhits += eid >= 0 ? 1 : 0; }
+                            if (lane == 0) {
+                                if (pass == 0 && eid >= 0) atomicMax(&s.lstamp[eid], clock0 + (uint32_t)q);
+                                sh_n[cur] = n_now + tot; sh_nfront[cur] = ends;
+                                if (pass == 0) sh_npts[cur] = npts + ends;
+                            }
                             __syncwarp();
                             attach(leaf, d, n_now, cl, tot, S.fol + li * FLFC);
-                            for (int c = lane; c < ends; c += 32) S.next[c] = n_now + c * t.FL + t.FL - 1;
-                            if (lane == 0) {
-                                sh_n = n_now + tot; sh_nnext = ends;
-                                if (pass == 0) {
-                                    ++sh_q;
-                                    if (eid >= 0) { ++sh_hits; atomicMax(&s.lstamp[eid], clock0 + (uint32_t)sh_q); }
-                                } else {
-                                    ++sh_fq;
-                                    if (eid >= 0) ++sh_fhits;
-                                }
+                            for (int c = lane; c < ends; c += 32) {
+                                const int end = n_now + c * t.FL + t.FL - 1;
+                                S.next[c] = end;
+                                if (pass == 0 && has_frozen) S.pts[npts + c] = end;
                             }
                         }
                     }
                 }
-                __syncthreads();
                 if (nfront == 1) break;
-                // (2) the sequential breadth-first order, planned by one thread or warp and filled in by all.  A query at the root (the only
+                __syncthreads();
+                // (2) the sequential breadth-first order, planned by one warp and filled in by all.  A query at the root (the only
                 // leaf of level 1, the first one of the frozen pass) is issued, and its followers attached, while the tree has fewer
                 // than max(1, T - crt) nodes; any other while fewer than T.  Below a leaf of depth d every follower is a chain of
                 // min(FL, max_depth - d) nodes, the chains follow one another until the cap cuts the last one short, and a chain of
                 // FL nodes ends in a leaf of the next level: so a leaf's nodes and frontier places follow from what the leaves
-                // before it want, a running sum that stops at the cap.
+                // before it want, a running sum that stops at the cap.  A leaf's lookup leaves one word for it and its plan is one word
+                // (with a word for each figure, and one thread for up to 16 leaves, planning took 1.6 to 3 k cycles a level).
                 const int lend = min(nfront, base + BS);
-                if (lend - base <= kSerialLeaves) {
-                    // few leaves: one after the other (800 cycles for one leaf against 1.8 k for the scan below, 1.6 k against 2.4 k for 8)
-                    if (tid == 0) {
-                        int n = n_now, q = 0, hits = 0, nn = sh_nnext;
-                        for (int l2 = base; l2 < lend; ++l2) {
-                            S.r_tot[l2] = 0;
-                            if (n >= T) continue;
-                            const int leaf = S.front[l2];
-                            const int cap = leaf == 0 ? max(1, T - crt) : T;
-                            if (n >= cap) continue;
-                            if (!S.r_ok[l2]) continue;
-                            ++q;                                // this query is issued: the dynamic table's clock ticks
-                            if (S.r_eid[l2] < 0) continue;
-                            ++hits;
-                            if (pass == 0) S.r_stamp[l2] = clock0 + (uint32_t)(sh_q + q);
-                            const int cl = min(t.FL, max_depth - S.dep[leaf]);
-                            const int tot = min(max(S.r_nf[l2], 0) * cl, cap - n);
-                            S.r_n0[l2] = n; S.r_cl[l2] = cl; S.r_tot[l2] = tot; S.r_nn0[l2] = nn;
-                            n += tot;
-                            if (cl == t.FL) nn += (int)(((uint32_t)tot * kInverse[cl]) >> 16);
-                        }
-                        sh_n = n; sh_nnext = nn;
-                        if (pass == 0) { sh_q += q; sh_hits += hits; } else { sh_fq += q; sh_fhits += hits; }
-                    }
-                } else if (warp == 0) {
-                    int n = n_now, q = 0, hits = 0, nn = sh_nnext;
-                    const int q0 = sh_q;
+                if (warp == 0) {
+                    int n = n_now, nn = sh_nfront[cur];
                     for (int l0 = base; l0 < lend; l0 += 32) {
                         const int l2 = l0 + lane;
-                        const int leaf = l2 < lend ? S.front[l2] : -1;
-                        const bool ok = leaf >= 0 && S.r_ok[l2] != 0, hit = ok && S.r_eid[l2] >= 0;
-                        const int cl = leaf >= 0 ? min(t.FL, max_depth - S.dep[leaf]) : 0;
-                        int want = hit ? max(S.r_nf[l2], 0) * cl : 0;
+                        const uint32_t x = l2 < lend ? S.r_want[l2] : 0u;
+                        const bool ok = (x >> 12) & 1u, hit = (x >> 13) & 1u;
+                        const int cl = (int)(x >> 16);
+                        int want = hit ? (int)(x & 0xFFFu) : 0;
                         bool open = true;
-                        if (leaf == 0) {                       // before every other leaf: n nodes stand when its turn comes
+                        if (l2 == 0 && S.front[0] == 0) {      // the root, before every other leaf: n nodes stand when its turn comes
                             const int cap = max(1, T - crt);
                             open = n < cap;
                             want = min(want, max(cap - n, 0));
@@ -884,8 +862,7 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                         const int start = min(T, n + incl - want);
                         const bool issued = ok && open && start < T;          // the dynamic table's clock ticks
                         const int tot = issued ? min(want, T - start) : 0;
-                        const uint32_t mi = __ballot_sync(CB_FULL, issued);
-                        hits += __popc(__ballot_sync(CB_FULL, issued && hit));
+                        const uint32_t mi = __ballot_sync(CB_FULL, issued), mh = __ballot_sync(CB_FULL, issued && hit);
                         const int leaves = cl == t.FL ? (int)(((uint32_t)tot * kInverse[cl]) >> 16) : 0;
                         int lincl = leaves;
 #pragma unroll
@@ -894,51 +871,50 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                             if (lane >= o) lincl += up;
                         }
                         if (l2 < lend) {
-                            if (pass == 0 && issued && hit) S.r_stamp[l2] = clock0 + (uint32_t)(q0 + q + __popc(mi & (0xFFFFFFFFu >> (31 - lane))));
-                            S.r_n0[l2] = start; S.r_cl[l2] = cl; S.r_tot[l2] = tot; S.r_nn0[l2] = nn + lincl - leaves;
+                            // the leaders that the sequential order reached get their stamp (two leaves of a level may share a leader)
+                            if (pass == 0 && issued && hit) atomicMax(&s.lstamp[S.r_eid[l2]], clock0 + (uint32_t)(q + __popc(mi & (0xFFFFFFFFu >> (31 - lane)))));
+                            S.r_plan[l2] = (uint32_t)start | (uint32_t)tot << 8 | (uint32_t)(nn + lincl - leaves) << 16 | (uint32_t)cl << 24;
                         }
-                        q += __popc(mi);
+                        if (pass == 0) { q += __popc(mi); hits += __popc(mh); } else { fq += __popc(mi); fhits += __popc(mh); }
                         n = min(T, n + __shfl_sync(CB_FULL, incl, 31));
                         nn += __shfl_sync(CB_FULL, lincl, 31);
                     }
                     if (lane == 0) {
-                        sh_n = n; sh_nnext = nn;
-                        if (pass == 0) { sh_q = q0 + q; sh_hits += hits; } else { sh_fq += q; sh_fhits += hits; }
+                        sh_n[cur] = n; sh_nfront[cur] = nn;
+                        if (pass == 0) sh_npts[cur] = npts + nn;
                     }
                 }
                 __syncthreads();
+                // (3) the leaves' nodes and the next frontier
                 for (int l2 = base + warp; l2 < lend; l2 += nwarps) {
-                    const int tot = S.r_tot[l2];
+                    const uint32_t x = S.r_plan[l2];
+                    const int n0 = (int)(x & 0xFFu), tot = (int)(x >> 8) & 0xFF, nn0 = (int)(x >> 16) & 0xFF, cl = (int)(x >> 24);
                     if (tot == 0) continue;
-                    const int leaf = S.front[l2], n0 = S.r_n0[l2], cl = S.r_cl[l2];
+                    const int leaf = S.front[l2];
                     attach(leaf, S.dep[leaf], n0, cl, tot, S.fol + l2 * FLFC);
                     if (cl == t.FL)
-                        for (int c = lane; c < (int)(((uint32_t)tot * kInverse[cl]) >> 16); c += 32) S.next[S.r_nn0[l2] + c] = n0 + c * t.FL + t.FL - 1;
+                        for (int c = lane; c < (int)(((uint32_t)tot * kInverse[cl]) >> 16); c += 32) {
+                            const int end = n0 + c * t.FL + t.FL - 1;
+                            S.next[nn0 + c] = end;
+                            if (pass == 0 && has_frozen) S.pts[npts + nn0 + c] = end;
+                        }
                 }
             }
-            // (3) stamp the leaders the sequential order reached; publish the next frontier
-            if (pass == 0 && nfront > 1)
-                for (int li = tid; li < nfront; li += blockDim.x)
-                    if (S.r_stamp[li] != 0u) atomicMax(&s.lstamp[S.r_eid[li]], S.r_stamp[li]);
-            const int nn = sh_nnext, np = sh_npts;
             __syncthreads();
-            for (int i = tid; i < nn; i += blockDim.x) {
-                S.front[i] = S.next[i];
-                if (pass == 0 && has_frozen) S.pts[np + i] = S.next[i];
-            }
-            if (tid == 0) { sh_nfront = nn; if (pass == 0 && has_frozen) sh_npts = np + nn; }
-            __syncthreads();
+            int32_t* const done = S.front;
+            S.front = S.next;
+            S.next = done;
         }
     }
 
-    const int n = sh_n;
+    const int n = sh_n[cur];
     if (tid == 0) {
-        s.hdr[0] = clock0 + (uint32_t)sh_q;
+        s.hdr[0] = clock0 + (uint32_t)q;
         o_n[b] = n;
-        if (sh_q) atomicAdd(&counters[CB_CNT_QUERIES], (unsigned long long)sh_q);
-        if (sh_hits) atomicAdd(&counters[CB_CNT_QUERY_HITS], (unsigned long long)sh_hits);
-        if (sh_fq) atomicAdd(&counters[CB_CNT_FROZEN_QUERIES], (unsigned long long)sh_fq);
-        if (sh_fhits) atomicAdd(&counters[CB_CNT_FROZEN_HITS], (unsigned long long)sh_fhits);
+        if (q) atomicAdd(&counters[CB_CNT_QUERIES], (unsigned long long)q);
+        if (hits) atomicAdd(&counters[CB_CNT_QUERY_HITS], (unsigned long long)hits);
+        if (fq) atomicAdd(&counters[CB_CNT_FROZEN_QUERIES], (unsigned long long)fq);
+        if (fhits) atomicAdd(&counters[CB_CNT_FROZEN_HITS], (unsigned long long)fhits);
     }
     for (int i = n + tid; i < T; i += blockDim.x) {              // places without a node
         const size_t at = (size_t)b * T + i;
@@ -1140,7 +1116,7 @@ static cb_status draft_launch(cb_ctx* ctx, const int32_t* tokens, int64_t row_st
     // A leaf can receive at most T - 1 followers (each adds a node), so no more than that many are staged per lookup.
     const int FCmax = ctx->has_frozen ? max(c.FC, ctx->frozen.FC) : c.FC;
     const int KF = max(1, min(FCmax, T - 1));
-    const size_t smem = sizeof(int32_t) * ((size_t)(3 + (T + 31) / 32) * T + (size_t)11 * NL + (size_t)NL * c.FL * KF);
+    const size_t smem = sizeof(int32_t) * ((size_t)(3 + (T + 31) / 32) * T + (size_t)kDraftArrays * NL + (size_t)NL * c.FL * KF);
     if (smem > 200 * 1024) return CB_ERR_UNSUPPORTED;
     if (smem > 48 * 1024) {
         static size_t opted[64] = {0};                         // largest size opted into so far, per device
@@ -1201,7 +1177,7 @@ extern "C" cb_status cb_accept_update_draft_tree(cb_ctx* ctx, const cb_accept_dr
     const int NL = min(T, (T - 1) / c.FL + 1);
     const int FCmax = ctx->has_frozen ? max(c.FC, ctx->frozen.FC) : c.FC;
     const int KF = max(1, min(FCmax, T - 1));
-    const size_t smem = sizeof(int32_t) * ((size_t)(3 + (T + 31) / 32) * T + (size_t)11 * NL + (size_t)NL * c.FL * KF);
+    const size_t smem = sizeof(int32_t) * ((size_t)(3 + (T + 31) / 32) * T + (size_t)kDraftArrays * NL + (size_t)NL * c.FL * KF);
     if (smem > 200 * 1024) return CB_ERR_UNSUPPORTED;
     const bool bf = a->logits_dtype == CB_DTYPE_BF16;
     const bool resident = (long long)cpr * T * c.batch <= 2ll * ctx->num_sms;

@@ -4,7 +4,7 @@
 // A window is LL + FL consecutive tokens; the corpus of N tokens has M = N - LL - FL + 1 of them.  Everything is counting
 // and selection on integers, done without sorting:
 //   1. leader counts: every window inserts-or-increments its leader in an open-addressing table whose slots hold the
-//      position of one occurrence (keys are compared by reading the corpus there) and, in the same 8 bytes, a counter; a
+//      position of one occurrence (keys are compared by reading the corpus there), with the counters in an array beside it; a
 //      window remembers its leader's slot for step 3;
 //   2. the LC best leaders under the order (count falling, tokens rising) are found by a most-significant-digit-first
 //      radix select over the distinct leaders (one histogram pass per 12 bits of the composite key; the block that comes
@@ -20,8 +20,9 @@
 // keys' counts and the lists are gathered per block in shared memory, so that a key that makes up a tenth of the corpus costs
 // an atomic per block and not one per occurrence.  Counting every selected window in a second hash table took 212 us of a build from 4 M
 // tokens (LL = 2, LC = 65,536, FC = 8: 167 MB of tables at random, more than the L2 holds), grouping its slots 49 us, ranking 187 us.
-// The whole call with the draft that follows it: 763 us that way, 547 us this way (60,000 tokens: 220 and 164; 8 launches of the selection
-// are one, which is most of it there).
+// The whole call with the draft that follows it: 763 us that way, 505 us this way (60,000 tokens: 220 and 165; 13 launches of the selection
+// are one, which is most of it there).  Of the 505: leader counts 94, windows into ranges 104, selection 75 (86 while the few threads with a
+// leader placed it between two barriers), ranking some 150 with its kernels side by side.
 // Which occurrence represents a key, and which entry id a leader gets, depends on timing; the table's content (and
 // cb_frozen_dump's output) does not.
 #include <algorithm>
@@ -31,7 +32,7 @@
 namespace {
 
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
-constexpr unsigned long long kEmptySlot = 0x00000000FFFFFFFFull;   // low word: position, high word: count
+constexpr unsigned long long kEmptySlot = 0x00000000FFFFFFFFull;   // second table; low word: position, high word: count
 constexpr int kMaxWords = 1 + CB_MAX_LL;      // composite selection key: count (complemented), then the leader's tokens
 constexpr int kDigitBits = 12, kBins = 1 << kDigitBits;
 constexpr int kMaxPasses = 1 + 3 * kMaxWords;  // leader counts below 4,095, then three digits for each word of the key
@@ -58,7 +59,7 @@ static_assert(offsetof(BuildState, hist) % 16 == 0, "histograms are read 16 byte
 
 struct BuildView {
     BuildState* st;
-    unsigned long long* h1;                                       // [S] leaders: position and count; a selected one: kTaken | entry id in the count's place
+    uint32_t* h1; uint32_t* h1_cnt;                               // [S1] leaders: position of an occurrence; count, later kTaken | entry id of a selected one
     unsigned long long* h2; uint32_t* h2_ord;                     // [S] windows of big leaders (big_slots in use); ordinal in the leader's group
     uint32_t* lslot;                                              // [M] leader slot of every window (kEmpty: left out)
     uint2* group;                                                 // [M] distinct windows of the big leaders, grouped by leader: position, count
@@ -68,7 +69,7 @@ struct BuildView {
     uint32_t* grp_n; uint32_t* grp_off;                           // [LC] windows placed (big: distinct ones); start, kBigFlag: of group, else of wpos
     uint32_t* listed; uint32_t* listed_big;                       // [LC] each: middling leaders from the front, large ones from the back; big ones
                                                                   // from the front, those that a warp takes from the back
-    uint32_t S;                                                   // slots of each hash table (a power of two)
+    uint32_t S1, S;                                               // slots of the first table (any number), of the second (a power of two)
     const int32_t* corpus;
     uint32_t M, n_tokens;
     int LL, FL, LC, FC;
@@ -85,6 +86,23 @@ __device__ __forceinline__ uint64_t hash_tokens(const int32_t* p, int n) {
 __device__ __forceinline__ bool same_tokens(const int32_t* a, const int32_t* b, int n) {
     for (int j = 0; j < n; ++j) if (a[j] != b[j]) return false;
     return true;
+}
+// The first table keeps positions and counts apart and has four slots for three windows (45 MB for 4 M windows; eight-byte slots, two a
+// window, were 67 MB: 547 against 542 us for the build).  Home slots are the hash's share of the table.
+__device__ __forceinline__ uint32_t home_leader(uint64_t h, uint32_t S1) { return __umulhi((uint32_t)(h >> 20), S1); }
+// Finds or creates the slot of the leader at corpus position i, from slot s on; kEmpty when every slot was visited.
+__device__ __forceinline__ uint32_t claim_leader(uint32_t* slots, uint32_t S1, uint32_t s, const int32_t* corpus, uint32_t i, int n, bool* created) {
+    *created = false;
+    for (uint32_t p = 0; p < S1; ++p) {
+        uint32_t pos = slots[s];
+        if (pos == kEmpty) {
+            pos = atomicCAS(&slots[s], kEmpty, i);
+            if (pos == kEmpty) { *created = true; return s; }
+        }
+        if (same_tokens(corpus + pos, corpus + i, n)) return s;
+        s = s + 1 == S1 ? 0u : s + 1;
+    }
+    return kEmpty;
 }
 // Finds or creates the slot of the n-token key at corpus position i, from slot s on.  Returns the slot, or kEmpty when every slot was
 // visited (cannot happen at the load factor the tables are sized for; reported as CB_ERR_PROBE_LIMIT).  A slot's position never
@@ -110,16 +128,18 @@ __device__ __forceinline__ uint32_t big_slots(const BuildView& v) {
     while (s < 2u * __ldcg(&v.st->big_cursor) && s < v.S) s <<= 1;
     return s;
 }
-__device__ __forceinline__ uint32_t* count_of(unsigned long long* slots, uint32_t s) { return reinterpret_cast<uint32_t*>(&slots[s]) + 1; }
+__device__ __forceinline__ uint32_t* counts_of(unsigned long long* slots) { return reinterpret_cast<uint32_t*>(slots) + 1; }   // two words apart
 
-// A block's counts of the slots it meets first in each of 512 places; other slots are counted in memory right away.
+// A block's counts of the slots it meets first in each of 512 places; other slots are counted in memory right away.  The count of
+// slot s is the word counts[s * STRIDE].
+template <int STRIDE>
 struct CountCache {
     uint32_t key[512], cnt[512];
     __device__ __forceinline__ void clear() {
         for (int i = threadIdx.x; i < 512; i += blockDim.x) { key[i] = kEmpty; cnt[i] = 0u; }
         __syncthreads();
     }
-    __device__ __forceinline__ void add(unsigned long long* slots, uint32_t s) {
+    __device__ __forceinline__ void add(uint32_t* counts, uint32_t s) {
         const uint32_t at = (s * 0x9E3779B1u) >> 23;
         uint32_t k = key[at];
         if (k == kEmpty) {
@@ -127,26 +147,26 @@ struct CountCache {
             if (k == kEmpty) k = s;
         }
         if (k == s) atomicAdd(&cnt[at], 1u);
-        else atomicAdd(count_of(slots, s), 1u);
+        else atomicAdd(counts + (size_t)s * STRIDE, 1u);
     }
-    __device__ __forceinline__ void flush(unsigned long long* slots) {
+    __device__ __forceinline__ void flush(uint32_t* counts) {
         __syncthreads();
         for (int i = threadIdx.x; i < 512; i += blockDim.x)
-            if (key[i] != kEmpty && cnt[i]) atomicAdd(count_of(slots, key[i]), cnt[i]);
+            if (key[i] != kEmpty && cnt[i]) atomicAdd(counts + (size_t)key[i] * STRIDE, cnt[i]);
     }
 };
 
 // Items that threads of a block append to a list in memory: gathered in shared memory, so that the list's counter takes an atomic
 // per thousand or so (one address takes one atomic in about 2 ns: an atomic per warp was 260 of 310 us of the leader count).
-template <typename T>
+template <typename T, uint32_t CAP = 2048>
 struct Appender {
-    static constexpr uint32_t kCap = 2048;
+    static constexpr uint32_t kCap = CAP;
     T item[kCap];
     uint32_t n, at;
     __device__ __forceinline__ void clear() { if (threadIdx.x == 0) n = 0u; __syncthreads(); }
-    // All threads of the block together, U items each at most; true (in all of them) if there may be no room for as many again.
+    // All threads of the block together, U items each at most.
     template <int U>
-    __device__ __forceinline__ bool gather(const bool (&has)[U], const T (&x)[U]) {
+    __device__ __forceinline__ void put(const bool (&has)[U], const T (&x)[U]) {
         const uint32_t lane = threadIdx.x & 31;
         uint32_t m[U], k = 0, total = 0;
 #pragma unroll
@@ -158,9 +178,16 @@ struct Appender {
             if (has[q]) item[k + __popc(m[q] & ((1u << lane) - 1u))] = x[q];
             k += (uint32_t)__popc(m[q]);
         }
-        // The block decides as one: every warp reads the count before it arrives at the barrier (the last to add sees all of it), and
-        // nobody adds again before all have.  Read after a barrier, the count could already hold the next call's additions.
-        return __syncthreads_or(n > kCap - blockDim.x * U) != 0;
+        __syncwarp();
+    }
+    __device__ __forceinline__ bool near_full(uint32_t u) const { return *(volatile const uint32_t*)&n > kCap - blockDim.x * u; }
+    // The same; true (in all threads) if there may be no room for as many again.  The block decides as one: every warp reads the count
+    // before it arrives at the barrier (the last to add sees all of it), and nobody adds again before all have.  Read after a barrier, the
+    // count could already hold the next call's additions.
+    template <int U>
+    __device__ __forceinline__ bool gather(const bool (&has)[U], const T (&x)[U]) {
+        put(has, x);
+        return __syncthreads_or(near_full(U)) != 0;
     }
     template <int U>
     __device__ __forceinline__ void add(const bool (&has)[U], const T (&x)[U], T* list, uint32_t* counter) {
@@ -198,9 +225,10 @@ __global__ void __launch_bounds__(256) fb_init_kernel(BuildView v, CbTables t) {
         atomicMax(&v.st->max_token, (uint32_t)hi);
         if (neg) { v.st->has_neg = 1u; if (v.M > 0) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_INVALID_ARG); }
     }
-    // last, so that as much of it as possible is in L2 when the leaders are counted
-    ulonglong2* a = reinterpret_cast<ulonglong2*>(v.h1);
-    for (size_t i = g; i < v.S / 2; i += stride) a[i] = make_ulonglong2(kEmptySlot, kEmptySlot);
+    // last, so that it is in L2 when the leaders are counted
+    uint4* const pos = reinterpret_cast<uint4*>(v.h1);
+    uint4* const cnt = reinterpret_cast<uint4*>(v.h1_cnt);       // whoever makes a slot has been counted
+    for (size_t i = g; i < v.S1 / 4; i += stride) { cnt[i] = make_uint4(1u, 1u, 1u, 1u); pos[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty); }
 }
 
 // 1. leader counts.  Four windows a thread, so that their chains (slot, tokens of the slot's occurrence) overlap; what the first look
@@ -208,7 +236,7 @@ __global__ void __launch_bounds__(256) fb_init_kernel(BuildView v, CbTables t) {
 template <int LL>
 __global__ void __launch_bounds__(256) fb_count_leaders_kernel(BuildView v) {
     CB_PDL_ENTRY();
-    __shared__ CountCache cache;
+    __shared__ CountCache<1> cache;
     __shared__ Appender<uint32_t> made;
     cache.clear();
     made.clear();
@@ -234,8 +262,8 @@ __global__ void __launch_bounds__(256) fb_count_leaders_kernel(BuildView v) {
         }
 #pragma unroll
         for (int q = 0; q < U; ++q) {
-            s[q] = home_slot(key[q], LL, v.S);
-            pos[q] = ok[q] ? *reinterpret_cast<const uint32_t*>(&v.h1[s[q]]) : kEmpty;
+            s[q] = home_leader(hash_tokens(key[q], LL), v.S1);
+            pos[q] = ok[q] ? v.h1[s[q]] : kEmpty;
         }
 #pragma unroll
         for (int q = 0; q < U; ++q)
@@ -249,16 +277,16 @@ __global__ void __launch_bounds__(256) fb_count_leaders_kernel(BuildView v) {
 #pragma unroll
                 for (int j = 0; j < LL; ++j) diff |= rep[q][j] ^ key[q][j];
                 if (diff != 0)                                  // an empty slot or another key's
-                    s[q] = find_or_claim(v.h1, v.S, pos[q] == kEmpty ? s[q] : (s[q] + 1) & (v.S - 1), v.corpus, (uint32_t)i, LL, &created[q]);
+                    s[q] = claim_leader(v.h1, v.S1, pos[q] == kEmpty ? s[q] : (s[q] + 1 == v.S1 ? 0u : s[q] + 1), v.corpus, (uint32_t)i, LL, &created[q]);
                 if (s[q] == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
-                else if (!created[q]) cache.add(v.h1, s[q]);
+                else if (!created[q]) cache.add(v.h1_cnt, s[q]);
             }
             if (i < v.M) v.lslot[i] = ok[q] ? s[q] : kEmpty;
         }
         made.add(created, s, v.uniq, &v.st->n_uniq);
     }
     made.flush(v.uniq, &v.st->n_uniq);
-    cache.flush(v.h1);
+    cache.flush(v.h1_cnt);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -266,8 +294,8 @@ __global__ void __launch_bounds__(256) fb_count_leaders_kernel(BuildView v) {
 // and every one needs the result of the one before (13 launches otherwise, for 60,000 tokens most of the build's time).
 constexpr int kSelThreads = 1024;
 struct SelSmem {
-    uint32_t bins[kBins], part[32], pick[2], last, cnt[33], start;
-    Appender<uint2> tied;
+    uint32_t bins[kBins], part[32], pick[2], last, start;
+    Appender<uint2, 8192> taken, tied;        // slot and count, slot and position
 };
 
 // All blocks of the launch; false after a wait that ran out (recorded as CB_ERR_TIMEOUT; the others run out too).
@@ -361,22 +389,15 @@ __device__ __forceinline__ void sel_histogram(uint32_t n, uint32_t* hist, SelSme
         if (S.bins[i]) atomicAdd(&hist[i], S.bins[i]);
 }
 
-// The leader in slot `at` of the first table gets the next entry (take; all threads of a block together, one atomic for all of
-// them); its key goes into the frozen table's index.
-__device__ __forceinline__ void place_leader(const BuildView& v, const CbTables& t, bool take, uint32_t at, unsigned long long slot, SelSmem& S) {
-    uint32_t total;
-    const uint32_t mine = sel_scan(take ? 1u : 0u, S.part, &total);
-    if (threadIdx.x == 0) S.start = total ? atomicAdd(&v.st->n_sel, total) : 0u;
-    __syncthreads();
-    if (!take) return;
-    const uint32_t eid = S.start + mine;
+// The leader in slot `at` of the first table gets entry eid; its key goes into the frozen table's index.
+__device__ __forceinline__ void place_leader(const BuildView& v, const CbTables& t, uint32_t eid, uint32_t at, uint32_t count) {
     if (eid >= (uint32_t)v.LC) { atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT); return; }
-    *count_of(v.h1, at) = kTaken | eid;
-    const int32_t* key = v.corpus + (uint32_t)slot;
+    v.h1_cnt[at] = kTaken | eid;
+    const int32_t* key = v.corpus + v.h1[at];
     uint32_t* e = t.entries + (size_t)eid * t.E;
     int32_t k4[4] = {0, 0, 0, 0};
     for (int j = 0; j < v.LL; ++j) { k4[j] = key[j]; e[j] = (uint32_t)key[j]; }
-    t.lstamp[eid] = (uint32_t)(slot >> 32);
+    t.lstamp[eid] = count;
     const uint64_t h = cb_hash4(k4[0], k4[1], k4[2], k4[3], v.LL);
     const uint32_t nb = t.nslots >> 5, word = (cb_hash_tag(h) << CB_EID_BITS) | eid;
     uint32_t bucket = cb_hash_bucket(h, t.nslots);
@@ -397,6 +418,20 @@ __device__ __forceinline__ void place_leader(const BuildView& v, const CbTables&
 }
 
 
+// All leaders gathered so far (slot and count) take entries, one atomic for all of them; all threads of the block together.  They are
+// gathered first because a placement is a chain of some 4 k cycles that the few threads with a leader would otherwise take between two
+// barriers of all.
+__device__ __forceinline__ void place_taken(const BuildView& v, const CbTables& t, SelSmem& S) {
+    __syncthreads();
+    const uint32_t n = S.taken.n;
+    if (threadIdx.x == 0) S.start = n ? atomicAdd(&v.st->n_sel, n) : 0u;
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < n; j += kSelThreads) place_leader(v, t, S.start + j, S.taken.item[j].x, S.taken.item[j].y);
+    __syncthreads();
+    if (threadIdx.x == 0) S.taken.n = 0u;
+    __syncthreads();
+}
+
 __global__ void __launch_bounds__(kSelThreads, 1) fb_select_kernel(BuildView v, CbTables t, int cbits) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     SelSmem& S = *reinterpret_cast<SelSmem*>(sel_smem);
@@ -405,7 +440,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) fb_select_kernel(BuildView v, 
     uint32_t round = 0, pass = 0, cut = 0, k = LC;
     if (!all) {
         // 2a. the count of the LC-th best leader: a bin per count below 4,095 (most comes first), the last one for all above
-        sel_histogram(n, v.st->hist[pass], S, [&](uint32_t i) { return kBins - 1 - min((uint32_t)(v.h1[v.uniq[i]] >> 32), (uint32_t)(kBins - 1)); });
+        sel_histogram(n, v.st->hist[pass], S, [&](uint32_t i) { return kBins - 1 - min(v.h1_cnt[v.uniq[i]], (uint32_t)(kBins - 1)); });
         if (!grid_barrier(v, &round, &S.last)) return;
         uint32_t rest, bin = pick_bin(v.st->hist[pass++], k, S, &rest);
         if (bin > 0u) {
@@ -417,7 +452,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) fb_select_kernel(BuildView v, 
             for (int shift = (cbits - 1) / kDigitBits * kDigitBits; shift >= 0; shift -= kDigitBits) {
                 const uint32_t hi_mask = shift + kDigitBits >= 32 ? 0u : (0xFFFFFFFFu << (shift + kDigitBits));
                 sel_histogram(n, v.st->hist[pass], S, [&](uint32_t i) {
-                    const uint32_t x = cmask - (uint32_t)(v.h1[v.uniq[i]] >> 32);
+                    const uint32_t x = cmask - v.h1_cnt[v.uniq[i]];
                     return (x & hi_mask) == (prefix & hi_mask) ? (x >> shift) & (kBins - 1) : kEmpty;
                 });
                 if (!grid_barrier(v, &round, &S.last)) return;
@@ -428,27 +463,34 @@ __global__ void __launch_bounds__(kSelThreads, 1) fb_select_kernel(BuildView v, 
         }
     }
     // 2b. the leaders with a larger count are placed, those with the same count listed
+    S.taken.clear();
     S.tied.clear();
     const uint32_t step = gridDim.x * kSelThreads;
     for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n; i0 += 4 * step) {
-        uint32_t at[4];
-        unsigned long long slot[4];
+        uint32_t at[4], cnt[4], pos[4];
+        bool take[4], tie[4];
+        uint2 x[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) at[q] = i0 + q * step + threadIdx.x < n ? v.uniq[i0 + q * step + threadIdx.x] : 0u;
+        for (int q = 0; q < 4; ++q) at[q] = i0 + q * step + threadIdx.x < n ? v.uniq[i0 + q * step + threadIdx.x] : kEmpty;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) slot[q] = i0 + q * step + threadIdx.x < n ? v.h1[at[q]] : 0ull;
-#pragma unroll 1
-        for (int q = 0; q < 4 && i0 + q * step < n; ++q) {
-            const bool in = i0 + q * step + threadIdx.x < n;
-            const uint32_t a = q == 0 ? at[0] : q == 1 ? at[1] : q == 2 ? at[2] : at[3];
-            const unsigned long long x = q == 0 ? slot[0] : q == 1 ? slot[1] : q == 2 ? slot[2] : slot[3];
-            const bool take = in && (all || (uint32_t)(x >> 32) > cut);
-            const bool tie[1] = {in && !take && (uint32_t)(x >> 32) == cut};
-            const uint2 item[1] = {make_uint2(a, (uint32_t)x)};
-            S.tied.add(tie, item, v.ties, &v.st->n_ties);
-            place_leader(v, t, take, a, x, S);
+        for (int q = 0; q < 4; ++q) cnt[q] = at[q] != kEmpty ? v.h1_cnt[at[q]] : 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            take[q] = at[q] != kEmpty && (all || cnt[q] > cut);
+            tie[q] = at[q] != kEmpty && !take[q] && cnt[q] == cut;
+            pos[q] = tie[q] ? v.h1[at[q]] : 0u;
+            x[q] = make_uint2(at[q], cnt[q]);
+        }
+        S.taken.put(take, x);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = make_uint2(at[q], pos[q]);
+        S.tied.put(tie, x);
+        if (__syncthreads_or(S.taken.near_full(4) || S.tied.near_full(4))) {
+            place_taken(v, t, S);
+            S.tied.flush(v.ties, &v.st->n_ties);
         }
     }
+    place_taken(v, t, S);
     S.tied.flush(v.ties, &v.st->n_ties);
     if (blockIdx.x == 0 && threadIdx.x == 0) t.hdr[1] = min(n, LC);
     if (!grid_barrier(v, &round, &S.last)) return;
@@ -478,12 +520,14 @@ __global__ void __launch_bounds__(kSelThreads, 1) fb_select_kernel(BuildView v, 
                 prefix[w] |= bin << shift;
             }
         // 2d. placed like the others
-        for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n_ties; i0 += gridDim.x * kSelThreads) {
+        for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n_ties; i0 += step) {
             const uint32_t i = i0 + threadIdx.x;
             const uint2 x = i < n_ties ? __ldcg(&v.ties[i]) : make_uint2(0u, 0u);
-            const bool take = i < n_ties && before_or_in(x.y, v.LL) <= 0;
-            place_leader(v, t, take, x.x, ((unsigned long long)cut << 32) | x.y, S);
+            const bool take[1] = {i < n_ties && before_or_in(x.y, v.LL) <= 0};
+            const uint2 item[1] = {make_uint2(x.x, cut)};
+            if (S.taken.gather(take, item)) place_taken(v, t, S);
         }
+        place_taken(v, t, S);
         if (!grid_barrier(v, &round, &S.last)) return;
     }
     // 3a. every selected leader takes a range (an atomic per block and 1,024 of them: their ranges lie side by side); those with more than
@@ -526,7 +570,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) fb_select_kernel(BuildView v, 
 // new one takes its ordinal in its leader's group.  Four windows a thread, whose chains (leader slot, leader, place) overlap.
 __global__ void __launch_bounds__(256) fb_windows_kernel(BuildView v) {
     CB_PDL_ENTRY();
-    __shared__ CountCache cache;
+    __shared__ CountCache<2> cache;
     constexpr int U = 4;
     const bool any_big = v.st->n_big != 0u;
     const uint32_t S2 = any_big ? big_slots(v) : 0u;
@@ -544,7 +588,7 @@ __global__ void __launch_bounds__(256) fb_windows_kernel(BuildView v) {
             if (j < n) {
                 s = find_or_claim(v.h2, S2, home_slot(v.corpus + x.x, v.LL + v.FL, S2), v.corpus, x.x, v.LL + v.FL, &created);
                 if (s == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
-                else if (!created) cache.add(v.h2, s);
+                else if (!created) cache.add(counts_of(v.h2), s);
             }
             // the new windows of one leader in a warp take their ordinals with one atomic
             if (__any_sync(CB_FULL, created)) {
@@ -569,7 +613,7 @@ __global__ void __launch_bounds__(256) fb_windows_kernel(BuildView v) {
             at[q] = i < v.M ? v.lslot[i] : kEmpty;
         }
 #pragma unroll
-        for (int q = 0; q < U; ++q) at[q] = at[q] != kEmpty ? *count_of(v.h1, at[q]) : 0u;    // kTaken | entry id, or a count
+        for (int q = 0; q < U; ++q) at[q] = at[q] != kEmpty ? v.h1_cnt[at[q]] : 0u;    // kTaken | entry id, or a count
 #pragma unroll
         for (int q = 0; q < U; ++q) off[q] = (at[q] & kTaken) ? v.grp_off[at[q] & ~kTaken] : 0u;
         uint32_t place[U];
@@ -592,7 +636,7 @@ __global__ void __launch_bounds__(256) fb_windows_kernel(BuildView v) {
     if (any_big) {
         __syncthreads();
         count_big();
-        cache.flush(v.h2);
+        cache.flush(counts_of(v.h2));
     }
 }
 // 3d. the distinct windows of the big leaders, grouped by leader: position and count
@@ -604,7 +648,7 @@ __global__ void __launch_bounds__(256) fb_group_scatter_kernel(BuildView v) {
     for (size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x; s < S2; s += stride) {
         const unsigned long long x = v.h2[s];
         if ((uint32_t)x == kEmpty) continue;
-        const uint32_t eid = *count_of(v.h1, v.lslot[(uint32_t)x]) & ~kTaken;
+        const uint32_t eid = v.h1_cnt[v.lslot[(uint32_t)x]] & ~kTaken;
         v.group[(v.grp_off[eid] & ~kBigFlag) + v.h2_ord[s]] = make_uint2((uint32_t)x, (uint32_t)(x >> 32));
     }
 }
@@ -763,9 +807,8 @@ template <int NT, int CAP>
 __global__ void __launch_bounds__(NT) fb_rank_block_kernel(BuildView v, CbTables t, uint32_t n_leaders_at) {
     fb_rank_begin();
     extern __shared__ uint32_t fb_smem[];
-    uint32_t* const tab = fb_smem;                               // [2 CAP]
-    uint32_t* const dist = tab + 2 * CAP;                        // [CAP] distinct windows
-    int32_t* const tok = reinterpret_cast<int32_t*>(dist + CAP); // [CAP][FL]
+    uint32_t* const tab = fb_smem;                               // [2 CAP], then the distinct windows at its front
+    int32_t* const tok = reinterpret_cast<int32_t*>(tab + 2 * CAP); // [CAP][FL]
     __shared__ Candidates cand;
     __shared__ uint32_t red[NT / 32], n_dist;
     const Crew<NT> crew = {red};
@@ -801,15 +844,21 @@ __global__ void __launch_bounds__(NT) fb_rank_block_kernel(BuildView v, CbTables
             }
         }
         __syncthreads();
-        for (uint32_t i0 = 0; i0 < slots; i0 += NT) {
-            const uint32_t i = i0 + me, y = i < slots ? tab[i] : 0u, m = __ballot_sync(CB_FULL, y != 0u);
+        constexpr int PER = 2 * CAP / NT;
+        uint32_t y[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) y[q] = (uint32_t)(q * NT) + me < slots ? tab[q * NT + me] : 0u;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const uint32_t m = __ballot_sync(CB_FULL, y[q] != 0u);
             uint32_t at = 0;
             if (m && lane == 0) at = atomicAdd(&n_dist, (uint32_t)__popc(m));
             at = __shfl_sync(CB_FULL, at, 0) + __popc(m & ((1u << lane) - 1u));
-            if (y) dist[at] = y;
+            if (y[q]) tab[at] = y[q];
         }
         __syncthreads();
-        const SharedGroup g = {dist, tok, v.FL};
+        const SharedGroup g = {tab, tok, v.FL};
         pick_followers<NT>(v, t, eid, g, n_dist, cand, crew);    // ends with a barrier
     }
     fb_rank_end();
@@ -1007,15 +1056,16 @@ __global__ void __launch_bounds__(256) fb_rank_kernel(BuildView v, CbTables t) {
         const uint32_t cnt = (uint32_t)__popc(same);
         const bool stands = mine && (same & ((1u << lane) - 1u)) == 0u;
         const uint32_t standing = __ballot_sync(CB_FULL, stands);
-        // Count and first token in one word (smaller comes first): four instructions for each of the others where the loop below, for two
-        // followers with the same word, takes twenty.
-        const uint32_t key = (32u - cnt) << 26 | (uint32_t)f[0];
+        // Count and first token in one word, the second token in another (smaller comes first): seven instructions for each of the others
+        // where the loop below, for two followers with the same words, takes twenty-five.
+        const uint32_t key = (32u - cnt) << 26 | (uint32_t)f[0], key2 = v.FL > 1 ? (uint32_t)f[1] : 0u;
         int rank = 0, alike = 0;
         if (short_tokens)
             for (uint32_t m = standing; m; m &= m - 1u) {
-                const uint32_t o = __shfl_sync(CB_FULL, key, __ffs(m) - 1);
-                rank += o < key ? 1 : 0;
-                alike += o == key ? 1 : 0;
+                const int k = __ffs(m) - 1;
+                const uint32_t o = __shfl_sync(CB_FULL, key, k), o2 = __shfl_sync(CB_FULL, key2, k);
+                rank += o < key || (o == key && o2 < key2) ? 1 : 0;
+                alike += o == key && o2 == key2 ? 1 : 0;
             }
         if (!short_tokens || __any_sync(CB_FULL, stands && alike > 1)) {
             rank = 0;
@@ -1045,7 +1095,7 @@ __global__ void __launch_bounds__(256) fb_rank_kernel(BuildView v, CbTables t) {
 size_t fb_align(size_t x) { return (x + 255) / 256 * 256; }
 
 struct BuildLayout {
-    uint32_t S;
+    uint32_t S1, S;
     size_t off_h1, off_h2, off_h2_ord, off_lslot, off_group, off_grp, total;
 };
 
@@ -1056,7 +1106,9 @@ cb_status fb_layout(const cb_frozen_config* c, int64_t n_tokens, BuildLayout* B)
     while (S < 2ull * (uint64_t)M) S <<= 1;
     B->S = (uint32_t)S;
     size_t o = fb_align(sizeof(BuildState));
-    B->off_h1 = o;      o = fb_align(o + S * 8);
+    uint64_t S1 = ((uint64_t)M + (uint64_t)M / 3 + 1024) / 4 * 4;
+    B->S1 = (uint32_t)S1;
+    B->off_h1 = o;      o = fb_align(o + S1 * 8);
     B->off_h2 = o;      o = fb_align(o + S * 8);
     B->off_h2_ord = o;  o = fb_align(o + S * 4);
     B->off_lslot = o;   o = fb_align(o + (size_t)(M > 0 ? M : 1) * 4);
@@ -1096,14 +1148,14 @@ extern "C" cb_status cb_frozen_build(const cb_frozen_config* cfg, const int32_t*
     char* base = (char*)dev_scratch;
     BuildView v;
     v.st = (BuildState*)base;
-    v.h1 = (unsigned long long*)(base + B.off_h1);
+    v.h1 = (uint32_t*)(base + B.off_h1); v.h1_cnt = v.h1 + B.S1;
     v.h2 = (unsigned long long*)(base + B.off_h2); v.h2_ord = (uint32_t*)(base + B.off_h2_ord);
     v.lslot = (uint32_t*)(base + B.off_lslot);
     v.group = (uint2*)(base + B.off_group); v.uniq = (uint32_t*)(base + B.off_group); v.ties = (uint2*)(v.uniq + B.S / 2);   // M <= S / 2
     v.wpos = (uint32_t*)(v.group + B.S / 2);                      // behind group's M places
     v.grp_n = (uint32_t*)(base + B.off_grp); v.grp_off = v.grp_n + cfg->LC; v.listed = v.grp_off + cfg->LC;
     v.listed_big = v.listed + cfg->LC;
-    v.S = B.S;
+    v.S1 = B.S1; v.S = B.S;
     v.corpus = dev_corpus;
     const int64_t M = n_tokens - cfg->LL - cfg->FL + 1;
     v.M = (uint32_t)(M > 0 ? M : 0);
@@ -1116,11 +1168,11 @@ extern "C" cb_status cb_frozen_build(const cb_frozen_config* cfg, const int32_t*
     CB_CUDA(cudaMemsetAsync(v.st, 0, sizeof(BuildState), st));
     CB_CUDA(cb_launch_pdl(fb_init_kernel, grid, block, 0, st, v, t));
     if (v.M > 0) {
-        // shared memory of step 4's blocks: table, distinct windows, follower tokens
-        auto block_smem = [&](uint32_t cap) { return (size_t)(3 + cfg->FL) * cap * 4; };
+        // shared memory of step 4's blocks: table, follower tokens
+        auto block_smem = [&](uint32_t cap) { return (size_t)(2 + cfg->FL) * cap * 4; };
         auto* const mid = fb_rank_block_kernel<128, kMidGroup>;
         auto* const large = fb_rank_block_kernel<512, kBigGroup>;
-        CB_CUDA(cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(3 + CB_MAX_FL) * kBigGroup * 4));
+        CB_CUDA(cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 + CB_MAX_FL) * kBigGroup * 4));
         int cbits = 1;                                        // counts are at most M
         while (cbits < 31 && (v.M >> cbits) != 0) ++cbits;
         CB_CUDA(cudaFuncSetAttribute(fb_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SelSmem)));
@@ -1141,7 +1193,7 @@ extern "C" cb_status cb_frozen_build(const cb_frozen_config* cfg, const int32_t*
         CB_CUDA(cb_launch_pdl(fb_windows_kernel, grid, block, 0, st, v));
         CB_CUDA(cb_launch_pdl(fb_group_scatter_kernel, grid, block, 0, st, v));
         CB_CUDA(cb_launch_pdl(fb_rank_big_kernel, dim3((unsigned)sms), dim3(1024), 0, st, v, t));
-        CB_CUDA(cb_launch_pdl(large, dim3((unsigned)sms), dim3(512), block_smem(kBigGroup), st, v, t, 1u));
+        CB_CUDA(cb_launch_pdl(large, dim3((unsigned)(sms * 2)), dim3(512), block_smem(kBigGroup), st, v, t, 1u));
         CB_CUDA(cb_launch_pdl(mid, dim3((unsigned)(sms * 8)), dim3(128), block_smem(kMidGroup), st, v, t, 0u));
         const size_t warp_smem = (size_t)kRankWarps * kWarpGroup * (2 + cfg->FL) * 4;
         CB_CUDA(cb_launch_pdl(fb_rank_warp_kernel, dim3((unsigned)(sms * 8)), dim3(32 * kRankWarps), warp_smem, st, v, t));

@@ -9,9 +9,12 @@
 // values (one (sequence, kv head), all its row groups) then lie a fixed fraction of the whole sequence apart, so that they
 // are worked on at the same time by different CTAs and the keys and values are fetched from HBM once and found in L2 by
 // the others; with the row group innermost one CTA would stream them again and again, each time after everything else
-// it holds has passed through L2.  A key tile of a unit with two row tiles takes about twice as long as one of a unit with one
-// (the two softmax chains share the latter's tiles; 3.1 k cycles at the 70B shape), so a tile counts w2 = 2 or w1 = 1 positions of the
-// sequence (batch 13 of small trees, head_dim 64: with one position each the CTAs ended between 42 k and 92 k cycles).  Starting a
+// it holds has passed through L2.  A key tile of a unit with two row tiles takes longer than one of a unit with one, so a tile counts w2
+// or w1 positions of the sequence: 2 and 1 with head_dim 64, where the softmax chains decide (two chains share the tiles of a unit with
+// one row tile; batch 13 of small trees: 47 us at 1 : 1, 43 at 3 : 2, 40 at 2 : 1, 43 at 5 : 2), 3 and 2 with head_dim 128, where the
+// copies of a tile weigh as much (ragged trees, 3 : 2 against 2 : 1: batch 30 58.7 against 65.7 us, batch 90 of short trees 135 against
+// 156, batch 8 of 64 heads 90 against 99, batch 20 61.0 against 62.8; 4 : 3 is 4% faster still on two of twelve shapes and 2% slower on three).
+// Starting a
 // unit costs about as much as two or three tiles (query load, pipeline refill, epilogue), so every unit is preceded by that many
 // padding positions: they carry no work, they only make a CTA that handles many short units receive fewer tiles.  A tile
 // belongs to the CTA whose range holds its first position.  A CTA therefore finishes whole units, plus at most one unit it shares
@@ -196,8 +199,8 @@ struct CbWalker {
             const int v0 = (int)(off - (long long)kh * vt);
             const int v1 = (int)min((long long)vt, (long long)v0 + (g1 - g));
             g += v1 - v0;
-            u->t0 = (max(v0 - ov, 0) + wt - 1) >> (wt - 1);  // wt is 1 or 2
-            u->t1 = (max(v1 - ov, 0) + wt - 1) >> (wt - 1);
+            u->t0 = (int)cb_quot(max(v0 - ov, 0) + wt - 1, wt);
+            u->t1 = (int)cb_quot(max(v1 - ov, 0) + wt - 1, wt);
             if (u->t1 <= u->t0) continue;                     // no tile of this unit begins in the range
             u->b = b; u->kh = kh; u->rg = rg; u->tiles = s.tiles; u->n = s.n; u->ctx = s.ctx;
             u->nrt = p.MT == 1 ? 1 : min(2, s.mtn - 2 * rg);

@@ -136,14 +136,15 @@ def oracle_attn_rows_by_head(oracle, cfg, prob, mask, rows, threads=None):
     return out, lse
 
 
-def stream_k_shares(cfg, ctx, n, n_ctas):
+def stream_k_shares(cfg, ctx, n, n_ctas, weights=(1, 2)):
     """What every persistent CTA of tree attention works on: n_ctas lists of (b, kh, row group, row tiles, tiles, t0, t1), key tiles
     [t0, t1) of the unit's `tiles`, in the order in which the CTA takes them.
 
     Restates the decomposition the attention kernel documents: work is counted in 128-key tiles; sequence b has
     ceil(ctx_b / 128) + 1 of them (the last holds the tree's own keys); a row tile packs 128 / G nodes with the G query
     heads of a kv head; a unit is one (sequence, kv head, row group), a row group being a pair of row tiles (one when the
-    whole tree cap fits one).  A tile of a unit with two row tiles counts two positions, of a unit with one it counts one; every
+    whole tree cap fits one).  A tile of a unit with two row tiles counts two positions, of a unit with one it counts one (`weights`
+    of head_dim 64; the kernel takes (2, 3) with head_dim 128, which cuts alike where all units have as many row tiles); every
     unit is preceded by three (two) tiles' worth of padding positions.  All units laid end to end in (row group, sequence, kv head)
     order, row group outermost, are cut into n_ctas equal ranges, range c = [total * c // n_ctas, total * (c + 1) // n_ctas); a
     tile belongs to the range that holds its first position."""
@@ -158,7 +159,7 @@ def stream_k_shares(cfg, ctx, n, n_ctas):
             if rg >= ((1 if mtn > 0 else 0) if MT == 1 else (mtn + 1) // 2):
                 continue
             tiles, nrt = -(-int(ctx[b]) // 128) + 1, 1 if MT == 1 else min(2, mtn - 2 * rg)
-            wt, ov = (2, 6) if nrt == 2 else (1, 2)
+            wt, ov = (weights[1], 3 * weights[1]) if nrt == 2 else (weights[0], 2 * weights[0])
             for kh in range(Hkv):
                 units.append((pos, ov, wt, tiles, b, kh, rg, nrt))
                 pos += ov + tiles * wt

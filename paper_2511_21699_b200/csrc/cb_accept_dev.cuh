@@ -18,17 +18,54 @@ __device__ __forceinline__ unsigned long long pack(float x, uint32_t idx) {
 }
 __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
 
+// The ordered values of a 16-byte vector of logits.
+template <bool BF16>
+__device__ __forceinline__ void ordered(const uint4& x, uint32_t (&o)[BF16 ? 8 : 4]) {
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (BF16) { o[2 * q] = f2ord(__uint_as_float(w[q] << 16)); o[(2 * q + 1) % (BF16 ? 8 : 4)] = f2ord(__uint_as_float(w[q] & 0xFFFF0000u)); }
+        else o[q] = f2ord(__uint_as_float(w[q]));
+    }
+}
+// A thread's running maximum over such vectors: the value, and the first vector that has it.  Which of the vector's logits it is is
+// looked up at the end, 5 instructions a logit where a packed (value, index) pair for each takes 8, for 16 registers more: for the grids
+// that are resident at once, whose threads have the registers and whose chain of round trips the packing lengthens (a third of the 4 k
+// cycles from the first load to the last comparison of one sequence over 32 k tokens); a larger grid waits for its logits either way.
+template <bool BF16>
+struct VectorMax {
+    static constexpr int N = BF16 ? 8 : 4;
+    uint32_t top = 0u, at = 0xFFFFFFFFu;      // ordered value; index of the vector's first logit
+    uint4 x = {0u, 0u, 0u, 0u};
+    __device__ __forceinline__ void take(const uint4& v, uint32_t id) {
+        uint32_t o[N];
+        ordered<BF16>(v, o);
+        uint32_t m = o[0];
+#pragma unroll
+        for (int j = 1; j < N; ++j) m = max(m, o[j]);
+        if (m > top || at == 0xFFFFFFFFu) { top = m; at = id; x = v; }
+    }
+    __device__ __forceinline__ unsigned long long packed() const {
+        if (at == 0xFFFFFFFFu) return 0ull;
+        uint32_t o[N], k = 0;
+        ordered<BF16>(x, o);
+#pragma unroll
+        for (int j = N - 1; j >= 0; --j) if (o[j] == top) k = (uint32_t)j;
+        return ((unsigned long long)top << 32) | (unsigned long long)(0xFFFFFFFFu - (at + k));
+    }
+};
+// The largest packed maximum of a warp's lanes.
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long x) {
+    const uint32_t hi = __reduce_max_sync(CB_FULL, (uint32_t)(x >> 32));
+    const uint32_t lo = __reduce_max_sync(CB_FULL, (uint32_t)(x >> 32) == hi ? (uint32_t)x : 0u);
+    return ((unsigned long long)hi << 32) | lo;
+}
+
 // The logits are read once: no L1 allocation, and first to leave L2 (the tables of the step's other kernels stay).
 __device__ __forceinline__ uint64_t l2_evict_first_policy() {
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     return pol;
-}
-__device__ __forceinline__ float4 ldg_stream4(const float* p, uint64_t pol) {
-    float4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "l"(pol));
-    return v;
 }
 __device__ __forceinline__ uint4 ldg_stream4u(const void* p, uint64_t pol) {
     uint4 v;
@@ -157,20 +194,26 @@ __device__ __forceinline__ bool accept_rows(
             v += head;
             const int nvec = (v1 - v) >> 2;
             const float* base = rowp + v;
+            VectorMax<false> vm;                                 // UN > 4
             for (int k = tid; k < nvec; k += blockDim.x * UN) {
-                float4 x[UN];
+                uint4 x[UN];
                 int kk[UN];
 #pragma unroll
-                for (int u = 0; u < UN; ++u) { kk[u] = k + u * blockDim.x; if (kk[u] < nvec) x[u] = ldg_stream4(base + 4 * (size_t)kk[u], pol); }
+                for (int u = 0; u < UN; ++u) { kk[u] = k + u * blockDim.x; if (kk[u] < nvec) x[u] = ldg_stream4u(base + 4 * (size_t)kk[u], pol); }
 #pragma unroll
                 for (int u = 0; u < UN; ++u) if (kk[u] < nvec) {
                     const uint32_t id = (uint32_t)(v + 4 * kk[u]);
-                    best = umax64(best, pack(x[u].x, id));
-                    best = umax64(best, pack(x[u].y, id + 1));
-                    best = umax64(best, pack(x[u].z, id + 2));
-                    best = umax64(best, pack(x[u].w, id + 3));
+                    if (UN > 4) {
+                        vm.take(x[u], id);
+                    } else {
+                        best = umax64(best, pack(__uint_as_float(x[u].x), id));
+                        best = umax64(best, pack(__uint_as_float(x[u].y), id + 1));
+                        best = umax64(best, pack(__uint_as_float(x[u].z), id + 2));
+                        best = umax64(best, pack(__uint_as_float(x[u].w), id + 3));
+                    }
                 }
             }
+            if (UN > 4) best = umax64(best, vm.packed());
             const int tail0 = v + 4 * nvec;
             if (tail0 + tid < v1) best = umax64(best, pack(rowp[tail0 + tid], (uint32_t)(tail0 + tid)));
         } else {
@@ -183,6 +226,7 @@ __device__ __forceinline__ bool accept_rows(
             v += head;
             const int nvec = (v1 - v) >> 3;
             const __nv_bfloat16* base = rowp + v;
+            VectorMax<true> vm;
             for (int k = tid; k < nvec; k += blockDim.x * UN) {
                 uint4 x[UN];
                 int kk[UN];
@@ -191,24 +235,28 @@ __device__ __forceinline__ bool accept_rows(
 #pragma unroll
                 for (int u = 0; u < UN; ++u) if (kk[u] < nvec) {
                     const uint32_t id = (uint32_t)(v + 8 * kk[u]);
-                    const uint32_t wds[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+                    if (UN > 4) {
+                        vm.take(x[u], id);
+                    } else {
+                        const uint32_t wds[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        best = umax64(best, pack(__uint_as_float(wds[q] << 16), id + 2 * q));
-                        best = umax64(best, pack(__uint_as_float(wds[q] & 0xFFFF0000u), id + 2 * q + 1));
+                        for (int q = 0; q < 4; ++q) {
+                            best = umax64(best, pack(__uint_as_float(wds[q] << 16), id + 2 * q));
+                            best = umax64(best, pack(__uint_as_float(wds[q] & 0xFFFF0000u), id + 2 * q + 1));
+                        }
                     }
                 }
             }
+            if (UN > 4) best = umax64(best, vm.packed());
             const int tail0 = v + 8 * nvec;
             if (tail0 + tid < v1) best = umax64(best, pack(__bfloat162float(rowp[tail0 + tid]), (uint32_t)(tail0 + tid)));
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) best = umax64(best, __shfl_xor_sync(CB_FULL, best, o));
+        best = warp_max(best);
         if ((tid & 31) == 0) s_red[tid >> 5] = best;
         __syncthreads();
-        if (tid == 0) {
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) best = umax64(best, s_red[w]);
-            atomicMax(&rowmax[(size_t)b * T + i], best);
+        if (tid < 32) {
+            best = warp_max(tid < (int)(blockDim.x >> 5) ? s_red[tid] : 0ull);
+            if (tid == 0) atomicMax(&rowmax[(size_t)b * T + i], best);
         }
     }
     // The last CTA of this sequence to arrive owns the walk (and re-zeroes the scratch for the next call).

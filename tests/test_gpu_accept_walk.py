@@ -68,3 +68,25 @@ def test_malformed_trees_are_not_followed():
         assert int(r["n_accept"][0]) == want, (at, p)
         assert r["accept_nodes"][0].cpu().tolist() == list(range(1, want + 1)) + [-1] * (dmax - want)
         assert r["out_tokens"][0].cpu().tolist() == list(range(2, want + 3)) + [-1] * (dmax - want)
+
+
+@pytest.mark.parametrize("batch", [1, 40])                       # a chunk's loads at once, and four at a time
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V", [1, 3, 4, 7, 8, 9, 1023, 1025, 2047, 2049, 8191, 8193, 16385, 32771])
+def test_first_maximum_among_ties(V, dtype, batch):
+    """Five values and -inf only, so that the maximum stands many times in a vector of logits, in several of a thread's, a warp's and a
+    block's; rows of one value throughout; rows at odd offsets.  The targets are exact."""
+    from paper_2511_21699_b200 import Cacheback
+    T = 12
+    g = torch.Generator().manual_seed(V)
+    store = torch.randint(-2, 3, (batch, T, V + 3), generator=g).float()
+    store[torch.rand(store.shape, generator=g) < 0.3] = float("-inf")
+    store[:, 1], store[:, 2] = -0.0, float("-inf")
+    store[:, 3, : V // 2] = -3.0
+    x = store.to(dtype).cuda()[:, :, :V]
+    cb = Cacheback(batch, 2, 4, 64, 4, T, 0, T, V, 8, 8, 64)
+    chain = torch.arange(T, dtype=torch.int32).repeat(batch, 1)
+    r = cb.cb_accept(dict(tokens=torch.zeros_like(chain).cuda(), parent=(chain - 1).cuda(), depth=chain.cuda(),
+                          n_nodes=torch.full((batch,), T, dtype=torch.int32).cuda()), logits=x)
+    assert np.array_equal(r["target_ids"].cpu().numpy(), store[:, :, :V].numpy().argmax(2))
+    assert cb.cb_poll_status()[0] == 0

@@ -345,11 +345,13 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                     uint32_t v[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int q = (int)q0 + j, f = q - LL, x = f - t.FC;
-                        const uint32_t fi = x < 0 ? (uint32_t)max(f, 0) : ((uint32_t)x * fl_inv) >> 16;
-                        const uint32_t pw = fi == 0u ? pw0 : (fi < n ? S.pair[S.group[g + fi]] : 0u);
+                        const int f = (int)q0 + j - LL, x = f - t.FC;       // follower of a stamp, place among the followers' tokens
+                        const uint32_t fi = x >= 0 ? ((uint32_t)x * fl_inv) >> 16 : (uint32_t)max(f, 0);
+                        uint32_t pw = pw0;
+                        if (fi != 0u) pw = fi < n ? S.pair[S.group[g + fi]] : 0u;
+                        const uint32_t at = f < 0 ? kpos + q0 + j : (pw >> 16) + (uint32_t)(LL - 1 + x) - fi * (uint32_t)t.FL;
                         v[j] = pw ? clock0 + (pw & 0xFFFFu) : 0u;
-                        if (f < 0 || (x >= 0 && pw)) v[j] = (uint32_t)S.tok[f < 0 ? kpos + q : (pw >> 16) - 1u + (uint32_t)(LL + x) - fi * (uint32_t)t.FL];
+                        if (f < 0 || (x >= 0 && pw)) v[j] = (uint32_t)S.tok[at];
                     }
                     *reinterpret_cast<uint4*>(e + q0) = make_uint4(v[0], v[1], v[2], v[3]);
                 }

@@ -516,7 +516,7 @@ def measure(args, cfg_name, rank, world, device, headline):
     bulk = {"ms": 1e3 * bulk_t, "windows": windows, "windows_per_s": windows / bulk_t, "algorithmic_bytes": bulk_bytes,
             "bytes_per_window": entry_bytes + (cfg.FL + 2) * 4, "gbs": bulk_bytes / bulk_t / 1e9,
             "frac_of_hbm": bulk_bytes / bulk_t / 1e9 / pk["hbm_gbs"], "scratch_bytes": scratch_bytes,
-            "path": "order-free (scratch attached: one thread per window, one warp per distinct leader)",
+            "path": "order-free (in shared memory up to 8,192 windows a sequence, through the attached scratch above)",
             "ms_without_scratch": float(np.median(bulk_plain_ms))}
 
     frozen_info, ft = None, None

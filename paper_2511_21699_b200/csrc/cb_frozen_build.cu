@@ -16,7 +16,7 @@
 //      (up to 32 windows: the lanes match their tokens against one another) or by a block with a table in shared memory; of a
 //      big leader's distinct windows a block picks the FC best from memory.  The pick: a threshold by bisection on the count, then on
 //      the tokens of the windows that tie with it where those are many; what is left is ranked.
-// What bounds it is random access: to the leader table (8 bytes a slot, 2 to 4 slots a window) and to the leaders' ranges.  The frequent
+// What bounds it is random access: to the leader table (positions and counts apart, four slots for three windows) and to the ranges.  The frequent
 // keys' counts and the lists are gathered per block in shared memory, so that a key that makes up a tenth of the corpus costs
 // an atomic per block and not one per occurrence.  Counting every selected window in a second hash table took 212 us of a build from 4 M
 // tokens (LL = 2, LC = 65,536, FC = 8: 167 MB of tables at random, more than the L2 holds), grouping its slots 49 us, ranking 187 us.

@@ -146,8 +146,7 @@ extern "C" cb_status cb_tree_attn(cb_ctx* ctx, const cb_attn_args* a, void* stre
     // The tensor-core kernel is persistent: one CTA per SM, each taking an equal share of all key tiles.
     p.nc = ctx->num_sms < CB_ATTN_MAX_CTAS ? ctx->num_sms : CB_ATTN_MAX_CTAS;
     p.cs = 0;
-    // What a tile of a unit with two row tiles weighs against one of a unit with one (cb_attn.cuh).
-    p.w1 = p.D == 128 ? 2 : 1; p.w2 = p.D == 128 ? 3 : 2;
+    cb_attn_weights(p);
     {
         const long long cap = (long long)a->max_pages * c.page_size;
         const long long mc = a->max_ctx > 0 && a->max_ctx < cap ? a->max_ctx : cap;

@@ -11,13 +11,17 @@
 // the others; with the row group innermost one CTA would stream them again and again, each time after everything else
 // it holds has passed through L2.  A key tile of a unit with two row tiles takes longer than one of a unit with one, so a tile counts w2
 // or w1 positions of the sequence: 2 and 1 with head_dim 64, where the softmax chains decide (two chains share the tiles of a unit with
-// one row tile; batch 13 of small trees: 47 us at 1 : 1, 43 at 3 : 2, 40 at 2 : 1, 43 at 5 : 2), 3 and 2 with head_dim 128, where the
+// one row tile; batch 13 of small trees: 47 us at 1 : 1, 43 at 3 : 2, 40 at 2 : 1, 43 at 5 : 2), 6 and 4 with head_dim 128, where the
 // copies of a tile weigh as much (ragged trees, 3 : 2 against 2 : 1: batch 30 58.7 against 65.7 us, batch 90 of short trees 135 against
 // 156, batch 8 of 64 heads 90 against 99, batch 20 61.0 against 62.8; 4 : 3 is 4% faster still on two of twelve shapes and 2% slower on three).
 // Starting a
 // unit costs about as much as two or three tiles (query load, pipeline refill, epilogue), so every unit is preceded by that many
 // padding positions: they carry no work, they only make a CTA that handles many short units receive fewer tiles.  A tile
-// belongs to the CTA whose range holds its first position.  A CTA therefore finishes whole units, plus at most one unit it shares
+// belongs to the CTA whose range holds the tile's deciding position, its d1-th or d2-th from zero.  Those are the first one at 2 : 1, and at
+// 6 : 4 the ones that cut a launch whose units have all one row tile, or all two, exactly as 2 : 1 cuts it: a range that starts at
+// the share x of the sequence leaves out the tiles i with 2x >= 2i + 1 (two) or x >= i + 1 (one), which is 6x >= 6i + 3 and 4x >= 4i + 4.
+// Where such launches are cut decides the last bit of rows that CTAs share.
+// A CTA therefore finishes whole units, plus at most one unit it shares
 // with earlier CTAs and one it shares with later CTAs; the CTAs of a shared unit combine unnormalised partials (in the kernel, or
 // in the merge pass of the CTA-pair kernel, which counts one position per tile).
 #pragma once
@@ -47,22 +51,30 @@ struct CbAttnParams {
     int MT;               // row tiles that T nodes need = ceil(T / NPT)
     int nc;               // persistent CTAs (= ranges of the global tile sequence)
     int w1, w2;           // positions that a key tile of a unit with one or with two row tiles counts
+    int d1, d2;           // which of them decides whose tile it is
     int max_tiles;        // host's upper bound on the key tiles of a unit (from max_ctx, else from the block table's width)
     int cs;               // > 0: cluster mode, one unit per cluster of cs CTAs (see cb_attn_tc.cu); 0: the stream-K split
     float scale_log2;     // softmax scale * log2(e)
     uint32_t* status;
 };
 
+// The weights of the persistent CTAs' split (see above).
+inline void cb_attn_weights(CbAttnParams& p) {
+    if (p.D == 128) { p.w1 = 4; p.w2 = 6; p.d1 = 3; p.d2 = 2; }
+    else { p.w1 = 1; p.w2 = 2; p.d1 = p.d2 = 0; }
+}
+
 // Per-sequence shape of the decomposition.
 struct CbSeqShape {
     int n, ctx, tiles, mtn, RG;
-    int w1, w2;
+    int w1, w2, d1, d2;
     bool one;             // the launch has one row tile per unit throughout
     long long W;          // positions (padding + key tiles) of all units of this sequence
     __device__ __forceinline__ bool two_rows(int rg) const { return !one && mtn - 2 * rg >= 2; }
     __device__ __forceinline__ int wt(int rg) const { return two_rows(rg) ? w2 : w1; }              // positions per key tile
     __device__ __forceinline__ int ov(int rg) const { return two_rows(rg) ? 3 * w2 : 2 * w1; }      // padding positions in front of a unit
     __device__ __forceinline__ int unit(int rg) const { return tiles * wt(rg) + ov(rg); }           // positions of one unit
+    __device__ __forceinline__ int dec(int rg) const { return ov(rg) + (two_rows(rg) ? d2 : d1); }  // deciding position of a unit's first tile
     // positions of this sequence's units of row group rg (all kv heads); 0 if the tree has no such row group
     __device__ __forceinline__ long long w_of(int Hkv, int rg) const { return rg < RG ? (long long)Hkv * unit(rg) : 0ll; }
 };
@@ -75,7 +87,7 @@ __device__ __forceinline__ CbSeqShape cb_seq_shape(const CbAttnParams& p, int b)
     s.mtn = (int)(((uint32_t)(s.n + p.NPT - 1) * p.npt_inv) >> 16);
     s.one = p.MT == 1;
     s.RG = s.one ? (s.mtn > 0 ? 1 : 0) : (s.mtn + 1) / 2;
-    s.w1 = p.w1; s.w2 = p.w2;
+    s.w1 = p.w1; s.w2 = p.w2; s.d1 = p.d1; s.d2 = p.d2;
     // every row group but the last has two row tiles
     s.W = s.RG > 0 ? (long long)p.Hkv * ((long long)(s.RG - 1) * s.unit(0) + s.unit(s.RG - 1)) : 0;
     return s;
@@ -99,7 +111,7 @@ __device__ __forceinline__ long long cb_quot(long long a, int b) {
     return cb_div(a, b);
 }
 __device__ __forceinline__ long long cb_range_start(long long total, int nc, int c) { return cb_quot(total * c, nc); }
-// CTA whose range holds global tile x.
+// CTA whose range holds position x.
 __device__ __forceinline__ int cb_cta_of(long long total, int nc, long long x) {
     const long long at = (x + 1) * nc - 1;
     return (int)(total < (1ll << 22) ? cb_quot(at, (int)total) : cb_div(at, total));
@@ -197,14 +209,14 @@ struct CbWalker {
             // with the roles' registers (with cb_quot: batch 39 of 40 heads over 220 tokens 82.1 us, so 74.8; batch 103 of 64 heads over 300
             // 154 and 135; batch 81 of 40 heads over 500 241 and 232.  Without any division but more state kept between two units: 76.8, 136, 239).
             const long long off = g - pre;
-            const int vt = s.unit(rg), wt = s.wt(rg), ov = s.ov(rg);
+            const int vt = s.unit(rg), wt = s.wt(rg), dec = s.dec(rg);
             const int kh = (int)cb_div(off, vt);
             const int v0 = (int)(off - (long long)kh * vt);
             const int v1 = (int)min((long long)vt, (long long)v0 + (g1 - g));
             g += v1 - v0;
-            u->t0 = (max(v0 - ov, 0) + wt - 1) / wt;
-            u->t1 = (max(v1 - ov, 0) + wt - 1) / wt;
-            if (u->t1 <= u->t0) continue;                     // no tile of this unit begins in the range
+            u->t0 = (max(v0 - dec, 0) + wt - 1) / wt;
+            u->t1 = (max(v1 - dec, 0) + wt - 1) / wt;
+            if (u->t1 <= u->t0) continue;                     // no tile of this unit is the range's
             u->b = b; u->kh = kh; u->rg = rg; u->tiles = s.tiles; u->n = s.n; u->ctx = s.ctx;
             u->nrt = p.MT == 1 ? 1 : min(2, s.mtn - 2 * rg);
             return true;

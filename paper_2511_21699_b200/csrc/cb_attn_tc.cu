@@ -316,9 +316,9 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     if (p.cs == 0 && !(u.t0 == 0 && u.t1 == u.tiles)) {
                         // a unit shared with other CTAs: who holds its first tile, and how many of them there are
                         // (ranges of at least one tile's positions: the CTAs from the first tile's to the last one's; shorter ranges
-                        // hold the beginning of one tile at most, so every tile has a CTA of its own)
+                        // hold the deciding position of one tile at most, so every tile has a CTA of its own)
                         const int wt = wk.s.wt(u.rg);
-                        const long long tot = *s_tot, x0 = wk.pre + (long long)u.kh * wk.s.unit(u.rg) + wk.s.ov(u.rg);
+                        const long long tot = *s_tot, x0 = wk.pre + (long long)u.kh * wk.s.unit(u.rg) + wk.s.dec(u.rg);
                         const int cf = cb_cta_of(tot, p.nc, x0);
                         const bool wide = tot >= (long long)p.nc * wt;
                         d->cf = cf;
@@ -1058,7 +1058,7 @@ cb_status launch_pairs(CbAttnParams p, const TcMaps& maps, cudaStream_t st, int 
     // same time, so that one fetch from HBM serves all of them.
     const int row_groups = (p.MT + 1) / 2;
     if (npairs > row_groups) npairs -= npairs % row_groups;
-    p.nc = npairs; p.cs = 0; p.w1 = p.w2 = 1;
+    p.nc = npairs; p.cs = 0; p.w1 = p.w2 = 1; p.d1 = p.d2 = 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * npairs)); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairCfg::SMEM_ALLOC; cfg.stream = st;
     cudaLaunchAttribute at[2];

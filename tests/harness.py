@@ -136,22 +136,22 @@ def oracle_attn_rows_by_head(oracle, cfg, prob, mask, rows, threads=None):
     return out, lse
 
 
-def stream_k_shares(cfg, ctx, n, n_ctas, weights=(1, 2)):
+def stream_k_shares(cfg, ctx, n, n_ctas):
     """What every persistent CTA of tree attention works on: n_ctas lists of (b, kh, row group, row tiles, tiles, t0, t1), key tiles
     [t0, t1) of the unit's `tiles`, in the order in which the CTA takes them.
 
     Restates the decomposition the attention kernel documents: work is counted in 128-key tiles; sequence b has
     ceil(ctx_b / 128) + 1 of them (the last holds the tree's own keys); a row tile packs 128 / G nodes with the G query
     heads of a kv head; a unit is one (sequence, kv head, row group), a row group being a pair of row tiles (one when the
-    whole tree cap fits one).  A tile of a unit with two row tiles counts two positions, of a unit with one it counts one (`weights`
-    of head_dim 64; the kernel takes (2, 3) with head_dim 128, which cuts alike where all units have as many row tiles); every
-    unit is preceded by three (two) tiles' worth of padding positions.  All units laid end to end in (row group, sequence, kv head)
-    order, row group outermost, are cut into n_ctas equal ranges, range c = [total * c // n_ctas, total * (c + 1) // n_ctas); a
-    tile belongs to the range that holds its first position."""
+    whole tree cap fits one).  A tile of a unit with two row tiles counts two positions, of a unit with one it counts one (head_dim 128:
+    six and four); every unit is preceded by three (two) tiles' worth of padding positions.  All units laid end to end in (row group,
+    sequence, kv head) order, row group outermost, are cut into n_ctas equal ranges, range c = [total * c // n_ctas, total * (c + 1) //
+    n_ctas); a tile belongs to the range that holds its first position (head_dim 128: its third of six, its fourth of four)."""
+    weights, decide = ((4, 6), (3, 2)) if cfg.head_dim == 128 else ((1, 2), (0, 0))
     G, Hkv, T = cfg.gqa, cfg.n_kv_heads, cfg.max_nodes
     npt = 128 // G
     MT = -(-T // npt)
-    units = []                                             # (first position, padding, positions per tile, tiles, b, kh, rg, row tiles)
+    units = []                                   # (first position, padding, positions per tile, tiles, b, kh, rg, row tiles, deciding place)
     pos = 0
     for rg in range(1 if MT == 1 else (MT + 1) // 2):
         for b in range(cfg.batch):
@@ -161,15 +161,15 @@ def stream_k_shares(cfg, ctx, n, n_ctas, weights=(1, 2)):
             tiles, nrt = -(-int(ctx[b]) // 128) + 1, 1 if MT == 1 else min(2, mtn - 2 * rg)
             wt, ov = (weights[1], 3 * weights[1]) if nrt == 2 else (weights[0], 2 * weights[0])
             for kh in range(Hkv):
-                units.append((pos, ov, wt, tiles, b, kh, rg, nrt))
+                units.append((pos, ov, wt, tiles, b, kh, rg, nrt, decide[nrt - 1]))
                 pos += ov + tiles * wt
     ctas, k = [], 0
     for c in range(n_ctas):
         g0, g1 = pos * c // n_ctas, pos * (c + 1) // n_ctas
         shares = []
         while k < len(units) and units[k][0] < g1:
-            p0, ov, wt, tiles, b, kh, rg, nrt = units[k]
-            t0, t1 = (-(-max(min(max(g, p0), p0 + ov + tiles * wt) - p0 - ov, 0) // wt) for g in (g0, g1))
+            p0, ov, wt, tiles, b, kh, rg, nrt, de = units[k]
+            t0, t1 = (-(-max(min(max(g, p0), p0 + ov + tiles * wt) - p0 - ov - de, 0) // wt) for g in (g0, g1))
             if t1 > t0:
                 shares.append((b, kh, rg, nrt, tiles, t0, t1))
             if p0 + ov + tiles * wt > g1:

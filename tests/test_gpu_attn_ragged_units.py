@@ -12,9 +12,9 @@ from tests.harness import (Problem, bf16_to_f64, dev, device_attn_inputs, oracle
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d,weights", [(64, (1, 2)), (128, (2, 3))])
+@pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("batch,hq,hkv,T,ctx", [(40, 8, 2, 61, (0, 1, 127, 128, 129, 700)), (150, 8, 4, 128, (5, 300)), (3, 64, 8, 100, (3000, 4000))])
-def test_attn_mixed_units(oracle, d, weights, batch, hq, hkv, T, ctx):
+def test_attn_mixed_units(oracle, d, batch, hq, hkv, T, ctx):
     from paper_2511_21699_b200 import Cacheback
     cfg = W.CbConfig("mixed_units", batch, 2, 2, 64, 2, T, 8, 0, hq, hkv, d, (0, max(ctx)), 100, 1.1, 0.3, (4, 8), 64)
     prob = Problem(cfg)
@@ -27,7 +27,7 @@ def test_attn_mixed_units(oracle, d, weights, batch, hq, hkv, T, ctx):
         par[b], dep[b] = W.random_tree(cfg.seed, b, int(n[b]), cfg.max_depth, T)
         mask[b] = tree_mask_from_parents(par[b], int(n[b]), (T + 31) // 32)
     owners, seams = {}, set()
-    for c, shares in enumerate(stream_k_shares(cfg, prob.ctx, n, min(torch.cuda.get_device_properties(0).multi_processor_count, 160), weights)):
+    for c, shares in enumerate(stream_k_shares(cfg, prob.ctx, n, min(torch.cuda.get_device_properties(0).multi_processor_count, 160))):
         for s in shares:
             owners.setdefault(s[:4], set()).add(c)
         for a, b in zip(shares, shares[1:]):

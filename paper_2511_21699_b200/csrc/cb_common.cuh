@@ -151,6 +151,21 @@ inline cudaError_t cb_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block
     cfg.attrs = at; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
+// Lets a kernel's blocks have `bytes` of dynamic shared memory.  Unasked a block gets 48 KB, its static part included.  *have: what it
+// may have so far, per device and kernel (0: not asked yet); the caller guards it.
+template <typename Kernel>
+inline cudaError_t cb_allow_smem(Kernel kernel, size_t bytes, size_t* have) {
+    if (*have == 0) {
+        cudaFuncAttributes at;
+        const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+        if (e != cudaSuccess) return e;
+        *have = 48 * 1024 - at.sharedSizeBytes;
+    }
+    if (bytes <= *have) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) *have = bytes;
+    return e;
+}
 #endif
 
 #define CB_CHECK_ARG(cond) do { if (!(cond)) return CB_ERR_INVALID_ARG; } while (0)

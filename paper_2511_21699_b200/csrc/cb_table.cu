@@ -1118,19 +1118,17 @@ static cb_status draft_launch(cb_ctx* ctx, const int32_t* tokens, int64_t row_st
     const int KF = max(1, min(FCmax, T - 1));
     const size_t smem = sizeof(int32_t) * ((size_t)(3 + (T + 31) / 32) * T + (size_t)kDraftArrays * NL + (size_t)NL * c.FL * KF);
     if (smem > 200 * 1024) return CB_ERR_UNSUPPORTED;
-    if (smem > 48 * 1024) {
-        static size_t opted[64] = {0};                         // largest size opted into so far, per device
-        const int d = ctx->device & 63;
-        if (opted[d] < smem) {
-            CB_CUDA(cudaFuncSetAttribute(cb_draft_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            CB_CUDA(cudaFuncSetAttribute(cb_draft_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            opted[d] = smem;
-        }
+    auto kernel = FCmax <= 32 ? cb_draft_kernel<1> : cb_draft_kernel<2>;
+    {
+        static std::mutex mu;
+        static size_t have[64][2] = {};                        // per device and kernel
+        std::lock_guard<std::mutex> lock(mu);
+        CB_CUDA(cb_allow_smem(kernel, smem, &have[ctx->device & 63][FCmax <= 32 ? 0 : 1]));
     }
     const int threads = upd_n_old ? 32 * kUpdWarps : 32 * max(1, min(8, NL));   // insertions: a warp per window
     CbTables tf = {};
     if (ctx->has_frozen) tf = ctx->frozen;
-    CB_CUDA(cb_launch_pdl(FCmax <= 32 ? cb_draft_kernel<1> : cb_draft_kernel<2>, dim3(c.batch), dim3(threads), smem, (cudaStream_t)stream, ctx->tables, tf, T, c.crt, c.max_depth, NL, KF,
+    CB_CUDA(cb_launch_pdl(kernel, dim3(c.batch), dim3(threads), smem, (cudaStream_t)stream, ctx->tables, tf, T, c.crt, c.max_depth, NL, KF,
                           tokens, row_stride, seq_len, upd_n_old, tree_tokens, tree_parent, tree_depth, tree_mask, n_nodes, ctx->d_status, ctx->d_counters));
     cb_count_launch(1);
     return CB_OK;
@@ -1184,15 +1182,11 @@ extern "C" cb_status cb_accept_update_draft_tree(cb_ctx* ctx, const cb_accept_dr
     auto kernel = FCmax > 32  ? (bf ? cb_accept_draft_kernel<2, true, 2> : cb_accept_draft_kernel<2, false, 2>)
                   : resident  ? (bf ? cb_accept_draft_kernel<1, true, 2> : cb_accept_draft_kernel<1, false, 2>)
                               : (bf ? cb_accept_draft_kernel<1, true, 4> : cb_accept_draft_kernel<1, false, 4>);
-    if (smem > 48 * 1024) {
+    {
         static std::mutex mu;
-        static size_t opted[64][6] = {};                       // largest size opted into so far, per device and kernel
+        static size_t have[64][6] = {};                        // per device and kernel
         std::lock_guard<std::mutex> lock(mu);
-        const int d = ctx->device & 63, k = (FCmax > 32 ? 0 : resident ? 2 : 4) + (bf ? 1 : 0);
-        if (opted[d][k] < smem) {
-            CB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            opted[d][k] = smem;
-        }
+        CB_CUDA(cb_allow_smem(kernel, smem, &have[ctx->device & 63][(FCmax > 32 ? 0 : resident ? 2 : 4) + (bf ? 1 : 0)]));
     }
     CbTables tf = {};
     if (ctx->has_frozen) tf = ctx->frozen;

@@ -50,6 +50,7 @@ struct BuildState {                           // head of the scratch buffer
     uint32_t n_ties;                          // leaders whose count is exactly that of the LC-th best
     uint32_t cursor, big_cursor;              // next free place of the window array, of the group array (the big leaders' windows)
     uint32_t arrived;                         // blocks of the selection that have come to its barriers so far
+    uint32_t aborted;                         // a block has given up on such a barrier: what the later kernels read is incomplete
     uint32_t max_token;                       // largest token of the corpus
     uint32_t has_neg;                         // some token is negative
     alignas(16) uint32_t hist[kMaxPasses][kBins];   // one histogram per pass of the selection (read 16 bytes at a time)
@@ -72,6 +73,7 @@ struct BuildView {
     uint32_t S1, S;                                               // slots of the first table (any number), of the second (a power of two)
     const int32_t* corpus;
     uint32_t M, n_tokens;
+    uint32_t wait_limit;                                          // looks at the selection's barriers before a block gives up
     int LL, FL, LC, FC;
 };
 
@@ -298,7 +300,8 @@ struct SelSmem {
     Appender<uint2, 8192> taken, tied;        // slot and count, slot and position
 };
 
-// All blocks of the launch; false after a wait that ran out (recorded as CB_ERR_TIMEOUT; the others run out too).
+// All blocks of the launch; false after a wait that ran out (the others run out too).  The call then returns CB_ERR_TIMEOUT, whatever
+// was recorded before, and the kernels behind this launch do nothing: a leader may have been selected by then without a range.
 __device__ __forceinline__ bool grid_barrier(const BuildView& v, uint32_t* round, uint32_t* s_flag) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -306,17 +309,19 @@ __device__ __forceinline__ bool grid_barrier(const BuildView& v, uint32_t* round
         __threadfence();
         atomicAdd(&v.st->arrived, 1u);
         uint32_t ok = 0u;
-        for (uint32_t k = 0; k < (1u << 24) && !ok; ++k) {
+        for (uint32_t k = 0; k < v.wait_limit && !ok; ++k) {
             uint32_t x;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(&v.st->arrived) : "memory");
             ok = x >= *round ? 1u : 0u;
         }
-        if (!ok) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_TIMEOUT);
+        if (!ok) { v.st->aborted = 1u; atomicExch(&v.st->status, (uint32_t)CB_ERR_TIMEOUT); }
         *s_flag = ok;
     }
     __syncthreads();
     return *s_flag != 0u;
 }
+// Asked by the kernels after that one, by every thread: a load that L1 serves (past it, thousands of warps at one word cost a kernel 2 us).
+__device__ __forceinline__ bool fb_aborted(const BuildView& v) { return v.st->aborted != 0u; }
 __device__ __forceinline__ uint32_t sel_scan(uint32_t x, uint32_t* part, uint32_t* total) {   // exclusive, over the block
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t incl = x;
@@ -570,6 +575,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) fb_select_kernel(BuildView v, 
 // new one takes its ordinal in its leader's group.  Four windows a thread, whose chains (leader slot, leader, place) overlap.
 __global__ void __launch_bounds__(256) fb_windows_kernel(BuildView v) {
     CB_PDL_ENTRY();
+    if (fb_aborted(v)) return;
     __shared__ CountCache<2> cache;
     constexpr int U = 4;
     const bool any_big = v.st->n_big != 0u;
@@ -642,7 +648,7 @@ __global__ void __launch_bounds__(256) fb_windows_kernel(BuildView v) {
 // 3d. the distinct windows of the big leaders, grouped by leader: position and count
 __global__ void __launch_bounds__(256) fb_group_scatter_kernel(BuildView v) {
     CB_PDL_ENTRY();
-    if (v.st->n_big == 0u) return;
+    if (fb_aborted(v) || v.st->n_big == 0u) return;
     const uint32_t S2 = big_slots(v);
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x; s < S2; s += stride) {
@@ -793,7 +799,7 @@ __global__ void __launch_bounds__(1024) fb_rank_big_kernel(BuildView v, CbTables
     __shared__ Candidates cand;
     __shared__ uint32_t red[32];
     const Crew<1024> crew = {red};
-    const uint32_t n = v.st->n_big;
+    const uint32_t n = fb_aborted(v) ? 0u : v.st->n_big;
     for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
         const uint32_t eid = v.listed_big[k];
         const MemoryGroup g = {v.group + (v.grp_off[eid] & ~kBigFlag), v.corpus, v.LL};
@@ -813,7 +819,7 @@ __global__ void __launch_bounds__(NT) fb_rank_block_kernel(BuildView v, CbTables
     __shared__ uint32_t red[NT / 32], n_dist;
     const Crew<NT> crew = {red};
     const int me = (int)threadIdx.x, lane = me & 31;
-    const uint32_t n = n_leaders_at ? v.st->n_large : v.st->n_mid;
+    const uint32_t n = fb_aborted(v) ? 0u : n_leaders_at ? v.st->n_large : v.st->n_mid;
     for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
         const uint32_t eid = v.listed[n_leaders_at ? (uint32_t)v.LC - 1 - k : k], nw = v.grp_n[eid];
         const uint32_t* const wp = v.wpos + v.grp_off[eid];
@@ -874,7 +880,7 @@ __global__ void __launch_bounds__(32 * kRankWarps) fb_rank_warp_kernel(BuildView
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* const tab = fb_smem + warp * (kWarpGroup * (2 + v.FL));      // [2 kWarpGroup]: index of the first claimant + 1, count
     int32_t* const tok = reinterpret_cast<int32_t*>(tab + 2 * kWarpGroup); // [kWarpGroup][FL]
-    const uint32_t n = v.st->n_warp, below = (1u << lane) - 1u;
+    const uint32_t n = fb_aborted(v) ? 0u : v.st->n_warp, below = (1u << lane) - 1u;
     for (uint32_t k = blockIdx.x * kRankWarps + warp; k < n; k += gridDim.x * kRankWarps) {
         const uint32_t eid = v.listed_big[(uint32_t)v.LC - 1 - k], nw = v.grp_n[eid];
         const uint32_t* const wp = v.wpos + v.grp_off[eid];
@@ -1013,7 +1019,7 @@ __global__ void __launch_bounds__(32 * kRankWarps) fb_rank_warp_kernel(BuildView
 __global__ void __launch_bounds__(256) fb_rank_kernel(BuildView v, CbTables t) {
     fb_rank_begin();
     const int lane = threadIdx.x & 31;
-    const uint32_t n = min(v.st->n_sel, (uint32_t)v.LC), nw = gridDim.x * 8;
+    const uint32_t n = fb_aborted(v) ? 0u : min(v.st->n_sel, (uint32_t)v.LC), nw = gridDim.x * 8;
     const bool short_tokens = v.st->max_token < (1u << 26);
     uint32_t eid = blockIdx.x * 8 + (threadIdx.x >> 5);
     // windows of leader e for this warp (0: another kernel's) and this lane's position
@@ -1132,8 +1138,8 @@ extern "C" cb_status cb_frozen_build_bytes(const cb_frozen_config* cfg, int64_t 
     return CB_OK;
 }
 
-extern "C" cb_status cb_frozen_build(const cb_frozen_config* cfg, const int32_t* dev_corpus, int64_t n_tokens, void* dev_table,
-                                     size_t table_bytes, void* dev_scratch, size_t scratch_bytes, void* stream) {
+static cb_status frozen_build(const cb_frozen_config* cfg, const int32_t* dev_corpus, int64_t n_tokens, void* dev_table,
+                              size_t table_bytes, void* dev_scratch, size_t scratch_bytes, void* stream, uint32_t wait_limit) {
     CbFrozenLayout L;
     BuildLayout B;
     cb_status s = cb_frozen_layout(cfg, &L);
@@ -1160,6 +1166,7 @@ extern "C" cb_status cb_frozen_build(const cb_frozen_config* cfg, const int32_t*
     const int64_t M = n_tokens - cfg->LL - cfg->FL + 1;
     v.M = (uint32_t)(M > 0 ? M : 0);
     v.n_tokens = (uint32_t)n_tokens;
+    v.wait_limit = wait_limit;
     v.LL = cfg->LL; v.FL = cfg->FL; v.LC = cfg->LC; v.FC = cfg->FC;
     int dev = 0, sms = 0;
     CB_CUDA(cudaGetDevice(&dev));
@@ -1206,3 +1213,16 @@ extern "C" cb_status cb_frozen_build(const cb_frozen_config* cfg, const int32_t*
     CB_CUDA(cudaStreamSynchronize(st));
     return (cb_status)status;
 }
+
+extern "C" cb_status cb_frozen_build(const cb_frozen_config* cfg, const int32_t* dev_corpus, int64_t n_tokens, void* dev_table,
+                                     size_t table_bytes, void* dev_scratch, size_t scratch_bytes, void* stream) {
+    return frozen_build(cfg, dev_corpus, n_tokens, dev_table, table_bytes, dev_scratch, scratch_bytes, stream, 1u << 24);
+}
+
+#ifdef CB_DEBUG
+// Checking build only: the same with the number of looks that a block of the selection takes at a barrier (0: it gives up at once).
+extern "C" cb_status cb_debug_frozen_build(const cb_frozen_config* cfg, const int32_t* dev_corpus, int64_t n_tokens, void* dev_table,
+                                           size_t table_bytes, void* dev_scratch, size_t scratch_bytes, void* stream, uint32_t wait_limit) {
+    return frozen_build(cfg, dev_corpus, n_tokens, dev_table, table_bytes, dev_scratch, scratch_bytes, stream, wait_limit);
+}
+#endif

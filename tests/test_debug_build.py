@@ -70,6 +70,41 @@ torch.cuda.synchronize()
 st, _ = cb.cb_poll_status()
 assert st == _lib.CB_ERR_INVALID_ARG, st
 assert torch.isfinite(out.float()).all()
+# a selection of the frozen builder that gives up at its first barrier: the call says so, and nothing behind it goes by what is missing
+import ctypes as C
+from oracle import cb_oracle
+L = _lib.load()
+L.cb_debug_frozen_build.argtypes = L.cb_frozen_build.argtypes + [C.c_uint32]
+L.cb_debug_frozen_build.restype = C.c_int32
+N, LL, FL, LC, FC = 20000, 2, 3, 1 << 15, 4
+corpus = np.random.default_rng(3).integers(0, 200, N).astype(np.int32)
+fc = _lib.CbFrozenConfigC(LL, FL, LC, FC)
+tb, sb = C.c_size_t(0), C.c_size_t(0)
+assert L.cb_frozen_bytes(C.byref(fc), C.byref(tb)) == 0 and L.cb_frozen_build_bytes(C.byref(fc), N, C.byref(sb)) == 0
+table = torch.empty(tb.value, dtype=torch.uint8, device="cuda")
+scratch = torch.full((sb.value,), 0xA5, dtype=torch.uint8, device="cuda")           # ranges that nobody wrote point far outside
+assert table.data_ptr() %% 256 == 0 and scratch.data_ptr() %% 256 == 0
+d = dev(corpus)
+args = (C.byref(fc), d.data_ptr(), N, table.data_ptr(), tb.value, scratch.data_ptr(), sb.value, torch.cuda.current_stream().cuda_stream)
+assert L.cb_debug_frozen_build(*args, 0) == 5                                       # CB_ERR_TIMEOUT
+# the windows' array: the last third of the region before the leaders' four words each at the scratch's end
+S = 1024
+while S < 2 * (N - LL - FL + 1):
+    S *= 2
+up = lambda x: (x + 255) // 256 * 256
+wpos = sb.value - up(LC * 16) - up(S * 6) + S * 4
+assert bool((scratch[wpos:wpos + S * 2] == 0xA5).all())
+assert bool((scratch[sb.value - up(LC * 16) + LC * 4:sb.value - up(LC * 16) + LC * 8] == 0xA5).all())       # no range was given out
+bad = dev(np.concatenate([[-1], corpus[1:]]).astype(np.int32))                      # reported even where a negative token was recorded first
+assert L.cb_debug_frozen_build(args[0], bad.data_ptr(), *args[2:], 0) == 5
+assert L.cb_frozen_build(*args) == 0
+nl = C.c_int32(0)
+lead, nf, fol = np.zeros((LC, LL), np.int32), np.zeros(LC, np.int32), np.zeros((LC, FC, FL), np.int32)
+ip = lambda a: a.ctypes.data_as(C.c_void_p)
+assert L.cb_frozen_dump(args[0], table.data_ptr(), tb.value, C.byref(nl), ip(lead), ip(nf), ip(fol)) == 0
+oL, onf, oF = cb_oracle.frozen_build(corpus, LL, FL, LC, FC)
+n = nl.value
+assert n == len(oL) and np.array_equal(lead[:n], oL) and np.array_equal(nf[:n], onf) and np.array_equal(fol[:n], oF)
 print("checking build ok")
 """
 

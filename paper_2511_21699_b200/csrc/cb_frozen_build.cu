@@ -51,6 +51,7 @@ struct BuildState {                           // head of the scratch buffer
     uint32_t cursor, big_cursor;              // next free place of the window array, of the group array (the big leaders' windows)
     uint32_t arrived;                         // blocks of the selection that have come to its barriers so far
     uint32_t aborted;                         // a block has given up on such a barrier: what the later kernels read is incomplete
+    uint32_t grouped;                         // kGo: step 3 is over and can be read (kGaveUp: it was not done)
     uint32_t max_token;                       // largest token of the corpus
     uint32_t has_neg;                         // some token is negative
     alignas(16) uint32_t hist[kMaxPasses][kBins];   // one histogram per pass of the selection (read 16 bytes at a time)
@@ -789,8 +790,26 @@ __device__ void pick_followers(const BuildView& v, const CbTables& t, uint32_t e
 
 // The five kernels of step 4 touch different leaders and depend on nothing but step 3, which is over when the first of them lets
 // the others start: so each of them starts as SMs become free and waits for the one before it only at its end (the stream's next
-// kernel is ordered behind the last of them only).
-__device__ __forceinline__ void fb_rank_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// kernel is ordered behind the last of them only).  A kernel that has not waited yet is promised nothing of what ran before it, so the
+// first one, which has, hands step 3 on with a release that every block of the others acquires; it is set when they start, but for a moment.
+constexpr uint32_t kGo = 1u, kGaveUp = 2u;
+__device__ __forceinline__ void fb_hand_on(const BuildView& v) {
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&v.st->grouped), "r"(fb_aborted(v) ? kGaveUp : kGo) : "memory");
+}
+__device__ __forceinline__ bool fb_rank_begin(const BuildView& v) {   // false: nothing to rank
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    __shared__ uint32_t s_go;
+    if (threadIdx.x == 0) {
+        uint32_t x = 0u;
+        for (uint32_t k = 0; k < (1u << 24) && x == 0u; ++k)
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(&v.st->grouped) : "memory");
+        if (x == 0u) atomicExch(&v.st->status, (uint32_t)CB_ERR_TIMEOUT);
+        s_go = x;
+    }
+    __syncthreads();
+    return s_go == kGo;
+}
 __device__ __forceinline__ void fb_rank_end() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // the big leaders, a block each
@@ -799,6 +818,7 @@ __global__ void __launch_bounds__(1024) fb_rank_big_kernel(BuildView v, CbTables
     __shared__ Candidates cand;
     __shared__ uint32_t red[32];
     const Crew<1024> crew = {red};
+    fb_hand_on(v);
     const uint32_t n = fb_aborted(v) ? 0u : v.st->n_big;
     for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
         const uint32_t eid = v.listed_big[k];
@@ -811,7 +831,7 @@ __global__ void __launch_bounds__(1024) fb_rank_big_kernel(BuildView v, CbTables
 // through a table there (a word per slot: index of the first claimant + 1, count).
 template <int NT, int CAP>
 __global__ void __launch_bounds__(NT) fb_rank_block_kernel(BuildView v, CbTables t, uint32_t n_leaders_at) {
-    fb_rank_begin();
+    const bool go = fb_rank_begin(v);
     extern __shared__ uint32_t fb_smem[];
     uint32_t* const tab = fb_smem;                               // [2 CAP], then the distinct windows at its front
     int32_t* const tok = reinterpret_cast<int32_t*>(tab + 2 * CAP); // [CAP][FL]
@@ -819,7 +839,7 @@ __global__ void __launch_bounds__(NT) fb_rank_block_kernel(BuildView v, CbTables
     __shared__ uint32_t red[NT / 32], n_dist;
     const Crew<NT> crew = {red};
     const int me = (int)threadIdx.x, lane = me & 31;
-    const uint32_t n = fb_aborted(v) ? 0u : n_leaders_at ? v.st->n_large : v.st->n_mid;
+    const uint32_t n = !go ? 0u : n_leaders_at ? v.st->n_large : v.st->n_mid;
     for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
         const uint32_t eid = v.listed[n_leaders_at ? (uint32_t)v.LC - 1 - k : k], nw = v.grp_n[eid];
         const uint32_t* const wp = v.wpos + v.grp_off[eid];
@@ -874,13 +894,13 @@ __global__ void __launch_bounds__(NT) fb_rank_block_kernel(BuildView v, CbTables
 // table in shared memory and the counts in registers.  A block of 128 threads took 12 us a leader.
 constexpr int kRankWarps = 8;
 __global__ void __launch_bounds__(32 * kRankWarps) fb_rank_warp_kernel(BuildView v, CbTables t) {
-    fb_rank_begin();
+    const bool go = fb_rank_begin(v);
     constexpr int PER = kWarpGroup / 32;
     extern __shared__ uint32_t fb_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* const tab = fb_smem + warp * (kWarpGroup * (2 + v.FL));      // [2 kWarpGroup]: index of the first claimant + 1, count
     int32_t* const tok = reinterpret_cast<int32_t*>(tab + 2 * kWarpGroup); // [kWarpGroup][FL]
-    const uint32_t n = fb_aborted(v) ? 0u : v.st->n_warp, below = (1u << lane) - 1u;
+    const uint32_t n = !go ? 0u : v.st->n_warp, below = (1u << lane) - 1u;
     for (uint32_t k = blockIdx.x * kRankWarps + warp; k < n; k += gridDim.x * kRankWarps) {
         const uint32_t eid = v.listed_big[(uint32_t)v.LC - 1 - k], nw = v.grp_n[eid];
         const uint32_t* const wp = v.wpos + v.grp_off[eid];
@@ -1017,10 +1037,10 @@ __global__ void __launch_bounds__(32 * kRankWarps) fb_rank_warp_kernel(BuildView
 
 // the common case, up to 32 windows: a warp per leader, a lane per window; the next leader's range is looked up while this one is ranked
 __global__ void __launch_bounds__(256) fb_rank_kernel(BuildView v, CbTables t) {
-    fb_rank_begin();
+    const bool go = fb_rank_begin(v);
     const int lane = threadIdx.x & 31;
-    const uint32_t n = fb_aborted(v) ? 0u : min(v.st->n_sel, (uint32_t)v.LC), nw = gridDim.x * 8;
-    const bool short_tokens = v.st->max_token < (1u << 26);
+    const uint32_t n = !go ? 0u : min(v.st->n_sel, (uint32_t)v.LC), nw = gridDim.x * 8;
+    const bool short_tokens = go && v.st->max_token < (1u << 26);
     uint32_t eid = blockIdx.x * 8 + (threadIdx.x >> 5);
     // windows of leader e for this warp (0: another kernel's) and this lane's position
     auto range_of = [&](uint32_t e, uint32_t* pos) {

@@ -13,7 +13,8 @@ __global__ void __launch_bounds__(256) cb_accept_logits_kernel(
     int32_t* __restrict__ n_accept, int32_t* __restrict__ accept_nodes, int32_t* __restrict__ out_tokens,
     int32_t* __restrict__ target_out) {
     CB_PDL_ENTRY();
-    accept_rows<BF16, UN>(T, V, Dmax, chunk, chunks_per_row, logits, row_stride, tok, par, dep, n_nodes, rowmax, ticket, n_accept, accept_nodes,
+    const int n = min(max(n_nodes[blockIdx.z], 0), T);
+    accept_rows<BF16, UN>(T, V, Dmax, chunk, chunks_per_row, logits, row_stride, tok, par, dep, n, rowmax, ticket, n_accept, accept_nodes,
                           out_tokens, target_out, [](int) {});
 }
 

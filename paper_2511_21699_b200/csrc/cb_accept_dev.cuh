@@ -160,18 +160,17 @@ __device__ __noinline__ void accept_walk(int b, int Dmax, const int32_t* tk, con
 // The work of one CTA of the acceptance grid (row chunk ck = blockIdx.x, node i = blockIdx.y, sequence b = blockIdx.z): its
 // chunk of the node's logits row is reduced into the row's packed maximum; the last CTA of the sequence to arrive turns the
 // maxima into the target's tokens, walks the tree and writes the result.  Returns true in that CTA (all its threads), after
-// the result has been written; false in all others.  beside(k): what the threads from 128 on (k = 0 ...) of that CTA do meanwhile.
+// the result has been written; false in all others.  n: nodes of the sequence's tree.  beside(k): what the threads from 128 on (k = 0 ...) of that CTA do meanwhile.
 // UN: 16-byte loads in flight per thread.  A grid that is resident at once is as long as its chain of round trips and takes all of
 // its 32 KB chunk (8 loads a thread) at once; a larger one has enough in flight with 4 and needs the registers for more CTAs.
 template <bool BF16, int UN, typename Beside>
 __device__ __forceinline__ bool accept_rows(
     int T, int V, int Dmax, int chunk, int chunks_per_row, const void* __restrict__ logits, int64_t row_stride,
     const int32_t* __restrict__ tok, const int32_t* __restrict__ par, const int32_t* __restrict__ dep,
-    const int32_t* __restrict__ n_nodes, unsigned long long* rowmax, uint32_t* ticket,
+    int n, unsigned long long* rowmax, uint32_t* ticket,
     int32_t* __restrict__ n_accept, int32_t* __restrict__ accept_nodes, int32_t* __restrict__ out_tokens,
     int32_t* __restrict__ target_out, Beside&& beside, int32_t* emit = nullptr, int* have = nullptr) {
     const int b = blockIdx.z, i = blockIdx.y, ck = blockIdx.x, tid = threadIdx.x;
-    const int n = min(max(n_nodes[b], 0), T);
     // Rows past the tree have nothing to add and do not queue for the ticket either (hundreds of atomics on one word at
     // batch 1); an empty tree keeps row 0's CTAs, one of which writes the empty result.
     if (i >= max(n, 1)) return false;

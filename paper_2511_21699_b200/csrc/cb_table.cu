@@ -605,13 +605,13 @@ constexpr int kDraftArrays = 6;                               // of NL words
 
 // The work of the CTA that drafts sequence b, whose history holds L tokens.  upd_n_old >= 0: the windows that the tokens
 // from upd_n_old on complete are inserted first (cb_update_draft_tree and the call that follows an acceptance).  row(i): token i of
-// the history (which this CTA may have extended just before).
-template <int FETCH, typename Tokens>
+// the history (which this CTA may have extended just before).  put_n(n): stores the new tree's node count (one thread, at the end).
+template <int FETCH, typename Tokens, typename PutN>
 __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf, int T, int crt, int max_depth, int NL, int KF,
                                            const Tokens& row, int b, int L, int upd_n_old,
                                            int32_t* __restrict__ o_tok, int32_t* __restrict__ o_par,
                                            int32_t* __restrict__ o_dep, uint32_t* __restrict__ o_mask,
-                                           int32_t* __restrict__ o_n, uint32_t* status,
+                                           PutN&& put_n, uint32_t* status,
                                            unsigned long long* counters, int32_t* smem) {
     DraftSmem S;
     const int W = (T + 31) >> 5;
@@ -910,7 +910,7 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
     const int n = sh_n[cur];
     if (tid == 0) {
         s.hdr[0] = clock0 + (uint32_t)q;
-        o_n[b] = n;
+        put_n(n);
         if (q) atomicAdd(&counters[CB_CNT_QUERIES], (unsigned long long)q);
         if (hits) atomicAdd(&counters[CB_CNT_QUERY_HITS], (unsigned long long)hits);
         if (fq) atomicAdd(&counters[CB_CNT_FROZEN_QUERIES], (unsigned long long)fq);
@@ -936,7 +936,7 @@ __global__ void __launch_bounds__(256) cb_draft_kernel(CbTables t, CbTables tf, 
     const int b = blockIdx.x;
     const int32_t* history = tokens + (size_t)b * row_stride;
     draft_body<FETCH>(t, tf, T, crt, max_depth, NL, KF, [=](int i) { return history[i]; }, b, seq_len[b], upd_n_old ? upd_n_old[b] : -1, o_tok, o_par,
-                      o_dep, o_mask, o_n, status, counters, smem);
+                      o_dep, o_mask, [=](int n) { o_n[b] = n; }, status, counters, smem);
 }
 
 // Acceptance of one step and update + draft of the next in one launch (the three are a chain per sequence: Fig. 2).  The
@@ -955,7 +955,14 @@ struct AcceptArgs {
 // of 72, 82.9 with four; batch 4 of 64: 61.3 and 59.6); one that is gains nothing from the bound and pays for it in the chain behind
 // the logits, and takes all of a thread's chunk at once instead.  With more than 32 followers a leader the code takes 109 registers and
 // stays at two.
-template <int FETCH, bool BF16, int CTAS>
+//
+// IN_PLACE: o_n is a.n_nodes.  Which rows a sequence's tree has decides which of its CTAs count for the acceptance, so its entry is stored only
+// when every CTA of the sequence has read the old one: those of the tree's rows have when the drafting CTA begins; those of the rows
+// past it (`waiting` of them) and the drafting CTA count themselves in a word of their own, and the last to come stores.  The word is the
+// packed maximum of row T - 1, which such a tree does not have: arrivals below, the new count above, zero between launches.  A CTA
+// that started late would otherwise take its row for one of the tree and leave a maximum and a ticket behind for the next launch.
+// (A form of its own: in the other one the two words that it keeps to the end cost a grid of four CTAs an SM 1.5% and batch 2 7%.)
+template <int FETCH, bool BF16, int CTAS, bool IN_PLACE>
 __global__ void __launch_bounds__(256, CTAS) cb_accept_draft_kernel(AcceptArgs a, CbTables t, CbTables tf, int T, int crt, int max_depth, int NL, int KF,
                                                               int32_t* tokens, int64_t row_stride, int32_t* seq_len,
                                                               int32_t* o_tok, int32_t* o_par, int32_t* o_dep, uint32_t* o_mask, int32_t* o_n,
@@ -967,6 +974,24 @@ __global__ void __launch_bounds__(256, CTAS) cb_accept_draft_kernel(AcceptArgs a
     __shared__ int32_t s_tail[CB_MAX_LL + CB_MAX_FL + 256], s_emit[256];
     __shared__ int s_have, s_len;
     const int b = blockIdx.z, tid = threadIdx.x, w = t.LL + t.FL;
+    const int n_old = min(max(a.n_nodes[b], 0), T);             // through L1: past it, thousands of warps at one word are a microsecond and more
+    uint32_t waiting = 0u;
+    auto arrive = [&](unsigned long long x) {
+        unsigned long long* const word = a.rowmax + (size_t)b * T + T - 1;
+        unsigned long long now;
+        asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;" : "=l"(now) : "l"(word), "l"(x) : "memory");
+        now += x;
+        if ((uint32_t)now == waiting + 1u) { o_n[b] = (int32_t)(now >> 32); *word = 0ull; }
+    };
+    if constexpr (IN_PLACE) {
+        const int rows = max(n_old, 1);
+        waiting = (uint32_t)(T - rows) * gridDim.x;
+        __syncthreads();                                        // all threads of this CTA have read the count
+        if ((int)blockIdx.y >= rows) {
+            if (tid == 0) arrive(1ull);
+            return;
+        }
+    }
     int32_t* const history = tokens + (size_t)b * row_stride;
     auto beside = [&](int k) {
         if (k >= 32) return;
@@ -975,7 +1000,7 @@ __global__ void __launch_bounds__(256, CTAS) cb_accept_draft_kernel(AcceptArgs a
         if (k == 0) s_len = L;
     };
     if (!accept_rows<BF16, CTAS == 2 && FETCH == 1 ? 8 : 4>(T, a.V, a.Dmax, a.chunk, a.chunks_per_row, a.logits, a.logits_row_stride, a.tok, a.par, a.dep,
-                                                            a.n_nodes, a.rowmax, a.ticket, a.n_accept, a.accept_nodes, a.out_tokens, a.target_out, beside,
+                                                            n_old, a.rowmax, a.ticket, a.n_accept, a.accept_nodes, a.out_tokens, a.target_out, beside,
                                                             s_emit, &s_have))
         return;
     __syncthreads();                                            // the walk (first warp) has written the sequence's result
@@ -993,7 +1018,10 @@ __global__ void __launch_bounds__(256, CTAS) cb_accept_draft_kernel(AcceptArgs a
     __syncthreads();
     if (tid == 0) seq_len[b] = L1;
     draft_body<FETCH>(t, tf, T, crt, max_depth, NL, KF, [&](int i) { return i >= tail0 && L <= row_stride ? s_tail[i - tail0] : history[i]; }, b, L1, L,
-                      o_tok, o_par, o_dep, o_mask, o_n, status, counters, smem);
+                      o_tok, o_par, o_dep, o_mask, [&](int n) {
+                          if (IN_PLACE && waiting) arrive((unsigned long long)n << 32 | 1ull);
+                          else o_n[b] = n;
+                      }, status, counters, smem);
 }
 
 }  // namespace
@@ -1179,14 +1207,19 @@ extern "C" cb_status cb_accept_update_draft_tree(cb_ctx* ctx, const cb_accept_dr
     if (smem > 200 * 1024) return CB_ERR_UNSUPPORTED;
     const bool bf = a->logits_dtype == CB_DTYPE_BF16;
     const bool resident = (long long)cpr * T * c.batch <= 2ll * ctx->num_sms;
-    auto kernel = FCmax > 32  ? (bf ? cb_accept_draft_kernel<2, true, 2> : cb_accept_draft_kernel<2, false, 2>)
-                  : resident  ? (bf ? cb_accept_draft_kernel<1, true, 2> : cb_accept_draft_kernel<1, false, 2>)
-                              : (bf ? cb_accept_draft_kernel<1, true, 4> : cb_accept_draft_kernel<1, false, 4>);
+    // [form][bf16][in place]
+    using Kernel = decltype(&cb_accept_draft_kernel<1, false, 2, false>);
+    static const Kernel kernels[3][2][2] = {
+        {{cb_accept_draft_kernel<2, false, 2, false>, cb_accept_draft_kernel<2, false, 2, true>}, {cb_accept_draft_kernel<2, true, 2, false>, cb_accept_draft_kernel<2, true, 2, true>}},
+        {{cb_accept_draft_kernel<1, false, 2, false>, cb_accept_draft_kernel<1, false, 2, true>}, {cb_accept_draft_kernel<1, true, 2, false>, cb_accept_draft_kernel<1, true, 2, true>}},
+        {{cb_accept_draft_kernel<1, false, 4, false>, cb_accept_draft_kernel<1, false, 4, true>}, {cb_accept_draft_kernel<1, true, 4, false>, cb_accept_draft_kernel<1, true, 4, true>}}};
+    const int form = FCmax > 32 ? 0 : resident ? 1 : 2, in_place = a->next_n_nodes == a->n_nodes ? 1 : 0;
+    const Kernel kernel = kernels[form][bf][in_place];
     {
         static std::mutex mu;
-        static size_t have[64][6] = {};                        // per device and kernel
+        static size_t have[64][3][2][2] = {};                  // per device and kernel
         std::lock_guard<std::mutex> lock(mu);
-        CB_CUDA(cb_allow_smem(kernel, smem, &have[ctx->device & 63][(FCmax > 32 ? 0 : resident ? 2 : 4) + (bf ? 1 : 0)]));
+        CB_CUDA(cb_allow_smem(kernel, smem, &have[ctx->device & 63][form][bf][in_place]));
     }
     CbTables tf = {};
     if (ctx->has_frozen) tf = ctx->frozen;

@@ -25,10 +25,14 @@ def _stale(target, deps):
 
 
 def build_binding(force=False):
-    src = os.path.join(CSRC, "cb_binding.cpp")
-    if not force and not _stale(SO_BINDING, [src, os.path.join(ROOT, "include", "cacheback.h")]):
-        return SO_BINDING
     import torch
+    src = os.path.join(CSRC, "cb_binding.cpp")
+    # The module is tied to torch's C++ classes and to the interpreter, so what it was built against lies beside it.
+    against = "torch %s, %s, C++11 ABI %d\n" % (torch.__version__, sys.implementation.cache_tag, int(torch._C._GLIBCXX_USE_CXX11_ABI))
+    stamp = SO_BINDING + ".stamp"
+    built = open(stamp).read() if os.path.exists(stamp) else None
+    if not force and built == against and not _stale(SO_BINDING, [src, os.path.join(ROOT, "include", "cacheback.h"), os.path.abspath(__file__)]):
+        return SO_BINDING
     t = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
     inc = [os.path.join(ROOT, "include"), os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
@@ -38,6 +42,9 @@ def build_binding(force=False):
                           [x for i in inc for x in ("-isystem" if i.startswith(t) else "-I", i)] +
                           [src, "-o", tmp, "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
     os.replace(tmp, SO_BINDING)
+    with open(stamp + ".tmp%d" % os.getpid(), "w") as f:
+        f.write(against)
+    os.replace(stamp + ".tmp%d" % os.getpid(), stamp)
     return SO_BINDING
 
 

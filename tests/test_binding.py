@@ -60,3 +60,29 @@ def test_arguments_of_the_wrong_number_or_kind(host):
         host.reset(C.c_void_p(None), None, object())             # not a stream
     with pytest.raises(KeyError):
         host.accept(C.c_void_p(None), {}, None, None, {}, _Stream())
+
+
+def test_module_is_built_again_for_another_torch_or_interpreter(monkeypatch, tmp_path):
+    """File times say nothing of what the module was compiled against."""
+    import os
+    import sys
+    import types
+    from paper_2511_21699_b200 import build
+    calls = []
+
+    def compiler(cmd, **kw):
+        calls.append(cmd)
+        open(cmd[cmd.index("-o") + 1], "w").close()
+    monkeypatch.setattr(build, "SO_BINDING", str(tmp_path / "_binding.so"))
+    monkeypatch.setattr(build.subprocess, "check_call", compiler)
+    for want in (1, 1):                                         # built once, then found as it is
+        build.build_binding()
+        assert len(calls) == want
+    monkeypatch.setattr(torch, "__version__", torch.__version__ + ".other")
+    build.build_binding()
+    build.build_binding()
+    assert len(calls) == 2
+    tag = types.SimpleNamespace(**dict(vars(sys.implementation), cache_tag="cpython-other"))
+    monkeypatch.setattr(build.sys, "implementation", tag)
+    build.build_binding()
+    assert len(calls) == 3 and os.path.exists(build.SO_BINDING)

@@ -8,6 +8,8 @@
 // (a stride of a tensor without dimensions, a tensor without memory) pass through as they do there.
 #include <Python.h>
 
+#include <algorithm>
+
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -133,6 +135,17 @@ PyObject* entry(PyObject*, PyObject* const* a, Py_ssize_t n) {
     END_HANDLE_TH_ERRORS
 }
 
+// The token history [batch, columns]: its pointer and the columns that a row has.  The stride of a dimension of size one says nothing:
+// the transpose of a [columns, 1] tensor is contiguous with a stride of 1.
+template <typename T = int32_t>
+T* history_of(PyObject* o, int64_t* row_stride) {
+    T* p = ptr<T>(o);
+    const at::Tensor& t = tensor_of(o);
+    *row_stride = t.stride(0);
+    if (t.dim() > 1 && t.size(0) == 1) *row_stride = std::max(*row_stride, t.numel());
+    return p;
+}
+
 // handle, seq_mask, stream
 void do_reset(PyObject* const* a) {
     cb_ctx* c = ctx_of(a[0]);
@@ -144,8 +157,8 @@ void do_reset(PyObject* const* a) {
 template <bool BULK>
 void do_update(PyObject* const* a) {
     cb_ctx* c = ctx_of(a[0]);
-    const int32_t* tok = ptr(a[1]);
-    const int64_t rs = tensor_of(a[1]).stride(0);
+    int64_t rs;
+    const int32_t* tok = history_of(a[1], &rs);
     const int32_t *n0 = ptr(a[2]), *n1 = ptr(a[3]);
     void* st = stream_of(a[4]);
     call(BULK ? "cb_update_bulk" : "cb_update", [&] { return (BULK ? g_lib.update_bulk : g_lib.update)(c, tok, rs, n0, n1, st); });
@@ -161,8 +174,8 @@ Tree tree_of(PyObject* t, bool mask) {
 // handle, tokens, seq_len, tree, stream
 void do_draft(PyObject* const* a) {
     cb_ctx* c = ctx_of(a[0]);
-    const int32_t* tok = ptr(a[1]);
-    const int64_t rs = tensor_of(a[1]).stride(0);
+    int64_t rs;
+    const int32_t* tok = history_of(a[1], &rs);
     const int32_t* n = ptr(a[2]);
     const Tree t = tree_of(a[3], true);
     void* st = stream_of(a[4]);
@@ -171,8 +184,8 @@ void do_draft(PyObject* const* a) {
 // handle, tokens, n_old, n_new, tree, stream
 void do_update_draft(PyObject* const* a) {
     cb_ctx* c = ctx_of(a[0]);
-    const int32_t* tok = ptr(a[1]);
-    const int64_t rs = tensor_of(a[1]).stride(0);
+    int64_t rs;
+    const int32_t* tok = history_of(a[1], &rs);
     const int32_t *n0 = ptr(a[2]), *n1 = ptr(a[3]);
     const Tree t = tree_of(a[4], true);
     void* st = stream_of(a[5]);
@@ -199,8 +212,7 @@ void do_accept_update_draft(PyObject* const* a) {
     x.tree_tokens = t.tok; x.tree_parent = t.par; x.tree_depth = t.dep; x.n_nodes = t.n;
     x.n_accept = item(a[6], s_n_accept); x.accept_nodes = item(a[6], s_accept_nodes);
     x.out_tokens = item(a[6], s_out_tokens); x.target_ids_out = item(a[6], s_target_ids);
-    x.tokens = ptr(a[3]);
-    x.row_stride = tensor_of(a[3]).stride(0);
+    x.tokens = history_of(a[3], &x.row_stride);
     x.seq_len = ptr(a[4]);
     const Tree n = tree_of(a[5], true);
     x.next_tokens = n.tok; x.next_parent = n.par; x.next_depth = n.dep; x.next_mask = n.mask; x.next_n_nodes = n.n;

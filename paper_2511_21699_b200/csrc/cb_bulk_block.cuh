@@ -104,11 +104,12 @@ __device__ __forceinline__ uint32_t blk_parts(uint32_t nwin, uint32_t spare, uin
     return max(min(share, max(nwin / 32u, 1u)), (nwin + kBlkPart - 1u) / kBlkPart);
 }
 
+// alone: no other kernel follows, so that no run may be longer than kBlkRun windows.
 // LL: the leader's tokens, FLX: a bound of the follower's (4 or 8), so that the loops over a window's tokens are straight code.
 template <int LL, int FLX>
 __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(CbTables t, int B, const int32_t* __restrict__ tokens, int64_t row_stride,
                                                                            const int32_t* __restrict__ n_old, const int32_t* __restrict__ n_new,
-                                                                           uint32_t* status, unsigned long long* counters) {
+                                                                           bool alone, uint32_t* status, unsigned long long* counters) {
     extern __shared__ __align__(16) unsigned char blk_smem[];
     BlkSmem& S = *reinterpret_cast<BlkSmem*>(blk_smem);
     auto clear_tables = [&] {
@@ -126,7 +127,10 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
             const uint2 h = *reinterpret_cast<const uint2*>(cb_seq(t, tid).hdr);
             const int first = max(0, n_old[tid] - w + 1);
             nwin = (uint32_t)max(0, n_new[tid] - w + 1 - first);
-            if (nwin > (uint32_t)kBlkRun) nwin = 0;             // left to the kernels after this one
+            if (nwin > (uint32_t)kBlkRun) {                     // left to the kernels after this one, or longer than its row
+                nwin = 0;
+                if (alone && blockIdx.x == 0) atomicCAS(status, 0u, (uint32_t)CB_ERR_INVALID_ARG);
+            }
             S.nwin[tid] = (uint16_t)nwin; S.first[tid] = first; S.clock[tid] = h.x; S.count[tid] = h.y;
         }
         (void)blk_scan(nwin, S.red, &all);

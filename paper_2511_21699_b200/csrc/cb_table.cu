@@ -1042,8 +1042,11 @@ extern "C" cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t 
     const int B = ctx->cfg.batch;
     int done = -1;
     if (ctx->tables.refresh && B <= kBlkMaxBatch) {
-        // Runs of up to kBlkRun windows by blocks that hold them in shared memory.  A row that has no room for more needs nothing else.
-        using Kernel = void (*)(CbTables, int, const int32_t*, int64_t, const int32_t*, const int32_t*, uint32_t*, unsigned long long*);
+        // Runs of up to kBlkRun windows by blocks that hold them in shared memory.  A row that has no room for more needs nothing else.  (A row
+        // without room for a window is a stride that means nothing: that of a batch of one.)
+        const int w = ctx->tables.LL + ctx->tables.FL;
+        const bool alone = row_stride >= w && row_stride - w + 1 <= (int64_t)kBlkRun;
+        using Kernel = void (*)(CbTables, int, const int32_t*, int64_t, const int32_t*, const int32_t*, bool, uint32_t*, unsigned long long*);
         static const Kernel kernels[CB_MAX_LL][2] = {{cb_update_bulk_block_kernel<1, 4>, cb_update_bulk_block_kernel<1, 8>},
                                                      {cb_update_bulk_block_kernel<2, 4>, cb_update_bulk_block_kernel<2, 8>},
                                                      {cb_update_bulk_block_kernel<3, 4>, cb_update_bulk_block_kernel<3, 8>},
@@ -1061,10 +1064,10 @@ extern "C" cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t 
             }
         }
         CB_CUDA(cb_launch_pdl(kernel, dim3((unsigned)ctx->num_sms), dim3(kBlkThreads), sizeof(BlkSmem), (cudaStream_t)stream, ctx->tables, B, tokens,
-                              row_stride, n_old, n_new, ctx->d_status, ctx->d_counters));
+                              row_stride, n_old, n_new, alone, ctx->d_status, ctx->d_counters));
         cb_count_launch(1);
         done = kBlkRun;
-        if (row_stride - (ctx->tables.LL + ctx->tables.FL) + 1 <= (int64_t)kBlkRun) return CB_OK;
+        if (alone) return CB_OK;
     }
     // enough warps per sequence to fill the GPU at small batch, fewer at large batch
     int wps = 1;

@@ -68,3 +68,41 @@ def test_bulk_runs_in_blocks(oracle, LL, FL, LC, FC, kind, first, second, scratc
         tabs[b].update(toks[b], 0, int(n1[b]))
     _assert_tables_equal(cb, tabs, check)
     assert cb.cb_poll_status()[0] == 0
+
+
+@pytest.mark.parametrize("form", ["rows", "transposed", "strided", "flat"])
+def test_one_sequence_whatever_its_stride(oracle, form):
+    """A batch of one: the stride of its only row means nothing, and a run longer than a block takes is not lost by it."""
+    from paper_2511_21699_b200 import Cacheback
+    LL, FL, LC, FC, n = 2, 3, 16384, 4, 10000
+    toks = _tokens("zipf", 1, n, np.random.default_rng(9))
+    d = dev(toks)
+    d = dict(rows=d, transposed=d.reshape(n, 1).clone().t(), strided=torch.as_strided(d, (1, n), (77, 1)), flat=d[0])[form]
+    assert d.is_contiguous() and (form == "rows") == (d.stride(0) == n)
+    cb = Cacheback(1, LL, FL, LC, FC, 32, 8, 8, 500, 8, 8, 64)
+    zero, n1, n2 = (dev(np.array([x], np.int32)) for x in (0, 9000, 9500))
+    tab = oracle.OracleTable(LL, FL, LC, FC)
+    cb.cb_update_bulk(d, zero, n1)
+    tab.update(toks[0], 0, 9000)
+    _assert_tables_equal(cb, {0: tab}, [0])
+    cb.cb_update_bulk(d, n1, n2)
+    tab.update(toks[0], 9000, 9500)
+    _assert_tables_equal(cb, {0: tab}, [0])
+    assert cb.cb_poll_status()[0] == 0
+    if form != "flat":                                          # the call that appends to the row takes its room from the tensor too
+        tree = cb.cb_draft_tree(d, n2)
+        logits = torch.zeros(1, 32, 500, device="cuda")
+        logits[..., 3] = 1.0
+        cb.cb_accept_update_draft_tree(tree, logits, d, n2)
+        assert cb.cb_poll_status()[0] == 0 and int(n2[0]) > 9500
+
+
+def test_run_longer_than_its_row_is_reported():
+    """n_new beyond the row of several: the windows that no kernel is left to take are reported."""
+    from paper_2511_21699_b200 import Cacheback
+    cb = Cacheback(3, 2, 3, 16384, 4, 32, 8, 8, 500, 8, 8, 64)
+    t = torch.zeros(3, 8000, dtype=torch.int32, device="cuda")
+    n = dev(np.array([100, 9000, 100], np.int32))
+    cb.cb_update_bulk(t, torch.zeros_like(n), n)
+    assert cb.cb_poll_status()[0] == 1                          # CB_ERR_INVALID_ARG
+    assert [len(cb.cb_table_dump_arrays(b)[0]) for b in range(3)] == [1, 0, 1]

@@ -120,8 +120,8 @@ cb_status cb_update(cb_ctx* ctx, const int32_t* tokens, int64_t row_stride, cons
  * over many warps where that cannot change the result (no leader can be evicted during the run: leaders stored + windows
  * <= LC, and at least 64 windows), and done by one warp in order otherwise.  Runs of up to 8,192 windows take one launch,
  * whose blocks reduce a run in shared memory without regard to its order (batches of up to 1,024 sequences, under the reading
- * that re-inserting a stored follower refreshes it); where row_stride has room for longer ones two more follow (seven with
- * scratch attached, see below).  CB_CNT_FOLLOWER_EVICTIONS counts the followers this call displaced from the lists; where a
+ * that re-inserting a stored follower refreshes it); where row_stride has room for longer ones, or for more windows than LC,
+ * two more belong to the call (seven with scratch attached, see below).  CB_CNT_FOLLOWER_EVICTIONS counts the followers this call displaced from the lists; where a
  * run is reduced, a follower that the run itself would have stored and displaced again is never stored and so is not counted.
  */
 cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t row_stride, const int32_t* n_old,

@@ -17,8 +17,11 @@
 //
 // What the blocks of a sequence share: hdr[0] and hdr[1] (clock, leaders) are read by all and not changed while any is at work;
 // entry ids come from hdr[2], arrivals are counted in hdr[3] (both zero between calls), and the last block to arrive folds them
-// into hdr[0] and hdr[1].  A sequence that does not qualify (fewer than 64 windows, or a leader could be evicted during the run) is
-// done in order by the first warp of its first part.
+// into hdr[0] and hdr[1].  A sequence that does not qualify (fewer than 64 windows, or a leader could be evicted during the run) stays one
+// (its leaders only grow in number) and is left to the kernels after this one, or, where there are none (`alone`), done in order
+// by one warp of the block that has its first part, side by side with the block's others: such a run is a chain of 1 to 2.5 k cycles a
+// window (batch 1,024 of 45 windows: 292 us with a block's one after the other, 64 so; batch 512 of 5,000 that evict, in the kernel
+// behind: 52.4 ms and 7.2).
 #pragma once
 
 namespace {
@@ -143,30 +146,28 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
     __syncthreads();
     const uint32_t n_parts = S.total;
     TblCounters cnt = {0, 0, 0, 0};
-    for (uint32_t u = blockIdx.x; u < n_parts; u += gridDim.x) {
+    auto sequence_of = [&](uint32_t u) {                        // the last sequence whose parts begin at or before u
         int b = 0;
-        for (int hi = B - 1; b < hi;) {                         // the last sequence whose parts begin at or before u
+        for (int hi = B - 1; b < hi;) {
             const int mid = (b + hi + 1) >> 1;
             if (S.pre[mid] <= u) b = mid; else hi = mid - 1;
         }
+        return b;
+    };
+    auto reduced = [&](int b) { return S.nwin[b] >= 64u && (unsigned long long)S.count[b] + S.nwin[b] <= (unsigned long long)t.LC; };
+    bool in_order = false;
+    for (uint32_t u = blockIdx.x; u < n_parts; u += gridDim.x) {
+        const int b = sequence_of(u);
         const uint32_t part = u - S.pre[b], np = S.pre[b + 1] - S.pre[b];
         const CbSeq s = cb_seq(t, b);
         const uint32_t clock0 = S.clock[b], count0 = S.count[b], nwin = S.nwin[b];
         const int first = S.first[b];
-        const bool together = nwin >= 64u && (unsigned long long)count0 + nwin <= (unsigned long long)t.LC;
         const int32_t* row = tokens + (size_t)b * row_stride;
-        if (!together) {
-            if (part == 0 && warp == 0) {
-                uint32_t clock = clock0, count = count0;
-                for (uint32_t k = 0; k < nwin; ++k) {
-                    const int i = first + (int)k;
-                    const int32_t mykey = lane < LL ? row[i + lane] : 0;
-                    const int32_t myfol = lane < t.FL ? row[i + LL + lane] : 0;
-                    tbl_insert(t, s, mykey, myfol, clock, count, lane, status, cnt);
-                }
-                if (lane == 0) { s.hdr[0] = clock; s.hdr[1] = count; }
-            }
-        } else {
+        if (!reduced(b)) {
+            in_order = in_order || part == 0u;
+            continue;
+        }
+        {
             // ---- the run's tokens
             {
                 if (u != blockIdx.x) clear_tables();
@@ -434,14 +435,29 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
             __threadfence();
             if (atomicAdd(&s.hdr[3], 1u) == np - 1u) {
                 __threadfence();
-                if (together) {
-                    s.hdr[1] = count0 + __ldcg(&s.hdr[2]);
-                    s.hdr[0] = clock0 + nwin;
-                }
+                s.hdr[1] = count0 + __ldcg(&s.hdr[2]);
+                s.hdr[0] = clock0 + nwin;
                 s.hdr[2] = 0u;
                 s.hdr[3] = 0u;
-                if (together) atomicAdd(&counters[CB_CNT_INSERTS], (unsigned long long)nwin);
+                atomicAdd(&counters[CB_CNT_INSERTS], (unsigned long long)nwin);
             }
+        }
+    }
+    if (alone && in_order) {
+        uint32_t k = 0;
+        for (uint32_t u = blockIdx.x; u < n_parts; u += gridDim.x) {
+            const int b = sequence_of(u);
+            if (u != S.pre[b] || reduced(b) || (k++ & 31u) != (uint32_t)warp) continue;
+            const CbSeq s = cb_seq(t, b);
+            const int32_t* row = tokens + (size_t)b * row_stride;
+            uint32_t clock = S.clock[b], count = S.count[b];
+            for (int i = S.first[b], end = i + (int)S.nwin[b]; i < end; ++i) {
+                const int32_t mykey = lane < LL ? row[i + lane] : 0;
+                const int32_t myfol = lane < t.FL ? row[i + LL + lane] : 0;
+                if (t.FC <= 32) tbl_insert<1>(t, s, mykey, myfol, clock, count, lane, status, cnt);
+                else tbl_insert<0>(t, s, mykey, myfol, clock, count, lane, status, cnt);
+            }
+            if (lane == 0) { s.hdr[0] = clock; s.hdr[1] = count; }
         }
     }
     const uint32_t mp = __reduce_max_sync(CB_FULL, cnt.maxprobe);

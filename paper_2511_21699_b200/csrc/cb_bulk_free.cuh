@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(1024) cb_bulk_free_plan_kernel(CbTables t, int
         p.first = (uint32_t)first;
         p.nwin = (uint32_t)nwin;
         p.parallel = (nwin >= 64 && (unsigned long long)s.hdr[1] + (unsigned long long)nwin <= (unsigned long long)t.LC) ? 1u : 0u;
-        if (nwin <= done) p.parallel = 2u;
+        if (nwin <= done && p.parallel == 1u) p.parallel = 2u;
         if (p.parallel == 1u) s.hdr[0] = p.clock0 + (uint32_t)nwin;
         plan[b] = p;
         s_nwin[b] = (p.parallel == 1u && t.refresh) ? (uint32_t)nwin : 0u;

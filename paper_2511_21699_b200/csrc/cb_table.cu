@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(128) cb_update_kernel(CbTables t, int B, const
 // sequences that do not qualify (short runs, possible eviction) are done by their first warp alone, in order.
 struct BulkPlan { uint32_t parallel, clock0, first, nwin; };   // parallel: 0 one warp in order, 1 warps by leader, 2 elsewhere (cb_bulk_block.cuh, cb_bulk_free.cuh)
 
-// done: runs of up to that many windows have been dealt with by the block kernel (cb_bulk_block.cuh)
+// done: runs of up to that many windows that qualify are the block kernel's (cb_bulk_block.cuh), which comes after this one
 __global__ void cb_bulk_plan_kernel(CbTables t, int B, const int32_t* __restrict__ n_old, const int32_t* __restrict__ n_new,
                                     BulkPlan* plan, int done) {
     CB_PDL_ENTRY();
@@ -411,7 +411,7 @@ __global__ void cb_bulk_plan_kernel(CbTables t, int B, const int32_t* __restrict
     p.first = (uint32_t)first;
     p.nwin = (uint32_t)nwin;
     p.parallel = (nwin >= 64 && (unsigned long long)s.hdr[1] + (unsigned long long)nwin <= (unsigned long long)t.LC) ? 1u : 0u;
-    if (nwin <= done) p.parallel = 2u;
+    if (nwin <= done && p.parallel == 1u) p.parallel = 2u;
     if (p.parallel == 1u) s.hdr[0] = p.clock0 + (uint32_t)nwin;   // the clock after the run; the warps take stamps from positions
     plan[b] = p;
 }
@@ -1040,12 +1040,28 @@ extern "C" cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t 
                                     const int32_t* n_new, void* stream) {
     CB_CHECK_ARG(ctx && tokens && n_old && n_new && row_stride >= 1);
     const int B = ctx->cfg.batch;
-    int done = -1;
-    if (ctx->tables.refresh && B <= kBlkMaxBatch) {
-        // Runs of up to kBlkRun windows by blocks that hold them in shared memory.  A row that has no room for more needs nothing else.  (A row
-        // without room for a window is a stride that means nothing: that of a batch of one.)
-        const int w = ctx->tables.LL + ctx->tables.FL;
-        const bool alone = row_stride >= w && row_stride - w + 1 <= (int64_t)kBlkRun;
+    // Runs of up to kBlkRun windows that qualify are reduced by blocks that hold them in shared memory.  Where a row has room for no
+    // other run (room for a window less than the leader capacity: then nothing can be evicted, unless the table holds more than the
+    // row's text; without room for one window the stride means nothing, as in a batch of one), that is all: one launch.  Otherwise it is told
+    // what is whose before (plan), and the longer runs and those in order follow: batch 32 of 1,024 to 8,192 tokens 32 us alone, 36 so.
+    const int w = ctx->tables.LL + ctx->tables.FL;
+    const bool blocks = ctx->tables.refresh && B <= kBlkMaxBatch;
+    const bool alone = blocks && row_stride >= w && row_stride - w + 1 <= (int64_t)std::min(kBlkRun, ctx->tables.LC);
+    const int done = blocks ? kBlkRun : -1;
+    // enough warps per sequence to fill the GPU at small batch, fewer at large batch
+    int wps = 1;
+    while (wps < 256 && (long long)B * wps * 2 <= (long long)ctx->num_sms * 64) wps *= 2;
+    BulkPlan* plan = reinterpret_cast<BulkPlan*>(ctx->d_bulk_plan);
+    const cudaStream_t st = (cudaStream_t)stream;
+    const bool free_path = ctx->bulk_scratch && B <= kBulkFreeMaxBatch && ctx->tables.refresh;
+    BulkFreeView v = {};
+    if (free_path) v = bulk_free_view(ctx->bulk_scratch, ctx->bulk_slots, B);
+    if (!alone) {
+        if (free_path) CB_CUDA(cb_launch_pdl(cb_bulk_free_plan_kernel, dim3(1), dim3(1024), 0, st, ctx->tables, B, n_old, n_new, plan, v, ctx->d_counters, done));
+        else CB_CUDA(cb_launch_pdl(cb_bulk_plan_kernel, dim3((B + 127) / 128), dim3(128), 0, st, ctx->tables, B, n_old, n_new, plan, done));
+        cb_count_launch(1);
+    }
+    if (blocks) {
         using Kernel = void (*)(CbTables, int, const int32_t*, int64_t, const int32_t*, const int32_t*, bool, uint32_t*, unsigned long long*);
         static const Kernel kernels[CB_MAX_LL][2] = {{cb_update_bulk_block_kernel<1, 4>, cb_update_bulk_block_kernel<1, 8>},
                                                      {cb_update_bulk_block_kernel<2, 4>, cb_update_bulk_block_kernel<2, 8>},
@@ -1063,35 +1079,37 @@ extern "C" cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t 
                 done_here = true;
             }
         }
-        CB_CUDA(cb_launch_pdl(kernel, dim3((unsigned)ctx->num_sms), dim3(kBlkThreads), sizeof(BlkSmem), (cudaStream_t)stream, ctx->tables, B, tokens,
-                              row_stride, n_old, n_new, alone, ctx->d_status, ctx->d_counters));
+        CB_CUDA(cb_launch_pdl(kernel, dim3((unsigned)ctx->num_sms), dim3(kBlkThreads), sizeof(BlkSmem), st, ctx->tables, B, tokens, row_stride, n_old, n_new,
+                              alone, ctx->d_status, ctx->d_counters));
         cb_count_launch(1);
-        done = kBlkRun;
         if (alone) return CB_OK;
     }
-    // enough warps per sequence to fill the GPU at small batch, fewer at large batch
-    int wps = 1;
-    while (wps < 256 && (long long)B * wps * 2 <= (long long)ctx->num_sms * 64) wps *= 2;
-    BulkPlan* plan = reinterpret_cast<BulkPlan*>(ctx->d_bulk_plan);
-    const bool free_path = ctx->bulk_scratch && B <= kBulkFreeMaxBatch && ctx->tables.refresh;
+    // The block kernel takes nearly all of an SM's memory as shared memory, and a kernel without a preference runs with what L1 that leaves
+    // (runs in order of batch 512: 11.9 ms a call, so 7.2; scratch, batch 128 of 32 k: 2.59 and 2.04): those behind it ask for theirs.
+    static std::mutex l1_mu;
+    static int l1_asked[64][2] = {};                           // per device: percent + 1 that the last kernel prefers, 1 where the others are done
+    auto prefer = [](auto kernel, int percent) { return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent); };
     if (free_path) {
-        // order-free path for the sequences that qualify and fit the attached scratch; the kernel below does the others
-        const BulkFreeView v = bulk_free_view(ctx->bulk_scratch, ctx->bulk_slots, B);
-        const cudaStream_t st = (cudaStream_t)stream;
-        const unsigned blocks = (unsigned)std::min<long long>((long long)v.S / 256, (long long)ctx->num_sms * 8);
+        {
+            std::lock_guard<std::mutex> lock(l1_mu);
+            int& asked = l1_asked[ctx->device & 63][1];
+            if (!asked) {
+                CB_CUDA(prefer(cb_bulk_free_clear_kernel, 10)); CB_CUDA(prefer(cb_bulk_free_reduce_kernel, 10)); CB_CUDA(prefer(cb_bulk_free_ranges_kernel, 10));
+                CB_CUDA(prefer(cb_bulk_free_scatter_kernel, 10)); CB_CUDA(prefer(cb_bulk_free_apply_kernel, 10));
+                asked = 1;
+            }
+        }
+        // order-free path for the longer sequences that qualify and fit the attached scratch; the kernel below does the others
+        const unsigned grid = (unsigned)std::min<long long>((long long)v.S / 256, (long long)ctx->num_sms * 8);
         const unsigned wide = (unsigned)std::min<long long>((long long)v.S / 256, (long long)ctx->num_sms * 32);   // one item per thread, or a few
-        CB_CUDA(cb_launch_pdl(cb_bulk_free_plan_kernel, dim3(1), dim3(1024), 0, st, ctx->tables, B, n_old, n_new, plan, v, ctx->d_counters, done));
         CB_CUDA(cb_launch_pdl(cb_bulk_free_clear_kernel, dim3(wide), dim3(256), 0, st, v));
         CB_CUDA(cb_launch_pdl(cb_bulk_free_reduce_kernel, dim3(wide), dim3(256), 0, st, ctx->tables, B, tokens, row_stride, (const BulkPlan*)plan, v,
                               ctx->d_status));
         CB_CUDA(cb_launch_pdl(cb_bulk_free_ranges_kernel, dim3(wide), dim3(256), 0, st, v));
         CB_CUDA(cb_launch_pdl(cb_bulk_free_scatter_kernel, dim3(wide), dim3(256), 0, st, v));
-        CB_CUDA(cb_launch_pdl(cb_bulk_free_apply_kernel, dim3(blocks), dim3(256), 0, st, ctx->tables, B, tokens, row_stride, (const BulkPlan*)plan, v,
+        CB_CUDA(cb_launch_pdl(cb_bulk_free_apply_kernel, dim3(grid), dim3(256), 0, st, ctx->tables, B, tokens, row_stride, (const BulkPlan*)plan, v,
                               ctx->d_status, ctx->d_counters));
-        cb_count_launch(6);
-    } else {
-        CB_CUDA(cb_launch_pdl(cb_bulk_plan_kernel, dim3((B + 127) / 128), dim3(128), 0, (cudaStream_t)stream, ctx->tables, B, n_old, n_new, plan, done));
-        cb_count_launch(1);
+        cb_count_launch(5);
     }
     const long long warps = (long long)B * wps;
     // kept entries per warp: four, fewer where 96 KB of shared memory per CTA (8 warps) do not hold that many
@@ -1107,7 +1125,13 @@ extern "C" cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t 
             opted[d] = smem;
         }
     }
-    CB_CUDA(cb_launch_pdl(cb_update_bulk_kernel, dim3((unsigned)((warps + 7) / 8)), dim3(256), smem, (cudaStream_t)stream, ctx->tables, B, wps, n_ways,
+    {
+        std::lock_guard<std::mutex> lock(l1_mu);
+        int& asked = l1_asked[ctx->device & 63][0];
+        const int percent = (int)std::min<size_t>(100, 4 * (smem + 1024) * 100 / (228 * 1024) + 1);   // four blocks an SM
+        if (asked != percent + 1) { CB_CUDA(prefer(cb_update_bulk_kernel, percent)); asked = percent + 1; }
+    }
+    CB_CUDA(cb_launch_pdl(cb_update_bulk_kernel, dim3((unsigned)((warps + 7) / 8)), dim3(256), smem, st, ctx->tables, B, wps, n_ways,
                           tokens, row_stride, n_old, n_new, (const BulkPlan*)plan, ctx->d_status, ctx->d_counters));
     cb_count_launch(1);
     return CB_OK;

@@ -70,6 +70,29 @@ def test_bulk_runs_in_blocks(oracle, LL, FL, LC, FC, kind, first, second, scratc
     assert cb.cb_poll_status()[0] == 0
 
 
+@pytest.mark.parametrize("few,many,n,LC", [(128, 512, 1500, 1024), (128, 1024, 50, 1024)])
+def test_runs_in_order_go_side_by_side(few, many, n, LC):
+    """Runs that could evict a leader, or are short, are chains of one warp each: four (eight) times as many sequences take about as long
+    where all of them are at work at once.  One block after the other took 3.5 (5.8) times as long, all at once 1.1 (1.4)."""
+    from paper_2511_21699_b200 import Cacheback
+    took = []
+    for B in (few, many):
+        cb = Cacheback(B, 2, 4, LC, 4, 32, 8, 8, 32000, 8, 8, 64)
+        d = dev(_tokens("zipf", 1, n, np.random.default_rng(3)).repeat(B, 0))
+        zero, end = torch.zeros(B, dtype=torch.int32, device="cuda"), torch.full((B,), n, dtype=torch.int32, device="cuda")
+        times = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            cb.cb_update_bulk(d, zero, end)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        took.append(min(times))
+        assert cb.cb_poll_status()[0] == 0
+    assert took[1] < 2.2 * took[0], took
+
+
 @pytest.mark.parametrize("form", ["rows", "transposed", "strided", "flat"])
 def test_one_sequence_whatever_its_stride(oracle, form):
     """A batch of one: the stride of its only row means nothing, and a run longer than a block takes is not lost by it."""

@@ -121,8 +121,9 @@ cb_status cb_update(cb_ctx* ctx, const int32_t* tokens, int64_t row_stride, cons
  * <= LC, and at least 64 windows), and done by one warp in order otherwise.  Runs of up to 8,192 windows take one launch,
  * whose blocks reduce a run in shared memory without regard to its order (batches of up to 1,024 sequences, under the reading
  * that re-inserting a stored follower refreshes it); where row_stride has room for longer ones, or for more windows than LC,
- * two more belong to the call (seven with scratch attached, see below).  CB_CNT_FOLLOWER_EVICTIONS counts the followers this call displaced from the lists; where a
- * run is reduced, a follower that the run itself would have stored and displaced again is never stored and so is not counted.
+ * two more belong to the call (seven with scratch attached, see below).  CB_CNT_FOLLOWER_EVICTIONS counts the followers this call displaced from the lists; with
+ * scratch attached, where a run is reduced, a follower that the run itself would have stored and displaced again is never stored and
+ * so is not counted.
  */
 cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t row_stride, const int32_t* n_old,
                          const int32_t* n_new, void* stream);

@@ -101,15 +101,158 @@ __device__ __forceinline__ uint32_t blk_slot(uint32_t* slots, const int32_t* tok
     return 0u;                                                  // excluded: there are as many slots as windows
 }
 
+// Hash of a window: of the leader's tokens, carried on over the follower's.
+template <int LL, int N>
+__device__ __forceinline__ uint32_t blk_leader_hash(const int32_t (&key)[N]) {
+    uint32_t x = 0x9E3779B9u;
+#pragma unroll
+    for (int j = 0; j < LL; ++j) { x = (x ^ (uint32_t)key[j]) * 0x85EBCA77u; x ^= x >> 15; }
+    return x;
+}
+template <int LL, int N>
+__device__ __forceinline__ uint32_t blk_pair_hash(uint32_t x, const int32_t (&key)[N], int n) {
+#pragma unroll
+    for (int j = LL; j < N; ++j) if (j < n) { x = (x ^ (uint32_t)key[j]) * 0x9E3779B1u; x ^= x >> 15; }
+    return x;
+}
+
+// Followers that the part's windows displace one after the other, which the reduction itself cannot say (it stores the latest only):
+// every listed leader that cannot keep all of its followers is marked, the marked ones' windows are listed in order, and a warp per
+// leader goes through its own among them with the leader's list in registers: lane l keeps places l, l + 32, ...: the stamp (0: free) and
+// the slot in `pair` of what is stored there.  All threads together; each warp gets its own share of the sum.  What it costs is some 300
+// cycles for each window of the most frequent leader, one after the other: batch 32 of 1,024 to 8,192 tokens,
+// reset and first draft included, 70 us where 32 do without (leaders of one token: 195 and 36).
+constexpr uint32_t kBlkMark = 0x80000000u;      // of a leader's word; windows stay below 2^14
+template <int LL, int FLX, int CH>
+__device__ __noinline__ uint32_t blk_evictions(BlkSmem& S, const uint32_t* entries, uint32_t E, int FL, int FC, uint32_t count0, uint32_t clock0,
+                                               uint32_t nwin, uint32_t part, uint32_t np) {
+    constexpr uint32_t kNone = 0xFFFFFFFFu;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, w = LL + FL;
+    auto find = [&](const uint32_t* slots, const int32_t (&key)[LL + FLX], int n, uint32_t h) {
+        uint32_t at = h & (kBlkSlots - 1);
+        for (int p = 0; p < kBlkSlots; ++p) {
+            const uint32_t x = slots[at] & ~kBlkMark;
+            if (x == 0u) break;
+            const int32_t* q = S.tok + (x >> 16) - 1u;
+            int32_t diff = 0;
+#pragma unroll
+            for (int j = 0; j < LL + FLX; ++j) if (j < n) diff |= q[j] ^ key[j];
+            if (diff == 0) return at;
+            at = (at + 1u) & (kBlkSlots - 1);
+        }
+        return kNone;
+    };
+    auto pair_of = [&](const int32_t (&key)[LL + FLX]) { return find(S.pair, key, w, blk_pair_hash<LL>(blk_leader_hash<LL>(key), key, w)); };
+    uint32_t id[CH], st[CH];
+    // Reads leader o's list as it was before the run; true if the run's followers do not all have room beside it.
+    auto crowded = [&](uint32_t o) {
+        const uint32_t at = ((S.lead[S.lslot[o]] & ~kBlkMark) >> 16) - 1u, x = count0 > 0u ? S.cur[o] : kBlkFresh;
+        const uint32_t* e = entries + (size_t)((x & kBlkFresh) ? 0u : x - 1u) * E;
+        uint32_t stored = 0, known = 0;
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+            const int f = c * 32 + lane;
+            id[c] = kNone;
+            st[c] = !(x & kBlkFresh) && f < FC ? e[LL + f] : 0u;
+            if (st[c]) {
+                int32_t key[LL + FLX];
+#pragma unroll
+                for (int j = 0; j < LL + FLX; ++j) key[j] = j < LL ? S.tok[at + j] : j < w ? (int32_t)e[LL + FC + f * FL + j - LL] : 0;
+                id[c] = pair_of(key);
+            }
+            stored += __popc(__ballot_sync(CB_FULL, st[c] != 0u));
+            known += __popc(__ballot_sync(CB_FULL, id[c] != kNone));
+        }
+        return stored + (S.gbase[o + 1] - S.gbase[o]) - known > (uint32_t)FC;
+    };
+    const uint32_t n_list = S.n_list;
+    bool any = false;
+    for (uint32_t i = warp; i < n_list; i += kBlkThreads / 32) {
+        const uint32_t o = S.pl[i];
+        if (!crowded(o)) continue;
+        any = true;
+        if (lane == 0) atomicOr(&S.lead[S.lslot[o]], kBlkMark);
+    }
+    if (!__syncthreads_or(any)) return 0u;
+    uint32_t m = 0;
+    for (uint32_t k0 = 0; k0 < nwin; k0 += kBlkThreads) {
+        const uint32_t k = k0 + tid;
+        bool in = false;
+        if (k < nwin) {
+            int32_t key[LL + FLX];
+            uint32_t x = 0x85EBCA6Bu;
+#pragma unroll
+            for (int j = 0; j < LL + FLX; ++j) {
+                key[j] = j < LL ? S.tok[k + j] : 0;
+                if (j < LL) { x = (x ^ (uint32_t)key[j]) * 0x9E3779B1u; x ^= x >> 16; }
+            }
+            if (__umulhi(x * 0xC2B2AE35u, np) == part) {
+                const uint32_t at = find(S.lead, key, LL, blk_leader_hash<LL>(key));
+                in = at != kNone && (S.lead[at] & kBlkMark);
+            }
+        }
+        uint32_t total;
+        const uint32_t before = blk_scan(in ? 1u : 0u, S.red, &total);
+        if (in) S.pslot[m + before] = (uint16_t)k;                // the pairs' list is not needed any more
+        m += total;
+    }
+    __syncthreads();
+    uint32_t out = 0;
+    for (uint32_t i = warp; i < n_list; i += kBlkThreads / 32) {
+        const uint32_t o = S.pl[i], lw = S.lead[S.lslot[o]];
+        if (!(lw & kBlkMark)) continue;
+        const uint32_t at = ((lw & ~kBlkMark) >> 16) - 1u;
+        (void)crowded(o);
+        uint32_t now = clock0;                                   // above every stored stamp; only their order matters here
+        for (uint32_t k0 = 0; k0 < m; k0 += 32) {
+            bool mine = k0 + lane < m;
+            const uint32_t k = mine ? S.pslot[k0 + lane] : 0u;
+#pragma unroll
+            for (int j = 0; j < LL; ++j) mine = mine && S.tok[k + j] == S.tok[at + j];
+            uint32_t ps = kNone;
+            if (mine) {
+                int32_t key[LL + FLX];
+#pragma unroll
+                for (int j = 0; j < LL + FLX; ++j) key[j] = j < w ? S.tok[k + j] : 0;
+                ps = pair_of(key);
+            }
+            for (uint32_t todo = __ballot_sync(CB_FULL, mine); todo; todo &= todo - 1u) {
+                const uint32_t x = __shfl_sync(CB_FULL, ps, __ffs(todo) - 1);
+                ++now;
+                bool hit = false;
+                uint32_t oldest = kNone;
+#pragma unroll
+                for (int c = 0; c < CH; ++c) {
+                    if (id[c] == x && st[c]) { st[c] = now; hit = true; }
+                    if (c * 32 + lane < FC) oldest = min(oldest, st[c]);
+                }
+                if (__any_sync(CB_FULL, hit)) continue;
+                // a free place has stamp 0 and there may be several; stamps in use are unique
+                const uint32_t g = __reduce_min_sync(CB_FULL, oldest);
+                out += g ? 1u : 0u;
+                if (lane == __ffs(__ballot_sync(CB_FULL, oldest == g)) - 1) {
+                    bool open = true;
+#pragma unroll
+                    for (int c = 0; c < CH; ++c)
+                        if (open && c * 32 + lane < FC && st[c] == g) { st[c] = now; id[c] = x; open = false; }
+                }
+            }
+        }
+    }
+    __syncthreads();                                             // the entries have been read
+    return out;
+}
+
 __device__ __forceinline__ uint32_t blk_parts(uint32_t nwin, uint32_t spare, uint32_t all) {
     if (nwin == 0u) return 0u;
     const uint32_t share = 1u + (uint32_t)((unsigned long long)nwin * spare / all);
     return max(min(share, max(nwin / 32u, 1u)), (nwin + kBlkPart - 1u) / kBlkPart);
 }
 
-// alone: no other kernel follows, so that no run may be longer than kBlkRun windows.
+// alone: no other kernel follows, so that no run may be longer than kBlkRun windows.  COUNT_ALL: every follower that the windows displace
+// one after the other is counted, also those that the run itself brought (else those displaced from the lists as they were).
 // LL: the leader's tokens, FLX: a bound of the follower's (4 or 8), so that the loops over a window's tokens are straight code.
-template <int LL, int FLX>
+template <int LL, int FLX, bool COUNT_ALL>
 __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(CbTables t, int B, const int32_t* __restrict__ tokens, int64_t row_stride,
                                                                            const int32_t* __restrict__ n_old, const int32_t* __restrict__ n_new,
                                                                            bool alone, uint32_t* status, unsigned long long* counters) {
@@ -206,13 +349,11 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                     int32_t lk[LL], wk[LL + FLX];
 #pragma unroll
                     for (int j = 0; j < LL + FLX; ++j) wk[j] = j < w ? S.tok[k + j] : 0;
-                    uint32_t x = 0x9E3779B9u;
 #pragma unroll
-                    for (int j = 0; j < LL; ++j) { lk[j] = wk[j]; x = (x ^ (uint32_t)lk[j]) * 0x85EBCA77u; x ^= x >> 15; }
+                    for (int j = 0; j < LL; ++j) lk[j] = wk[j];
+                    const uint32_t x = blk_leader_hash<LL>(wk);
                     ls = blk_slot<LL>(S.lead, S.tok, lk, LL, x, k, &new_l);
-#pragma unroll
-                    for (int j = LL; j < LL + FLX; ++j) if (j < w) { x = (x ^ (uint32_t)wk[j]) * 0x9E3779B1u; x ^= x >> 15; }
-                    ps = blk_slot<LL + FLX>(S.pair, S.tok, wk, w, x, k, &new_p);
+                    ps = blk_slot<LL + FLX>(S.pair, S.tok, wk, w, blk_pair_hash<LL>(x, wk, w), k, &new_p);
                     if (new_p) { S.pl[ps] = (uint16_t)ls; atomicAdd(&S.cur[ls], 1u); }
                 }
                 // what is new goes into the lists
@@ -306,7 +447,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                 if (o < nl) {
                     const uint32_t eid = entry_of(o, &c.open);
                     c.open = c.open && eid < (uint32_t)t.LC;
-                    c.h = leader_hash((S.lead[S.lslot[o]] >> 16) - 1u);
+                    c.h = leader_hash(((S.lead[S.lslot[o]] & ~kBlkMark) >> 16) - 1u);
                     c.word = (cb_hash_tag(c.h) << CB_EID_BITS) | eid;
                 }
                 return c;
@@ -364,8 +505,12 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
             __syncthreads();
             // ---- the listed ones by a warp each
             const uint32_t n_list = S.n_list;
+            uint32_t displaced = cnt.fevict;
+            if (COUNT_ALL && n_list)
+                displaced += t.FC <= 32 ? blk_evictions<LL, FLX, 1>(S, s.entries, t.E, t.FL, t.FC, count0, clock0, nwin, part, np)
+                                        : blk_evictions<LL, FLX, CB_MAX_FC / 32>(S, s.entries, t.E, t.FL, t.FC, count0, clock0, nwin, part, np);
             for (uint32_t i = warp; i < n_list; i += kBlkThreads / 32) {
-                const uint32_t o = S.pl[i], lw = S.lead[S.lslot[o]], kpos = (lw >> 16) - 1u, g = S.gbase[o], n = S.gbase[o + 1] - g;
+                const uint32_t o = S.pl[i], lw = S.lead[S.lslot[o]] & ~kBlkMark, kpos = (lw >> 16) - 1u, g = S.gbase[o], n = S.gbase[o + 1] - g;
                 bool fresh;
                 const uint32_t eid = entry_of(o, &fresh);
                 if (eid >= (uint32_t)t.LC) continue;
@@ -422,6 +567,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                     }
                 }
             }
+            if (COUNT_ALL) cnt.fevict = displaced;
             // ---- the rest of the publication
             if (mine.open) finish(mine, mine_old);
             for (uint32_t o = tid + kBlkThreads; o < nl; o += kBlkThreads) {

@@ -1063,17 +1063,17 @@ extern "C" cb_status cb_update_bulk(cb_ctx* ctx, const int32_t* tokens, int64_t 
     }
     if (blocks) {
         using Kernel = void (*)(CbTables, int, const int32_t*, int64_t, const int32_t*, const int32_t*, bool, uint32_t*, unsigned long long*);
-        static const Kernel kernels[CB_MAX_LL][2] = {{cb_update_bulk_block_kernel<1, 4>, cb_update_bulk_block_kernel<1, 8>},
-                                                     {cb_update_bulk_block_kernel<2, 4>, cb_update_bulk_block_kernel<2, 8>},
-                                                     {cb_update_bulk_block_kernel<3, 4>, cb_update_bulk_block_kernel<3, 8>},
-                                                     {cb_update_bulk_block_kernel<4, 4>, cb_update_bulk_block_kernel<4, 8>}};
-        const int l = ctx->tables.LL - 1, f = ctx->tables.FL <= 4 ? 0 : 1;
-        const Kernel kernel = kernels[l][f];
+        // [leader][follower][every displaced follower counted: with scratch attached the call does not promise that]
+#define CB_BLK(l) {{cb_update_bulk_block_kernel<l, 4, false>, cb_update_bulk_block_kernel<l, 4, true>}, {cb_update_bulk_block_kernel<l, 8, false>, cb_update_bulk_block_kernel<l, 8, true>}}
+        static const Kernel kernels[CB_MAX_LL][2][2] = {CB_BLK(1), CB_BLK(2), CB_BLK(3), CB_BLK(4)};
+#undef CB_BLK
+        const int l = ctx->tables.LL - 1, f = ctx->tables.FL <= 4 ? 0 : 1, all = ctx->bulk_scratch ? 0 : 1;
+        const Kernel kernel = kernels[l][f][all];
         static std::mutex mu;
-        static bool opted[64][CB_MAX_LL][2] = {};              // per device
+        static bool opted[64][CB_MAX_LL][2][2] = {};              // per device
         {
             std::lock_guard<std::mutex> lock(mu);
-            bool& done_here = opted[ctx->device & 63][l][f];
+            bool& done_here = opted[ctx->device & 63][l][f][all];
             if (!done_here) {
                 CB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlkSmem)));
                 done_here = true;

@@ -61,6 +61,12 @@ def test_bulk_runs_in_blocks(oracle, LL, FL, LC, FC, kind, first, second, scratc
     _assert_tables_equal(cb, tabs, check)
     st, cnt = cb.cb_poll_status()
     assert st == 0 and cnt["inserts"] == int(np.maximum(n2 - w + 1, 0).sum())
+    if not scratch:                                             # the counters are those of the windows one after the other
+        one = Cacheback(B, LL, FL, LC, FC, 32, 8, 8, 32000, 8, 8, 64)
+        one.cb_update(d, zero, dev(n1))
+        one.cb_update(d, dev(n1), dev(n2))
+        ref = one.cb_poll_status()[1]
+        assert [cnt[k] for k in ("inserts", "leader_evictions", "follower_evictions")] == [ref[k] for k in ("inserts", "leader_evictions", "follower_evictions")]
     cb.cb_reset()                                               # a table that was in use, empty again
     cb.cb_update_bulk(d, zero, dev(n1))
     tabs = {b: oracle.OracleTable(LL, FL, LC, FC) for b in check}

@@ -1005,15 +1005,16 @@ __global__ void __launch_bounds__(256, CTAS) cb_accept_draft_kernel(AcceptArgs a
         return;
     __syncthreads();                                            // the walk (first warp) has written the sequence's result
     const int have = s_have;                                    // tokens emitted (an empty tree emits none)
-    const int L = s_len, tail0 = max(0, L - w + 1);
+    // (a malformed tree may name a depth beyond any of its own: more places than are kept here are read from the history)
+    const int L = s_len, tail0 = have <= 256 ? max(0, L - w + 1) : 0x7FFFFFFF;
     int L1 = L + have;
-    if (L1 > row_stride) {
-        // no room in the history: nothing is appended and the step is reported; the draft below continues from what is there
+    if (L < 0 || L1 > row_stride) {
+        // no room in the history, or no length: nothing is appended and the step is reported; the draft below continues from what is there
         if (tid == 0) atomicCAS(status, 0u, (uint32_t)CB_ERR_INVALID_ARG);
         L1 = L;
     } else if (tid < have) {
         history[L + tid] = s_emit[tid];
-        s_tail[L - tail0 + tid] = s_emit[tid];
+        if (have <= 256) s_tail[L - tail0 + tid] = s_emit[tid];
     }
     __syncthreads();
     if (tid == 0) seq_len[b] = L1;

@@ -59,3 +59,30 @@ def test_fused_call_equals_separate_calls_from_short_histories(LL, FL, FC, T, de
     sa, ca = a.cb_poll_status()
     sb, cb_ = b.cb_poll_status()
     assert sa == sb == 0 and ca["inserts"] == cb_["inserts"] and ca["query_hits"] == cb_["query_hits"]
+
+
+def test_a_depth_beyond_the_tree_and_a_length_below_zero_stay_inside_the_kept_tail():
+    """Malformed inputs: a tree whose one accepted node names a depth of 300 (the step emits 301 places, of which the launch keeps 256 on
+    chip), and a sequence of negative length (nothing is appended, reported)."""
+    from paper_2511_21699_b200 import Cacheback
+    V, T, N = 64, 8, 1000
+    cb = Cacheback(2, 2, 3, 256, 4, T, 2, 400, V, 8, 8, 64)
+    toks = torch.zeros(2, N, dtype=torch.int32, device="cuda")
+    toks[:, :500] = torch.arange(500, device="cuda") % 50
+    tree = cb.alloc_tree()
+    for k, fill in (("tokens", -1), ("parent", -1), ("depth", -1), ("mask", 0)):
+        tree[k].fill_(fill)
+    tree["n_nodes"].copy_(dev(np.array([2, 1], np.int32)))
+    tree["tokens"][:, 0] = 49
+    tree["depth"][:, 0] = 0
+    tree["tokens"][0, 1], tree["parent"][0, 1], tree["depth"][0, 1] = 7, 0, 300
+    logits = torch.zeros(2, T, V, device="cuda")
+    logits[..., 7] = 1.0
+    n = dev(np.array([500, -5], np.int32))
+    nxt = cb.alloc_tree()
+    res = cb.cb_accept_update_draft_tree(tree, logits, toks, n, next_tree=nxt)
+    assert cb.cb_poll_status()[0] == 1                          # CB_ERR_INVALID_ARG, of the second sequence
+    assert res["n_accept"].tolist() == [300, 0] and n.tolist() == [801, -5]
+    assert (res["out_tokens"][0, :299] == -1).all() and res["out_tokens"][0, 299:301].tolist() == [7, 7]
+    assert (toks[0, 500:756] == -1).all() and not toks[0, 756:].any() and torch.equal(toks[1, :500], torch.arange(500, device="cuda", dtype=torch.int32) % 50)
+    assert int(nxt["n_nodes"][1]) == 0

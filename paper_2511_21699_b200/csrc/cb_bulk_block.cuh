@@ -277,6 +277,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                 nwin = 0;
                 if (alone && blockIdx.x == 0) atomicCAS(status, 0u, (uint32_t)CB_ERR_INVALID_ARG);
             }
+            if (!cb_dbg_in(h.y, (long long)t.LC + 1, t.dbg_status)) nwin = 0;
             S.nwin[tid] = (uint16_t)nwin; S.first[tid] = first; S.clock[tid] = h.x; S.count[tid] = h.y;
         }
         (void)blk_scan(nwin, S.red, &all);
@@ -406,7 +407,8 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                             for (int q = 0; q < 4; ++q) {
                                 empty = empty || xs[q] == CB_IDX_EMPTY;
                                 const uint32_t eid = xs[q] & CB_EID_MASK;
-                                if (xs[q] == CB_IDX_EMPTY || xs[q] == CB_IDX_TOMB || (xs[q] >> CB_EID_BITS) != tag || eid >= count0) continue;
+                                if (xs[q] == CB_IDX_EMPTY || xs[q] == CB_IDX_TOMB || (xs[q] >> CB_EID_BITS) != tag) continue;
+                                if (!cb_dbg_in(eid, t.LC, t.dbg_status) || eid >= count0) continue;   // (from count0 on: a leader of another part)
                                 bool eq = true;
                                 for (int j = 0; j < LL; ++j) eq = eq && (int32_t)__ldcg(&s.entries[(size_t)eid * t.E + j]) == S.tok[kpos + j];
                                 if (eq) found = eid + 1u;

@@ -70,9 +70,40 @@ torch.cuda.synchronize()
 st, _ = cb.cb_poll_status()
 assert st == _lib.CB_ERR_INVALID_ARG, st
 assert torch.isfinite(out.float()).all()
+# prompts through the block kernel: the oracle's tables, then a planted index word that names an entry the table cannot have
+from oracle import cb_oracle
+LL, FL, LC, FC, n = 2, 3, 4096, 4, 1500
+toks = np.minimum(np.random.default_rng(4).zipf(1.3, (2, 2 * n)) - 1, 900).astype(np.int32)
+cb = Cacheback(2, LL, FL, LC, FC, 32, 8, 8, 1000, 8, 8, 64)
+tab = [cb_oracle.OracleTable(LL, FL, LC, FC) for _ in range(2)]
+z, n1, n2 = (dev(np.full(2, x, np.int32)) for x in (0, n, 2 * n))
+for a, b, ha, hb in ((z, n1, 0, n), (n1, n2, n, 2 * n)):
+    cb.cb_update_bulk(dev(toks), a, b)
+    for s in range(2):
+        tab[s].update(toks[s], ha, hb)
+        assert all(np.array_equal(x, y) for x, y in zip(cb.cb_table_dump_arrays(s), tab[s].dump_arrays()))
+assert cb.cb_poll_status()[0] == 0
+M64 = (1 << 64) - 1
+h = 0x9E3779B97F4A7C15 ^ LL                             # the key's hash: its tag and its bucket
+key = toks[0, :2] * 0 + 950                               # a leader that the tables do not have
+for k in key:
+    h = ((h ^ int(k)) * 0xFF51AFD7ED558CCD) & M64
+    h ^= h >> 32
+h ^= h >> 33
+h = (h * 0xC4CEB9FE1A85EC53) & M64
+h ^= h >> 33
+nslots = 4 * LC
+base = (cb.workspace.data_ptr() + 255) // 256 * 256 - cb.workspace.data_ptr()
+index = cb.workspace[base + 512:base + 512 + 4 * nslots].view(torch.int32)           # behind the headers and their guard area
+bucket = index[32 * ((h >> 32) & (nslots // 32 - 1)):][:32]
+free = int((bucket == 0).nonzero()[0])
+bucket[free] = int(np.uint32(((h & 0xFFFFFFFF) %% 4094 + 1) << 20 | (LC + 7)).view(np.int32))
+more = np.concatenate([toks, np.full((2, 80), 950, np.int32)], 1)
+cb.cb_update_bulk(dev(more), n2, dev(np.full(2, 2 * n + 80, np.int32)))
+assert cb.cb_poll_status()[0] == _lib.CB_ERR_INVALID_ARG
+bucket[free] = 0
 # a selection of the frozen builder that gives up at its first barrier: the call says so, and nothing behind it goes by what is missing
 import ctypes as C
-from oracle import cb_oracle
 L = _lib.load()
 L.cb_debug_frozen_build.argtypes = L.cb_frozen_build.argtypes + [C.c_uint32]
 L.cb_debug_frozen_build.restype = C.c_int32

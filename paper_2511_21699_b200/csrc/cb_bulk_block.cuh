@@ -6,9 +6,9 @@
 // of the run, the table of the part's leaders and that of its (leader, follower) pairs lie in shared memory, so claims, "last
 // index" maxima and the grouping of pairs by leader are shared-memory operations, and what is left in global memory is an atomic per
 // new leader and the entry itself.  Through scratch in global memory the same run is six launches whose every step is a chain of L2
-// round trips: batch 32 of 1,024 to 8,192 tokens (147 k windows), reset and first draft with it, 118 us against 35.5 us this way
-// (some 20 of them this kernel's: 31 k cycles, of which the entries take 10 k, claiming 5.5 k, the reads of lengths and tokens 5 k).
-// What bounds it is the chain of phases in a block, a thread or two per window; no unit of the SM is busy.
+// round trips: batch 32 of 1,024 to 8,192 tokens (147 k windows), reset and first draft with it, 118 us against 32.7 us this way
+// (some 17 of them this kernel's: 31 k cycles in its first form, of which the entries took 10 k, claiming 5.5 k, the reads of lengths and
+// tokens 5 k).  What bounds it is the chain of phases in a block, a thread or two per window.
 //
 // Parts: every block reads all lengths and deals gridDim.x parts to the sequences in proportion to their windows (at least one
 // each, and no more than kBlkPart windows expected in one, so that the tables stay at most half full), so no plan kernel and no host

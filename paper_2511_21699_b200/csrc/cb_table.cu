@@ -950,10 +950,10 @@ struct AcceptArgs {
     int32_t* n_accept; int32_t* accept_nodes; int32_t* out_tokens; int32_t* target_out;
 };
 
-// CTAS: CTAs that an SM has registers for.  The drafting code takes 106 registers, room for two.  A grid that is not resident at
-// once that way streams the logits with half in flight of what four CTAs of 59 have (a step of batch 6 with trees of 96: 86.6 us with three
+// CTAS: CTAs that an SM has registers for.  The drafting code takes 102 registers, room for two.  A grid that is not resident at
+// once that way streams the logits with half in flight of what four CTAs of 62 have (a step of batch 6 with trees of 96: 86.6 us with three
 // of 72, 82.9 with four; batch 4 of 64: 61.3 and 59.6); one that is gains nothing from the bound and pays for it in the chain behind
-// the logits, and takes all of a thread's chunk at once instead.  With more than 32 followers a leader the code takes 109 registers and
+// the logits, and takes all of a thread's chunk at once instead.  With more than 32 followers a leader the code takes 120 registers and
 // stays at two.
 //
 // IN_PLACE: o_n is a.n_nodes.  Which rows a sequence's tree has decides which of its CTAs count for the acceptance, so its entry is stored only

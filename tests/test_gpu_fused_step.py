@@ -23,7 +23,7 @@ def test_accept_update_draft_in_one_launch(oracle, name, dtype, steps):
 
 @pytest.mark.parametrize("batch,dtype", [(1, "f32"), (2, "f32"), (2, "bf16"), (3, "bf16")])
 def test_grids_on_both_sides_of_two_ctas_a_sm(oracle, batch, dtype):
-    """64 nodes x 32 k tokens in four (two) chunks a row: 256 CTAs run at once two to an SM, 384 and 512 take the form for three."""
+    """64 nodes x 32 k tokens in four (two) chunks a row: 256 CTAs run at once two to an SM, 384 and 512 take the form for four."""
     from dataclasses import replace
     _loop(oracle, replace(W.get_config("c2_7b"), name="c2_small_batch", batch=batch, max_nodes=64), dtype, 3)
 

@@ -8,7 +8,8 @@
 // new leader and the entry itself.  Through scratch in global memory the same run is six launches whose every step is a chain of L2
 // round trips: batch 32 of 1,024 to 8,192 tokens (147 k windows), reset and first draft with it, 118 us against 32.7 us this way
 // (some 17 of them this kernel's: 31 k cycles in its first form, of which the entries took 10 k, claiming 5.5 k, the reads of lengths and
-// tokens 5 k).  What bounds it is the chain of phases in a block, a thread or two per window.
+// tokens 5 k).  What bounds it is the chain of phases in a block, a thread or two per window: a quarter of the SM's issue
+// rate, 18% of the shared-memory pipe, 5 MB from DRAM; half of the stalled warps wait at a barrier.
 //
 // Parts: every block reads all lengths and deals gridDim.x parts to the sequences in proportion to their windows (at least one
 // each, and no more than kBlkPart windows expected in one, so that the tables stay at most half full), so no plan kernel and no host

@@ -172,8 +172,9 @@ __device__ __forceinline__ void cb_sched_locate(const CbAttnParams& p, long long
 
 // One unit's share of a CTA's range: key tiles [t0, t1) of the unit's `tiles`.
 struct CbUnit {
-    int b, kh, rg, t0, t1, tiles, n, ctx, nrt;   // nrt = valid row tiles in the group (1 or 2)
+    int b, kh, rg, t0, t1, tiles, n, ctx, nrt;   // nrt = valid row tiles in the group (1 or 2), or kTwoHeads
 };
+constexpr int kTwoHeads = 3;                     // the units of heads kh and kh + 1, both whole and of one row tile, side by side (next_pair)
 
 // Walks the units of the range [g, g1).  Every role of a CTA runs its own copy and sees the same units.
 struct CbWalker {
@@ -221,6 +222,17 @@ struct CbWalker {
             u->nrt = p.MT == 1 ? 1 : min(2, s.mtn - 2 * rg);
             return true;
         }
+    }
+    // The same with two whole units of one row tile at a time where the range holds the next head's as well.
+    __device__ __forceinline__ bool next_pair(const CbAttnParams& p, CbUnit* u) {
+        if (!next(p, u)) return false;
+        if (fixed || u->nrt != 1 || u->t0 > 0 || u->t1 < u->tiles || u->kh + 1 >= p.Hkv) return true;
+        const long long end = pre + (long long)(u->kh + 2) * s.unit(rg);                    // of the next head's unit
+        const int last = (u->tiles - 1) * s.wt(rg) + s.dec(rg) - s.unit(rg);                // its last tile's deciding position, from there
+        if (end + last >= g1) return true;
+        g = min(end, g1);
+        u->nrt = kTwoHeads;
+        return true;
     }
 };
 

@@ -12,6 +12,11 @@
 //   * a unit with two row tiles gives each chain a row tile, and both walk all key tiles;
 //   * a unit with one row tile deals its key tiles to the two chains in turn; every chain keeps its own reference maximum and
 //     accumulator and the two are put together at the end of the unit.
+//   * where a range holds two heads' whole units of one row tile, they are taken together, a chain each with a query tile of its own: the
+//     key tiles come in turn as before, but nothing is put together at the end, and what lies between two units (query load, refill,
+//     epilogue; some 12 k cycles of a unit of two tiles) is paid once for both.  Batch 69 of 40 heads over 10 to 77 tokens 124 -> 91 us,
+//     batch 128 of 32 heads (64 dims) over 65 tokens 141 -> 103, 28 x 8 heads of 110-node trees over 377 tokens 91.8 -> 80.2, batch 64 of 40
+//     heads over 2,048 tokens 463 -> 455.
 // A row's 128 scores are split over two threads (64 each): one warp per scheduler and chain left half of the issue slots empty
 // (2.1 k cycles a tile with a row per thread, spills included).
 //
@@ -227,8 +232,9 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             uint32_t seq = isV ? 1u : 0u;                    // K and V tiles alternate in the ring
             bool ok = true;
             const uint64_t pol = l2_evict_first_policy();
-            while (ok && wk.next(p, &u)) {
+            while (ok && wk.next_pair(p, &u)) {
                 const int npages = (u.ctx + 15) / 16, nct = u.tiles - 1;   // pages of 16 tokens (checked by the launcher)
+                const int heads = u.nrt == kTwoHeads ? 2 : 1;              // their tiles come in turn
                 const int32_t* bt = p.block_table + (size_t)u.b * p.max_pages;
                 // The page number of a lane's box comes from the block table: a memory round trip that the copy depends on.
                 // It is fetched one tile ahead, so that it is under way while this tile's copies are issued and waited for.
@@ -245,16 +251,19 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     int page = page_next;
                     if (i + 1 < u.t1) page_next = page_of(i + 1);
                     if (!cb_dbg_in(page, p.num_pages + 1, p.status)) page = p.num_pages;   // the copy then fills zeros
-                    const uint32_t sl = seq % ns;
-                    if (seq >= ns && !(ok = mbar_wait(bar_free(sl), (seq / ns - 1) & 1, s_abort, p.status))) break;
-                    if (lane == 0) mbar_expect_tx(bar_full(sl), C::TILE_BYTES);
-                    __syncwarp();
-                    if (i < nct) {
-                        if (active) tma_load_5d_hint(slot_base(sl) + j * 2 * GROUP, isV ? &maps.v_pool : &maps.k_pool, bar_full(sl), 0, 0, 0, page * 2, u.kh, pol);
-                    } else if (lane < 16) {
-                        tma_load_5d(slot_base(sl) + lane * GROUP, isV ? &maps.v_tree : &maps.k_tree, bar_full(sl), 0, 8 * lane, 0, u.kh, u.b);
+                    for (int hd = 0; hd < heads; ++hd) {
+                        const uint32_t sl = seq % ns;
+                        if (seq >= ns && !(ok = mbar_wait(bar_free(sl), (seq / ns - 1) & 1, s_abort, p.status))) break;
+                        if (lane == 0) mbar_expect_tx(bar_full(sl), C::TILE_BYTES);
+                        __syncwarp();
+                        if (i < nct) {
+                            if (active) tma_load_5d_hint(slot_base(sl) + j * 2 * GROUP, isV ? &maps.v_pool : &maps.k_pool, bar_full(sl), 0, 0, 0, page * 2, u.kh + hd, pol);
+                        } else if (lane < 16) {
+                            tma_load_5d(slot_base(sl) + lane * GROUP, isV ? &maps.v_tree : &maps.k_tree, bar_full(sl), 0, 8 * lane, 0, u.kh + hd, u.b);
+                        }
+                        seq += 2;
                     }
-                    seq += 2;
+                    if (!ok) break;
                 }
             }
         } else if (warp == 1) {
@@ -264,9 +273,9 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                 constexpr uint32_t idesc_o = make_idesc(128, D, true);
                 uint32_t seq0 = 0, uq = 0, c_p[2] = {0u, 0u};
                 bool ok = true;
-                while (ok && wk.next(p, &u)) {
-                    const bool two = u.nrt == 2;
-                    const int nt = u.t1 - u.t0, nev = two ? 2 * nt : nt;   // products of either kind in this unit
+                while (ok && wk.next_pair(p, &u)) {
+                    const bool two = u.nrt == 2, heads = u.nrt == kTwoHeads;
+                    const int nt = heads ? 2 * u.tiles : u.t1 - u.t0, nev = two ? 2 * nt : nt;   // products of either kind in this unit
                     if (!(ok = mbar_wait(bar_qfull, uq & 1, s_abort, p.status))) break;
                     // Turn e belongs to chain e & 1: the P V of its turn before (key tile iv), then S of this turn's key tile ik.
                     for (int e = 0; e < nev + 2; ++e) {
@@ -284,7 +293,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                                 tc_fence_after();
                                 mma_pv_halves_block<D>(tmem + C::O_COL + l * D, tmem + l * 128, desc_lo(slot_base(vs), 1024), idesc_o, e < 4 ? 0u : 1u);
                                 if (!two || l == 1) tc_commit(bar_free(vs));
-                                if (iv == nt - 1) tc_commit(two ? bar_odone(l) : bar_odone_both);
+                                if (iv >= nt - (heads ? 2 : 1)) tc_commit(two || heads ? bar_odone(l) : bar_odone_both);
                             }
                         }
                         if (ik < nt) {
@@ -293,7 +302,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                                 if (!(ok = mbar_wait(bar_full(ks), (kseq / ns) & 1, s_abort, p.status))) break;
                                 tc_fence_after();
                             }
-                            mma_s_grouped_block<D>(tmem + l * 128, desc_lo(sbase + C::OFF_Q + (two ? l : 0) * C::Q_BYTES, 16), desc_lo(slot_base(ks), 16), idesc_s);
+                            mma_s_grouped_block<D>(tmem + l * 128, desc_lo(sbase + C::OFF_Q + (u.nrt > 1 ? l : 0) * C::Q_BYTES, 16), desc_lo(slot_base(ks), 16), idesc_s);
                             tc_commit(bar_sfull(l));
                             if (!two || l == 1) {
                                 tc_commit(bar_free(ks));
@@ -310,7 +319,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             uint32_t uq = 0;
             if (lane == 0) {
                 bool ok = true;
-                while (ok && wk.next(p, &u)) {
+                while (ok && wk.next_pair(p, &u)) {
                     volatile UnitDesc* d = &s_units[uq % kUnitRing];
                     d->b = u.b; d->kh = u.kh; d->rg = u.rg; d->t0 = u.t0; d->t1 = u.t1; d->tiles = u.tiles; d->n = u.n; d->ctx = u.ctx; d->nrt = u.nrt;
                     if (p.cs == 0 && !(u.t0 == 0 && u.t1 == u.tiles)) {
@@ -329,11 +338,12 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     }
                     mbar_arrive(bar_ufull(uq % kUnitRing));
                     if (uq > 0 && !(ok = mbar_wait(bar_qfree, (uq - 1) & 1, s_abort, p.status))) break;
-                    mbar_expect_tx(bar_qfull, (uint32_t)(u.nrt * C::DB * RT * 128));
-                    for (int rt = 0; rt < u.nrt; ++rt)
+                    const int nq = min(u.nrt, 2), head = u.nrt == kTwoHeads ? 1 : 0;   // query tiles: two row tiles, or two heads' only one
+                    mbar_expect_tx(bar_qfull, (uint32_t)(nq * C::DB * RT * 128));
+                    for (int k = 0; k < nq; ++k)
                         for (int db = 0; db < C::DB; ++db)
-                            tma_load_4d(sbase + C::OFF_Q + rt * C::Q_BYTES + db * (CB_MT * 128), &maps.q, bar_qfull, db * 64, u.kh * p.G,
-                                        (u.rg * 2 + rt) * p.NPT, u.b);
+                            tma_load_4d(sbase + C::OFF_Q + k * C::Q_BYTES + db * (CB_MT * 128), &maps.q, bar_qfull, db * 64, (u.kh + k * head) * p.G,
+                                        (u.rg * 2 + k * (1 - head)) * p.NPT, u.b);
                     ++uq;
                 }
                 if (ok) {
@@ -392,9 +402,10 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             if (!(ok = mbar_wait(bar_ufull(uq % kUnitRing), (uq / kUnitRing) & 1, s_abort, p.status))) break;
             const volatile UnitDesc* u = &s_units[uq % kUnitRing];   // read again where it is needed: registers are short
             if (u->nrt == 0) break;
-            const bool two = u->nrt == 2;
+            const bool two = u->nrt > 1;                      // a chain has its own rows: a row tile, or a head's only one
+            const int lr = u->nrt == 2 ? l : 0;               // row tile of the unit
             const int step = two ? 1 : 2, tfirst = u->t0 + (two ? 0 : l), t1 = u->t1, nfull = min(u->ctx / CB_KT, u->tiles - 1);
-            const int node = (u->rg * 2 + (two ? l : 0)) * p.NPT + row / p.G;
+            const int node = (u->rg * 2 + lr) * p.NPT + row / p.G;
             const bool row_valid = row < RT && node < u->n;
             const bool warp_active = (wq * 32) < RT && node - row / p.G + (wq * 32) / p.G < u->n;   // row 0 of the warp is valid
             // this row's ancestor bits: word 0 (the reference is taken from the tile's first 32 keys) and this half's two words
@@ -550,7 +561,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             }
             if (!ok) break;
             // ---- epilogue of this unit's share
-            const int ub = u->b, t0 = u->t0, h = u->kh * p.G + row % p.G;
+            const int ub = u->b, t0 = u->t0, h = (u->kh + (u->nrt == kTwoHeads ? l : 0)) * p.G + row % p.G;
             const bool whole = t0 == 0 && t1 == u->tiles;
             // this thread's columns of the output row, 16 at a time: half a row with two row tiles, a quarter with one
             int npc, c0;

@@ -139,6 +139,7 @@ extern "C" cb_status cb_tree_attn(cb_ctx* ctx, const cb_attn_args* a, void* stre
     p.max_pages = a->max_pages; p.num_pages = a->num_pages;
     p.NPT = CB_MT / p.G;
     p.npt_inv = 65536u / (uint32_t)p.NPT + 1u;
+    p.g_inv = 65536u / (uint32_t)p.G + 1u;
     p.MT = (p.T + p.NPT - 1) / p.NPT;
     const float scale = a->scale > 0.f ? a->scale : 1.0f / sqrtf((float)c.head_dim);
     p.scale_log2 = scale * 1.4426950408889634f;

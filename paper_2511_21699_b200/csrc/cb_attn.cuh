@@ -48,6 +48,7 @@ struct CbAttnParams {
     int B, T, W, Hq, Hkv, G, D, P, max_pages, num_pages;
     int NPT;              // tree nodes per row tile = 128 / G
     uint32_t npt_inv;     // x / NPT = x * npt_inv >> 16 for x < 256
+    uint32_t g_inv;       // x / G = x * g_inv >> 16 for x < 256
     int MT;               // row tiles that T nodes need = ceil(T / NPT)
     int nc;               // persistent CTAs (= ranges of the global tile sequence)
     int w1, w2;           // positions that a key tile of a unit with one or with two row tiles counts

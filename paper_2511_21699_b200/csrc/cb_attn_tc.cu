@@ -380,6 +380,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
         const int sw = warp - 4, l = sw >> 3, hf = (sw >> 2) & 1;   // chain, half of the tile's keys
         const int wq = warp & 3;                              // TMEM lane quarter this warp may access
         const int row = wq * 32 + lane;
+        auto node_of = [&](int r) { return (int)((uint32_t)r * p.g_inv >> 16); };   // r / G: a row is node * G + head of the group
         const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
         const int pair_id = 1 + l * 4 + wq;                   // named barrier of the two warps that share these rows
         constexpr int CW = D / 4;                             // accumulator columns handled at a time
@@ -412,9 +413,9 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             const bool two = u->nrt > 1;                      // a chain has its own rows: a row tile, or a head's only one
             const int lr = u->nrt == 2 ? l : 0;               // row tile of the unit
             const int step = two ? 1 : 2, tfirst = u->t0 + (two ? 0 : l), t1 = u->t1, nfull = min(u->ctx / CB_KT, u->tiles - 1);
-            const int node = (u->rg * 2 + lr) * p.NPT + row / p.G;
+            const int node = (u->rg * 2 + lr) * p.NPT + node_of(row);
             const bool row_valid = row < RT && node < u->n;
-            const bool warp_active = (wq * 32) < RT && node - row / p.G + (wq * 32) / p.G < u->n;   // row 0 of the warp is valid
+            const bool warp_active = (wq * 32) < RT && node - node_of(row) + node_of(wq * 32) < u->n;   // row 0 of the warp is valid
             // this row's ancestor bits: word 0 (the reference is taken from the tile's first 32 keys) and this half's two words
             uint32_t mref = 0u, mlo = 0u, mhi = 0u;
             if (row_valid && t1 == u->tiles) {
@@ -568,7 +569,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             }
             if (!ok) break;
             // ---- epilogue of this unit's share
-            const int ub = u->b, t0 = u->t0, h = (u->kh + (u->nrt == kTwoHeads ? l : 0)) * p.G + row % p.G;
+            const int ub = u->b, t0 = u->t0, h = (u->kh + (u->nrt == kTwoHeads ? l : 0)) * p.G + row - node_of(row) * p.G;
             const bool whole = t0 == 0 && t1 == u->tiles;
             // this thread's columns of the output row, 16 at a time: half a row with two row tiles, a quarter with one
             int npc, c0;

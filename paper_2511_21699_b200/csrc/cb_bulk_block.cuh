@@ -6,9 +6,9 @@
 // of the run, the table of the part's leaders and that of its (leader, follower) pairs lie in shared memory, so claims, "last
 // index" maxima and the grouping of pairs by leader are shared-memory operations, and what is left in global memory is an atomic per
 // new leader and the entry itself.  Through scratch in global memory the same run is six launches whose every step is a chain of L2
-// round trips: batch 32 of 1,024 to 8,192 tokens (147 k windows), reset and first draft with it, 118 us against 32.7 us this way
-// (some 17 of them this kernel's: 31 k cycles in its first form, of which the entries took 10 k, claiming 5.5 k, the reads of lengths and
-// tokens 5 k).  What bounds it is the chain of phases in a block, a thread or two per window: a quarter of the SM's issue
+// round trips: batch 32 of 1,024 to 8,192 tokens (147 k windows), reset and first draft with it, 118 us against 30.2 us this way
+// (some 17 of them this kernel's, 35 k cycles: lengths, parts and tokens 6 k, listing the part's windows 3 k, claims 7 k with the second
+// turn of those beyond 1,024, ranges and grouping 2.5 k, entries and their index words 12 k, the rest at the end).  What bounds it is the chain of phases in a block, a thread or two per window: a quarter of the SM's issue
 // rate, 18% of the shared-memory pipe, 5 MB from DRAM; half of the stalled warps wait at a barrier.
 //
 // Parts: every block reads all lengths and deals gridDim.x parts to the sequences in proportion to their windows (at least one
@@ -48,7 +48,8 @@ struct BlkSmem {
     int32_t first[kBlkMaxBatch];       // first position, clock, leaders and windows of every sequence
     uint32_t clock[kBlkMaxBatch], count[kBlkMaxBatch];
     uint16_t nwin[kBlkMaxBatch];
-    uint32_t red[32], total, n_own, n_lead, n_pair, n_fresh, n_list, base;
+    float inv;                         // one over the windows of a part
+    uint32_t red[32], total, n_multi, n_own, n_lead, n_pair, n_fresh, n_list, base;
 };
 static_assert(sizeof(BlkSmem) <= 227 * 1024, "shared memory of one CTA");
 constexpr uint32_t kBlkFresh = 0x80000000u;
@@ -244,10 +245,33 @@ __device__ __noinline__ uint32_t blk_evictions(BlkSmem& S, const uint32_t* entri
     return out;
 }
 
-__device__ __forceinline__ uint32_t blk_parts(uint32_t nwin, uint32_t spare, uint32_t all) {
-    if (nwin == 0u) return 0u;
-    const uint32_t share = 1u + (uint32_t)((unsigned long long)nwin * spare / all);
-    return max(min(share, max(nwin / 32u, 1u)), (nwin + kBlkPart - 1u) / kBlkPart);
+// Parts of a run of n windows where a part is to have 1 / inv of them: no more than kBlkPart expected in one.
+__device__ __forceinline__ uint32_t blk_parts(uint32_t n, float inv) {
+    return n == 0u ? 0u : max((uint32_t)ceilf((float)n * inv), (n + kBlkPart - 1u) / kBlkPart);
+}
+// One warp: about the smallest number of windows a part with which the parts of all sequences are no more than the blocks (a part too many
+// is a second turn for some block, and the longest part is what the launch waits for: shares rounded down left 16 of 148 blocks without a
+// part at batch 32 and gave 1,270 windows to one where 1,050 do).
+// (Parts of 32, 96, 224 and 448 windows at least, 22 shapes, time against the shares before: 0.978, 0.976, 0.982, 1.001; single shapes of
+// few windows lie 1 to 3% to either side.)
+constexpr int kBlkLeast = 64;
+constexpr int kBlkSearch = 8;                                   // sequences a lane
+__device__ __forceinline__ float blk_share(const uint16_t* nwin, int B, uint32_t blocks, int lane) {
+    uint32_t n[kBlkSearch], all = 0;
+#pragma unroll
+    for (int q = 0; q < kBlkSearch; ++q) { n[q] = q * 32 + lane < B ? nwin[q * 32 + lane] : 0u; all += n[q]; }
+    all = __reduce_add_sync(CB_FULL, all);
+    float share = fmaxf((float)all / ((float)blocks - 0.5f * (float)B), (float)kBlkLeast), inv = 1.f / share;   // rounding up adds half a part a sequence
+    for (int k = 0; k < 16; ++k) {
+        uint32_t parts = 0;
+#pragma unroll
+        for (int q = 0; q < kBlkSearch; ++q) if (q * 32 < B) parts += blk_parts(n[q], inv);
+        parts = __reduce_add_sync(CB_FULL, parts);
+        if (parts <= blocks) break;
+        share += share * (float)(parts - blocks) / (float)blocks + 1.f;
+        inv = 1.f / share;
+    }
+    return inv;
 }
 
 // alone: no other kernel follows, so that no run may be longer than kBlkRun windows.  COUNT_ALL: every follower that the windows displace
@@ -269,7 +293,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
     const int w = LL + t.FL;
     {
         // the parts of all sequences
-        uint32_t nwin = 0, all = 0, parts = 0;
+        uint32_t nwin = 0, parts = 0;
         if (tid < B) {
             const uint2 h = *reinterpret_cast<const uint2*>(cb_seq(t, tid).hdr);
             const int first = max(0, n_old[tid] - w + 1);
@@ -281,9 +305,14 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
             if (!cb_dbg_in(h.y, (long long)t.LC + 1, t.dbg_status)) nwin = 0;
             S.nwin[tid] = (uint16_t)nwin; S.first[tid] = first; S.clock[tid] = h.x; S.count[tid] = h.y;
         }
-        (void)blk_scan(nwin, S.red, &all);
-        const uint32_t spare = gridDim.x > (uint32_t)B ? gridDim.x - (uint32_t)B : 0u;
-        const uint32_t mine = blk_parts(nwin, spare, max(all, 1u));
+        float inv = 1.f / (float)kBlkPart;
+        if ((uint32_t)B < gridDim.x && B <= 32 * kBlkSearch) {
+            __syncthreads();
+            if (warp == 0) { const float x = blk_share(S.nwin, B, gridDim.x, lane); if (lane == 0) S.inv = x; }
+            __syncthreads();
+            inv = S.inv;
+        }
+        const uint32_t mine = blk_parts(nwin, inv);
         const uint32_t before = blk_scan(mine, S.red, &parts);
         if (tid < B) S.pre[tid] = before;
         if (tid == 0) { S.pre[B] = parts; S.total = parts; }
@@ -316,8 +345,20 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
             // ---- the run's tokens
             {
                 if (u != blockIdx.x) clear_tables();
-                for (uint32_t i = tid; i < nwin + (uint32_t)w - 1u; i += kBlkThreads) S.tok[i] = row[first + (int)i];
-                if (tid == 0) { S.n_own = 0u; S.n_lead = 0u; S.n_pair = 0u; S.n_fresh = 0u; S.n_list = 0u; }
+                // all of a thread's loads at once (one after the other they were 3.6 k cycles)
+                auto fetch = [&](auto loads) {
+                    constexpr int U = decltype(loads)::value;
+                    const uint32_t len = nwin + (uint32_t)w - 1u;
+                    int32_t x[U];
+#pragma unroll
+                    for (int q = 0; q < U; ++q) x[q] = (uint32_t)(q * kBlkThreads + tid) < len ? row[first + q * kBlkThreads + tid] : 0;
+#pragma unroll
+                    for (int q = 0; q < U; ++q) if ((uint32_t)(q * kBlkThreads + tid) < len) S.tok[q * kBlkThreads + tid] = x[q];
+                };
+                constexpr int kMost = (kBlkRun + CB_MAX_LL + CB_MAX_FL + kBlkThreads - 1) / kBlkThreads;
+                if (nwin + (uint32_t)w <= 2u * kBlkThreads) fetch(std::integral_constant<int, 2>{});
+                else fetch(std::integral_constant<int, kMost>{});
+                if (tid == 0) { S.n_multi = 0u; S.n_own = 0u; S.n_lead = 0u; S.n_pair = 0u; S.n_fresh = 0u; S.n_list = 0u; }
             }
             __syncthreads();
             // ---- the part's windows are listed first (in `group`), so that the claims below run with full warps
@@ -327,17 +368,25 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                 for (int j = 0; j < LL; ++j) k4[j] = S.tok[k + j];
                 return cb_hash4(k4[0], k4[1], k4[2], k4[3], LL);
             };
-            for (uint32_t k0 = warp * 32; k0 < nwin; k0 += kBlkThreads) {
-                const uint32_t k = k0 + lane;
+            uint32_t own[kBlkRun / kBlkThreads], mine_n = 0;
+#pragma unroll
+            for (int q = 0; q < kBlkRun / kBlkThreads; ++q) {
+                const uint32_t k = (uint32_t)(q * kBlkThreads + tid);
+                own[q] = 0u;
+                if ((uint32_t)(q * kBlkThreads + warp * 32) >= nwin) continue;
                 uint32_t x = 0x85EBCA6Bu;
 #pragma unroll
                 for (int j = 0; j < LL; ++j) { x = (x ^ (uint32_t)S.tok[k + j]) * 0x9E3779B1u; x ^= x >> 16; }
-                const bool own = k < nwin && __umulhi(x * 0xC2B2AE35u, np) == part;
-                const uint32_t m = __ballot_sync(CB_FULL, own);
-                uint32_t at = 0;
-                if (m && lane == 0) at = atomicAdd(&S.n_own, (uint32_t)__popc(m));
-                at = __shfl_sync(CB_FULL, at, 0) + __popc(m & ((1u << lane) - 1u));
-                if (own) S.group[at] = (uint16_t)k;
+                own[q] = __ballot_sync(CB_FULL, k < nwin && __umulhi(x * 0xC2B2AE35u, np) == part);
+                mine_n += (uint32_t)__popc(own[q]);
+            }
+            uint32_t own_at = 0;
+            if (lane == 0 && mine_n) own_at = atomicAdd(&S.n_own, mine_n);
+            own_at = __shfl_sync(CB_FULL, own_at, 0);
+#pragma unroll
+            for (int q = 0; q < kBlkRun / kBlkThreads; ++q) {
+                if ((own[q] >> lane) & 1u) S.group[own_at + __popc(own[q] & ((1u << lane) - 1u))] = (uint16_t)(q * kBlkThreads + tid);
+                own_at += (uint32_t)__popc(own[q]);
             }
             __syncthreads();
             const uint32_t n_own = S.n_own;
@@ -370,6 +419,9 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
             __syncthreads();
             // ---- every leader takes a range of the pairs
             const uint32_t nl = S.n_lead, n_pair = S.n_pair;
+            // the ids of new leaders; where all are new, under way while the pairs are grouped
+            uint32_t got = 0;
+            if (tid == 0 && count0 == 0u && nl) got = atomicAdd(&s.hdr[2], nl);
             for (uint32_t o0 = 0, g0 = 0; o0 < nl; o0 += kBlkThreads) {
                 const uint32_t o = o0 + tid, ls = o < nl ? S.lslot[o] : 0u, c = o < nl ? S.cur[ls] : 0u;
                 uint32_t tot;
@@ -431,8 +483,12 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                 }
                 __syncthreads();
             }
-            const uint32_t n_fresh = count0 > 0u ? S.n_fresh : nl;
-            if (tid == 0) S.base = count0 + (n_fresh ? atomicAdd(&s.hdr[2], n_fresh) : 0u);
+            if (tid == 0) {
+                if (count0 > 0u && S.n_fresh) got = atomicAdd(&s.hdr[2], S.n_fresh);
+                S.base = count0 + got;
+            }
+            // (the hash of this thread's first leader, meanwhile)
+            const uint64_t mine_h = (uint32_t)tid < nl ? leader_hash((S.lead[S.lslot[tid]] >> 16) - 1u) : 0ull;
             __syncthreads();
             const uint32_t base = S.base;
             // entry id of leader o: the plan excludes that ids run out
@@ -445,12 +501,12 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
             // launch is over (the look-up above passes over ids from count0 on), so it may go out before the entry is written, and
             // the entries are written while the first attempts are under way.
             struct Claim { uint64_t h; uint32_t word, tries; bool open; };
-            auto claim_of = [&](uint32_t o) {
+            auto claim_of = [&](uint32_t o, uint64_t h) {
                 Claim c = {0, 0, 0, false};
                 if (o < nl) {
                     const uint32_t eid = entry_of(o, &c.open);
                     c.open = c.open && eid < (uint32_t)t.LC;
-                    c.h = leader_hash(((S.lead[S.lslot[o]] & ~kBlkMark) >> 16) - 1u);
+                    c.h = h;
                     c.word = (cb_hash_tag(c.h) << CB_EID_BITS) | eid;
                 }
                 return c;
@@ -459,7 +515,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                 const uint32_t nb = t.nslots >> 5, bucket = (cb_hash_bucket(c.h, t.nslots) + (c.tries >> 5)) & (nb - 1);
                 return &s.index[bucket * 32u + (((uint32_t)(c.h >> 20) + c.tries) & 31u)];
             };
-            Claim mine = claim_of((uint32_t)tid);
+            Claim mine = claim_of((uint32_t)tid, mine_h);
             uint32_t mine_old = CB_IDX_EMPTY;
             if (mine.open) mine_old = atomicCAS(attempt(mine), CB_IDX_EMPTY, mine.word);
             auto finish = [&](Claim& c, uint32_t old) {              // old: what the first attempt met
@@ -471,23 +527,15 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                 }
                 cnt.maxprobe = max(cnt.maxprobe, (c.tries >> 5) + 1u);
             };
-            // ---- entries: as many lanes to a leader as there are threads for (8 at most) write a new one that has room for its followers,
-            // 16 bytes at a time; the others are listed
+            // ---- entries, 16 bytes at a time: key, stamps (0: free), tokens of the followers that there are; zeros behind them up to 16
+            // bytes.  A new leader that has room for its followers is written by a team of lanes, the others are listed.
             const uint32_t fl_inv = 65536u / (uint32_t)t.FL + 1u;          // x * fl_inv >> 16 = x / FL for x < 8,192
-            const int lg = nl > kBlkThreads / 2 ? 0 : nl > kBlkThreads / 4 ? 1 : nl > kBlkThreads / 8 ? 2 : 3;
-            const uint32_t team = (uint32_t)tid & ((1u << lg) - 1u);
-            for (uint32_t o = (uint32_t)tid >> lg; o < nl; o += (uint32_t)kBlkThreads >> lg) {
-                const uint32_t lw = S.lead[S.lslot[o]], kpos = (lw >> 16) - 1u, g = S.gbase[o], n = S.gbase[o + 1] - g;
-                bool fresh;
-                const uint32_t eid = entry_of(o, &fresh);
-                if (!fresh || n > (uint32_t)t.FC) {
-                    if (team == 0u) S.pl[atomicAdd(&S.n_list, 1u)] = (uint16_t)o;
-                    continue;
-                }
-                if (eid >= (uint32_t)t.LC) continue;
+            auto team_of = [](uint32_t n) { return n > kBlkThreads / 2 ? 0 : n > kBlkThreads / 4 ? 1 : n > kBlkThreads / 8 ? 2 : 3; };   // log2 of its lanes
+            auto write_entry = [&](uint32_t o, uint32_t eid, int lg) {
+                if (eid >= (uint32_t)t.LC) return;
+                const uint32_t lw = S.lead[S.lslot[o]], kpos = (lw >> 16) - 1u, g = S.gbase[o], n = S.gbase[o + 1] - g, team = (uint32_t)tid & ((1u << lg) - 1u);
                 uint32_t* e = s.entries + (size_t)eid * t.E;
                 if (team == 0u) s.lstamp[eid] = clock0 + (lw & 0xFFFFu);
-                // key, stamps (0: free), tokens of the followers that there are; zeros behind them up to 16 bytes
                 // (most leaders have one follower, which is looked up once)
                 const uint32_t end = (uint32_t)(LL + t.FC) + n * (uint32_t)t.FL, pw0 = S.pair[S.group[g]];
                 for (uint32_t q0 = 4u * team; q0 < end; q0 += 4u << lg) {
@@ -503,6 +551,45 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                         if (f < 0 || (x >= 0 && pw)) v[j] = (uint32_t)S.tok[at];
                     }
                     *reinterpret_cast<uint4*>(e + q0) = make_uint4(v[0], v[1], v[2], v[3]);
+                }
+            };
+            if (nl > kBlkThreads / 2) {
+                // A thread to a leader: those with one follower, as most are, are their first window's tokens and one stamp and need no look at
+                // the pairs; the few with more come after them (all in one loop: 8.1 k cycles, so 6).  Shorter lists go to teams as they are:
+                // a second loop and its barrier cost a part of 60 leaders more than it gains.
+                for (uint32_t o = (uint32_t)tid; o < nl; o += kBlkThreads) {
+                    const uint32_t lw = S.lead[S.lslot[o]], kpos = (lw >> 16) - 1u, n = S.gbase[o + 1] - S.gbase[o];
+                    bool fresh;
+                    const uint32_t eid = entry_of(o, &fresh);
+                    if (!fresh || n > (uint32_t)t.FC) { S.pl[atomicAdd(&S.n_list, 1u)] = (uint16_t)o; continue; }
+                    if (n > 1u) { S.pslot[atomicAdd(&S.n_multi, 1u)] = (uint16_t)o; continue; }       // the pairs' list is not needed any more
+                    if (eid >= (uint32_t)t.LC) continue;
+                    uint32_t* e = s.entries + (size_t)eid * t.E;
+                    const uint32_t stamp = clock0 + (lw & 0xFFFFu);
+                    s.lstamp[eid] = stamp;
+                    for (int q0 = 0; q0 < LL + t.FC + t.FL; q0 += 4) {
+                        uint32_t v[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int x = q0 + j, y = x < LL ? x : x - t.FC;    // its place among the window's tokens
+                            v[j] = (x < LL || x >= LL + t.FC) && y < w ? (uint32_t)S.tok[kpos + y] : (x == LL ? stamp : 0u);
+                        }
+                        *reinterpret_cast<uint4*>(e + q0) = make_uint4(v[0], v[1], v[2], v[3]);
+                    }
+                }
+                __syncthreads();
+                const int lg = team_of(S.n_multi);
+                for (uint32_t i = (uint32_t)tid >> lg; i < S.n_multi; i += (uint32_t)kBlkThreads >> lg) {
+                    bool fresh;
+                    write_entry(S.pslot[i], entry_of(S.pslot[i], &fresh), lg);
+                }
+            } else {
+                const int lg = team_of(nl);
+                for (uint32_t o = (uint32_t)tid >> lg; o < nl; o += (uint32_t)kBlkThreads >> lg) {
+                    bool fresh;
+                    const uint32_t eid = entry_of(o, &fresh);
+                    if (fresh && S.gbase[o + 1] - S.gbase[o] <= (uint32_t)t.FC) write_entry(o, eid, lg);
+                    else if (((uint32_t)tid & ((1u << lg) - 1u)) == 0u) S.pl[atomicAdd(&S.n_list, 1u)] = (uint16_t)o;
                 }
             }
             __syncthreads();
@@ -574,16 +661,14 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
             // ---- the rest of the publication
             if (mine.open) finish(mine, mine_old);
             for (uint32_t o = tid + kBlkThreads; o < nl; o += kBlkThreads) {
-                Claim c = claim_of(o);
+                Claim c = claim_of(o, leader_hash(((S.lead[S.lslot[o]] & ~kBlkMark) >> 16) - 1u));
                 if (c.open) finish(c, atomicCAS(attempt(c), CB_IDX_EMPTY, c.word));
             }
         }
         // ---- the last block of the sequence folds the run into its header
         __syncthreads();
         if (tid == 0) {
-            __threadfence();
-            if (atomicAdd(&s.hdr[3], 1u) == np - 1u) {
-                __threadfence();
+            if (add_acq_rel(&s.hdr[3], 1u) == np - 1u) {
                 s.hdr[1] = count0 + __ldcg(&s.hdr[2]);
                 s.hdr[0] = clock0 + nwin;
                 s.hdr[2] = 0u;

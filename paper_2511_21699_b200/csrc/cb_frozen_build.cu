@@ -3,12 +3,12 @@
 //
 // A window is LL + FL consecutive tokens; the corpus of N tokens has M = N - LL - FL + 1 of them.  Everything is counting
 // and selection on integers, done without sorting:
-//   1. leader counts: every window inserts-or-increments its leader in an open-addressing table whose slots hold the
-//      position of one occurrence (keys are compared by reading the corpus there), with the counters in an array beside it; a
+//   1. leader counts: every window inserts-or-increments its leader in an open-addressing table whose slots hold the leader's tokens as
+//      one number (or, where they do not fit 63 bits, the position of one occurrence), with the counters in an array beside it; a
 //      window remembers its leader's slot for step 3;
 //   2. the LC best leaders under the order (count falling, tokens rising) are found by a most-significant-digit-first
-//      radix select over the distinct leaders (one histogram pass per 12 bits of the composite key; the block that comes
-//      last picks the digit), then written into the frozen table's entries and hashed into its index;
+//      radix select over the table (one histogram pass per 12 bits of the composite key; every block picks the digit for
+//      itself), then take a range for their windows and are written into the frozen table's entries and hashed into its index;
 //   3. the windows of the selected leaders go into the leaders' ranges of one array (a counting sort: the leader counts are known
 //      from step 1), all but those of the few leaders with more than kBigGroup windows: these insert-or-increment the whole window in
 //      a second hash table, and the distinct ones are grouped by leader afterwards;
@@ -16,22 +16,25 @@
 //      (up to 32 windows: the lanes match their tokens against one another) or by a block with a table in shared memory; of a
 //      big leader's distinct windows a block picks the FC best from memory.  The pick: a threshold by bisection on the count, then on
 //      the tokens of the windows that tie with it where those are many; what is left is ranked.
-// What bounds it is random access: to the leader table (positions and counts apart, four slots for three windows) and to the ranges.  The frequent
+// What bounds it is random access: to the leader table (four slots for three windows) and to the ranges.  The frequent
 // keys' counts and the lists are gathered per block in shared memory, so that a key that makes up a tenth of the corpus costs
 // an atomic per block and not one per occurrence.  Counting every selected window in a second hash table took 212 us of a build from 4 M
 // tokens (LL = 2, LC = 65,536, FC = 8: 167 MB of tables at random, more than the L2 holds), grouping its slots 49 us, ranking 187 us.
-// The whole call with the draft that follows it: 763 us that way, 505 us this way (60,000 tokens: 220 and 165; 13 launches of the selection
-// are one, which is most of it there).  Of the 505: leader counts 94, windows into ranges 104, selection 75 (86 while the few threads with a
-// leader placed it between two barriers), ranking some 150 with its kernels side by side.
+// The whole call with the draft that follows it: 763 us that way, 508 with windows in ranges, and 470 with keys in the leader table, read from
+// end to end by the selection, and ranges taken as the leaders are placed (a table of positions with a list of its used slots: the same
+// call from 302 k tokens 218, so 183; 949 k, LL = 3: 256 and 218).  Of the 470: leader counts 91, windows into ranges 105, selection 60,
+// ranking some 150 with its kernels side by side.
 // Which occurrence represents a key, and which entry id a leader gets, depends on timing; the table's content (and
 // cb_frozen_dump's output) does not.
 #include <algorithm>
+#include <type_traits>
 
 #include "cb_common.cuh"
 
 namespace {
 
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
+constexpr unsigned long long kNoLeader = ~0ull;                    // first table: a free slot
 constexpr unsigned long long kEmptySlot = 0x00000000FFFFFFFFull;   // second table; low word: position, high word: count
 constexpr int kMaxWords = 1 + CB_MAX_LL;      // composite selection key: count (complemented), then the leader's tokens
 constexpr int kDigitBits = 12, kBins = 1 << kDigitBits;
@@ -44,7 +47,7 @@ static_assert(kCand >= 2 * CB_MAX_FC, "the FC best and as many ties fit");
 
 struct BuildState {                           // head of the scratch buffer
     uint32_t status;                          // (the state is cleared before the first launch)
-    uint32_t n_uniq;                          // distinct leaders
+    uint32_t n_once;                          // leaders that occur once (counted where that matters)
     uint32_t n_sel;                           // entry ids handed out
     uint32_t n_warp, n_mid, n_large, n_big;   // leaders with more than 32, kWarpGroup, kMidGroup, kBigGroup windows
     uint32_t n_ties;                          // leaders whose count is exactly that of the LC-th best
@@ -61,12 +64,13 @@ static_assert(offsetof(BuildState, hist) % 16 == 0, "histograms are read 16 byte
 
 struct BuildView {
     BuildState* st;
-    uint32_t* h1; uint32_t* h1_cnt;                               // [S1] leaders: position of an occurrence; count, later kTaken | entry id of a selected one
+    unsigned long long* h1;                                       // [S1] leaders: the tokens as one number where they fit, else the position of an occurrence
+    uint32_t* h1_cnt;                                             // [S1] occurrences but one; of a selected one later kTaken | next free place of its range,
+                                                                  // with more than kBigGroup windows kTaken | kBigLeader | entry id
     unsigned long long* h2; uint32_t* h2_ord;                     // [S] windows of big leaders (big_slots in use); ordinal in the leader's group
     uint32_t* lslot;                                              // [M] leader slot of every window (kEmpty: left out)
     uint2* group;                                                 // [M] distinct windows of the big leaders, grouped by leader: position, count
-    uint32_t* uniq; uint2* ties;                                  // [M] slots of the distinct leaders; slot and position of those that tie with the LC-th best
-                                                                  // (both share group's memory: dead before that is filled)
+    uint32_t* ties;                                               // [M] slots of the leaders that tie with the LC-th best (in group's memory: dead before that is filled)
     uint32_t* wpos;                                               // [M] windows of the other selected leaders, grouped by leader
     uint32_t* grp_n; uint32_t* grp_off;                           // [LC] windows placed (big: distinct ones); start, kBigFlag: of group, else of wpos
     uint32_t* listed; uint32_t* listed_big;                       // [LC] each: middling leaders from the front, large ones from the back; big ones
@@ -78,7 +82,7 @@ struct BuildView {
     int LL, FL, LC, FC;
 };
 
-constexpr uint32_t kTaken = 0x80000000u, kBigFlag = 0x80000000u;   // counts and positions stay below 2^30
+constexpr uint32_t kTaken = 0x80000000u, kBigLeader = 0x40000000u, kBigFlag = 0x80000000u;   // counts, positions and entry ids stay below 2^30
 
 __device__ __forceinline__ uint64_t hash_tokens(const int32_t* p, int n) {
     uint64_t h = 0x9E3779B97F4A7C15ull ^ (uint64_t)n;
@@ -90,20 +94,36 @@ __device__ __forceinline__ bool same_tokens(const int32_t* a, const int32_t* b, 
     for (int j = 0; j < n; ++j) if (a[j] != b[j]) return false;
     return true;
 }
-// The first table keeps positions and counts apart and has four slots for three windows (45 MB for 4 M windows; eight-byte slots, two a
-// window, were 67 MB: 547 against 542 us for the build).  Home slots are the hash's share of the table.
+// A leader's tokens as one number, the first one highest, so that the numbers' order is that of the tokens: bits each, as many as the
+// corpus' largest token has.  0: they do not fit 63 bits (four tokens of 16 bits or more); the table then holds positions.  With
+// positions, every look at a slot is followed by one at the corpus (4 M windows, LL = 2: count of the leaders 94 us).
+__device__ __forceinline__ int key_bits(const BuildView& v) {
+    const int bits = max(32 - __clz((int)v.st->max_token), 1);
+    return bits * v.LL <= 63 ? bits : 0;
+}
+__device__ __forceinline__ uint64_t hash_key(uint64_t k) {
+    k *= 0xFF51AFD7ED558CCDull; k ^= k >> 32;
+    k *= 0xC4CEB9FE1A85EC53ull; return k ^ (k >> 29);
+}
+// Token j of the leader in a slot that holds x.
+__device__ __forceinline__ int32_t leader_token(const BuildView& v, int bits, uint64_t x, int j) {
+    return bits ? (int32_t)((x >> (bits * (v.LL - 1 - j))) & ((1ull << bits) - 1ull)) : v.corpus[(uint32_t)x + j];
+}
+// The first table keeps keys and counts apart and has four slots for three windows.  Home slots are the hash's share of the table.
 __device__ __forceinline__ uint32_t home_leader(uint64_t h, uint32_t S1) { return __umulhi((uint32_t)(h >> 20), S1); }
-// Finds or creates the slot of the leader at corpus position i, from slot s on; kEmpty when every slot was visited.
-__device__ __forceinline__ uint32_t claim_leader(uint32_t* slots, uint32_t S1, uint32_t s, const int32_t* corpus, uint32_t i, int n, bool* created) {
+// Finds or creates the slot of leader `me` (same(x): the one that a slot holds is this), from slot s on, whose word is x; kEmpty when every
+// slot was visited.
+template <typename Same>
+__device__ __forceinline__ uint32_t claim_leader(unsigned long long* slots, uint32_t S1, uint32_t s, unsigned long long x, unsigned long long me, bool* created, Same&& same) {
     *created = false;
     for (uint32_t p = 0; p < S1; ++p) {
-        uint32_t pos = slots[s];
-        if (pos == kEmpty) {
-            pos = atomicCAS(&slots[s], kEmpty, i);
-            if (pos == kEmpty) { *created = true; return s; }
+        if (x == kNoLeader) {
+            x = atomicCAS(&slots[s], kNoLeader, me);
+            if (x == kNoLeader) { *created = true; return s; }
         }
-        if (same_tokens(corpus + pos, corpus + i, n)) return s;
+        if (same(x)) return s;
         s = s + 1 == S1 ? 0u : s + 1;
+        x = slots[s];
     }
     return kEmpty;
 }
@@ -229,67 +249,153 @@ __global__ void __launch_bounds__(256) fb_init_kernel(BuildView v, CbTables t) {
         if (neg) { v.st->has_neg = 1u; if (v.M > 0) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_INVALID_ARG); }
     }
     // last, so that it is in L2 when the leaders are counted
-    uint4* const pos = reinterpret_cast<uint4*>(v.h1);
-    uint4* const cnt = reinterpret_cast<uint4*>(v.h1_cnt);       // whoever makes a slot has been counted
-    for (size_t i = g; i < v.S1 / 4; i += stride) { cnt[i] = make_uint4(1u, 1u, 1u, 1u); pos[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty); }
+    uint4* const key = reinterpret_cast<uint4*>(v.h1);
+    uint4* const cnt = reinterpret_cast<uint4*>(v.h1_cnt);
+    for (size_t i = g; i < v.S1 / 4; i += stride) cnt[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (size_t i = g; i < v.S1 / 2; i += stride) key[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
 }
 
-// 1. leader counts.  Four windows a thread, so that their chains (slot, tokens of the slot's occurrence) overlap; what the first look
-// does not settle is looked up slot by slot.
+// 1. leader counts.  Four windows a thread, so that their chains (slot, atomic) overlap.
+// What a block has met lies in shared memory, a key to each place: the windows with such a key are counted there and never look at the
+// table, and where the corpus begins, a frequent key's free slot is tried once a block and not by every thread that has it (733 k
+// windows, LL = 1: 38 us, 75 without it).
+template <int U>
+__device__ __forceinline__ void left_out(const BuildView& v, size_t i0, int LL, bool (&ok)[U]) {   // the windows with a negative token
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+        for (int j = 0; j < LL + v.FL && ok[q]; ++j) ok[q] = v.corpus[i0 + q * 256 + threadIdx.x + j] >= 0;
+}
+struct KeyCache {
+    static constexpr uint32_t N = 1024;
+    unsigned long long key[N];
+    uint32_t slot[N], cnt[N];
+};
 template <int LL>
-__global__ void __launch_bounds__(256) fb_count_leaders_kernel(BuildView v) {
-    CB_PDL_ENTRY();
-    __shared__ CountCache<1> cache;
-    __shared__ Appender<uint32_t> made;
-    cache.clear();
-    made.clear();
+__device__ __forceinline__ void count_packed(const BuildView& v, int bits, KeyCache& cache) {
     constexpr int U = 4;
+    for (uint32_t i = threadIdx.x; i < KeyCache::N; i += 256) { cache.key[i] = kNoLeader; cache.cnt[i] = 0u; }
+    __syncthreads();
     const size_t stride = (size_t)gridDim.x * 256 * U;
     const bool has_neg = v.st->has_neg != 0u;
     for (size_t i0 = (size_t)blockIdx.x * 256 * U; i0 < v.M; i0 += stride) {
-        uint32_t s[U], pos[U];
-        bool ok[U], created[U];
-        int32_t key[U][LL], rep[U][LL];
+        uint32_t s[U], at[U];
+        unsigned long long x[U], me[U];
+        bool ok[U], look[U], first[U];                          // look: this thread finds or makes the slot; first: it has a place in the cache
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const size_t i = i0 + q * 256 + threadIdx.x;
             ok[q] = i < v.M;
-            created[q] = false;
+            me[q] = 0ull;
 #pragma unroll
-            for (int j = 0; j < LL; ++j) key[q][j] = ok[q] ? v.corpus[i + j] : 0;
+            for (int j = 0; j < LL; ++j) me[q] = me[q] << bits | (ok[q] ? (uint32_t)v.corpus[i + j] : 0u);
+            const uint64_t h = hash_key(me[q]);
+            s[q] = home_leader(h, v.S1);
+            at[q] = (uint32_t)h & (KeyCache::N - 1);
         }
-        if (has_neg) {                                          // the windows with a negative token are left out
-#pragma unroll 1
-            for (int q = 0; q < U; ++q)
-                for (int j = 0; j < LL + v.FL && ok[q]; ++j) ok[q] = v.corpus[i0 + q * 256 + threadIdx.x + j] >= 0;
-        }
+        if (has_neg) left_out(v, i0, LL, ok);
 #pragma unroll
         for (int q = 0; q < U; ++q) {
-            s[q] = home_leader(hash_tokens(key[q], LL), v.S1);
-            pos[q] = ok[q] ? v.h1[s[q]] : kEmpty;
+            look[q] = first[q] = false;
+            if (!ok[q]) continue;
+            unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&cache.key[at[q]]);
+            if (k == kNoLeader) {
+                k = atomicCAS(&cache.key[at[q]], kNoLeader, me[q]);
+                first[q] = k == kNoLeader;
+            }
+            look[q] = k != me[q];
+            if (!look[q]) atomicAdd(&cache.cnt[at[q]], 1u);
         }
+        // A slot never changes once it is set, so an ordinary load will do; one that still shows a free slot is put right by the
+        // compare-and-swap.
 #pragma unroll
-        for (int q = 0; q < U; ++q)
+        for (int q = 0; q < U; ++q) x[q] = look[q] ? v.h1[s[q]] : kNoLeader;
 #pragma unroll
-            for (int j = 0; j < LL; ++j) rep[q][j] = pos[q] != kEmpty ? v.corpus[pos[q] + j] : -1;
+        for (int q = 0; q < U; ++q) {
+            if (!look[q]) continue;
+            bool created = false;
+            if (x[q] != me[q]) s[q] = claim_leader(v.h1, v.S1, s[q], x[q], me[q], &created, [&](unsigned long long y) { return y == me[q]; });
+            if (s[q] == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
+            if (first[q]) cache.slot[at[q]] = s[q];
+            if (created || s[q] == kEmpty) continue;
+            if (first[q]) atomicAdd(&cache.cnt[at[q]], 1u);
+            else atomicAdd(&v.h1_cnt[s[q]], 1u);
+        }
+        __syncthreads();                                        // the new places' slots are known
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const size_t i = i0 + q * 256 + threadIdx.x;
+            if (i < v.M) v.lslot[i] = !ok[q] ? kEmpty : (look[q] ? s[q] : cache.slot[at[q]]);
+        }
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < KeyCache::N; i += 256)
+        if (cache.cnt[i] && cache.slot[i] != kEmpty) atomicAdd(&v.h1_cnt[cache.slot[i]], cache.cnt[i]);
+}
+// The same for longer leaders, most of which a block meets once: no places for keys, the counts alone are gathered.
+template <int LL>
+__device__ __forceinline__ void count_packed(const BuildView& v, int bits, CountCache<1>& cache) {
+    constexpr int U = 4;
+    cache.clear();
+    const size_t stride = (size_t)gridDim.x * 256 * U;
+    const bool has_neg = v.st->has_neg != 0u;
+    for (size_t i0 = (size_t)blockIdx.x * 256 * U; i0 < v.M; i0 += stride) {
+        uint32_t s[U];
+        unsigned long long x[U], me[U];
+        bool ok[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const size_t i = i0 + q * 256 + threadIdx.x;
+            ok[q] = i < v.M;
+            me[q] = 0ull;
+#pragma unroll
+            for (int j = 0; j < LL; ++j) me[q] = me[q] << bits | (ok[q] ? (uint32_t)v.corpus[i + j] : 0u);
+            s[q] = home_leader(hash_key(me[q]), v.S1);
+        }
+        if (has_neg) left_out(v, i0, LL, ok);
+#pragma unroll
+        for (int q = 0; q < U; ++q) x[q] = ok[q] ? v.h1[s[q]] : kNoLeader;
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const size_t i = i0 + q * 256 + threadIdx.x;
             if (ok[q]) {
-                int32_t diff = 0;
-#pragma unroll
-                for (int j = 0; j < LL; ++j) diff |= rep[q][j] ^ key[q][j];
-                if (diff != 0)                                  // an empty slot or another key's
-                    s[q] = claim_leader(v.h1, v.S1, pos[q] == kEmpty ? s[q] : (s[q] + 1 == v.S1 ? 0u : s[q] + 1), v.corpus, (uint32_t)i, LL, &created[q]);
+                bool created = false;
+                if (x[q] != me[q]) s[q] = claim_leader(v.h1, v.S1, s[q], x[q], me[q], &created, [&](unsigned long long y) { return y == me[q]; });
                 if (s[q] == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
-                else if (!created[q]) cache.add(v.h1_cnt, s[q]);
+                else if (!created) cache.add(v.h1_cnt, s[q]);
             }
             if (i < v.M) v.lslot[i] = ok[q] ? s[q] : kEmpty;
         }
-        made.add(created, s, v.uniq, &v.st->n_uniq);
     }
-    made.flush(v.uniq, &v.st->n_uniq);
     cache.flush(v.h1_cnt);
+}
+// The same with positions in the table: every look at a slot is followed by one at the tokens there.
+template <int LL>
+__device__ __forceinline__ void count_positions(const BuildView& v, CountCache<1>& cache) {
+    cache.clear();
+    const bool has_neg = v.st->has_neg != 0u;
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < v.M; i += (size_t)gridDim.x * 256) {
+        bool ok = true, created = false;
+        for (int j = 0; has_neg && j < LL + v.FL; ++j) ok = ok && v.corpus[i + j] >= 0;
+        uint32_t s = kEmpty;
+        if (ok) {
+            s = home_leader(hash_tokens(v.corpus + i, LL), v.S1);
+            s = claim_leader(v.h1, v.S1, s, v.h1[s], i, &created, [&](unsigned long long y) { return same_tokens(v.corpus + (uint32_t)y, v.corpus + i, LL); });
+            if (s == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
+            else if (!created) cache.add(v.h1_cnt, s);
+        }
+        v.lslot[i] = s;
+    }
+    cache.flush(v.h1_cnt);
+}
+constexpr int kCachedKeys = 2;                // up to that many tokens a leader's keys are kept (LL = 3: 36 us with the counts alone, 52 with keys; LL = 2: 117 and 90)
+template <int LL>
+__global__ void __launch_bounds__(256) fb_count_leaders_kernel(BuildView v) {
+    CB_PDL_ENTRY();
+    using Cache = std::conditional_t<LL <= kCachedKeys, KeyCache, CountCache<1>>;
+    __shared__ union { Cache keys; CountCache<1> slots; } cache;
+    const int bits = key_bits(v);
+    if (bits) count_packed<LL>(v, bits, cache.keys);
+    else count_positions<LL>(v, cache.slots);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -297,8 +403,9 @@ __global__ void __launch_bounds__(256) fb_count_leaders_kernel(BuildView v) {
 // and every one needs the result of the one before (13 launches otherwise, for 60,000 tokens most of the build's time).
 constexpr int kSelThreads = 1024;
 struct SelSmem {
-    uint32_t bins[kBins], part[32], pick[2], last, start;
-    Appender<uint2, 8192> taken, tied;        // slot and count, slot and position
+    uint32_t bins[kBins], part[32], pick[2], last, start, range, made[4], from[4];
+    Appender<uint2, 12288> taken;             // slot and count
+    Appender<uint32_t, 12288> tied;           // slot
 };
 
 // All blocks of the launch; false after a wait that ran out (the others run out too).  The call then returns CB_ERR_TIMEOUT, whatever
@@ -345,11 +452,12 @@ __device__ __forceinline__ uint32_t sel_scan(uint32_t x, uint32_t* part, uint32_
     return incl - x + (warp > 0 ? before : 0u);
 }
 // The bin of a finished histogram in which the k-th smallest key lies; *rest: its rank inside the bin.  Every block for itself.
-__device__ __forceinline__ uint32_t pick_bin(const uint32_t* hist, uint32_t k, SelSmem& S, uint32_t* rest) {
+__device__ __forceinline__ uint32_t pick_bin(const uint32_t* hist, uint32_t k, SelSmem& S, uint32_t* rest, uint32_t* all = nullptr) {
     const uint4 c = __ldcg(reinterpret_cast<const uint4*>(hist) + threadIdx.x);      // four bins a thread
     const uint32_t cs[4] = {c.x, c.y, c.z, c.w};
     uint32_t total;
     uint32_t cum = sel_scan(cs[0] + cs[1] + cs[2] + cs[3], S.part, &total);
+    if (all) *all = total;                                      // (fewer than k keys: the bin means nothing)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         if (cum < k && k <= cum + cs[j]) { S.pick[0] = threadIdx.x * 4 + j; S.pick[1] = k - cum; }
@@ -395,44 +503,99 @@ __device__ __forceinline__ void sel_histogram(uint32_t n, uint32_t* hist, SelSme
         if (S.bins[i]) atomicAdd(&hist[i], S.bins[i]);
 }
 
-// The leader in slot `at` of the first table gets entry eid; its key goes into the frozen table's index.
-__device__ __forceinline__ void place_leader(const BuildView& v, const CbTables& t, uint32_t eid, uint32_t at, uint32_t count) {
-    if (eid >= (uint32_t)v.LC) { atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT); return; }
-    v.h1_cnt[at] = kTaken | eid;
-    const int32_t* key = v.corpus + v.h1[at];
+// The same over the counts of the first table, four slots a load: bin_of(count, slot), for counts of two or more.
+template <typename F>
+__device__ __forceinline__ void sel_count_histogram(const BuildView& v, uint32_t* hist, SelSmem& S, F&& bin_of) {
+    for (int i = threadIdx.x; i < kBins; i += kSelThreads) S.bins[i] = 0u;
+    __syncthreads();
+    const uint4* const cnt = reinterpret_cast<const uint4*>(v.h1_cnt);
+    constexpr int U = 4;
+    const uint32_t n = v.S1 / 4, step = gridDim.x * kSelThreads;
+    for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n; i0 += U * step) {
+        uint4 c[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) { const uint32_t i = i0 + q * step + threadIdx.x; c[q] = i < n ? cnt[i] : make_uint4(0u, 0u, 0u, 0u); }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const uint32_t x[4] = {c[q].x, c[q].y, c[q].z, c[q].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) add_bin(S.bins, x[j] ? bin_of(x[j] + 1u) : kEmpty);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kBins; i += kSelThreads)
+        if (S.bins[i]) atomicAdd(&hist[i], S.bins[i]);
+}
+
+// The leader in slot `at` of the first table, which says `word` from now on, gets entry eid; its key goes into the frozen table's index.
+__device__ __forceinline__ void place_leader(const BuildView& v, const CbTables& t, int bits, uint32_t eid, uint32_t at, uint32_t count, uint32_t word) {
+    v.h1_cnt[at] = word;
+    const uint64_t key = v.h1[at];
     uint32_t* e = t.entries + (size_t)eid * t.E;
     int32_t k4[4] = {0, 0, 0, 0};
-    for (int j = 0; j < v.LL; ++j) { k4[j] = key[j]; e[j] = (uint32_t)key[j]; }
+#pragma unroll
+    for (int j = 0; j < CB_MAX_LL; ++j) if (j < v.LL) { k4[j] = leader_token(v, bits, key, j); e[j] = (uint32_t)k4[j]; }
     t.lstamp[eid] = count;
     const uint64_t h = cb_hash4(k4[0], k4[1], k4[2], k4[3], v.LL);
-    const uint32_t nb = t.nslots >> 5, word = (cb_hash_tag(h) << CB_EID_BITS) | eid;
+    const uint32_t nb = t.nslots >> 5, tagged = (cb_hash_tag(h) << CB_EID_BITS) | eid;
+    // From a place of its own on through the bucket, then through the next one: with the bucket's first free slot tried first, the eight leaders
+    // that it gets at once took eight rounds of a compare-and-swap each (placing 65,536 leaders 27 us).
     uint32_t bucket = cb_hash_bucket(h, t.nslots);
     for (uint32_t p = 0; p < nb; ++p) {
-        // the bucket's 32 words at once; only those seen empty are tried
-        const uint4* bp = reinterpret_cast<const uint4*>(t.index + (size_t)bucket * 32);
-        uint32_t empty = 0u;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const uint4 x = __ldcg(bp + q);
-            empty |= ((x.x == CB_IDX_EMPTY ? 1u : 0u) | (x.y == CB_IDX_EMPTY ? 2u : 0u) | (x.z == CB_IDX_EMPTY ? 4u : 0u) | (x.w == CB_IDX_EMPTY ? 8u : 0u)) << (4 * q);
-        }
-        for (; empty; empty &= empty - 1u)
-            if (atomicCAS(&t.index[bucket * 32 + __ffs(empty) - 1], CB_IDX_EMPTY, word) == CB_IDX_EMPTY) return;
+        for (uint32_t j = 0; j < 32u; ++j)
+            if (atomicCAS(&t.index[bucket * 32 + (((uint32_t)(h >> 20) + j) & 31u)], CB_IDX_EMPTY, tagged) == CB_IDX_EMPTY) return;
         bucket = (bucket + 1) & (nb - 1);
     }
     atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
 }
 
 
-// All leaders gathered so far (slot and count) take entries, one atomic for all of them; all threads of the block together.  They are
+// All leaders gathered so far (slot and count) take entries and ranges for their windows, an atomic for the entries and one per 1,024
+// ranges, which lie side by side; those with more than 32 windows are listed by size.  All threads of the block together.  They are
 // gathered first because a placement is a chain of some 4 k cycles that the few threads with a leader would otherwise take between two
 // barriers of all.
-__device__ __forceinline__ void place_taken(const BuildView& v, const CbTables& t, SelSmem& S) {
+__device__ __forceinline__ void place_taken(const BuildView& v, const CbTables& t, int bits, SelSmem& S) {
     __syncthreads();
     const uint32_t n = S.taken.n;
     if (threadIdx.x == 0) S.start = n ? atomicAdd(&v.st->n_sel, n) : 0u;
-    __syncthreads();
-    for (uint32_t j = threadIdx.x; j < n; j += kSelThreads) place_leader(v, t, S.start + j, S.taken.item[j].x, S.taken.item[j].y);
+    for (uint32_t j0 = 0; j0 < n; j0 += kSelThreads) {
+        const uint32_t j = j0 + threadIdx.x;
+        const bool has = j < n;
+        const uint2 item = has ? S.taken.item[j] : make_uint2(0u, 0u);
+        const bool big = item.y > kBigGroup;
+        const uint32_t c = big ? 0u : item.y;
+        uint32_t total;
+        const uint32_t before = sel_scan(c, S.part, &total);
+        if (threadIdx.x == 0) S.range = total ? atomicAdd(&v.st->cursor, total) : 0u;
+        if (threadIdx.x < 4) S.made[threadIdx.x] = 0u;
+        __syncthreads();
+        const uint32_t eid = S.start + j;
+        const bool fits = has && eid < (uint32_t)v.LC;
+        if (has && !fits) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
+        // the listed kinds take their places in the block first (one address takes one atomic in about 2 ns)
+        const int kind = !fits ? -1 : big ? 3 : c > kMidGroup ? 2 : c > kWarpGroup ? 1 : c > 32u ? 0 : -1;
+        const uint32_t place = kind >= 0 ? atomicAdd(&S.made[kind], 1u) : 0u;
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            uint32_t* const lists[4] = {&v.st->n_warp, &v.st->n_mid, &v.st->n_large, &v.st->n_big};
+            S.from[threadIdx.x] = S.made[threadIdx.x] ? atomicAdd(lists[threadIdx.x], S.made[threadIdx.x]) : 0u;
+        }
+        __syncthreads();
+        const uint32_t at = kind >= 0 ? S.from[kind] + place : 0u;
+        if (kind == 0) v.listed_big[v.LC - 1 - at] = eid;
+        else if (kind == 1) v.listed[at] = eid;
+        else if (kind == 2) v.listed[v.LC - 1 - at] = eid;
+        else if (kind == 3) v.listed_big[at] = eid;
+        if (!fits) continue;
+        const uint32_t start = S.range + before;
+        if (big) {
+            v.grp_off[eid] = kBigFlag | atomicAdd(&v.st->big_cursor, item.y);   // no more distinct windows than windows
+        } else {
+            v.grp_off[eid] = start;
+            v.grp_n[eid] = c;
+        }
+        place_leader(v, t, bits, eid, item.x, item.y, kTaken | (big ? kBigLeader | eid : start));
+    }
     __syncthreads();
     if (threadIdx.x == 0) S.taken.n = 0u;
     __syncthreads();
@@ -441,138 +604,135 @@ __device__ __forceinline__ void place_taken(const BuildView& v, const CbTables& 
 __global__ void __launch_bounds__(kSelThreads, 1) fb_select_kernel(BuildView v, CbTables t, int cbits) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     SelSmem& S = *reinterpret_cast<SelSmem*>(sel_smem);
-    const uint32_t n = v.st->n_uniq, LC = (uint32_t)v.LC, cmask = (1u << cbits) - 1u;
-    const bool all = n <= LC;                                   // all of them are taken
-    uint32_t round = 0, pass = 0, cut = 0, k = LC;
-    if (!all) {
-        // 2a. the count of the LC-th best leader: a bin per count below 4,095 (most comes first), the last one for all above
-        sel_histogram(n, v.st->hist[pass], S, [&](uint32_t i) { return kBins - 1 - min(v.h1_cnt[v.uniq[i]], (uint32_t)(kBins - 1)); });
-        if (!grid_barrier(v, &round, &S.last)) return;
-        uint32_t rest, bin = pick_bin(v.st->hist[pass++], k, S, &rest);
-        if (bin > 0u) {
-            cut = kBins - 1 - bin;
-            k = rest;
-        } else {
-            // 4,095 or more: digit by digit over the complemented count
-            uint32_t prefix = 0;
-            for (int shift = (cbits - 1) / kDigitBits * kDigitBits; shift >= 0; shift -= kDigitBits) {
-                const uint32_t hi_mask = shift + kDigitBits >= 32 ? 0u : (0xFFFFFFFFu << (shift + kDigitBits));
-                sel_histogram(n, v.st->hist[pass], S, [&](uint32_t i) {
-                    const uint32_t x = cmask - v.h1_cnt[v.uniq[i]];
-                    return (x & hi_mask) == (prefix & hi_mask) ? (x >> shift) & (kBins - 1) : kEmpty;
-                });
-                if (!grid_barrier(v, &round, &S.last)) return;
-                bin = pick_bin(v.st->hist[pass++], k, S, &k);
-                prefix |= bin << shift;
-            }
-            cut = cmask - prefix;
+    const uint32_t LC = (uint32_t)v.LC, cmask = (1u << cbits) - 1u;
+    const int bits = key_bits(v);
+    bool all = false;                                           // all of them are taken
+    uint32_t round = 0, pass = 0, cut = 1, k = LC, n = LC;
+    // 2a. the count of the LC-th best leader: a bin per count from two to 4,094 (most comes first), the last one for all above.  The table is
+    // read from one end to the other; by a list of its used slots every look was one at random (and the list took the count
+    // kernel's blocks a barrier for every four windows of a thread).
+    sel_count_histogram(v, v.st->hist[pass], S, [&](uint32_t c) { return kBins - 1 - min(c, (uint32_t)(kBins - 1)); });
+    if (!grid_barrier(v, &round, &S.last)) return;
+    uint32_t rest, more, bin = pick_bin(v.st->hist[pass++], k, S, &rest, &more);
+    if (more < LC) {
+        // not enough occur twice: those that occur once tie, or all are taken
+        const uint4* const cnt = reinterpret_cast<const uint4*>(v.h1_cnt);
+        const ulonglong2* const key = reinterpret_cast<const ulonglong2*>(v.h1);
+        uint32_t once = 0;
+        for (uint32_t i = blockIdx.x * kSelThreads + threadIdx.x; i < v.S1 / 4; i += gridDim.x * kSelThreads) {
+            const uint4 c = cnt[i];
+            const ulonglong2 a = key[2 * i], b = key[2 * i + 1];
+            once += (c.x == 0u && a.x != kNoLeader) + (c.y == 0u && a.y != kNoLeader) + (c.z == 0u && b.x != kNoLeader) + (c.w == 0u && b.y != kNoLeader);
         }
+        once = __reduce_add_sync(CB_FULL, once);
+        if ((threadIdx.x & 31) == 0 && once) atomicAdd(&v.st->n_once, once);
+        if (!grid_barrier(v, &round, &S.last)) return;
+        n = more + __ldcg(&v.st->n_once);
+        all = n <= LC;
+        k = LC - more;
+    } else if (bin > 0u) {
+        cut = kBins - 1 - bin;
+        k = rest;
+    } else {
+        // 4,095 or more: digit by digit over the complemented count
+        uint32_t prefix = 0;
+        for (int shift = (cbits - 1) / kDigitBits * kDigitBits; shift >= 0; shift -= kDigitBits) {
+            const uint32_t hi_mask = shift + kDigitBits >= 32 ? 0u : (0xFFFFFFFFu << (shift + kDigitBits));
+            sel_count_histogram(v, v.st->hist[pass], S, [&](uint32_t c) {
+                const uint32_t x = cmask - c;
+                return (x & hi_mask) == (prefix & hi_mask) ? (x >> shift) & (kBins - 1) : kEmpty;
+            });
+            if (!grid_barrier(v, &round, &S.last)) return;
+            bin = pick_bin(v.st->hist[pass++], k, S, &k);
+            prefix |= bin << shift;
+        }
+        cut = cmask - prefix;
     }
     // 2b. the leaders with a larger count are placed, those with the same count listed
     S.taken.clear();
     S.tied.clear();
     const uint32_t step = gridDim.x * kSelThreads;
-    for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n; i0 += 4 * step) {
-        uint32_t at[4], cnt[4], pos[4];
-        bool take[4], tie[4];
-        uint2 x[4];
+    {
+        constexpr int U = 8;                                    // slots of a thread between two barriers
+        const uint4* const cnt = reinterpret_cast<const uint4*>(v.h1_cnt);
+        const uint32_t n4 = v.S1 / 4;
+        for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n4; i0 += U / 4 * step) {
+            uint4 c4[U / 4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) at[q] = i0 + q * step + threadIdx.x < n ? v.uniq[i0 + q * step + threadIdx.x] : kEmpty;
+            for (int h = 0; h < U / 4; ++h) { const uint32_t i = i0 + h * step + threadIdx.x; c4[h] = i < n4 ? cnt[i] : make_uint4(0u, 0u, 0u, 0u); }
+            uint32_t at[U];
+            bool take[U], tie[U];
+            uint2 x[U];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) cnt[q] = at[q] != kEmpty ? v.h1_cnt[at[q]] : 0u;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            take[q] = at[q] != kEmpty && (all || cnt[q] > cut);
-            tie[q] = at[q] != kEmpty && !take[q] && cnt[q] == cut;
-            pos[q] = tie[q] ? v.h1[at[q]] : 0u;
-            x[q] = make_uint2(at[q], cnt[q]);
-        }
-        S.taken.put(take, x);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = make_uint2(at[q], pos[q]);
-        S.tied.put(tie, x);
-        if (__syncthreads_or(S.taken.near_full(4) || S.tied.near_full(4))) {
-            place_taken(v, t, S);
-            S.tied.flush(v.ties, &v.st->n_ties);
+            for (int q = 0; q < U; ++q) {
+                const uint32_t i = i0 + (q / 4) * step + threadIdx.x, c = (q % 4 == 0 ? c4[q / 4].x : q % 4 == 1 ? c4[q / 4].y : q % 4 == 2 ? c4[q / 4].z : c4[q / 4].w) + 1u;
+                at[q] = 4 * i + q % 4;
+                // a count of one may be a free slot's
+                const bool there = c > 1u || (cut == 1u && i < n4 && v.h1[at[q]] != kNoLeader);
+                take[q] = there && (all || c > cut);
+                tie[q] = there && !take[q] && c == cut;
+                x[q] = make_uint2(at[q], c);
+            }
+            S.taken.put(take, x);
+            S.tied.put(tie, at);
+            if (__syncthreads_or(S.taken.near_full(U) || S.tied.near_full(U))) {
+                place_taken(v, t, bits, S);
+                S.tied.flush(v.ties, &v.st->n_ties);
+            }
         }
     }
-    place_taken(v, t, S);
+    // (what is gathered by now is placed with the ties that are taken)
+    if (all) place_taken(v, t, bits, S);
     S.tied.flush(v.ties, &v.st->n_ties);
     if (blockIdx.x == 0 && threadIdx.x == 0) t.hdr[1] = min(n, LC);
     if (!grid_barrier(v, &round, &S.last)) return;
     if (!all) {
-        // 2c. of those the k first by tokens, digit by digit; leading digits that are zero in every token are passed over
+        // 2c. of those the k first by tokens, digit by digit: over the whole number that the slot holds, or token by token
         const uint32_t n_ties = __ldcg(&v.st->n_ties);
-        uint32_t prefix[CB_MAX_LL] = {0u, 0u, 0u, 0u};
-        auto before_or_in = [&](uint32_t pos, int words) {      // -1, 0, 1: the leader's first words against the prefix
-            for (int j = 0; j < words; ++j) {
-                const uint32_t x = (uint32_t)v.corpus[pos + j];
-                if (x != prefix[j]) return x < prefix[j] ? -1 : 1;
+        const int words = bits ? 1 : v.LL, wbits = bits ? bits * v.LL : max(32 - __clz((int)v.st->max_token), 1);
+        uint64_t prefix[CB_MAX_LL] = {0ull, 0ull, 0ull, 0ull};
+        // a thread's first tie stays in its registers: most have no other
+        const uint32_t i_mine = blockIdx.x * kSelThreads + threadIdx.x, at_mine = i_mine < n_ties ? __ldcg(&v.ties[i_mine]) : 0u;
+        const uint64_t x_mine = v.h1[at_mine];
+        auto word = [&](uint64_t x, int w) { return bits ? x : (uint64_t)(uint32_t)v.corpus[(uint32_t)x + w]; };
+        auto before_or_in = [&](uint64_t x, int upto) {         // -1, 0, 1: the leader's first words against the prefix
+            for (int j = 0; j < upto; ++j) {
+                const uint64_t y = word(x, j);
+                if (y != prefix[j]) return y < prefix[j] ? -1 : 1;
             }
             return 0;
         };
-        for (int w = 0; w < v.LL; ++w)
-            for (int shift = 24; shift >= 0; shift -= kDigitBits) {
-                if (shift > 0 && (v.st->max_token >> shift) == 0u) continue;
-                const uint32_t hi_mask = shift + kDigitBits >= 32 ? 0u : (0xFFFFFFFFu << (shift + kDigitBits));
+        for (int w = 0; w < words; ++w)
+            for (int shift = (wbits - 1) / kDigitBits * kDigitBits; shift >= 0; shift -= kDigitBits) {
+                const uint64_t hi_mask = shift + kDigitBits >= 64 ? 0ull : (~0ull << (shift + kDigitBits));
                 sel_histogram(n_ties, v.st->hist[pass], S, [&](uint32_t i) {
-                    const uint32_t pos = __ldcg(&v.ties[i]).y;
-                    if (before_or_in(pos, w) != 0) return kEmpty;
-                    const uint32_t x = (uint32_t)v.corpus[pos + w];
-                    return (x & hi_mask) == (prefix[w] & hi_mask) ? (x >> shift) & (kBins - 1) : kEmpty;
+                    const uint64_t x = i == i_mine ? x_mine : v.h1[__ldcg(&v.ties[i])];
+                    if (before_or_in(x, w) != 0) return kEmpty;
+                    const uint64_t y = word(x, w);
+                    return (y & hi_mask) == (prefix[w] & hi_mask) ? (uint32_t)(y >> shift) & (kBins - 1) : kEmpty;
                 });
                 if (!grid_barrier(v, &round, &S.last)) return;
-                const uint32_t bin = pick_bin(v.st->hist[pass++], k, S, &k);
-                prefix[w] |= bin << shift;
+                const uint32_t digit = pick_bin(v.st->hist[pass++], k, S, &k);
+                prefix[w] |= (uint64_t)digit << shift;
             }
         // 2d. placed like the others
         for (uint32_t i0 = blockIdx.x * kSelThreads; i0 < n_ties; i0 += step) {
-            const uint32_t i = i0 + threadIdx.x;
-            const uint2 x = i < n_ties ? __ldcg(&v.ties[i]) : make_uint2(0u, 0u);
-            const bool take[1] = {i < n_ties && before_or_in(x.y, v.LL) <= 0};
-            const uint2 item[1] = {make_uint2(x.x, cut)};
-            if (S.taken.gather(take, item)) place_taken(v, t, S);
+            const uint32_t i = i0 + threadIdx.x, at = i == i_mine ? at_mine : i < n_ties ? __ldcg(&v.ties[i]) : 0u;
+            const bool take[1] = {i < n_ties && before_or_in(i == i_mine ? x_mine : v.h1[at], words) <= 0};
+            const uint2 item[1] = {make_uint2(at, cut)};
+            if (S.taken.gather(take, item)) place_taken(v, t, bits, S);
         }
-        place_taken(v, t, S);
+        place_taken(v, t, bits, S);
         if (!grid_barrier(v, &round, &S.last)) return;
     }
-    // 3a. every selected leader takes a range (an atomic per block and 1,024 of them: their ranges lie side by side); those with more than
-    // 32 windows are listed by size
-    const uint32_t n_sel = min(__ldcg(&v.st->n_sel), LC);
-    for (uint32_t e0 = blockIdx.x * kSelThreads; e0 < n_sel; e0 += gridDim.x * kSelThreads) {
-        const uint32_t e = e0 + threadIdx.x, windows = e < n_sel ? __ldcg(&t.lstamp[e]) : 0u;
-        const bool big = windows > kBigGroup;
-        const uint32_t c = big ? 0u : windows;
-        uint32_t total;
-        const uint32_t before = sel_scan(c, S.part, &total);
-        if (threadIdx.x == 0) S.start = total ? atomicAdd(&v.st->cursor, total) : 0u;
-        // the most frequent of the listed kinds: an atomic per warp
-        const int lane = threadIdx.x & 31;
-        const bool by_warp = c > 32u && c <= kWarpGroup;
-        const uint32_t m = __ballot_sync(CB_FULL, by_warp);
-        uint32_t k2 = 0;
-        if (m && lane == 0) k2 = atomicAdd(&v.st->n_warp, (uint32_t)__popc(m));
-        k2 = __shfl_sync(CB_FULL, k2, 0) + __popc(m & ((1u << lane) - 1u));
-        if (by_warp) v.listed_big[v.LC - 1 - k2] = e;
-        __syncthreads();
-        if (big) {
-            v.grp_off[e] = kBigFlag | atomicAdd(&v.st->big_cursor, windows);   // no more distinct windows than windows
-            v.listed_big[atomicAdd(&v.st->n_big, 1u)] = e;
-        } else if (e < n_sel) {
-            v.grp_off[e] = S.start + before;
-            if (c > kMidGroup) v.listed[v.LC - 1 - atomicAdd(&v.st->n_large, 1u)] = e;
-            else if (c > kWarpGroup) v.listed[atomicAdd(&v.st->n_mid, 1u)] = e;
-        }
-    }
-    // 3b. the part of the second table that the big leaders' windows need
-    if (!grid_barrier(v, &round, &S.last)) return;
+    // 3a. the part of the second table that the big leaders' windows need
     if (__ldcg(&v.st->n_big) == 0u) return;
     const uint32_t S2 = big_slots(v);
     ulonglong2* a = reinterpret_cast<ulonglong2*>(v.h2);
     for (size_t i = (size_t)blockIdx.x * kSelThreads + threadIdx.x; i < S2 / 2; i += (size_t)gridDim.x * kSelThreads) a[i] = make_ulonglong2(kEmptySlot, kEmptySlot);
 }
 
-// 3c. every window of a selected leader goes into its leader's range; a big leader's window is counted in the second table, where a
+// 3b. every window of a selected leader goes into its leader's range; a big leader's window is counted in the second table, where a
 // new one takes its ordinal in its leader's group.  Four windows a thread, whose chains (leader slot, leader, place) overlap.
 __global__ void __launch_bounds__(256) fb_windows_kernel(BuildView v) {
     CB_PDL_ENTRY();
@@ -582,71 +742,64 @@ __global__ void __launch_bounds__(256) fb_windows_kernel(BuildView v) {
     const bool any_big = v.st->n_big != 0u;
     const uint32_t S2 = any_big ? big_slots(v) : 0u;
     if (any_big) cache.clear();
-    __shared__ Appender<uint2> big;
-    big.clear();
+    __shared__ uint2 s_big[8][160];                             // by warp: position and entry id
     const int lane = threadIdx.x & 31;
-    auto count_big = [&] {                                      // all threads of the block together
-        const uint32_t n = big.n;
-        for (uint32_t j0 = 0; j0 < n; j0 += blockDim.x) {
-            const uint32_t j = j0 + threadIdx.x;
-            const uint2 x = j < n ? big.item[j] : make_uint2(0u, 0u);
-            bool created = false;
-            uint32_t s = kEmpty;
-            if (j < n) {
-                s = find_or_claim(v.h2, S2, home_slot(v.corpus + x.x, v.LL + v.FL, S2), v.corpus, x.x, v.LL + v.FL, &created);
-                if (s == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
-                else if (!created) cache.add(counts_of(v.h2), s);
-            }
-            // the new windows of one leader in a warp take their ordinals with one atomic
-            if (__any_sync(CB_FULL, created)) {
-                const uint32_t peers = __match_any_sync(CB_FULL, created ? (int)x.y : -1 - lane);
-                const int head = __ffs(peers) - 1;
-                uint32_t o = 0;
-                if (created && lane == head) o = atomicAdd(&v.grp_n[x.y], (uint32_t)__popc(peers));
-                o = __shfl_sync(CB_FULL, o, head) + __popc(peers & ((1u << lane) - 1u));
-                if (created) v.h2_ord[s] = o;
-            }
+    uint2* const list = s_big[threadIdx.x >> 5];
+    uint32_t n_list = 0;
+    auto count_big = [&](bool has) {                            // the last 32 of the list
+        const uint2 x = has ? list[n_list + lane] : make_uint2(0u, 0u);
+        __syncwarp();
+        bool created = false;
+        uint32_t s = kEmpty;
+        if (has) {
+            s = find_or_claim(v.h2, S2, home_slot(v.corpus + x.x, v.LL + v.FL, S2), v.corpus, x.x, v.LL + v.FL, &created);
+            if (s == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
+            else if (!created) cache.add(counts_of(v.h2), s);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) big.n = 0u;
-        __syncthreads();
+        // the new windows of one leader in a warp take their ordinals with one atomic
+        if (__any_sync(CB_FULL, created)) {
+            const uint32_t peers = __match_any_sync(CB_FULL, created ? (int)x.y : -1 - lane);
+            const int head = __ffs(peers) - 1;
+            uint32_t o = 0;
+            if (created && lane == head) o = atomicAdd(&v.grp_n[x.y], (uint32_t)__popc(peers));
+            o = __shfl_sync(CB_FULL, o, head) + __popc(peers & ((1u << lane) - 1u));
+            if (created) v.h2_ord[s] = o;
+        }
     };
     const size_t stride = (size_t)gridDim.x * blockDim.x * U;
     for (size_t i0 = (size_t)blockIdx.x * blockDim.x * U; i0 < v.M; i0 += stride) {
-        uint32_t at[U], off[U];
+        uint32_t slot[U], word[U];
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const size_t i = i0 + (size_t)q * blockDim.x + threadIdx.x;
-            at[q] = i < v.M ? v.lslot[i] : kEmpty;
+            slot[q] = i < v.M ? v.lslot[i] : kEmpty;
         }
 #pragma unroll
-        for (int q = 0; q < U; ++q) at[q] = at[q] != kEmpty ? v.h1_cnt[at[q]] : 0u;    // kTaken | entry id, or a count
+        for (int q = 0; q < U; ++q) word[q] = slot[q] != kEmpty ? v.h1_cnt[slot[q]] : 0u;    // (the flags and an entry id do not change here)
 #pragma unroll
-        for (int q = 0; q < U; ++q) off[q] = (at[q] & kTaken) ? v.grp_off[at[q] & ~kTaken] : 0u;
-        uint32_t place[U];
+        for (int q = 0; q < U; ++q) slot[q] = (word[q] & kTaken) && !(word[q] & kBigLeader) ? atomicAdd(&v.h1_cnt[slot[q]], 1u) & ~kTaken : kEmpty;
 #pragma unroll
-        for (int q = 0; q < U; ++q) place[q] = (at[q] & kTaken) && !(off[q] & kBigFlag) ? atomicAdd(&v.grp_n[at[q] & ~kTaken], 1u) : 0u;
-#pragma unroll
-        for (int q = 0; q < U; ++q)
-            if ((at[q] & kTaken) && !(off[q] & kBigFlag)) v.wpos[off[q] + place[q]] = (uint32_t)(i0 + (size_t)q * blockDim.x + threadIdx.x);
+        for (int q = 0; q < U; ++q) if (slot[q] != kEmpty) v.wpos[slot[q]] = (uint32_t)(i0 + (size_t)q * blockDim.x + threadIdx.x);
         if (!any_big) continue;
         // The big leaders' windows are gathered and counted with full warps: they are a seventh of the windows here, some in every warp.
-        bool is_big[U];
-        uint2 item[U];
 #pragma unroll
         for (int q = 0; q < U; ++q) {
-            is_big[q] = (at[q] & kTaken) && (off[q] & kBigFlag);
-            item[q] = make_uint2((uint32_t)(i0 + (size_t)q * blockDim.x + threadIdx.x), at[q] & ~kTaken);
+            const bool is_big = (word[q] & kTaken) && (word[q] & kBigLeader);
+            const uint32_t m = __ballot_sync(CB_FULL, is_big);
+            if (is_big) list[n_list + __popc(m & ((1u << lane) - 1u))] = make_uint2((uint32_t)(i0 + (size_t)q * blockDim.x + threadIdx.x), word[q] & (kBigLeader - 1u));
+            n_list += (uint32_t)__popc(m);
         }
-        if (big.gather(is_big, item)) count_big();
+        __syncwarp();
+        while (n_list >= 32u) { n_list -= 32u; count_big(true); }
     }
     if (any_big) {
-        __syncthreads();
-        count_big();
+        const uint32_t n = n_list;
+        n_list = 0;
+        count_big((uint32_t)lane < n);
         cache.flush(counts_of(v.h2));
     }
 }
-// 3d. the distinct windows of the big leaders, grouped by leader: position and count
+// 3c. the distinct windows of the big leaders, grouped by leader: position and count
 __global__ void __launch_bounds__(256) fb_group_scatter_kernel(BuildView v) {
     CB_PDL_ENTRY();
     if (fb_aborted(v) || v.st->n_big == 0u) return;
@@ -655,7 +808,7 @@ __global__ void __launch_bounds__(256) fb_group_scatter_kernel(BuildView v) {
     for (size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x; s < S2; s += stride) {
         const unsigned long long x = v.h2[s];
         if ((uint32_t)x == kEmpty) continue;
-        const uint32_t eid = v.h1_cnt[v.lslot[(uint32_t)x]] & ~kTaken;
+        const uint32_t eid = v.h1_cnt[v.lslot[(uint32_t)x]] & (kBigLeader - 1u);
         v.group[(v.grp_off[eid] & ~kBigFlag) + v.h2_ord[s]] = make_uint2((uint32_t)x, (uint32_t)(x >> 32));
     }
 }
@@ -1122,7 +1275,7 @@ size_t fb_align(size_t x) { return (x + 255) / 256 * 256; }
 
 struct BuildLayout {
     uint32_t S1, S;
-    size_t off_h1, off_h2, off_h2_ord, off_lslot, off_group, off_grp, total;
+    size_t off_cnt, off_h2, off_h2_ord, off_lslot, off_group, off_grp, total;
 };
 
 cb_status fb_layout(const cb_frozen_config* c, int64_t n_tokens, BuildLayout* B) {
@@ -1134,8 +1287,8 @@ cb_status fb_layout(const cb_frozen_config* c, int64_t n_tokens, BuildLayout* B)
     size_t o = fb_align(sizeof(BuildState));
     uint64_t S1 = ((uint64_t)M + (uint64_t)M / 3 + 1024) / 4 * 4;
     B->S1 = (uint32_t)S1;
-    B->off_h1 = o;      o = fb_align(o + S1 * 8);
-    B->off_h2 = o;      o = fb_align(o + S * 8);
+    B->off_cnt = o;     o = fb_align(o + S1 * 4);
+    B->off_h2 = o;      o = fb_align(o + std::max(S, S1) * 8);   // until the selection's end it holds the first table's words
     B->off_h2_ord = o;  o = fb_align(o + S * 4);
     B->off_lslot = o;   o = fb_align(o + (size_t)(M > 0 ? M : 1) * 4);
     B->off_group = o;   o = fb_align(o + S * 6);   // M x 8 bytes, then M x 4
@@ -1174,10 +1327,10 @@ static cb_status frozen_build(const cb_frozen_config* cfg, const int32_t* dev_co
     char* base = (char*)dev_scratch;
     BuildView v;
     v.st = (BuildState*)base;
-    v.h1 = (uint32_t*)(base + B.off_h1); v.h1_cnt = v.h1 + B.S1;
-    v.h2 = (unsigned long long*)(base + B.off_h2); v.h2_ord = (uint32_t*)(base + B.off_h2_ord);
+    v.h1_cnt = (uint32_t*)(base + B.off_cnt);
+    v.h2 = v.h1 = (unsigned long long*)(base + B.off_h2); v.h2_ord = (uint32_t*)(base + B.off_h2_ord);
     v.lslot = (uint32_t*)(base + B.off_lslot);
-    v.group = (uint2*)(base + B.off_group); v.uniq = (uint32_t*)(base + B.off_group); v.ties = (uint2*)(v.uniq + B.S / 2);   // M <= S / 2
+    v.group = (uint2*)(base + B.off_group); v.ties = (uint32_t*)(base + B.off_group);   // M <= S / 2
     v.wpos = (uint32_t*)(v.group + B.S / 2);                      // behind group's M places
     v.grp_n = (uint32_t*)(base + B.off_grp); v.grp_off = v.grp_n + cfg->LC; v.listed = v.grp_off + cfg->LC;
     v.listed_big = v.listed + cfg->LC;

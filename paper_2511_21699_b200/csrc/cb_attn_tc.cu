@@ -71,7 +71,7 @@ struct Cfg {
     static constexpr uint32_t O_COL = 256;                   // TMEM columns: S0 at 0, S1 at 128, O0 at 256, O1 at 256 + D
 };
 
-struct SchedSmem { long long g0, g1, pre0; int b0, rg0; int c_b, c_kh, c_t0, c_t1, c_tiles, c_n, c_ctx, c_has; };
+struct SchedSmem { long long g0, g1, pre0; int b0, rg0; int c_b, c_kh, c_n, c_has; };   // c_*: cluster mode
 static_assert(sizeof(SchedSmem) <= 64, "the schedule block is followed by the tmem base and the abort flag");
 
 }  // namespace
@@ -150,6 +150,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             for (int k = 0; k < kUnitRing; ++k) mbar_init(bar_ufull(k), 1);
             mbar_init(bar_cready, p.cs > 0 ? (uint32_t)p.cs : 1u); mbar_init(bar_cdata, 1);
             *s_abort = 0;
+            s_sched->c_has = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             tma_prefetch_desc(&maps.k_pool); tma_prefetch_desc(&maps.v_pool); tma_prefetch_desc(&maps.q);
             tma_prefetch_desc(&maps.k_tree); tma_prefetch_desc(&maps.v_tree);
@@ -164,7 +165,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
         ticket_set = (int)(*reinterpret_cast<volatile uint32_t*>(p.part_turn) & 1u) * CB_ATTN_TICKETS;
         if (lane < 16) p.part_ticket[CB_ATTN_TICKETS - ticket_set + cta * 16 + lane] = 0u;
     }
-    if (warp == 3) {
+    if (warp == 3 && p.cs == 0) {
         // The block table into L2, a slice per CTA: the first copies' addresses come from it, and which part of it a CTA needs is
         // known only after the schedule below (two memory round trips one after the other otherwise).
         const long long lines = ((long long)p.B * p.max_pages * 4 + 127) / 128;
@@ -172,19 +173,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
             asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p.block_table) + k * 128));
     }
 
-    if (warp == 0 && p.cs > 0) {
-        // Cluster mode: cluster k works on unit k = (sequence, kv head) and its CTAs take equal parts of the unit's key tiles.
-        if (lane == 0) {
-            const int uid = cta / p.cs, rank = cta % p.cs;
-            const int b = uid / p.Hkv;
-            const CbSeqShape sh = cb_seq_shape(p, b);
-            s_sched->c_b = b; s_sched->c_kh = uid % p.Hkv; s_sched->c_tiles = sh.tiles; s_sched->c_n = sh.n; s_sched->c_ctx = sh.ctx;
-            s_sched->c_has = sh.RG > 0 ? 1 : 0;
-            s_sched->c_t0 = sh.RG > 0 ? (int)((long long)sh.tiles * rank / p.cs) : 0;
-            s_sched->c_t1 = sh.RG > 0 ? (int)((long long)sh.tiles * (rank + 1) / p.cs) : 0;
-            s_sched->g0 = 0; s_sched->g1 = 0; s_sched->pre0 = 0; s_sched->b0 = 0; s_sched->rg0 = 0;
-        }
-    } else if (warp == 0) {
+    if (p.cs == 0 && warp == 0) {
         // this CTA's range of the global tile sequence
         const long long tot = cb_sched_total(p, lane);
         const long long g0 = cb_range_start(tot, p.nc, cta), g1 = cb_range_start(tot, p.nc, cta + 1);
@@ -198,10 +187,6 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
     constexpr uint32_t ns = (uint32_t)C::NSLOT;
-    // Cluster mode: the peers' barriers must exist before anything arrives on them.  Every thread reports here and waits where its
-    // role first reaches over, or at its end (a CTA must not leave before the others' report either).
-    // What they must see of this CTA, its initialised barriers, went out with the fence behind the initialisation, so the report itself
-    // releases nothing (a releasing one waits for every access before it: 0.9 k of the cycles before batch 1's first copy).
     if (p.cs > 0) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     auto cluster_wait = [&]() {
         if (p.cs > 0) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -210,12 +195,31 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
     if (warp < 4) {
         reg_dealloc<64>();
         CbWalker wk;
+        // Cluster mode: cluster k works on unit k = (sequence, kv head); its CTAs take equal parts of the unit's key tiles.  Every role works its
+        // share out for itself (through one warp and shared memory, with divisions by the cluster size, batch 1 took 18.9 us, so 18.2).
         if (p.cs > 0) {
+            const int lcs = 31 - __clz(p.cs);                 // the cluster size is a power of two
+            const int uid = cta >> lcs, rank = cta & (p.cs - 1), b = uid / p.Hkv;
+            int guess = -1, page_guess = 0;                   // a tile, and the page of this lane's box in it
+            if ((warp == 0 || warp == 3) && lane < 8) {
+                // The first tile if the context is as long as the caller's bound: its page is asked for beside the lengths that say whether it is
+                // (one memory round trip instead of two).
+                guess = (int)((long long)p.max_tiles * rank >> lcs);
+                const long long at = (long long)guess * (CB_KT / 16) + lane;
+                if (at < p.max_pages) page_guess = p.block_table[(size_t)b * p.max_pages + at];
+            }
+            const CbSeqShape sh = cb_seq_shape(p, b);
             CbUnit u0;
-            u0.b = s_sched->c_b; u0.kh = s_sched->c_kh; u0.rg = 0; u0.t0 = s_sched->c_t0; u0.t1 = s_sched->c_t1;
-            u0.tiles = s_sched->c_tiles; u0.n = s_sched->c_n; u0.ctx = s_sched->c_ctx; u0.nrt = 1;
+            u0.b = b; u0.kh = uid - b * p.Hkv; u0.rg = 0; u0.tiles = sh.tiles; u0.n = sh.n; u0.ctx = sh.ctx; u0.nrt = 1;
+            u0.t0 = sh.RG > 0 ? (int)((long long)sh.tiles * rank >> lcs) : 0;
+            u0.t1 = sh.RG > 0 ? (int)((long long)sh.tiles * (rank + 1) >> lcs) : 0;
             wk.init_fixed(u0);
-        } else {
+            wk.rg = guess; wk.b = page_guess;                 // (a fixed walk has no use for them)
+            if (warp == 2 && lane == 0) {
+                // read by the softmax warps, behind the barrier on which the unit is published
+                s_sched->c_b = b; s_sched->c_kh = u0.kh; s_sched->c_n = sh.n; s_sched->c_has = sh.RG > 0 ? 1 : 0;
+            }
+        } else if (warp != 1) {                               // (the issuer reads the published units)
             wk.init(p, s_sched->g0, s_sched->g1, s_sched->rg0, s_sched->b0, s_sched->pre0);
         }
         CbUnit u;
@@ -242,7 +246,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                     int page = p.num_pages;                  // out of range: the copy fills zeros
                     if (active && i < nct) {
                         const int pidx = i * (CB_KT / 16) + j;
-                        if (pidx < npages) page = bt[pidx];
+                        if (pidx < npages) page = wk.fixed && i == wk.rg ? wk.b : bt[pidx];
                     }
                     return page;
                 };

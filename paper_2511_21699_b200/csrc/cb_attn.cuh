@@ -177,6 +177,11 @@ struct CbUnit {
 };
 constexpr int kTwoHeads = 3;                     // the units of heads kh and kh + 1, both whole and of one row tile, side by side (next_pair)
 
+// x / wt for the weights that there are (1, 2, 4 and 6) and x >= 0: a division is a chain of 100 to 200 cycles, two of them in the first unit.
+__device__ __forceinline__ int cb_tiles_of(int x, int wt) {
+    return wt == 6 ? (int)((unsigned long long)(uint32_t)x * 0xAAAAAAABull >> 34) : x >> (wt >> 1);
+}
+
 // Walks the units of the range [g, g1).  Every role of a CTA runs its own copy and sees the same units.
 struct CbWalker {
     long long g, g1, pre;     // pre: global position at which the units of (rg, b) start
@@ -216,8 +221,8 @@ struct CbWalker {
             const int v0 = (int)(off - (long long)kh * vt);
             const int v1 = (int)min((long long)vt, (long long)v0 + (g1 - g));
             g += v1 - v0;
-            u->t0 = (max(v0 - dec, 0) + wt - 1) / wt;
-            u->t1 = (max(v1 - dec, 0) + wt - 1) / wt;
+            u->t0 = cb_tiles_of(max(v0 - dec, 0) + wt - 1, wt);
+            u->t1 = cb_tiles_of(max(v1 - dec, 0) + wt - 1, wt);
             if (u->t1 <= u->t0) continue;                     // no tile of this unit is the range's
             u->b = b; u->kh = kh; u->rg = rg; u->tiles = s.tiles; u->n = s.n; u->ctx = s.ctx;
             u->nrt = p.MT == 1 ? 1 : min(2, s.mtn - 2 * rg);

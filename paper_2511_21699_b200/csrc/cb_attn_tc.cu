@@ -48,7 +48,6 @@ namespace {
 // A unit as the softmax warps see it (nrt = 0: no more units).  cf, np: the CTA that holds the unit's first key tile and the number of
 // CTAs that hold one; ticket: where its parts are counted; xpos: position of that tile where a CTA holds one tile at most, else -1.
 struct UnitDesc { int b, kh, rg, t0, t1, tiles, n, ctx, nrt, cf, np, xpos, wt, ticket; };
-constexpr int kFmaExpPhase = 3;                              // of every four pairs of exponentials this one is taken by the FMA pipe
 constexpr int kUnitRing = 4;                                 // units published ahead of the slowest softmax thread: at most two
 
 template <int D>
@@ -68,6 +67,12 @@ struct Cfg {
     static constexpr uint32_t OFF_MISC = OFF_X + 2 * 2 * CB_MT * 4;                  // schedule, tmem base, abort flag, pair counters
     static constexpr uint32_t SMEM = OFF_MISC + 96 + 64;
     static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
+    // Of so many pairs of exponentials the last is taken by the FMA pipe.  With head_dim 64, whose products take half as long, the exponential
+    // unit decides, and a quarter off it is worth 1 to 4% (batch 85 of 32/8 heads over 1,283 tokens: 60.1 us without, 58.6 an eighth,
+    // 57.8 a quarter).  With 128 the chains' hand-overs decide and the polynomial's 17 instructions are mostly power: an
+    // eighth is as fast as a quarter in short runs (70B shape, batch 8: 238.5 and 240.9 us) and faster at the power cap
+    // (its full batch 19.2 ms and 19.5, none 19.15; batch 64 of 40 heads 498 us and 501).
+    static constexpr int FMA_EXP = (D == 128) ? 8 : 4;
     static constexpr uint32_t O_COL = 256;                   // TMEM columns: S0 at 0, S1 at 128, O0 at 256, O1 at 256 + D
 };
 
@@ -531,7 +536,7 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
                             for (int q = 0; q < 8; ++q) {
                                 const uint64_t x = f2_fma(f2_pack(__uint_as_float(cur[2 * q]), __uint_as_float(cur[2 * q + 1])), scale2, negmu2);
                                 float p0, p1;
-                                if (!MASKED && q % 4 == kFmaExpPhase) {
+                                if (!MASKED && q % C::FMA_EXP == C::FMA_EXP - 1) {
                                     ex2_pair_fma(x, p0, p1);
                                 } else {
                                     f2_unpack(x, p0, p1);

@@ -283,7 +283,7 @@ __device__ __forceinline__ void update_seq(const CbTables& t, int b, const int32
 // entry in L1 (a write by this CTA goes through that L1, so what it finds there is current; no other CTA writes this sequence's table).
 constexpr int kUpdWarps = 8;
 template <int FETCH, typename Tokens, typename Idle>
-__device__ __forceinline__ void update_seq_cta(const CbTables& t, int b, const Tokens& row, int n0, int n1,
+__device__ __forceinline__ uint32_t update_seq_cta(const CbTables& t, int b, const Tokens& row, int n0, int n1,
                                                int warp, int lane, uint32_t* status, unsigned long long* counters, Idle&& idle) {
     __shared__ unsigned long long sh_h[kUpdWarps];
     __shared__ uint32_t sh_state[kUpdWarps], sh_bucket[kUpdWarps], sh_count[2];
@@ -369,6 +369,7 @@ __device__ __forceinline__ void update_seq_cta(const CbTables& t, int b, const T
         if (cnt.fevict) atomicAdd(&counters[CB_CNT_FOLLOWER_EVICTIONS], (unsigned long long)cnt.fevict);
         if (cnt.maxprobe) atomicMax(&counters[CB_CNT_MAX_PROBE], (unsigned long long)cnt.maxprobe);
     }
+    return clock;                                                // all threads know it
 }
 
 template <int FETCH>
@@ -626,9 +627,22 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const CbSeq s = cb_seq(t, b);
+    // The root needs no look at the table: a thread of the last warp, which most often has no window to insert, puts it there.
+    if (tid == (int)blockDim.x - 32) {
+        const bool root = L >= 1;
+        sh_n[0] = sh_nfront[0] = sh_npts[0] = root ? 1 : 0;
+        if (root) {
+            const int tk = row(L - 1);
+            S.tok[0] = tk; S.par[0] = -1; S.dep[0] = 0; S.front[0] = 0; S.pts[0] = 0;
+            const size_t at = (size_t)b * T;
+            o_tok[at] = tk; o_par[at] = -1; o_dep[at] = 0;
+            for (int k = 0; k < W; ++k) { S.mask[k] = k == 0 ? 1u : 0u; o_mask[at * W + k] = k == 0 ? 1u : 0u; }
+        }
+    }
+    uint32_t clock0;
     if (upd_n_old >= 0) {
         // cb_update_draft_tree: the sequence's new windows go into the table first, then the CTA drafts from the updated table.
-        update_seq_cta<FETCH>(t, b, row, upd_n_old, L, warp, lane, status, counters, [&] {
+        clock0 = update_seq_cta<FETCH>(t, b, row, upd_n_old, L, warp, lane, status, counters, [&] {
             if (L < t.LL) return;
             const int32_t mykey = lane < t.LL ? row(L - t.LL + lane) : 0;
             EntryRegs er;
@@ -643,11 +657,11 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                 for (int c = 0; c < CB_MAX_FC / 32; ++c) asm volatile("" ::"r"(er.fs4[c]));
             }
         });
-        __threadfence_block();
-        __syncthreads();
+    } else {
+        clock0 = s.hdr[0];
     }
+    __syncthreads();
     const int FLFC = t.FL * KF;                               // staged followers per leaf: the KF best
-    const uint32_t clock0 = s.hdr[0];
     const bool has_frozen = tf.index != nullptr;
 
     // Nodes [0, tot) of leaf `leaf` (depth d), numbered from n0 on, by one warp: node x is token x % cl of follower x / cl.
@@ -668,19 +682,6 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
             }
         }
     };
-    if (tid == 0) {
-        const bool root = L >= 1;
-        sh_n[0] = sh_nfront[0] = sh_npts[0] = root ? 1 : 0;
-        if (root) {
-            const int tk = row(L - 1);
-            S.tok[0] = tk; S.par[0] = -1; S.dep[0] = 0; S.front[0] = 0; S.pts[0] = 0;
-            const size_t at = (size_t)b * T;
-            o_tok[at] = tk; o_par[at] = -1; o_dep[at] = 0;
-            for (int k = 0; k < W; ++k) { S.mask[k] = k == 0 ? 1u : 0u; o_mask[at * W + k] = k == 0 ? 1u : 0u; }
-        }
-    }
-    __syncthreads();
-
     int cur = 0;
     for (int pass = 0; pass < (has_frozen ? 2 : 1); ++pass) {
         const CbTables& tt = pass ? tf : t;
@@ -758,11 +759,18 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                             }
                             // no more than the tree has room for chains of this length
                             const int cl = min(tt.FL, max_depth - d), room = (leaf == 0 ? max(1, T - crt) : T) - n_now;
-                            nf = min(nf, min(KF, (max(room, 0) + cl - 1) / cl));
+                            nf = min(nf, min(KF, (int)(((uint32_t)(max(room, 0) + cl - 1) * kInverse[cl]) >> 16)));
                             int rank[CH];
 #pragma unroll
                             for (int c = 0; c < CH; ++c) rank[c] = -1;
-                            if (FETCH == 1 || nf <= 40) {     // about where a maximum each costs what the counting below does
+                            if (FETCH == 1 && tt.FC <= 8 && nf > 2) {
+                                // eight places: the larger stamps are counted by shuffles that do not wait for one another (a maximum for each
+                                // follower wanted is a chain of some 45 cycles a step)
+                                int larger = 0;
+#pragma unroll
+                                for (int l = 0; l < 8; ++l) larger += __shfl_sync(CB_FULL, fs[0], l) > fs[0] ? 1 : 0;
+                                if (fs[0] != 0u && larger < nf) rank[0] = larger;
+                            } else if (FETCH == 1 || nf <= 40) {     // about where a maximum each costs what the counting below does
                                 for (int r = 0; r < nf; ++r) {
                                     uint32_t m = fs[0];
 #pragma unroll

@@ -255,77 +255,62 @@ __global__ void __launch_bounds__(256) fb_init_kernel(BuildView v, CbTables t) {
     for (size_t i = g; i < v.S1 / 2; i += stride) key[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
 }
 
-// 1. leader counts.  Four windows a thread, so that their chains (slot, atomic) overlap.
+// 1. leader counts.  A window a thread at a time, so that eight blocks of 256 fit an SM (32 registers); four at a time, whose chains overlap,
+// leave room for four: 4 M windows, LL = 2, 472 us the whole build, 450 with two windows and eight blocks, 446 with one.
 // What a block has met lies in shared memory, a key to each place: the windows with such a key are counted there and never look at the
 // table, and where the corpus begins, a frequent key's free slot is tried once a block and not by every thread that has it (733 k
 // windows, LL = 1: 38 us, 75 without it).
-template <int U>
-__device__ __forceinline__ void left_out(const BuildView& v, size_t i0, int LL, bool (&ok)[U]) {   // the windows with a negative token
-#pragma unroll
-    for (int q = 0; q < U; ++q)
-        for (int j = 0; j < LL + v.FL && ok[q]; ++j) ok[q] = v.corpus[i0 + q * 256 + threadIdx.x + j] >= 0;
-}
 struct KeyCache {
     static constexpr uint32_t N = 1024;
     unsigned long long key[N];
     uint32_t slot[N], cnt[N];
 };
+// The window at i as one number; false where it has a negative token, which leaves it out.
+template <int LL>
+__device__ __forceinline__ bool packed_key(const BuildView& v, int bits, bool has_neg, size_t i, unsigned long long* key) {
+    *key = 0ull;
+#pragma unroll
+    for (int j = 0; j < LL; ++j) *key = *key << bits | (uint32_t)v.corpus[i + j];
+    bool ok = true;
+    for (int j = 0; has_neg && j < LL + v.FL && ok; ++j) ok = v.corpus[i + j] >= 0;
+    return ok;
+}
 template <int LL>
 __device__ __forceinline__ void count_packed(const BuildView& v, int bits, KeyCache& cache) {
-    constexpr int U = 4;
     for (uint32_t i = threadIdx.x; i < KeyCache::N; i += 256) { cache.key[i] = kNoLeader; cache.cnt[i] = 0u; }
     __syncthreads();
-    const size_t stride = (size_t)gridDim.x * 256 * U;
     const bool has_neg = v.st->has_neg != 0u;
-    for (size_t i0 = (size_t)blockIdx.x * 256 * U; i0 < v.M; i0 += stride) {
-        uint32_t s[U], at[U];
-        unsigned long long x[U], me[U];
-        bool ok[U], look[U], first[U];                          // look: this thread finds or makes the slot; first: it has a place in the cache
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const size_t i = i0 + q * 256 + threadIdx.x;
-            ok[q] = i < v.M;
-            me[q] = 0ull;
-#pragma unroll
-            for (int j = 0; j < LL; ++j) me[q] = me[q] << bits | (ok[q] ? (uint32_t)v.corpus[i + j] : 0u);
-            const uint64_t h = hash_key(me[q]);
-            s[q] = home_leader(h, v.S1);
-            at[q] = (uint32_t)h & (KeyCache::N - 1);
-        }
-        if (has_neg) left_out(v, i0, LL, ok);
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            look[q] = first[q] = false;
-            if (!ok[q]) continue;
-            unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&cache.key[at[q]]);
+    for (size_t i0 = (size_t)blockIdx.x * 256; i0 < v.M; i0 += (size_t)gridDim.x * 256) {
+        const size_t i = i0 + threadIdx.x;
+        unsigned long long me = kNoLeader;
+        const bool ok = i < v.M && packed_key<LL>(v, bits, has_neg, i, &me);
+        uint32_t s = kEmpty, at = 0u;
+        bool look = false;                                      // this thread finds or makes the slot
+        if (ok) {
+            const uint64_t h = hash_key(me);
+            at = (uint32_t)h & (KeyCache::N - 1);
+            unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&cache.key[at]);
+            bool first = false;                                 // and has a place in the cache
             if (k == kNoLeader) {
-                k = atomicCAS(&cache.key[at[q]], kNoLeader, me[q]);
-                first[q] = k == kNoLeader;
+                k = atomicCAS(&cache.key[at], kNoLeader, me);
+                first = k == kNoLeader;
             }
-            look[q] = k != me[q];
-            if (!look[q]) atomicAdd(&cache.cnt[at[q]], 1u);
-        }
-        // A slot never changes once it is set, so an ordinary load will do; one that still shows a free slot is put right by the
-        // compare-and-swap.
-#pragma unroll
-        for (int q = 0; q < U; ++q) x[q] = look[q] ? v.h1[s[q]] : kNoLeader;
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            if (!look[q]) continue;
-            bool created = false;
-            if (x[q] != me[q]) s[q] = claim_leader(v.h1, v.S1, s[q], x[q], me[q], &created, [&](unsigned long long y) { return y == me[q]; });
-            if (s[q] == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
-            if (first[q]) cache.slot[at[q]] = s[q];
-            if (created || s[q] == kEmpty) continue;
-            if (first[q]) atomicAdd(&cache.cnt[at[q]], 1u);
-            else atomicAdd(&v.h1_cnt[s[q]], 1u);
+            look = k != me;
+            if (!look) {
+                atomicAdd(&cache.cnt[at], 1u);
+            } else {
+                // A slot never changes once it is set, so an ordinary load will do; one that still shows a free slot is put right by
+                // the compare-and-swap.
+                bool created = false;
+                s = home_leader(h, v.S1);
+                s = claim_leader(v.h1, v.S1, s, v.h1[s], me, &created, [&](unsigned long long y) { return y == me; });
+                if (s == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
+                if (first) cache.slot[at] = s;
+                if (!created && s != kEmpty) atomicAdd(first ? &cache.cnt[at] : &v.h1_cnt[s], 1u);
+            }
         }
         __syncthreads();                                        // the new places' slots are known
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const size_t i = i0 + q * 256 + threadIdx.x;
-            if (i < v.M) v.lslot[i] = !ok[q] ? kEmpty : (look[q] ? s[q] : cache.slot[at[q]]);
-        }
+        if (i < v.M) v.lslot[i] = !ok ? kEmpty : (look ? s : cache.slot[at]);
     }
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < KeyCache::N; i += 256)
@@ -334,37 +319,19 @@ __device__ __forceinline__ void count_packed(const BuildView& v, int bits, KeyCa
 // The same for longer leaders, most of which a block meets once: no places for keys, the counts alone are gathered.
 template <int LL>
 __device__ __forceinline__ void count_packed(const BuildView& v, int bits, CountCache<1>& cache) {
-    constexpr int U = 4;
     cache.clear();
-    const size_t stride = (size_t)gridDim.x * 256 * U;
     const bool has_neg = v.st->has_neg != 0u;
-    for (size_t i0 = (size_t)blockIdx.x * 256 * U; i0 < v.M; i0 += stride) {
-        uint32_t s[U];
-        unsigned long long x[U], me[U];
-        bool ok[U];
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const size_t i = i0 + q * 256 + threadIdx.x;
-            ok[q] = i < v.M;
-            me[q] = 0ull;
-#pragma unroll
-            for (int j = 0; j < LL; ++j) me[q] = me[q] << bits | (ok[q] ? (uint32_t)v.corpus[i + j] : 0u);
-            s[q] = home_leader(hash_key(me[q]), v.S1);
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < v.M; i += (size_t)gridDim.x * 256) {
+        unsigned long long me;
+        uint32_t s = kEmpty;
+        if (packed_key<LL>(v, bits, has_neg, i, &me)) {
+            bool created = false;
+            s = home_leader(hash_key(me), v.S1);
+            s = claim_leader(v.h1, v.S1, s, v.h1[s], me, &created, [&](unsigned long long y) { return y == me; });
+            if (s == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
+            else if (!created) cache.add(v.h1_cnt, s);
         }
-        if (has_neg) left_out(v, i0, LL, ok);
-#pragma unroll
-        for (int q = 0; q < U; ++q) x[q] = ok[q] ? v.h1[s[q]] : kNoLeader;
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const size_t i = i0 + q * 256 + threadIdx.x;
-            if (ok[q]) {
-                bool created = false;
-                if (x[q] != me[q]) s[q] = claim_leader(v.h1, v.S1, s[q], x[q], me[q], &created, [&](unsigned long long y) { return y == me[q]; });
-                if (s[q] == kEmpty) atomicCAS(&v.st->status, 0u, (uint32_t)CB_ERR_PROBE_LIMIT);
-                else if (!created) cache.add(v.h1_cnt, s[q]);
-            }
-            if (i < v.M) v.lslot[i] = ok[q] ? s[q] : kEmpty;
-        }
+        v.lslot[i] = s;
     }
     cache.flush(v.h1_cnt);
 }
@@ -389,7 +356,7 @@ __device__ __forceinline__ void count_positions(const BuildView& v, CountCache<1
 }
 constexpr int kCachedKeys = 2;                // up to that many tokens a leader's keys are kept (LL = 3: 36 us with the counts alone, 52 with keys; LL = 2: 117 and 90)
 template <int LL>
-__global__ void __launch_bounds__(256) fb_count_leaders_kernel(BuildView v) {
+__global__ void __launch_bounds__(256, 8) fb_count_leaders_kernel(BuildView v) {
     CB_PDL_ENTRY();
     using Cache = std::conditional_t<LL <= kCachedKeys, KeyCache, CountCache<1>>;
     __shared__ union { Cache keys; CountCache<1> slots; } cache;

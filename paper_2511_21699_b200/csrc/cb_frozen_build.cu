@@ -932,18 +932,59 @@ __device__ __forceinline__ bool fb_rank_begin(const BuildView& v) {   // false: 
 }
 __device__ __forceinline__ void fb_rank_end() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// the big leaders, a block each
-__global__ void __launch_bounds__(1024) fb_rank_big_kernel(BuildView v, CbTables t) {
+// The big leaders, a block each.  A frequent token of a large corpus has 100 k distinct windows and more, of which the few with the largest counts
+// are wanted: a histogram of the counts says from which count on there are FC, and those from there on are copied to shared memory, two looks
+// at memory where the bisections of pick_followers took one a step (3.7 M windows, LL = 1, FC = 64: 275 us for the longest leader).  Where too many
+// tie, or fewer than FC occur twice, it goes over all of them as they are.
+constexpr uint32_t kShort = 2048, kCountBins = 1024;
+__global__ void __launch_bounds__(kCountBins) fb_rank_big_kernel(BuildView v, CbTables t) {
     CB_PDL_ENTRY();
     __shared__ Candidates cand;
-    __shared__ uint32_t red[32];
-    const Crew<1024> crew = {red};
+    __shared__ uint32_t red[32], bins[kCountBins], n_short, from;
+    __shared__ uint2 best[kShort];
+    const Crew<kCountBins> crew = {red};
     fb_hand_on(v);
-    const uint32_t n = fb_aborted(v) ? 0u : v.st->n_big;
-    for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
-        const uint32_t eid = v.listed_big[k];
-        const MemoryGroup g = {v.group + (v.grp_off[eid] & ~kBigFlag), v.corpus, v.LL};
-        pick_followers<1024>(v, t, eid, g, v.grp_n[eid], cand, crew);
+    const int me = (int)threadIdx.x, lane = me & 31;
+    const uint32_t n_big = fb_aborted(v) ? 0u : v.st->n_big;
+    for (uint32_t k = blockIdx.x; k < n_big; k += gridDim.x) {
+        const uint32_t eid = v.listed_big[k], n = v.grp_n[eid];
+        const uint2* const g = v.group + (v.grp_off[eid] & ~kBigFlag);
+        bool few = false;
+        if (n > kShort) {
+            bins[me] = 0u;
+            if (me == 0) { n_short = 0u; from = 0u; }
+            __syncthreads();
+            constexpr int U = 4;
+            for (uint32_t i0 = 0; i0 < n; i0 += U * kCountBins) {
+                uint32_t c[U];
+#pragma unroll
+                for (int q = 0; q < U; ++q) { const uint32_t i = i0 + q * kCountBins + me; c[q] = i < n ? g[i].y : 0u; }
+#pragma unroll
+                for (int q = 0; q < U; ++q) add_bin(bins, c[q] > 1u ? min(c[q], kCountBins - 1u) : kEmpty);
+            }
+            __syncthreads();
+            uint32_t total;                                     // thread t: how many have the count kCountBins - 1 - t or more
+            const uint32_t own = bins[kCountBins - 1 - me], above = sel_scan(own, red, &total);
+            if (above < (uint32_t)v.FC && above + own >= (uint32_t)v.FC && above + own <= kShort) from = kCountBins - 1u - (uint32_t)me;
+            __syncthreads();
+            few = from != 0u;
+            for (uint32_t i0 = 0; few && i0 < n; i0 += U * kCountBins) {
+                uint2 x[U];
+#pragma unroll
+                for (int q = 0; q < U; ++q) { const uint32_t i = i0 + q * kCountBins + me; x[q] = i < n ? g[i] : make_uint2(0u, 0u); }
+#pragma unroll
+                for (int q = 0; q < U; ++q) {
+                    const uint32_t m = __ballot_sync(CB_FULL, x[q].y >= from);
+                    uint32_t at = 0;
+                    if (m && lane == 0) at = atomicAdd(&n_short, (uint32_t)__popc(m));
+                    at = __shfl_sync(CB_FULL, at, 0) + __popc(m & ((1u << lane) - 1u));
+                    if (x[q].y >= from) best[at] = x[q];
+                }
+            }
+            __syncthreads();
+        }
+        const MemoryGroup group = {few ? best : g, v.corpus, v.LL};
+        pick_followers<kCountBins>(v, t, eid, group, few ? n_short : n, cand, crew);
     }
 }
 
@@ -1339,7 +1380,7 @@ static cb_status frozen_build(const cb_frozen_config* cfg, const int32_t* dev_co
         }
         CB_CUDA(cb_launch_pdl(fb_windows_kernel, grid, block, 0, st, v));
         CB_CUDA(cb_launch_pdl(fb_group_scatter_kernel, grid, block, 0, st, v));
-        CB_CUDA(cb_launch_pdl(fb_rank_big_kernel, dim3((unsigned)sms), dim3(1024), 0, st, v, t));
+        CB_CUDA(cb_launch_pdl(fb_rank_big_kernel, dim3((unsigned)sms), dim3(kCountBins), 0, st, v, t));
         CB_CUDA(cb_launch_pdl(large, dim3((unsigned)(sms * 2)), dim3(512), block_smem(kBigGroup), st, v, t, 1u));
         CB_CUDA(cb_launch_pdl(mid, dim3((unsigned)(sms * 8)), dim3(128), block_smem(kMidGroup), st, v, t, 0u));
         const size_t warp_smem = (size_t)kRankWarps * kWarpGroup * (2 + cfg->FL) * 4;

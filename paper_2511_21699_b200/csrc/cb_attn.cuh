@@ -182,7 +182,7 @@ __device__ __forceinline__ int cb_tiles_of(int x, int wt) {
     return wt == 6 ? (int)((unsigned long long)(uint32_t)x * 0xAAAAAAABull >> 34) : x >> (wt >> 1);
 }
 
-// Walks the units of the range [g, g1).  Every role of a CTA runs its own copy and sees the same units.
+// Walks the units of the range [g, g1).  Every role that walks runs its own copy and sees the same units.
 struct CbWalker {
     long long g, g1, pre;     // pre: global position at which the units of (rg, b) start
     int rg, b;

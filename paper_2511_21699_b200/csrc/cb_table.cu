@@ -283,7 +283,7 @@ __device__ __forceinline__ void update_seq(const CbTables& t, int b, const int32
 // entry in L1 (a write by this CTA goes through that L1, so what it finds there is current; no other CTA writes this sequence's table).
 constexpr int kUpdWarps = 8;
 template <int FETCH, typename Tokens, typename Idle>
-__device__ __forceinline__ uint32_t update_seq_cta(const CbTables& t, int b, const Tokens& row, int n0, int n1,
+__device__ __forceinline__ void update_seq_cta(const CbTables& t, int b, const Tokens& row, int n0, int n1,
                                                int warp, int lane, uint32_t* status, unsigned long long* counters, Idle&& idle) {
     __shared__ unsigned long long sh_h[kUpdWarps];
     __shared__ uint32_t sh_state[kUpdWarps], sh_bucket[kUpdWarps], sh_count[2];
@@ -369,7 +369,6 @@ __device__ __forceinline__ uint32_t update_seq_cta(const CbTables& t, int b, con
         if (cnt.fevict) atomicAdd(&counters[CB_CNT_FOLLOWER_EVICTIONS], (unsigned long long)cnt.fevict);
         if (cnt.maxprobe) atomicMax(&counters[CB_CNT_MAX_PROBE], (unsigned long long)cnt.maxprobe);
     }
-    return clock;                                                // all threads know it
 }
 
 template <int FETCH>
@@ -639,10 +638,9 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
             for (int k = 0; k < W; ++k) { S.mask[k] = k == 0 ? 1u : 0u; o_mask[at * W + k] = k == 0 ? 1u : 0u; }
         }
     }
-    uint32_t clock0;
     if (upd_n_old >= 0) {
         // cb_update_draft_tree: the sequence's new windows go into the table first, then the CTA drafts from the updated table.
-        clock0 = update_seq_cta<FETCH>(t, b, row, upd_n_old, L, warp, lane, status, counters, [&] {
+        update_seq_cta<FETCH>(t, b, row, upd_n_old, L, warp, lane, status, counters, [&] {
             if (L < t.LL) return;
             const int32_t mykey = lane < t.LL ? row(L - t.LL + lane) : 0;
             EntryRegs er;
@@ -657,11 +655,13 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                 for (int c = 0; c < CB_MAX_FC / 32; ++c) asm volatile("" ::"r"(er.fs4[c]));
             }
         });
-    } else {
-        clock0 = s.hdr[0];
+        __syncthreads();
     }
-    __syncthreads();
     const int FLFC = t.FL * KF;                               // staged followers per leaf: the KF best
+    // Read back from memory although update_seq_cta's threads know it: handed on from there, with one barrier less, the compiler gave the kernel
+    // of short lists 92 registers instead of 80, two blocks an SM instead of three (batch 300 12.4 us, so 9.6), and long lists
+    // (one leader token, 128 followers) took 10.9 us, 15.3 with a cold L2, instead of 10.0 and 12.9; batch 1 of short lists gained 0.1.
+    const uint32_t clock0 = s.hdr[0];
     const bool has_frozen = tf.index != nullptr;
 
     // Nodes [0, tot) of leaf `leaf` (depth d), numbered from n0 on, by one warp: node x is token x % cl of follower x / cl.
@@ -682,6 +682,8 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
             }
         }
     };
+    __syncthreads();
+
     int cur = 0;
     for (int pass = 0; pass < (has_frozen ? 2 : 1); ++pass) {
         const CbTables& tt = pass ? tf : t;
@@ -763,14 +765,7 @@ __device__ __forceinline__ void draft_body(const CbTables& t, const CbTables& tf
                             int rank[CH];
 #pragma unroll
                             for (int c = 0; c < CH; ++c) rank[c] = -1;
-                            if (FETCH == 1 && tt.FC <= 8 && nf > 2) {
-                                // eight places: the larger stamps are counted by shuffles that do not wait for one another (a maximum for each
-                                // follower wanted is a chain of some 45 cycles a step)
-                                int larger = 0;
-#pragma unroll
-                                for (int l = 0; l < 8; ++l) larger += __shfl_sync(CB_FULL, fs[0], l) > fs[0] ? 1 : 0;
-                                if (fs[0] != 0u && larger < nf) rank[0] = larger;
-                            } else if (FETCH == 1 || nf <= 40) {     // about where a maximum each costs what the counting below does
+                            if (FETCH == 1 || nf <= 40) {     // about where a maximum each costs what the counting below does
                                 for (int r = 0; r < nf; ++r) {
                                     uint32_t m = fs[0];
 #pragma unroll
@@ -958,10 +953,10 @@ struct AcceptArgs {
     int32_t* n_accept; int32_t* accept_nodes; int32_t* out_tokens; int32_t* target_out;
 };
 
-// CTAS: CTAs that an SM has registers for.  The drafting code takes 102 registers, room for two.  A grid that is not resident at
+// CTAS: CTAs that an SM has registers for.  The drafting code takes 112 registers, room for two.  A grid that is not resident at
 // once that way streams the logits with half in flight of what four CTAs of 62 have (a step of batch 6 with trees of 96: 86.6 us with three
 // of 72, 82.9 with four; batch 4 of 64: 61.3 and 59.6); one that is gains nothing from the bound and pays for it in the chain behind
-// the logits, and takes all of a thread's chunk at once instead.  With more than 32 followers a leader the code takes 120 registers and
+// the logits, and takes all of a thread's chunk at once instead.  With more than 32 followers a leader the code takes 119 registers and
 // stays at two.
 //
 // IN_PLACE: o_n is a.n_nodes.  Which rows a sequence's tree has decides which of its CTAs count for the acceptance, so its entry is stored only

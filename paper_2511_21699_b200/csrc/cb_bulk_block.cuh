@@ -252,9 +252,9 @@ __device__ __forceinline__ uint32_t blk_parts(uint32_t n, float inv) {
 // One warp: about the smallest number of windows a part with which the parts of all sequences are no more than the blocks (a part too many
 // is a second turn for some block, and the longest part is what the launch waits for: shares rounded down left 16 of 148 blocks without a
 // part at batch 32 and gave 1,270 windows to one where 1,050 do).
-// (Parts of 32, 96, 224 and 448 windows at least, 22 shapes, time against the shares before: 0.978, 0.976, 0.982, 1.001; single shapes of
-// few windows lie 1 to 3% to either side.)
-constexpr int kBlkLeast = 64;
+// At least 32 windows a part: batch 13 of 294 to 450 tokens 18.5 us, 19.0 with 48 or 64; batch 13 of 344 to 688 18.8, 18.9 and 19.3; longer runs are
+// cut by the number of blocks.
+constexpr int kBlkLeast = 32;
 constexpr int kBlkSearch = 8;                                   // sequences a lane
 __device__ __forceinline__ float blk_share(const uint16_t* nwin, int B, uint32_t blocks, int lane) {
     uint32_t n[kBlkSearch], all = 0;
@@ -368,25 +368,19 @@ __global__ void __launch_bounds__(kBlkThreads, 1) cb_update_bulk_block_kernel(Cb
                 for (int j = 0; j < LL; ++j) k4[j] = S.tok[k + j];
                 return cb_hash4(k4[0], k4[1], k4[2], k4[3], LL);
             };
-            uint32_t own[kBlkRun / kBlkThreads], mine_n = 0;
-#pragma unroll
-            for (int q = 0; q < kBlkRun / kBlkThreads; ++q) {
-                const uint32_t k = (uint32_t)(q * kBlkThreads + tid);
-                own[q] = 0u;
-                if ((uint32_t)(q * kBlkThreads + warp * 32) >= nwin) continue;
+            // (One atomic a warp, with the votes of all its rounds unrolled into registers, gains 1% on runs of some thousand windows and costs a run of
+            // 300 a twentieth: code that it jumps over, 13 against 14 us.)
+            for (uint32_t k0 = warp * 32; k0 < nwin; k0 += kBlkThreads) {
+                const uint32_t k = k0 + lane;
                 uint32_t x = 0x85EBCA6Bu;
 #pragma unroll
                 for (int j = 0; j < LL; ++j) { x = (x ^ (uint32_t)S.tok[k + j]) * 0x9E3779B1u; x ^= x >> 16; }
-                own[q] = __ballot_sync(CB_FULL, k < nwin && __umulhi(x * 0xC2B2AE35u, np) == part);
-                mine_n += (uint32_t)__popc(own[q]);
-            }
-            uint32_t own_at = 0;
-            if (lane == 0 && mine_n) own_at = atomicAdd(&S.n_own, mine_n);
-            own_at = __shfl_sync(CB_FULL, own_at, 0);
-#pragma unroll
-            for (int q = 0; q < kBlkRun / kBlkThreads; ++q) {
-                if ((own[q] >> lane) & 1u) S.group[own_at + __popc(own[q] & ((1u << lane) - 1u))] = (uint16_t)(q * kBlkThreads + tid);
-                own_at += (uint32_t)__popc(own[q]);
+                const bool own = k < nwin && __umulhi(x * 0xC2B2AE35u, np) == part;
+                const uint32_t m = __ballot_sync(CB_FULL, own);
+                uint32_t at = 0;
+                if (m && lane == 0) at = atomicAdd(&S.n_own, (uint32_t)__popc(m));
+                at = __shfl_sync(CB_FULL, at, 0) + __popc(m & ((1u << lane) - 1u));
+                if (own) S.group[at] = (uint16_t)k;
             }
             __syncthreads();
             const uint32_t n_own = S.n_own;

@@ -212,10 +212,6 @@ struct Appender {
         put(has, x);
         return __syncthreads_or(near_full(U)) != 0;
     }
-    template <int U>
-    __device__ __forceinline__ void add(const bool (&has)[U], const T (&x)[U], T* list, uint32_t* counter) {
-        if (gather(has, x)) flush(list, counter);
-    }
     __device__ __forceinline__ void flush(T* list, uint32_t* counter) {
         __syncthreads();
         if (threadIdx.x == 0) at = n ? atomicAdd(counter, n) : 0u;
@@ -354,15 +350,20 @@ __device__ __forceinline__ void count_positions(const BuildView& v, CountCache<1
     }
     cache.flush(v.h1_cnt);
 }
-constexpr int kCachedKeys = 2;                // up to that many tokens a leader's keys are kept (LL = 3: 36 us with the counts alone, 52 with keys; LL = 2: 117 and 90)
+// Up to that many tokens a leader's keys are kept, of the longer ones the counts alone (4 M windows: LL = 2 75 us with keys, 90 with counts; LL = 3
+// 101 and 92; 700 k windows: 24 and 29, 30 and 28).
+constexpr int kCachedKeys = 2;
 template <int LL>
 __global__ void __launch_bounds__(256, 8) fb_count_leaders_kernel(BuildView v) {
     CB_PDL_ENTRY();
-    using Cache = std::conditional_t<LL <= kCachedKeys, KeyCache, CountCache<1>>;
-    __shared__ union { Cache keys; CountCache<1> slots; } cache;
+    __shared__ std::conditional_t<LL <= kCachedKeys, KeyCache, CountCache<1>> cache;
     const int bits = key_bits(v);
-    if (bits) count_packed<LL>(v, bits, cache.keys);
-    else count_positions<LL>(v, cache.slots);
+    if constexpr (LL * 31 <= 63) {                              // a token has 31 bits at most: one and two of them always fit
+        count_packed<LL>(v, bits, cache);
+    } else {
+        if (bits) count_packed<LL>(v, bits, cache);
+        else count_positions<LL>(v, cache);
+    }
 }
 
 // ---------------------------------------------------------------------------------------------------

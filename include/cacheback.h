@@ -205,10 +205,13 @@ cb_status cb_tree_add_branches(cb_ctx* ctx, const int32_t* branches, const int32
  *   tree_mask    uint32 [batch, T, W], n_nodes int32 [batch]   as written by cb_draft_tree
  *   out          bf16 [batch, T, Hq, D]         rows >= n_nodes are written as zero
  *   lse          float [batch, Hq, T] or NULL   natural-log sum of exponentials per row (0 for padding)
- *   max_ctx      host upper bound on every ctx_len (0 = max_pages * P); used only to size the grid
+ *   max_ctx      host upper bound on every ctx_len (0 = max_pages * P); sizes the grid and, with few units, names the page-table entry of
+ *                each sequence that is read ahead of its length (the entry is used only if the length says it is the one wanted)
  *   scale        softmax scale; 0 selects 1/sqrt(D)
  * Row (b, i, h) = softmax_j(scale * q.k_j) v_j over j in {cached tokens of kv head h / (Hq/Hkv)}
  * U {tree nodes in mask row i}; fp32 accumulation and softmax, output rounded to bf16.
+ * Equal calls give equal bits.  How a row's keys are split for the sum follows from ctx_len and n_nodes of the whole batch, so the last
+ * bits of a sequence's rows may depend on the other sequences.
  * All base pointers must be 16-byte aligned.
  * Keys and values are fetched a tile at a time and what lies outside a row's key set is given probability 0, not skipped,
  * so everything a tile covers must be finite (0 x NaN would reach the output): all T rows of k_tree / v_tree of every

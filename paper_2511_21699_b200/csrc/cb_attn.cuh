@@ -20,7 +20,9 @@
 // belongs to the CTA whose range holds the tile's deciding position, its d1-th or d2-th from zero.  Those are the first one at 2 : 1, and at
 // 6 : 4 the ones that cut a launch whose units have all one row tile, or all two, exactly as 2 : 1 cuts it: a range that starts at
 // the share x of the sequence leaves out the tiles i with 2x >= 2i + 1 (two) or x >= i + 1 (one), which is 6x >= 6i + 3 and 4x >= 4i + 4.
-// Where such launches are cut decides the last bit of rows that CTAs share.
+// Where a launch is cut decides the last bits of rows: of a unit that CTAs share (its parts are put together), and of a whole unit of one row
+// tile, whose keys one chain takes where the range holds the next head's whole unit as well (CbWalker::next_pair), else two chains in turn.  The cuts
+// follow from the lengths and node counts of the whole batch; equal calls give equal bits.
 // A CTA therefore finishes whole units, plus at most one unit it shares
 // with earlier CTAs and one it shares with later CTAs; the CTAs of a shared unit combine unnormalised partials (in the kernel, or
 // in the merge pass of the CTA-pair kernel, which counts one position per tile).

@@ -70,9 +70,10 @@ struct Cfg {
     static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
     // Of so many pairs of exponentials the last is taken by the FMA pipe.  With head_dim 64, whose products take half as long, the exponential
     // unit decides, and a quarter off it is worth 1 to 4% (batch 85 of 32/8 heads over 1,283 tokens: 60.1 us without, 58.6 an eighth,
-    // 57.8 a quarter).  With 128 the chains' hand-overs decide and the polynomial's 17 instructions are mostly power: an
-    // eighth is as fast as a quarter in short runs (70B shape, batch 8: 238.5 and 240.9 us) and faster at the power cap
-    // (its full batch 19.2 ms and 19.5, none 19.15; batch 64 of 40 heads 498 us and 501).
+    // 57.8 a quarter).  With 128 the chains' hand-overs decide and the polynomial's 17 instructions are mostly power.  Runs of 2 s at the
+    // power cap, four in turn, a quarter / an eighth / none: 70B shape, batch 128 18.69 / 18.49 / 18.46 ms; batch 8 of it over 4 k to 16 k tokens
+    // 347.2 / 343.9 / 345.4 us; batch 64 of 40 heads 473.9 / 470.0 / 469.0; batch 32 of 32/8 heads 184.6 / 183.7 / 184.1.  None is as good as an
+    // eighth within half a percent either way, a quarter is slower in all.
     static constexpr int FMA_EXP = (D == 128) ? 8 : 4;
     static constexpr uint32_t O_COL = 256;                   // TMEM columns: S0 at 0, S1 at 128, O0 at 256, O1 at 256 + D
 };
@@ -195,6 +196,11 @@ cb_attn_tc_kernel(const CbAttnParams p, const __grid_constant__ TcMaps maps) {
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
     constexpr uint32_t ns = (uint32_t)C::NSLOT;
+    // Cluster mode: the peers' barriers must exist before anything arrives on them.  Every thread reports here and waits where its
+    // role first reaches over, or at its end (a CTA must not leave before the others' report either).
+    // What the peers must see of this CTA, its initialised barriers and nothing else, went out with the fence behind the initialisation, so the
+    // report itself releases nothing (a releasing one waits for every access before it: 0.9 k of the cycles before batch 1's first copy).
+    // What else was written before it (c_has, the abort flag) is for this CTA's threads, behind the block's barriers.
     if (p.cs > 0) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     auto cluster_wait = [&]() {
         if (p.cs > 0) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");

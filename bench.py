@@ -56,26 +56,28 @@ def parse(argv=None):
 
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one cb_attn_tc_kernel launch with full trees, from the ncu
-# captures summarised under profiles/.  Reported only while the kernel sources still hash to the captured ones; after any
-# change to them the figure is stale and `traffic` is null until the capture is redone.
-ATTN_TRAFFIC = {"sources_sha1": "fc7fecd6be57e41dc2fc4344c4ea26fe35fb495d",
-                "bytes_per_launch": {"c2_7b": 70.2e6, "c3_8b_gqa": 554.6e6, "c4_13b_turns": 2762.9e6},
+# captures summarised under profiles/.  Reported only while the kernel sources, without comments and white space, still hash to the
+# captured ones; after any change to their code the figure is stale and `traffic` is null until the capture is redone.
+ATTN_TRAFFIC = {"sources_sha1": "602bea24e6267c9f91efa99da628ec602b3a4ff6",
+                "bytes_per_launch": {"c2_7b": 69.9e6, "c3_8b_gqa": 554.7e6, "c4_13b_turns": 2762.3e6},
                 "source": {k: "profiles/cb_attn_tc_kernel_c2_c3_c4_c5b8.md" for k in ("c2_7b", "c3_8b_gqa", "c4_13b_turns")},
                 # config 5 holds 25 GB and runs 20 ms per launch: too large to capture.  The same shape at batch 8 was captured
-                # (1,618.9 + 7.1 and 1,526.6 + 7.3 MB per launch); keys and values are streamed per sequence, so the traffic is taken
+                # (1,568.7 + 7.2 and 1,554.9 + 7.2 MB per launch); keys and values are streamed per sequence, so the traffic is taken
                 # to grow with the batch: mean x 128 / 8.
-                "scaled": {"c5_70b_long": (1580.0e6 * 16.0,
+                "scaled": {"c5_70b_long": (1569.0e6 * 16.0,
                                            "profiles/cb_attn_tc_kernel_c2_c3_c4_c5b8.md: c5_70b_b8 (same shape, batch 8), mean of two captures "
                                            "x 16 sequences' worth; not a capture of this workload")}}
-ATTN_SOURCES = ("cb_attn_tc.cu", "cb_tc_dev.cuh", "cb_attn_pair.cuh", "cb_attn.cuh", "cb_attn.cu")
+ATTN_SOURCES = ("cb_attn_tc.cu", "cb_attn_sched32.cuh", "cb_tc_dev.cuh", "cb_attn_pair.cuh", "cb_attn.cuh", "cb_attn.cu")
 
 
 def attn_sources_sha1():
     import hashlib
+    import re
     h = hashlib.sha1()
     for f in ATTN_SOURCES:
-        with open(os.path.join(ROOT, "paper_2511_21699_b200", "csrc", f), "rb") as fh:
-            h.update(fh.read())
+        with open(os.path.join(ROOT, "paper_2511_21699_b200", "csrc", f), encoding="utf-8") as fh:
+            text = re.sub(r'("(?:\\.|[^"\\])*")|//[^\n]*|/\*.*?\*/', lambda m: m.group(1) or " ", fh.read(), flags=re.S)
+        h.update("".join(text.split()).encode())
     return h.hexdigest()
 
 

@@ -6,10 +6,10 @@
 // of the run, the table of the part's leaders and that of its (leader, follower) pairs lie in shared memory, so claims, "last
 // index" maxima and the grouping of pairs by leader are shared-memory operations, and what is left in global memory is an atomic per
 // new leader and the entry itself.  Through scratch in global memory the same run is six launches whose every step is a chain of L2
-// round trips: batch 32 of 1,024 to 8,192 tokens (147 k windows), reset and first draft with it, 118 us against 30.2 us this way
-// (some 17 of them this kernel's, 35 k cycles: lengths, parts and tokens 6 k, listing the part's windows 3 k, claims 7 k with the second
+// round trips: batch 32 of 1,024 to 8,192 tokens (147 k windows), reset and first draft with it, 118 us against 30.0 us this way
+// (some 17 of them this kernel's, 36 k cycles: lengths, parts and tokens 6 k, listing the part's windows 4 k, claims 7 k with the second
 // turn of those beyond 1,024, ranges and grouping 2.5 k, entries and their index words 12 k, the rest at the end).  What bounds it is the chain of phases in a block, a thread or two per window: a quarter of the SM's issue
-// rate, 18% of the shared-memory pipe, 5 MB from DRAM; half of the stalled warps wait at a barrier.
+// rate, a fifth of the shared-memory pipe, 5 MB from DRAM; half of the stalled warps wait at a barrier.
 //
 // Parts: every block reads all lengths and deals gridDim.x parts to the sequences in proportion to their windows (at least one
 // each, and no more than kBlkPart windows expected in one, so that the tables stay at most half full), so no plan kernel and no host

@@ -20,9 +20,9 @@
 // keys' counts and the lists are gathered per block in shared memory, so that a key that makes up a tenth of the corpus costs
 // an atomic per block and not one per occurrence.  Counting every selected window in a second hash table took 212 us of a build from 4 M
 // tokens (LL = 2, LC = 65,536, FC = 8: 167 MB of tables at random, more than the L2 holds), grouping its slots 49 us, ranking 187 us.
-// The whole call with the draft that follows it: 763 us that way, 508 with windows in ranges, 450 with keys in the leader table, read from
+// The whole call with the draft that follows it: 763 us that way, 508 with windows in ranges, 453 with keys in the leader table, read from
 // end to end by the selection, and ranges taken as the leaders are placed (a table of positions with a list of its used slots: the same
-// call from 302 k tokens 218, so 178; 949 k, LL = 3: 256 and 198).  Of the 450: leader counts 73, windows into ranges 105, selection 60,
+// call from 302 k tokens 218, so 178; 949 k, LL = 3: 256 and 198).  Of the 453: leader counts 72, windows into ranges 106, selection 60,
 // ranking some 150 with its kernels side by side.
 // Which occurrence represents a key, and which entry id a leader gets, depends on timing; the table's content (and
 // cb_frozen_dump's output) does not.
